@@ -37,6 +37,7 @@ extern "C" void fdvlm_destroy(fdvlm_t* h) {
   if (h->loop_exec) cudaGraphExecDestroy(h->loop_exec);
   if (h->kv) cudaFree(h->kv);
   if (h->slab) cudaFree(h->slab);
+  if (h->pf_slab) cudaFree(h->pf_slab);
   for (cudaEvent_t ev : h->prof_ev) cudaEventDestroy(ev);
   if (h->info_host) cudaFreeHost(h->info_host);
   if (h->host_stage) cudaFreeHost(h->host_stage);
@@ -96,6 +97,7 @@ extern "C" int fdvlm_create(const fdvlm_config* cfg, const fdvlm_weights* w, voi
   h->loop_exec = nullptr;
   h->q_d = nullptr; h->q_mask = nullptr; h->q_pos_off = nullptr; h->quad_B = 0;
   h->f_rows = nullptr; h->f_mask = nullptr;
+  h->pf_slab = nullptr; h->pf_rows = 0;
   cudaGetDevice(&h->device);
 
   const int R = cfg->max_block, H = cfg->hidden, I = cfg->intermediate, d = cfg->head_dim;
@@ -162,7 +164,28 @@ extern "C" int fdvlm_create(const fdvlm_config* cfg, const fdvlm_weights* w, voi
   };
   size_t slab_bytes = 0;
   for (auto& a : allocs) slab_bytes += (a.bytes + 255) / 256 * 256;
-  e = cudaMalloc((void**)&h->slab, slab_bytes);
+  // Prompt path: as many rows as one forward of it takes (PF_MAX_ROWS: above that its tiles fill the GPU many times over
+  // and more rows only cost memory).  W8A8 prompts run through the decode path's quantising GEMM.
+  size_t pf_bytes = 0;
+  if (h->use_tc && !h->act8 && cfg->max_seq > PF_MIN_ROWS) {
+    const int max_rows = (cfg->max_seq + 127) / 128 * 128;
+    const size_t P = max_rows < PF_MAX_ROWS ? max_rows : PF_MAX_ROWS;
+    h->pf_rows = (int)P;
+    h->pf_part_bytes = (size_t)sm_count() * 256 * 256 * sizeof(float);
+    struct { void** p; size_t bytes; } pf[] = {
+        {(void**)&h->pf_h, P * H * 4},        {(void**)&h->pf_cs, P * d * 4},
+        {(void**)&h->pf_ssq, P * h->nt * 4},  {(void**)&h->pf_a, P * H * 2 * a_planes},
+        {(void**)&h->pf_q, P * NQ * 2},       {(void**)&h->pf_ao, P * NQ * 2 * planes},
+        {(void**)&h->pf_act, P * I * 2 * planes}, {(void**)&h->pf_part, h->pf_part_bytes},
+    };
+    for (auto& a : pf) pf_bytes += (a.bytes + 255) / 256 * 256;
+    e = cudaMalloc((void**)&h->pf_slab, pf_bytes);
+    if (e == cudaSuccess) {
+      char* cur = h->pf_slab;
+      for (auto& a : pf) { *a.p = cur; cur += (a.bytes + 255) / 256 * 256; }
+    }
+  }
+  if (e == cudaSuccess) e = cudaMalloc((void**)&h->slab, slab_bytes);
   if (e == cudaSuccess) e = cudaMalloc((void**)&h->kv, (size_t)cfg->n_layers * 2 * kv_plane(h));
   if (e != cudaSuccess) {
     fail(nullptr, FDVLM_ERR_OOM, "cudaMalloc of the work buffers (%zu bytes) or the KV cache failed: %s", slab_bytes, cudaGetErrorString(e));
@@ -217,7 +240,15 @@ extern "C" int fdvlm_prefill(fdvlm_t* h, const void* embeds, int n_embeds, const
   if ((long long)h->cache_len + total > h->cfg.max_seq)
     return fail(h, FDVLM_ERR_CAPACITY, "prefill: %d + %d rows exceed max_seq %d", h->cache_len, total, h->cfg.max_seq);
   h->launches = 0;
-  const int R = h->cfg.max_block, H = h->cfg.hidden;
+  const int H = h->cfg.hidden;
+  // Above PF_MIN_ROWS rows the prompt path; its forwards are of equal size (in whole 128-row tiles).
+  const bool large = h->pf_rows > 0 && total > PF_MIN_ROWS;
+  int R = h->cfg.max_block;
+  if (large) {
+    const int parts = (total + h->pf_rows - 1) / h->pf_rows;
+    R = ((total + parts - 1) / parts + 127) / 128 * 128;
+  }
+  auto stage = large ? stage_prefill_rows : stage_rows;
   int done = 0;
   while (done < total) {
     const int n = total - done < R ? total - done : R;
@@ -225,15 +256,15 @@ extern "C" int fdvlm_prefill(fdvlm_t* h, const void* embeds, int n_embeds, const
     int rc;
     if (done < n_embeds) {
       ne = n_embeds - done < n ? n_embeds - done : n;
-      rc = stage_rows(h, 0, ne, nullptr, (const char*)embeds + (size_t)done * H * h->act_sz);
+      rc = stage(h, 0, ne, nullptr, (const char*)embeds + (size_t)done * H * h->act_sz);
       if (rc) return rc;
     }
     if (ne < n) {
-      rc = stage_rows(h, ne, n - ne, tokens + (done + ne - n_embeds), nullptr);
+      rc = stage(h, ne, n - ne, tokens + (done + ne - n_embeds), nullptr);
       if (rc) return rc;
     }
     const bool last = (done + n == total);
-    rc = forward_rows(h, n, MODE_CAUSAL, (last && last_logits) ? 1 : 0, 1);
+    rc = large ? forward_prefill(h, n, last && last_logits) : forward_rows(h, n, MODE_CAUSAL, (last && last_logits) ? 1 : 0, 1);
     if (rc) return rc;
     h->cache_len += n;
     done += n;

@@ -97,6 +97,112 @@ int stage_rows(fdvlm_t* h, int row0, int n, const int32_t* tokens, const void* e
   return FDVLM_OK;
 }
 
+int stage_prefill_rows(fdvlm_t* h, int row0, int n, const int32_t* tokens, const void* embeds) {
+  const size_t H = h->cfg.hidden;
+  launch_embed_prep(h->w.embed, tokens, embeds, h->pf_h + row0 * H, (char*)h->pf_a + row0 * H * 2, h->pf_rows * H, h->xfmt,
+                    h->layers[0].g_attn, h->pf_ssq + (size_t)row0 * h->nt, h->nt, n, (int)H, h->cfg.vocab, h->info + 3, h->st);
+  h->launches++;
+  CU(h, cudaGetLastError());
+  return FDVLM_OK;
+}
+
+// ---- prompt path ---------------------------------------------------------------------------------------------------------
+// per layer: [QKV GEMM + norm factor, bias, rotary, K/V rows] [causal attention] [O GEMM + residual, gain, ssq]
+//            [gate/up GEMM + SwiGLU] [down GEMM + residual, gain, ssq]
+// O and down of a short prompt: split-K partial sums + fin_resid (see prefill_splits).
+int forward_prefill(fdvlm_t* h, int n, int want_last_logits) {
+  const fdvlm_config& c = h->cfg;
+  const int H = c.hidden, I = c.intermediate, d = c.head_dim, nt = h->nt;
+  const int NQ = c.n_q_heads * d, NKV = c.n_kv_heads * d;
+  const size_t R = h->pf_rows;
+  const bool fp8 = h->dt == DT_FP8;
+  cudaError_t e = cudaSuccess;
+  auto gemm = [&](int mode, const void* x, size_t ld, int k) {
+    PfGemm g;
+    memset(&g, 0, sizeof(g));
+    g.mode = mode; g.m = n; g.k = k; g.x_rows = (int)R; g.fp8 = fp8; g.n_mats = 1;
+    g.x = x; g.x_lo = fp8 ? nullptr : (const char*)x + R * ld * 2;
+    g.nt = nt; g.inv_h = 1.f / (float)H; g.eps = c.rms_eps; g.status = h->info + 3;
+    return g;
+  };
+  auto run = [&](const PfGemm& g) {
+    prof_begin(h, 0);
+    e = prefill_gemm_launch(g, h->st);
+    prof_end(h);
+    h->launches++;
+    return e == cudaSuccess;
+  };
+  // residual add of x w^T, the next norm's gain and sums of squares
+  auto resid = [&](const void* x, size_t ld, int k, const void* w, const float* scale, const float* gain, int fmt) {
+    PfGemm g = gemm(PF_RESID, x, ld, k);
+    g.w[0] = w; g.n[0] = H;
+    g.splits = prefill_splits(n, H, k, fp8);
+    if (g.splits > 1 && (size_t)g.splits * n * H * sizeof(float) <= h->pf_part_bytes) {
+      g.mode = PF_PARTIAL; g.part = h->pf_part;
+      if (!run(g)) return false;
+      launch_fin_resid(h->pf_part, g.splits, n, H, h->pf_h, gain, h->pf_a, R * H, fmt, h->pf_ssq, nt, scale, h->st);
+      h->launches++;
+      return true;
+    }
+    g.scale[0] = scale; g.h = h->pf_h; g.gain = gain; g.out = h->pf_a; g.out_lo_off = R * H; g.out_fmt = fmt; g.ssq_out = h->pf_ssq;
+    return run(g);
+  };
+  launch_rope_table(h->pf_cs, n, h->cache_len, d, c.rope_theta, h->st);
+  h->launches++;
+  for (int l = 0; l < c.n_layers; ++l) {
+    const fdvlm_layer_weights& lw = h->layers[l];
+    PfGemm g = gemm(PF_QKV, h->pf_a, H, H);
+    g.n_mats = 3;
+    g.w[0] = lw.wq; g.w[1] = lw.wk; g.w[2] = lw.wv; g.n[0] = NQ; g.n[1] = g.n[2] = NKV;
+    g.scale[0] = lw.s_q; g.scale[1] = lw.s_k; g.scale[2] = lw.s_v; g.bias[0] = lw.bq; g.bias[1] = lw.bk; g.bias[2] = lw.bv;
+    g.ssq_in = h->pf_ssq; g.out = h->pf_q; g.kc = kv_ptr(h, l, 0); g.vc = kv_ptr(h, l, 1); g.cs = h->pf_cs;
+    g.pos0 = h->cache_len; g.max_seq = c.max_seq; g.d = d; g.kv_type = h->kv_type;
+    if (!run(g)) return fail(h, FDVLM_ERR_CUDA, "qkv projection launch: %s", cudaGetErrorString(e));
+    AttnArgs at;
+    memset(&at, 0, sizeof(at));
+    at.q = h->pf_q; at.kc = kv_ptr(h, l, 0); at.vc = kv_ptr(h, l, 1); at.out = h->pf_ao; at.n = n; at.cache_len = h->cache_len;
+    at.max_seq = c.max_seq; at.hq = c.n_q_heads; at.hkv = c.n_kv_heads; at.d = d; at.causal = 1; at.kv_type = h->kv_type;
+    at.out_fmt = h->xfmt; at.out_lo_off = R * NQ; at.status = h->info + 3;
+    prof_begin(h, 1);
+    e = launch_prefill_attention(at, h->st);
+    prof_end(h);
+    h->launches++;
+    if (e != cudaSuccess) return fail(h, FDVLM_ERR_CUDA, "attention launch: %s", cudaGetErrorString(e));
+    if (!resid(h->pf_ao, NQ, NQ, lw.wo, lw.s_o, lw.g_mlp, h->xfmt))
+      return fail(h, FDVLM_ERR_CUDA, "o projection launch: %s", cudaGetErrorString(e));
+    g = gemm(PF_SWIGLU, h->pf_a, H, H);
+    g.n_mats = 2;
+    g.w[0] = lw.w_gate; g.w[1] = lw.w_up; g.n[0] = g.n[1] = I; g.scale[0] = lw.s_gate; g.scale[1] = lw.s_up;
+    g.ssq_in = h->pf_ssq; g.out = h->pf_act; g.out_lo_off = R * I; g.out_fmt = h->xfmt;
+    if (!run(g)) return fail(h, FDVLM_ERR_CUDA, "gate/up projection launch: %s", cudaGetErrorString(e));
+    const bool last = l + 1 == c.n_layers;
+    if (!resid(h->pf_act, I, I, lw.w_down, lw.s_down, last ? h->w.g_final : h->layers[l + 1].g_attn, last ? h->head_fmt : h->xfmt))
+      return fail(h, FDVLM_ERR_CUDA, "down projection launch: %s", cudaGetErrorString(e));
+  }
+  if (want_last_logits) {
+    TcOut o;
+    memset(&o, 0, sizeof(o));
+    o.mode = TC_MODE_LOGITS; o.status = h->info + 3; o.y = h->logits; o.ld = c.vocab; o.write_logits = 1;
+    o.ssq_in = h->pf_ssq + (size_t)(n - 1) * nt; o.nt_in = nt; o.hidden = H; o.eps = c.rms_eps; o.stats = h->stats; o.mask_id = c.mask_id;
+    TcGroup lm;
+    memset(&lm, 0, sizeof(lm));
+    lm.m = 1; lm.k = H; lm.n_mats = 1; lm.n[0] = c.vocab;
+    lm.w[0] = c.tie_embeddings ? h->w.embed : h->w.lm_head;
+    lm.x = (const char*)h->pf_a + (size_t)(n - 1) * H * 2;
+    lm.x_lo = h->head_fmt == XF_BF16X2 ? (const char*)lm.x + R * H * 2 : nullptr;
+    lm.fp8 = h->head_fmt == XF_F16;
+    if (!c.tie_embeddings) lm.scale[0] = h->w.s_lm_head;
+    prof_begin(h, 0);
+    e = tc_group_launch(lm, o, h->st);
+    prof_end(h);
+    h->launches++;
+    if (e != cudaSuccess) return fail(h, FDVLM_ERR_CUDA, "lm head launch: %s", cudaGetErrorString(e));
+  }
+  e = cudaGetLastError();
+  if (e != cudaSuccess) return fail(h, FDVLM_ERR_CUDA, "kernel launch: %s", cudaGetErrorString(e));
+  return FDVLM_OK;
+}
+
 // ---- exact CUDA-core path: one kernel per operator ---------------------------------------------------
 static int forward_rows_simt(fdvlm_t* h, int n, int mode, int logits_rows) {
   const fdvlm_config& c = h->cfg;

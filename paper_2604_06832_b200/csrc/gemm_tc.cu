@@ -98,22 +98,6 @@ struct TcSmem {
   static constexpr int TOTAL = ROWSC_OFF + 512 + 1024;  // + alignment slack
 };
 
-// sixteen e4m3 bytes -> sixteen f16 (exact: every e4m3 value, subnormals included, is an f16 value)
-__device__ __forceinline__ void e4m3x16_to_f16(const uint4& in, uint4& lo, uint4& hi) {
-  const uint32_t w[4] = {in.x, in.y, in.z, in.w};
-  uint32_t o[8];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-#pragma unroll
-    for (int hsel = 0; hsel < 2; ++hsel) {
-      const unsigned short two = (unsigned short)(hsel ? (w[i] >> 16) : (w[i] & 0xffffu));
-      asm("cvt.rn.f16x2.e4m3x2 %0, %1;" : "=r"(o[2 * i + hsel]) : "h"(two));
-    }
-  }
-  lo = make_uint4(o[0], o[1], o[2], o[3]);
-  hi = make_uint4(o[4], o[5], o[6], o[7]);
-}
-
 // Widen NP 16-byte pieces (tid, tid + stride, ...) of an 8 KB e4m3 tile (rows of 64 bytes) into the 128-byte-swizzled
 // f16 tile the MMA descriptor expects.
 template <int NP>
@@ -632,7 +616,7 @@ bool make_tmap(CUtensorMap* tm, const void* ptr, int rows, int cols, int box_row
 }
 
 // SM count of the current device (cached per device: one process may drive several GPUs)
-static int sm_count() {
+int sm_count() {
   static int n[MAX_DEVICES] = {};
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= MAX_DEVICES) return 148;

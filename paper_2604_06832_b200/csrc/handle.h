@@ -67,6 +67,13 @@ struct fdvlm {
   unsigned long long* f_mask;   // [64]
   void* ws;        // GEMM split-K / attention split-KV workspace
   size_t ws_bytes;
+  // prompt path (forward_prefill): buffers of pf_rows rows in an allocation of their own, so that the decode path's small
+  // buffers stay close together; pf_rows = 0: prompts run through the decode path in chunks of max_block rows
+  int pf_rows;
+  char* pf_slab;
+  float *pf_h, *pf_cs, *pf_ssq, *pf_part;
+  void *pf_a, *pf_ao, *pf_act, *pf_q;
+  size_t pf_part_bytes;
   int32_t* info_host;  // pinned
   char* host_stage;    // pinned staging for *_host variants
   int nt;          // ceil(H / 128)
@@ -133,11 +140,16 @@ int stage_rows(fdvlm_t* h, int row0, int n, const int32_t* tokens, const void* e
 // logits_rows: 0 none; n = all rows (logits into h->logits when want_logits, and conf / pred always);
 // 1 = last row only, raw logits into h->logits[0 .. V).
 int forward_rows(fdvlm_t* h, int n, int mode, int logits_rows, int want_logits);
+// The causal forward over the n rows staged in pf_h / pf_a (n <= pf_rows); the last row's logits into h->logits.
+int forward_prefill(fdvlm_t* h, int n, int want_last_logits);
+int stage_prefill_rows(fdvlm_t* h, int row0, int n, const int32_t* tokens, const void* embeds);
 int forward_rows_enqueue(fdvlm_t* h, int n, int mode, int logits_rows, int want_logits);
 
 size_t linear_workspace_bytes(int m, int n, int k, int dtype);
 size_t attention_workspace_bytes(int n, int hq, int hkv, int d);
 
+constexpr int PF_MIN_ROWS = 64;      // a prompt of at most this many rows is one forward of the decode path
+constexpr int PF_MAX_ROWS = 4096;    // rows of one forward of the prompt path
 constexpr int FDVLM_MAX_STAMPS = 1024;
 // Bytes at the start of an operator-level workspace that hold the kernels' two status words.
 constexpr size_t OP_HEAD = 256;

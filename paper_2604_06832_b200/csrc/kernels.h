@@ -107,6 +107,31 @@ bool tc_linear_supported(int m, int n, int k, int dtype);
 size_t tc_workspace_bytes(int m, int ld, int tiles, int k);
 cudaError_t tc_group_launch(const TcGroup& g, const TcOut& o, cudaStream_t st);
 
+// SM count of the current device (cached per device: one process may drive several GPUs).
+int sm_count();
+
+// ---- large-M GEMM of the prompt path (prefill_gemm.cu) ---------------------------------------------------------
+//   QKV    : w = q, k, v; out = q rows [m][n0] after bias and rotary (cs), K / V into the cache planes kc, vc at pos0
+//   RESID  : h += x w^T * scale; out = h * gain (XF_*, lo plane out_lo_off on); ssq_out[row][nt] = sums of h^2 per 128 columns
+//   SWIGLU : w = gate, up; out[m][n0] = silu(gate) * up
+//   PARTIAL: part[splits][m][n0] = split-K partial sums, left to fin_resid
+// The folded norm factor comes from ssq_in as in TcOut.  fp8: e4m3 weights and f16 rows; else bf16 weights and hi / lo planes.
+enum { PF_QKV = 0, PF_RESID = 1, PF_SWIGLU = 2, PF_PARTIAL = 3 };
+struct PfGemm {
+  int mode, m, k, x_rows, fp8, n_mats;        // x_rows >= m: rows that x holds
+  const void *x, *x_lo;
+  const void* w[3]; int n[3];
+  const float *scale[3], *bias[3];
+  const float* ssq_in; int nt; float inv_h, eps;
+  void* out; size_t out_lo_off; int out_fmt;
+  void *kc, *vc; const float* cs; int pos0, max_seq, d, kv_type;
+  float* h; const float* gain; float* ssq_out;
+  float* part; int splits;
+  int* status;
+};
+int prefill_splits(int m, int n, int k, bool fp8);
+cudaError_t prefill_gemm_launch(const PfGemm& g, cudaStream_t st);
+
 // Tensor-core path glue.  ssq[row][nt] holds per-128-column partial sums of h^2; xg / lo_off / fmt: a GEMM input
 // stored as XF_* (common.cuh).  q, kc, vc of fin_qkv are KV_BF16 or KV_F16 elements (kv_type).
 void launch_embed_prep(const void* table, const int32_t* tokens, const void* rows, float* h, void* xg, size_t lo_off, int fmt,
@@ -142,6 +167,8 @@ struct AttnArgs {
   float* amax_out;      // nullable (tensor-core kernel): [n][hq] maxima of |out| as stored, per row and head
   KStamp* stamp;        // nullable: two consecutive entries (attention, chunk merge)
 };
+// Prompt path: causal attention of any number of rows, one CTA per (128 rows, query head), no key split (prefill_attn.cu).
+cudaError_t launch_prefill_attention(const AttnArgs& a, cudaStream_t st);
 size_t attention_workspace_bytes(int n, int hq, int hkv, int d);
 bool attention_long_cache(int keys);   // whether the tensor-core kernel takes its long-cache shape for this many keys
 
