@@ -109,7 +109,7 @@ int stage_prefill_rows(fdvlm_t* h, int row0, int n, const int32_t* tokens, const
 // ---- prompt path ---------------------------------------------------------------------------------------------------------
 // per layer: [QKV GEMM + norm factor, bias, rotary, K/V rows] [causal attention] [O GEMM + residual, gain, ssq]
 //            [gate/up GEMM + SwiGLU] [down GEMM + residual, gain, ssq]
-// O and down of a short prompt: split-K partial sums + fin_resid (see prefill_splits).
+// O and down of a short prompt: split-K partial sums + fin_resid_rows (see prefill_splits).
 int forward_prefill(fdvlm_t* h, int n, int want_last_logits) {
   const fdvlm_config& c = h->cfg;
   const int H = c.hidden, I = c.intermediate, d = c.head_dim, nt = h->nt;
@@ -136,11 +136,11 @@ int forward_prefill(fdvlm_t* h, int n, int want_last_logits) {
   auto resid = [&](const void* x, size_t ld, int k, const void* w, const float* scale, const float* gain, int fmt) {
     PfGemm g = gemm(PF_RESID, x, ld, k);
     g.w[0] = w; g.n[0] = H;
-    g.splits = prefill_splits(n, H, k, fp8);
+    g.splits = prefill_splits(n, H, k);
     if (g.splits > 1 && (size_t)g.splits * n * H * sizeof(float) <= h->pf_part_bytes) {
       g.mode = PF_PARTIAL; g.part = h->pf_part;
       if (!run(g)) return false;
-      launch_fin_resid(h->pf_part, g.splits, n, H, h->pf_h, gain, h->pf_a, R * H, fmt, h->pf_ssq, nt, scale, h->st);
+      launch_fin_resid_rows(h->pf_part, g.splits, n, H, h->pf_h, gain, h->pf_a, R * H, fmt, h->pf_ssq, nt, scale, h->st);
       h->launches++;
       return true;
     }

@@ -148,7 +148,7 @@ int forward_rows_enqueue(fdvlm_t* h, int n, int mode, int logits_rows, int want_
 size_t linear_workspace_bytes(int m, int n, int k, int dtype);
 size_t attention_workspace_bytes(int n, int hq, int hkv, int d);
 
-constexpr int PF_MIN_ROWS = 64;      // a prompt of at most this many rows is one forward of the decode path
+constexpr int PF_MIN_ROWS = 128;     // a prompt of at most this many rows is one forward of the decode path
 constexpr int PF_MAX_ROWS = 4096;    // rows of one forward of the prompt path
 constexpr int FDVLM_MAX_STAMPS = 1024;
 // Bytes at the start of an operator-level workspace that hold the kernels' two status words.

@@ -535,6 +535,61 @@ __global__ void __launch_bounds__(128) fin_resid_kernel(const float* __restrict_
     stamp_end(stamp, true);
   }
 }
+// The same for the many rows of a prompt (hidden a multiple of 4, no W8A8): one warp per (row, tile of 128 columns), four
+// columns per lane.  Bound by the bytes it moves; the kernel above, whose CTAs exist to have every load of a few rows in
+// flight at once, took 35 us for 1024 x 2048 with two splits.
+__global__ void __launch_bounds__(256) fin_resid_rows_kernel(const float* __restrict__ part, int S, int m, int hidden,
+                                                             float* __restrict__ h, const float* __restrict__ g, void* __restrict__ xg,
+                                                             size_t lo_off, int fmt, float* __restrict__ ssq, int nt,
+                                                             const float* __restrict__ scale) {
+  pdl_trigger();
+  const int idx_w = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  const int r = idx_w / nt, t = idx_w - r * nt, c = t * 128 + lane * 4;
+  pdl_wait();
+  if (r >= m) return;
+  float ss = 0.f;
+  if (c < hidden) {
+    const size_t idx = (size_t)r * hidden + c, sstride = (size_t)m * hidden;
+    const float4 hv = *reinterpret_cast<const float4*>(h + idx);
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int s0 = 0; s0 < S; s0 += 4) {
+      float4 v[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        v[j] = (s0 + j < S) ? __ldcs(reinterpret_cast<const float4*>(part + idx + (size_t)(s0 + j) * sstride)) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) { a.x += v[j].x; a.y += v[j].y; a.z += v[j].z; a.w += v[j].w; }
+    }
+    float x[4] = {a.x, a.y, a.z, a.w};
+    const float hh[4] = {hv.x, hv.y, hv.z, hv.w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      x[e] = hh[e] + x[e] * (scale ? scale[c + e] : 1.f);
+      ss = fmaf(x[e], x[e], ss);
+    }
+    *reinterpret_cast<float4*>(h + idx) = make_float4(x[0], x[1], x[2], x[3]);
+    unsigned short hi[4], lo[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const float y = x[e] * g[c + e];
+      if (fmt == XF_F16) {
+        hi[e] = f16_bits_sat(y);
+      } else {
+        const bf16 b = __float2bfloat16_rn(y);
+        hi[e] = __bfloat16_as_ushort(b);
+        lo[e] = __bfloat16_as_ushort(__float2bfloat16_rn(y - __bfloat162float(b)));
+      }
+    }
+    *reinterpret_cast<ushort4*>((unsigned short*)xg + idx) = make_ushort4(hi[0], hi[1], hi[2], hi[3]);
+    if (fmt == XF_BF16X2) *reinterpret_cast<ushort4*>((unsigned short*)xg + lo_off + idx) = make_ushort4(lo[0], lo[1], lo[2], lo[3]);
+  }
+  ss = warp_sum(ss);
+  if (lane == 0) ssq[(size_t)r * nt + t] = ss;
+}
+void launch_fin_resid_rows(const float* part, int S, int m, int hidden, float* h, const float* g, void* xg, size_t lo_off, int fmt,
+                           float* ssq, int nt, const float* scale, cudaStream_t st) {
+  launch_pdl(fin_resid_rows_kernel, dim3((m * nt + 7) / 8), dim3(256), 0, st, part, S, m, hidden, h, g, xg, lo_off, fmt, ssq, nt, scale);
+}
 void launch_fin_resid(const float* part, int S, int m, int hidden, float* h, const float* g, void* xg, size_t lo_off, int fmt,
                       float* ssq, int nt, const float* scale, cudaStream_t st, KStamp* stamp, const float* amax_in, int n_amax_in,
                       float* amax_out) {

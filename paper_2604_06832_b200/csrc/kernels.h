@@ -129,7 +129,7 @@ struct PfGemm {
   float* part; int splits;
   int* status;
 };
-int prefill_splits(int m, int n, int k, bool fp8);
+int prefill_splits(int m, int n, int k);
 cudaError_t prefill_gemm_launch(const PfGemm& g, cudaStream_t st);
 
 // Tensor-core path glue.  ssq[row][nt] holds per-128-column partial sums of h^2; xg / lo_off / fmt: a GEMM input
@@ -145,6 +145,8 @@ void launch_fin_qkv(const float* part, int S, int m, const float* cs, const floa
 void launch_fin_resid(const float* part, int S, int m, int hidden, float* h, const float* g, void* xg, size_t lo_off, int fmt,
                       float* ssq, int nt, const float* scale, cudaStream_t st, KStamp* stamp = nullptr,
                       const float* amax_in = nullptr, int n_amax_in = 0, float* amax_out = nullptr);
+void launch_fin_resid_rows(const float* part, int S, int m, int hidden, float* h, const float* g, void* xg, size_t lo_off, int fmt,
+                           float* ssq, int nt, const float* scale, cudaStream_t st);
 void launch_stats_merge(const void* stats, int n_part, int m, float* conf, int32_t* pred, cudaStream_t st, KStamp* stamp = nullptr);
 
 // ---- attention -----------------------------------------------------------------------------------
