@@ -59,7 +59,7 @@ typedef enum {
 /* Storage type of the linear weights.  For FDVLM_F32 everything is fp32.  Otherwise the embedding table and the
  * embedding rows given to fdvlm_prefill are bf16, and the accumulation, residual stream, norms and softmax are
  * fp32; the 16-bit tensors between the operators are internal: GEMM inputs are pairs of bf16 (value = hi + lo, ~16
- * significant bits) for bf16 weights and f16 for fp8 weights (e4m3 widens exactly to f16), q and the KV cache are
+ * significant bits) for bf16 weights and f16 values for fp8 weights, q and the KV cache are
  * of fdvlm_kv_dtype. */
 typedef enum {
   FDVLM_F32 = 0,
@@ -332,7 +332,7 @@ int fdvlm_util_stream_read(const void *device_buf, size_t bytes, void *device_si
  * x: device [m, k], fp32 for F32 else bf16; w: device [n, k] in `dtype` storage; scale: device fp32
  * [n] (fp8) or NULL; bias: device fp32 [n] or NULL; y: device fp32 [m, n].
  * workspace: device scratch of at least fdvlm_op_linear_workspace_bytes(m, n, k, dtype) bytes (never 0): the
- * kernels' status words, split-K partial sums and, for fp8 weights, the f16 copy of x that GEMM multiplies by.
+ * kernels' status words, split-K partial sums and, for fp8 weights, the copy of x that GEMM multiplies by.
  * The call is asynchronous; fdvlm_op_linear_status(workspace, stream) waits for the stream and returns
  * FDVLM_ERR_TIMEOUT if a bounded wait inside the kernels of the LAST call on that workspace gave up (y is then
  * undefined), else FDVLM_OK.  workspace = NULL asks about the built-in scratch of fdvlm_op_linear_static on the

@@ -341,8 +341,12 @@ __device__ __forceinline__ void attn_merge_warp(const float* att_o, const float2
   }
   den = warp_sum(den);
   const float inv = 1.f / den;
+  if (VPL == 4) {
+    store_act4(out, lo_off, out_idx + lane * VPL, make_float4(acc[0] * inv, acc[1] * inv, acc[VPL - 2] * inv, acc[VPL - 1] * inv), fmt);
+  } else {
 #pragma unroll
-  for (int i = 0; i < VPL; ++i) store_act(out, lo_off, out_idx + lane * VPL + i, acc[i] * inv, fmt);
+    for (int i = 0; i < VPL; ++i) store_act(out, lo_off, out_idx + lane * VPL + i, acc[i] * inv, fmt);
+  }
   if (amax_out) {     // W8A8: the O projection quantises this row; its maximum as stored (f16) over this head
     float am = 0.f;
 #pragma unroll

@@ -118,11 +118,13 @@ extern "C" int fdvlm_create(const fdvlm_config* cfg, const fdvlm_weights* w, voi
     delete h;
     return fail(nullptr, FDVLM_ERR_UNSUPPORTED, "an f16 KV cache needs shapes the tensor-core kernels take");
   }
-  // GEMM inputs: bf16 hi + lo planes for bf16 weights, one f16 plane for fp8 weights (CUDA-core path: one plane)
-  h->xfmt = !h->use_tc ? XF_BF16 : (h->dt == DT_FP8 ? XF_F16 : XF_BF16X2);
-  h->head_fmt = (h->xfmt == XF_F16 && cfg->tie_embeddings) ? XF_BF16X2 : h->xfmt;
-  const int planes = h->xfmt == XF_BF16X2 ? 2 : 1;
-  const int a_planes = (h->xfmt == XF_BF16X2 || h->head_fmt == XF_BF16X2) ? 2 : 1;
+  // GEMM inputs: bf16 hi + lo planes for bf16 weights; for fp8 weights e5m2 planes, or one f16 plane where the rows are
+  // quantised (W8A8) or meet widened weights (prompts).  CUDA-core path: one plane.
+  h->xfmt = !h->use_tc ? XF_BF16 : (h->dt == DT_FP8 ? (h->act8 ? XF_F16 : XF_E5M2X3) : XF_BF16X2);
+  h->pf_fmt = h->dt == DT_FP8 ? XF_F16 : XF_BF16X2;
+  h->head_fmt = !h->use_tc ? XF_BF16 : ((h->dt == DT_FP8 && !cfg->tie_embeddings) ? XF_E5M2X3 : XF_BF16X2);
+  const int planes = (h->xfmt == XF_BF16X2 || h->xfmt == XF_E5M2X3) ? 2 : 1;       // of 16 bits (XF_E5M2X3 takes 3 bytes)
+  const int a_planes = h->use_tc ? 2 : 1;
   h->a_lo = (size_t)R * H; h->ao_lo = (size_t)R * NQ; h->act_lo = (size_t)R * I;
   if (h->use_tc) {
     const size_t g3[] = {tc_workspace_bytes(R, NQKV, (NQ + 127) / 128 + 2 * ((NKV + 127) / 128), H),

@@ -16,11 +16,12 @@ void launch_splitk_epilogue(const float* part, int S, int m, int n, const float*
 thread_local char g_create_error[512] = "";
 
 // Stand-alone projection.  The caller's workspace starts with OP_HEAD bytes for the two status words (see
-// TcOut::status; cleared here on the stream), then -- fp8 weights only -- an f16 copy of the bf16 rows (W8A8: followed
-// by one 256-byte-rounded array of per-row maxima), then the split-K partial sums.
+// TcOut::status; cleared here on the stream), then -- fp8 weights only -- the bf16 rows as XF_E5M2X3 planes (W8A8: as f16 rows,
+// followed by one 256-byte-rounded array of per-row maxima), then the split-K partial sums.
 static size_t op_amax_bytes(int m, int dtype) { return dtype == DT_A8 ? (((size_t)m * 4 + 255) / 256) * 256 : 0; }
 static size_t op_x16_bytes(int m, int k, int dtype) {
-  return (dtype == DT_FP8 || dtype == DT_A8) ? (((size_t)m * k * 2 + 255) / 256) * 256 + op_amax_bytes(m, dtype) : 0;
+  if (dtype == DT_FP8) return (((size_t)m * k * 3 + 255) / 256) * 256;
+  return dtype == DT_A8 ? (((size_t)m * k * 2 + 255) / 256) * 256 + op_amax_bytes(m, dtype) : 0;
 }
 size_t linear_workspace_bytes(int m, int n, int k, int dtype) {
   const int wdt = dtype == DT_A8 ? DT_FP8 : dtype;
@@ -55,9 +56,10 @@ int launch_linear(const LinearArgs& a, cudaStream_t st, cudaError_t* err) {
     launch_bf16_rows_to_f16_amax(a.x, b.workspace, a.m, a.k, row_amax, st);
     g.x = b.workspace;
     ++launched;
-  } else if (g.fp8) {     // the fp8 GEMM multiplies f16 by f16
-    launch_bf16_to_f16(a.x, b.workspace, (size_t)a.m * a.k, st);
-    g.x = b.workspace;
+  } else if (g.fp8) {
+    const size_t plane = (size_t)a.m * a.k;
+    launch_bf16_to_e5m2x3(a.x, b.workspace, plane, st);
+    g.x = b.workspace; g.x_lo = (const char*)g.x + plane; g.x_3 = (const char*)g.x + 2 * plane;
     ++launched;
   }
   float* part = (float*)((char*)b.workspace + x16);
@@ -84,7 +86,7 @@ int stage_rows(fdvlm_t* h, int row0, int n, const int32_t* tokens, const void* e
   const int H = h->cfg.hidden;
   const int edt = h->dt == DT_F32 ? DT_F32 : DT_BF16;
   if (h->use_tc) {
-    launch_embed_prep(h->w.embed, tokens, embeds, h->h + (size_t)row0 * H, (char*)h->a + (size_t)row0 * H * 2, h->a_lo, h->xfmt,
+    launch_embed_prep(h->w.embed, tokens, embeds, h->h + (size_t)row0 * H, (char*)h->a + (size_t)row0 * H * xf_bytes(h->xfmt), h->a_lo, h->xfmt,
                       h->layers[0].g_attn, h->ssq + (size_t)row0 * h->nt, h->nt, n, H, h->cfg.vocab, h->info + 3, h->st, nullptr,
                       h->act8 ? h->amax_a + (size_t)row0 * h->nt : nullptr);
   } else if (tokens) {
@@ -97,9 +99,17 @@ int stage_rows(fdvlm_t* h, int row0, int n, const int32_t* tokens, const void* e
   return FDVLM_OK;
 }
 
+// The rows of a group: a GEMM input stored as `fmt`, planes lo_off elements apart, from element row0_elems on.
+static void set_rows(TcGroup* g, const void* x, size_t lo_off, size_t row0_elems, int fmt) {
+  const char* p = (const char*)x + row0_elems * xf_bytes(fmt);
+  g->x = p;
+  g->x_lo = (fmt == XF_BF16X2 || fmt == XF_E5M2X3) ? p + lo_off * xf_bytes(fmt) : nullptr;
+  g->x_3 = fmt == XF_E5M2X3 ? p + 2 * lo_off : nullptr;
+  g->fp8 = fmt == XF_E5M2X3 || fmt == XF_F16;
+}
 int stage_prefill_rows(fdvlm_t* h, int row0, int n, const int32_t* tokens, const void* embeds) {
   const size_t H = h->cfg.hidden;
-  launch_embed_prep(h->w.embed, tokens, embeds, h->pf_h + row0 * H, (char*)h->pf_a + row0 * H * 2, h->pf_rows * H, h->xfmt,
+  launch_embed_prep(h->w.embed, tokens, embeds, h->pf_h + row0 * H, (char*)h->pf_a + row0 * H * 2, h->pf_rows * H, h->pf_fmt,
                     h->layers[0].g_attn, h->pf_ssq + (size_t)row0 * h->nt, h->nt, n, (int)H, h->cfg.vocab, h->info + 3, h->st);
   h->launches++;
   CU(h, cudaGetLastError());
@@ -162,21 +172,21 @@ int forward_prefill(fdvlm_t* h, int n, int want_last_logits) {
     memset(&at, 0, sizeof(at));
     at.q = h->pf_q; at.kc = kv_ptr(h, l, 0); at.vc = kv_ptr(h, l, 1); at.out = h->pf_ao; at.n = n; at.cache_len = h->cache_len;
     at.max_seq = c.max_seq; at.hq = c.n_q_heads; at.hkv = c.n_kv_heads; at.d = d; at.causal = 1; at.kv_type = h->kv_type;
-    at.out_fmt = h->xfmt; at.out_lo_off = R * NQ; at.status = h->info + 3;
+    at.out_fmt = h->pf_fmt; at.out_lo_off = R * NQ; at.status = h->info + 3;
     prof_begin(h, 1);
     e = launch_prefill_attention(at, h->st);
     prof_end(h);
     h->launches++;
     if (e != cudaSuccess) return fail(h, FDVLM_ERR_CUDA, "attention launch: %s", cudaGetErrorString(e));
-    if (!resid(h->pf_ao, NQ, NQ, lw.wo, lw.s_o, lw.g_mlp, h->xfmt))
+    if (!resid(h->pf_ao, NQ, NQ, lw.wo, lw.s_o, lw.g_mlp, h->pf_fmt))
       return fail(h, FDVLM_ERR_CUDA, "o projection launch: %s", cudaGetErrorString(e));
     g = gemm(PF_SWIGLU, h->pf_a, H, H);
     g.n_mats = 2;
     g.w[0] = lw.w_gate; g.w[1] = lw.w_up; g.n[0] = g.n[1] = I; g.scale[0] = lw.s_gate; g.scale[1] = lw.s_up;
-    g.ssq_in = h->pf_ssq; g.out = h->pf_act; g.out_lo_off = R * I; g.out_fmt = h->xfmt;
+    g.ssq_in = h->pf_ssq; g.out = h->pf_act; g.out_lo_off = R * I; g.out_fmt = h->pf_fmt;
     if (!run(g)) return fail(h, FDVLM_ERR_CUDA, "gate/up projection launch: %s", cudaGetErrorString(e));
     const bool last = l + 1 == c.n_layers;
-    if (!resid(h->pf_act, I, I, lw.w_down, lw.s_down, last ? h->w.g_final : h->layers[l + 1].g_attn, last ? h->head_fmt : h->xfmt))
+    if (!resid(h->pf_act, I, I, lw.w_down, lw.s_down, last ? h->w.g_final : h->layers[l + 1].g_attn, last ? h->head_fmt : h->pf_fmt))
       return fail(h, FDVLM_ERR_CUDA, "down projection launch: %s", cudaGetErrorString(e));
   }
   if (want_last_logits) {
@@ -188,9 +198,7 @@ int forward_prefill(fdvlm_t* h, int n, int want_last_logits) {
     memset(&lm, 0, sizeof(lm));
     lm.m = 1; lm.k = H; lm.n_mats = 1; lm.n[0] = c.vocab;
     lm.w[0] = c.tie_embeddings ? h->w.embed : h->w.lm_head;
-    lm.x = (const char*)h->pf_a + (size_t)(n - 1) * H * 2;
-    lm.x_lo = h->head_fmt == XF_BF16X2 ? (const char*)lm.x + R * H * 2 : nullptr;
-    lm.fp8 = h->head_fmt == XF_F16;
+    set_rows(&lm, h->pf_a, R * H, (size_t)(n - 1) * H, h->head_fmt);
     if (!c.tie_embeddings) lm.scale[0] = h->w.s_lm_head;
     prof_begin(h, 0);
     e = tc_group_launch(lm, o, h->st);
@@ -293,17 +301,16 @@ static int forward_rows_tc(fdvlm_t* h, int n, int mode, int logits_rows, int wan
     h->stamp_kind.push_back(kind);
     return h->stamps + h->stamp_used++;
   };
-  const bool fp8 = (h->dt == DT_FP8);
   const bool a8 = h->act8 != 0;                      // W8A8: the four layer projections quantise their input rows
   // a GEMM input buffer: hi (or only) plane, and its lo plane when the format has one
   auto group = [&](const void* x, size_t lo_off, size_t row0_elems, int m, int k, int nm, const void* w0, int n0, const void* w1, int n1,
                    const void* w2, int n2) {
     TcGroup g;
     memset(&g, 0, sizeof(g));
-    g.x = (const char*)x + row0_elems * 2; g.m = m; g.k = k; g.n_mats = nm;
-    g.x_lo = (h->xfmt == XF_BF16X2) ? (const char*)x + (lo_off + row0_elems) * 2 : nullptr;
+    set_rows(&g, x, lo_off, row0_elems, h->xfmt);
+    g.m = m; g.k = k; g.n_mats = nm;
     g.w[0] = w0; g.n[0] = n0; g.w[1] = w1; g.n[1] = n1; g.w[2] = w2; g.n[2] = n2;
-    g.fp8 = fp8; g.a8 = a8;
+    g.a8 = a8;
     return g;
   };
   auto out = [&](int tc_mode, int kind) {
@@ -386,9 +393,8 @@ static int forward_rows_tc(fdvlm_t* h, int n, int mode, int logits_rows, int wan
     o.ssq_in = h->ssq + (size_t)first * nt; o.nt_in = nt; o.hidden = H; o.eps = c.rms_eps;
     o.stats = h->stats; o.mask_id = c.mask_id;
     TcGroup lm = group(h->a, h->a_lo, (size_t)first * H, m, H, 1, table, c.vocab, nullptr, 0, nullptr, 0);
-    lm.fp8 = (h->head_fmt == XF_F16);
+    set_rows(&lm, h->a, h->a_lo, (size_t)first * H, h->head_fmt);
     lm.a8 = 0;                                       // the LM head keeps 16-bit input rows
-    lm.x_lo = (h->head_fmt == XF_BF16X2) ? (const char*)h->a + (h->a_lo + (size_t)first * H) * 2 : nullptr;
     if (!c.tie_embeddings) lm.scale[0] = h->w.s_lm_head;
     if (!gemm(lm, o))
       return fail(h, FDVLM_ERR_CUDA, "lm head launch: %s", cudaGetErrorString(e));

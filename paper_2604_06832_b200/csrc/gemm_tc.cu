@@ -10,10 +10,11 @@
 // work items (tile, K-split).  bf16 weights: the activations arrive as two bf16 planes, hi = bf16(v) and
 // lo = bf16(v - hi); both land side by side in the stage and form ONE MMA operand of twice the rows, so every streamed
 // weight tile is read from shared memory once and multiplied by both; the epilogue adds the two halves of the
-// accumulator.  The activation side of the product thus carries ~16 significant bits at no extra HBM traffic.  FP8-E4M3 weights take the
-// same road with half the bytes: the byte tile lands in the stage, four converter warps widen it exactly to f16
-// (one cvt per pair) into a swizzled buffer of its own, and the MMA (f16 x f16, activations stored as f16) reads
-// that buffer; the per-channel scales are applied by the epilogues.
+// accumulator.  The activation side of the product thus carries ~16 significant bits at no extra HBM traffic.
+// FP8-E4M3 weights: the byte tile is the MMA operand as it lands.  The rows are f16 values, stored as three planes of
+// e5m2 bytes whose weighted sum they are (XF_E5M2X3), again one MMA operand (of three times the rows, kind::f8f6f4, fp32
+// accumulation); the epilogue adds the three parts of the accumulator and applies the per-channel scales.  (Widening the
+// bytes to f16 in converter warps made the converters the bottleneck: 7B gate/up 34.5 us a layer.)
 // Every mbarrier wait is bounded: on a timeout the CTA records an
 // error code in a status word, drains its own bulk copies, frees its tensor memory and returns.
 #include <cuda.h>
@@ -28,16 +29,17 @@
 namespace fdk {
 
 constexpr int TC_THREADS = 192;       // warp 0 TMA producer, warp 1 MMA issuer, warps 2..5 epilogue
-constexpr int TC_THREADS_FP8 = 320;   // + warps 6..9: e4m3 -> bf16 converters
+constexpr int TC_THREADS_A8 = 320;    // + warps 6..9: quantise the rows (W8A8)
 constexpr int TC_A_BYTES = TC_BM * TC_BK * 2;   // a bf16 weight tile
-constexpr int TC_NCONV = 2;           // converted-tile buffers (fp8 only)
+constexpr int TC_NCONV = 2;           // quantised-tile buffers (W8A8 only)
 
 enum { TC_ERR_PRODUCER = ST_PRODUCER, TC_ERR_MMA = ST_MMA, TC_ERR_EPILOGUE = ST_EPILOGUE };
 
 struct TcParams {
   CUtensorMap tm_w[3];  // weight matrices, box {64 k, 64 rows}
   CUtensorMap tm_x;     // activations (hi plane, or the only one), box {64 k, m_pad rows}
-  CUtensorMap tm_xl;    // lo plane of the activations (has_lo)
+  CUtensorMap tm_xl;    // lo plane of the activations (has_lo); fp8: second plane
+  CUtensorMap tm_x3;    // fp8: third plane
   int has_lo;
   int n_out[3];         // rows (output features) of each matrix
   int tile_begin[4];    // first tile of each matrix; [n_mats] = total tiles
@@ -73,7 +75,7 @@ struct TcParams {
 
 // Operand kinds of the kernel:
 //   TC_KIND_BF16: bf16 weights x bf16 hi/lo activation planes
-//   TC_KIND_FP8 : e4m3 weights widened to f16 by converter warps x f16 activations
+//   TC_KIND_FP8 : e4m3 weights x three e5m2 planes of the activations; a k-block is 128 elements
 //   TC_KIND_A8  : e4m3 weights x activations quantised to e4m3 per row inside the kernel (W8A8, Sec. 3.4 "System
 //                 integration"); a k-block is 128 elements, the byte tile of the weights is the MMA operand as it lands
 enum { TC_KIND_BF16 = 0, TC_KIND_FP8 = 1, TC_KIND_A8 = 2 };
@@ -81,14 +83,14 @@ enum { TC_KIND_BF16 = 0, TC_KIND_FP8 = 1, TC_KIND_A8 = 2 };
 template <int M_PAD, int KIND>
 struct TcSmem {
   static constexpr bool FP8 = KIND == TC_KIND_FP8, A8 = KIND == TC_KIND_A8;
-  static constexpr int STAGES = FP8 ? 6 : (M_PAD <= 32 ? 4 : 3);       // two CTAs per SM must fit (A8, M_PAD > 32: one)
-  static constexpr int KB_ELEMS = A8 ? 2 * TC_BK : TC_BK;              // k per stage
-  static constexpr int W_BYTES = FP8 ? TC_BM * TC_BK : TC_A_BYTES;     // weight tile as it is streamed
-  static constexpr int B_BYTES = M_PAD * TC_BK * 2;                    // one activation plane (A8: one 64-k half, f16)
-  static constexpr int X_PLANES = FP8 ? 1 : 2;                         // f16; bf16 hi + lo; A8: two 64-k halves
+  static constexpr int STAGES = FP8 ? (M_PAD <= 16 ? 4 : (M_PAD <= 48 ? 3 : 2)) : (M_PAD <= 32 ? 4 : 3);   // two CTAs per SM must fit (A8, M_PAD > 32: one)
+  static constexpr int KB_ELEMS = (A8 || FP8) ? 2 * TC_BK : TC_BK;     // k per stage
+  static constexpr int W_BYTES = TC_A_BYTES;                           // weight tile
+  static constexpr int B_BYTES = M_PAD * 128;                          // one activation plane (A8: one 64-k half, f16)
+  static constexpr int X_PLANES = FP8 ? 3 : 2;                         // e5m2 planes; bf16 hi + lo; A8: two 64-k halves
   static constexpr int STAGE_BYTES = W_BYTES + X_PLANES * B_BYTES;
-  static constexpr int CONV_OFF = STAGES * STAGE_BYTES;                // tiles made by the converters
-  static constexpr int CONV_BYTES = FP8 ? TC_A_BYTES : (A8 ? M_PAD * 128 : 0);   // f16 weight tile / e4m3 activation tile
+  static constexpr int CONV_OFF = STAGES * STAGE_BYTES;                // tiles made by the quantising warps
+  static constexpr int CONV_BYTES = A8 ? M_PAD * 128 : 0;              // e4m3 activation tile
   static constexpr int EX_OFF = CONV_OFF + TC_NCONV * CONV_BYTES;      // SwiGLU epilogue: gate/up exchange
   static constexpr int EX_ROWS = KIND != TC_KIND_BF16 ? 16 : 32;       // rows that pass through it per round
   static constexpr int EX_ROUNDS = (M_PAD + EX_ROWS - 1) / EX_ROWS;
@@ -97,22 +99,6 @@ struct TcSmem {
   static constexpr int ROWSC_OFF = BAR_OFF + 256;                      // A8: the rows' quantisation scales and their reciprocals
   static constexpr int TOTAL = ROWSC_OFF + 512 + 1024;  // + alignment slack
 };
-
-// Widen NP 16-byte pieces (tid, tid + stride, ...) of an 8 KB e4m3 tile (rows of 64 bytes) into the 128-byte-swizzled
-// f16 tile the MMA descriptor expects.
-template <int NP>
-__device__ __forceinline__ void convert_pieces(const uint8_t* src, uint32_t dst, int tid, int stride) {
-#pragma unroll
-  for (int i = 0; i < NP; ++i) {
-    const int piece = tid + stride * i, r = piece >> 2, c = piece & 3;     // row, 16-byte piece of the row
-    const uint4 in = *reinterpret_cast<const uint4*>(src + piece * 16);
-    uint4 lo, hi;
-    e4m3x16_to_f16(in, lo, hi);
-    const uint32_t row = dst + r * 128;
-    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(row + (((2 * c) ^ (r & 7)) << 4)), "r"(lo.x), "r"(lo.y), "r"(lo.z), "r"(lo.w) : "memory");
-    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(row + (((2 * c + 1) ^ (r & 7)) << 4)), "r"(hi.x), "r"(hi.y), "r"(hi.z), "r"(hi.w) : "memory");
-  }
-}
 
 // Quantise NP 16-byte pieces (tid, tid + stride, ...) of the activation tile of one stage -- two 128-byte-swizzled f16
 // halves of 64 k each -- into the 128-byte-swizzled e4m3 tile [M_PAD rows][128 k] the MMA reads: code = e4m3(x / scale
@@ -152,12 +138,12 @@ __device__ __forceinline__ void quantize_pieces(const uint8_t* x_tile, uint32_t 
 }
 
 template <int M_PAD, int KIND>
-__global__ void __launch_bounds__(KIND != TC_KIND_BF16 ? TC_THREADS_FP8 : TC_THREADS, 1) gemm_tc_kernel(const __grid_constant__ TcParams p) {
+__global__ void __launch_bounds__(KIND == TC_KIND_A8 ? TC_THREADS_A8 : TC_THREADS, 1) gemm_tc_kernel(const __grid_constant__ TcParams p) {
   extern __shared__ uint8_t smem_raw[];
   using L = TcSmem<M_PAD, KIND>;
   constexpr bool A8 = KIND == TC_KIND_A8;
-  constexpr bool FP8 = KIND != TC_KIND_BF16;       // a converter stage sits between the ring and the MMA
-  constexpr bool WIDEN = KIND == TC_KIND_FP8;      // ... which widens the weight tile (A8: quantises the activation tile)
+  constexpr bool W8 = KIND != TC_KIND_BF16;        // weight bytes: a k-block is 128 elements
+  constexpr bool X3 = KIND == TC_KIND_FP8;
   constexpr int TC_STAGES = L::STAGES;
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
@@ -178,18 +164,16 @@ __global__ void __launch_bounds__(KIND != TC_KIND_BF16 ? TC_THREADS_FP8 : TC_THR
   volatile float2* row_scale = reinterpret_cast<volatile float2*>(sm + L::ROWSC_OFF);   // A8 only: (scale, RN(1 / scale))
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // two accumulator buffers; bf16 weights: each holds the hi-plane product in columns [0, M_PAD) and the lo-plane
-  // product in [M_PAD, 2 M_PAD)
-  constexpr int ACC_COLS = FP8 ? M_PAD : 2 * M_PAD;
-  constexpr int TMEM_COLS = (2 * ACC_COLS <= 32) ? 32 : ((2 * ACC_COLS <= 64) ? 64 : ((2 * ACC_COLS <= 128) ? 128 : 256));
+  // two accumulator buffers; each holds the products of plane i in columns [i M_PAD, (i + 1) M_PAD)
+  constexpr int ACC_COLS = A8 ? M_PAD : L::X_PLANES * M_PAD;
+  // (one buffer where two would leave no tensor memory for a second CTA on the SM)
+  constexpr int NACC = 2 * ACC_COLS <= 256 ? 2 : 1;
+  constexpr int TMEM_COLS = (NACC * ACC_COLS <= 32) ? 32 : ((NACC * ACC_COLS <= 64) ? 64 : ((NACC * ACC_COLS <= 128) ? 128 : 256));
 
-  // fp8 launches in which no CTA has a second work item: the epilogue warps, idle until the accumulator is complete,
-  // widen half of every weight tile beside the four converter warps
-  const bool helpers = WIDEN && p.tile_begin[p.n_mats] * p.splits <= (int)gridDim.x;
   if (threadIdx.x == 0) {
     for (int s = 0; s < TC_STAGES; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
     for (int a = 0; a < 2; ++a) { mbar_init(tfull_bar(a), 1); mbar_init(tempty_bar(a), 4); }
-    for (int c = 0; c < TC_NCONV; ++c) { mbar_init(cfull_bar(c), helpers ? 8 : 4); mbar_init(cempty_bar(c), 1); }
+    for (int c = 0; c < TC_NCONV; ++c) { mbar_init(cfull_bar(c), 4); mbar_init(cempty_bar(c), 1); }
     for (int pr = 0; pr < 2; ++pr) { mbar_init(exw_bar(pr), 2); mbar_init(exr_bar(pr), 2); }
     stamp_start(p.stamp);
     *abort_flag = 0;
@@ -212,7 +196,7 @@ __global__ void __launch_bounds__(KIND != TC_KIND_BF16 ? TC_THREADS_FP8 : TC_THR
   const int n_items = total_tiles * p.splits;
 
   const int kbps = p.kb_per_split, kblocks = p.kblocks;
-  auto convert_all = [&](int cvt_tid) -> bool {
+  auto quantize_all = [&](int cvt_tid) -> bool {
     int stage = 0, cbuf = 0;
     uint32_t phase = 0, cphase = 0;
     for (int it = blockIdx.x; it < n_items; it += gridDim.x) {
@@ -223,9 +207,7 @@ __global__ void __launch_bounds__(KIND != TC_KIND_BF16 ? TC_THREADS_FP8 : TC_THR
         if (!mbar_wait(full_bar(stage), phase, abort_flag) || !mbar_wait(cempty_bar(cbuf), cphase ^ 1u, abort_flag)) return false;
         const uint8_t* src = sm + stage * L::STAGE_BYTES;
         const uint32_t dst = base + L::CONV_OFF + cbuf * L::CONV_BYTES;
-        if (A8) quantize_pieces<M_PAD, (M_PAD * 8 + 127) / 128>(src + L::W_BYTES, dst, row_scale, cvt_tid, 128);
-        else if (helpers) convert_pieces<2>(src, dst, cvt_tid, 256);
-        else convert_pieces<4>(src, dst, cvt_tid, 128);
+        quantize_pieces<M_PAD, (M_PAD * 8 + 127) / 128>(src + L::W_BYTES, dst, row_scale, cvt_tid, 128);
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic writes -> the MMA's async-proxy reads
         __syncwarp();
         if (lane == 0) mbar_arrive(cfull_bar(cbuf));
@@ -252,12 +234,13 @@ __global__ void __launch_bounds__(KIND != TC_KIND_BF16 ? TC_THREADS_FP8 : TC_THR
       bool ok = !poisoned;
       bool waited = false;
       int n_pend = 0, pend_stage[TC_STAGES], pend_kb[TC_STAGES];
-      const uint32_t stage_tx = L::W_BYTES + ((A8 || p.has_lo) ? 2 : 1) * L::B_BYTES;
+      const uint32_t stage_tx = L::W_BYTES + (X3 ? 3 : ((A8 || p.has_lo) ? 2 : 1)) * L::B_BYTES;
       auto load_x = [&](int st_, int kb_) {
         const uint32_t dst = base + st_ * L::STAGE_BYTES + L::W_BYTES;
         tma_load_2d(dst, &p.tm_x, full_bar(st_), kb_ * L::KB_ELEMS, 0, pol_x);
         if (A8) tma_load_2d(dst + L::B_BYTES, &p.tm_x, full_bar(st_), kb_ * L::KB_ELEMS + TC_BK, 0, pol_x);   // second 64 k
-        if (!FP8 && p.has_lo) tma_load_2d(dst + L::B_BYTES, &p.tm_xl, full_bar(st_), kb_ * TC_BK, 0, pol_x);
+        if (!A8 && (X3 || p.has_lo)) tma_load_2d(dst + L::B_BYTES, &p.tm_xl, full_bar(st_), kb_ * L::KB_ELEMS, 0, pol_x);
+        if (X3) tma_load_2d(dst + 2 * L::B_BYTES, &p.tm_x3, full_bar(st_), kb_ * L::KB_ELEMS, 0, pol_x);
       };
       for (int it = blockIdx.x; it < n_items && ok; it += gridDim.x) {
         const int tile = it % total_tiles, split = it / total_tiles;
@@ -322,33 +305,31 @@ __global__ void __launch_bounds__(KIND != TC_KIND_BF16 ? TC_THREADS_FP8 : TC_THR
   } else if (warp == 1) {
     // ------------------------------------------------ MMA issuer --------------------------------------------------
     if (lane == 0) {
-      const bool two_planes = !FP8 && p.has_lo;
-      const uint32_t idesc = A8 ? umma_idesc_e4m3(M_PAD) : (FP8 ? umma_idesc_f16(M_PAD) : umma_idesc_bf16(two_planes ? 2 * M_PAD : M_PAD));
+      const uint32_t idesc = A8 ? umma_idesc_e4m3(M_PAD) : (X3 ? umma_idesc_e4m3_e5m2(3 * M_PAD) : umma_idesc_bf16(p.has_lo ? 2 * M_PAD : M_PAD));
       int stage = 0, cbuf = 0;
       uint32_t phase = 0, cphase = 0;
       int local = 0;
       bool ok = true;
       for (int it = blockIdx.x; it < n_items && ok; it += gridDim.x, ++local) {
         const int split = it / total_tiles;
-        const int acc = local & 1;
-        const uint32_t acc_phase = (uint32_t)(local >> 1) & 1u;
+        const int acc = local % NACC;
+        const uint32_t acc_phase = (uint32_t)(local / NACC) & 1u;
         if (!mbar_wait(tempty_bar(acc), acc_phase ^ 1u, abort_flag)) { ok = false; break; }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const uint32_t d_tmem = tmem_base + (uint32_t)(acc * ACC_COLS);
         const int kb0 = split * p.kb_per_split;
         const int kb1 = min(p.kblocks, kb0 + p.kb_per_split);
         for (int kb = kb0; kb < kb1; ++kb) {
-          // fp8: the converters have waited for the stage and left their tile in buffer cbuf (the widened weights; A8:
-          // the quantised activations, the weight bytes being read from the stage itself, whose barrier this thread
-          // then observes too)
-          if (!mbar_wait(FP8 ? cfull_bar(cbuf) : full_bar(stage), FP8 ? cphase : phase, abort_flag)) { ok = false; break; }
+          // A8: the quantising warps have waited for the stage and left the activations in buffer cbuf; the weight bytes
+          // are read from the stage itself, whose barrier this thread then observes too
+          if (!mbar_wait(A8 ? cfull_bar(cbuf) : full_bar(stage), A8 ? cphase : phase, abort_flag)) { ok = false; break; }
           if (A8 && !mbar_wait(full_bar(stage), phase, abort_flag)) { ok = false; break; }
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           const uint32_t a_addr = base + stage * L::STAGE_BYTES;
           const uint32_t c_addr = base + L::CONV_OFF + cbuf * L::CONV_BYTES;
-          const uint64_t adesc = umma_desc_sw128(WIDEN ? c_addr : a_addr);
+          const uint64_t adesc = umma_desc_sw128(a_addr);
           const uint64_t bdesc = umma_desc_sw128(A8 ? c_addr : a_addr + L::W_BYTES);
-          if (A8) {
+          if (W8) {
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk)      // 32 bytes of k per instruction
               umma_f8(d_tmem, adesc + 2u * kk, bdesc + 2u * kk, idesc, (kb > kb0 || kk > 0) ? 1u : 0u);
@@ -358,7 +339,7 @@ __global__ void __launch_bounds__(KIND != TC_KIND_BF16 ? TC_THREADS_FP8 : TC_THR
               umma_bf16(d_tmem, adesc + 2u * kk, bdesc + 2u * kk, idesc, (kb > kb0 || kk > 0) ? 1u : 0u);
           }
           umma_commit(empty_bar(stage));
-          if (FP8) {
+          if (A8) {
             umma_commit(cempty_bar(cbuf));
             if (++cbuf == TC_NCONV) { cbuf = 0; cphase ^= 1u; }
           }
@@ -368,12 +349,11 @@ __global__ void __launch_bounds__(KIND != TC_KIND_BF16 ? TC_THREADS_FP8 : TC_THR
       }
       if (!ok) atomicCAS(p.status, 0, TC_ERR_MMA);
     }
-  } else if (FP8 && warp >= 6) {
-    // ------------------------------------------------ converters -----------------------------------------------------
-    // TC_KIND_FP8: 128 threads (256 with the epilogue warps helping): thread t widens the 16-byte pieces t, t + 128
-    // (256), ... of each 8 KB byte tile.  TC_KIND_A8: the same threads quantise the activation tile; first they form
-    // every row's scale = max of the producer's partial maxima / 448 (two threads per row; 1 for an all-zero row).
-    if (A8) {
+  } else if (A8 && warp >= 6) {
+    // ------------------------------------------------ quantising warps (W8A8) ---------------------------------------
+    // First every row's scale = max of the producer's partial maxima / 448 (two threads per row; 1 for an all-zero row),
+    // then the activation tile of each stage, thread t taking the 16-byte pieces t, t + 128, ...
+    {
       const int t = (int)threadIdx.x - 192, r = t >> 1;
       pdl_wait();                      // the partial maxima are the predecessor's
       float mx = 0.f;
@@ -396,13 +376,12 @@ __global__ void __launch_bounds__(KIND != TC_KIND_BF16 ? TC_THREADS_FP8 : TC_THR
       }
       asm volatile("bar.sync 2, 128;" ::: "memory");
     }
-    if (!convert_all(threadIdx.x - 192) && threadIdx.x == 192) atomicCAS(p.status, 0, TC_ERR_MMA);
+    if (!quantize_all(threadIdx.x - 192) && threadIdx.x == 192) atomicCAS(p.status, 0, TC_ERR_MMA);
   } else {
     // ------------------------------------------------ epilogue warps ----------------------------------------------
     const int q = warp & 3;  // TMEM lane quarter this warp may read
     int local = 0;
     bool ok = true;
-    if (helpers) ok = convert_all(128 + (int)threadIdx.x - 64);
     pdl_wait();   // the epilogue reads the predecessor's row statistics and overwrites buffers it may still be reading
     // folded RMSNorm: lane l keeps the factor of rows l and l + 32; broadcast by shuffle where needed
     float rs0 = 1.f, rs1 = 1.f;
@@ -420,8 +399,8 @@ __global__ void __launch_bounds__(KIND != TC_KIND_BF16 ? TC_THREADS_FP8 : TC_THR
     }
     for (int it = blockIdx.x; it < n_items && ok; it += gridDim.x, ++local) {
       const int tile = it % total_tiles, split = it / total_tiles;
-      const int acc = local & 1;
-      const uint32_t acc_phase = (uint32_t)(local >> 1) & 1u;
+      const int acc = local % NACC;
+      const uint32_t acc_phase = (uint32_t)(local / NACC) & 1u;
       if (!mbar_wait(tfull_bar(acc), acc_phase, abort_flag)) { ok = false; break; }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       if (A8 && local == 0) {
@@ -434,7 +413,17 @@ __global__ void __launch_bounds__(KIND != TC_KIND_BF16 ? TC_THREADS_FP8 : TC_THR
       const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * ACC_COLS);
 #pragma unroll
       for (int c = 0; c < M_PAD; c += 16) tmem_ld16(taddr + c, v + c);
-      if (!FP8 && p.has_lo) {      // the low-order plane's product sits M_PAD columns further on
+      if (X3) {                    // x = p0 + p1 / 4 + p2 / 128
+#pragma unroll
+        for (int c = 0; c < M_PAD; c += 16) {
+          float b1[16], b2[16];
+          tmem_ld16(taddr + M_PAD + c, b1);
+          tmem_ld16(taddr + 2 * M_PAD + c, b2);
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+          for (int i = 0; i < 16; ++i) v[c + i] += fmaf(b2[i], 0.0078125f, b1[i] * 0.25f);
+        }
+      } else if (!A8 && p.has_lo) {      // the low-order plane's product sits M_PAD columns further on
 #pragma unroll
         for (int c = 0; c < M_PAD; c += 16) {
           float lo[16];
@@ -588,7 +577,7 @@ static EncodeTiledFn encode_fn() {
 
 // 2-D row-major [rows, cols] tensor, box {64 columns, box_rows}, zero OOB fill.  16-bit elements (TM_BF16, TM_F16):
 // 128-byte swizzle (rows of the box are 128 bytes); e4m3 bytes: TM_E4M3 no swizzle (rows of 64 bytes, widened by the
-// converter warps), TM_E4M3_128 a box of 128 columns with the 128-byte swizzle (the tile is an MMA operand as it lands).
+// converter warps of the prompt path), TM_E4M3_128 a box of 128 columns with the 128-byte swizzle (the tile is an MMA operand as it lands).
 bool make_tmap(CUtensorMap* tm, const void* ptr, int rows, int cols, int box_rows, int kind) {
   typedef std::tuple<const void*, int, int, int, int> Key;
   static std::map<Key, CUtensorMap> cache;
@@ -651,9 +640,10 @@ bool tc_linear_supported(int m, int n, int k, int dtype) {
 }
 
 size_t tc_workspace_bytes(int m, int ld, int tiles, int k) {
-  int s, kbps;
+  int s, s8, kbps;       // (k-blocks of 64 elements, of 128 with fp8 weights)
   tc_plan(tiles, ceil_div(k, TC_BK), &s, &kbps);
-  return (size_t)s * m * ld * sizeof(float);
+  tc_plan(tiles, ceil_div(k, 2 * TC_BK), &s8, &kbps);
+  return (size_t)(s > s8 ? s : s8) * m * ld * sizeof(float);
 }
 
 template <int M_PAD, int KIND>
@@ -661,7 +651,7 @@ static cudaError_t tc_launch_t(const TcParams& p, int grid, cudaStream_t st) {
   static bool attr_set[MAX_DEVICES] = {};
   cudaError_t e = ensure_dynamic_smem(gemm_tc_kernel<M_PAD, KIND>, TcSmem<M_PAD, KIND>::TOTAL, attr_set);
   if (e != cudaSuccess) return e;
-  return launch_pdl(gemm_tc_kernel<M_PAD, KIND>, dim3(grid), dim3(KIND != TC_KIND_BF16 ? TC_THREADS_FP8 : TC_THREADS),
+  return launch_pdl(gemm_tc_kernel<M_PAD, KIND>, dim3(grid), dim3(KIND == TC_KIND_A8 ? TC_THREADS_A8 : TC_THREADS),
                     (size_t)TcSmem<M_PAD, KIND>::TOTAL, st, p);
 }
 
@@ -687,16 +677,18 @@ cudaError_t tc_group_launch(const TcGroup& g, const TcOut& o, cudaStream_t st) {
   memset(&p, 0, sizeof(p));
   const int mode = o.mode;
   const int mp = pad_m(g.m);
-  const int xkind = g.fp8 ? TM_F16 : TM_BF16;     // fp8 weights are widened to f16 and meet f16 activations
-  const bool a8 = g.fp8 && g.a8;                  // ... unless the kernel quantises the activations to e4m3 itself
+  const bool a8 = g.fp8 && g.a8;                  // f16 rows that the kernel quantises to e4m3 itself
+  const bool x3 = g.fp8 && !a8;                   // rows as e5m2 planes
+  const int xkind = a8 ? TM_F16 : (x3 ? TM_E4M3_128 : TM_BF16);     // (bytes are bytes: e5m2 planes take the same map)
   if (a8 && (mode == TC_MODE_DIRECT || mode == TC_MODE_LOGITS)) return cudaErrorInvalidValue;
   if (a8 && (!o.amax_in || o.n_amax_in < 1)) return cudaErrorInvalidValue;
   if (!make_tmap(&p.tm_x, g.x, g.m, g.k, mp, xkind)) return cudaErrorInvalidValue;
   p.has_lo = (!g.fp8 && g.x_lo) ? 1 : 0;
-  if (p.has_lo && !make_tmap(&p.tm_xl, g.x_lo, g.m, g.k, mp, xkind)) return cudaErrorInvalidValue;
+  if ((x3 || p.has_lo) && !make_tmap(&p.tm_xl, g.x_lo, g.m, g.k, mp, xkind)) return cudaErrorInvalidValue;
+  if (x3 && !make_tmap(&p.tm_x3, g.x_3, g.m, g.k, mp, xkind)) return cudaErrorInvalidValue;
   int tiles = 0, col = 0;
   for (int i = 0; i < g.n_mats; ++i) {
-    if (!make_tmap(&p.tm_w[i], g.w[i], g.n[i], g.k, 64, a8 ? TM_E4M3_128 : (g.fp8 ? TM_E4M3 : TM_BF16))) return cudaErrorInvalidValue;
+    if (!make_tmap(&p.tm_w[i], g.w[i], g.n[i], g.k, 64, g.fp8 ? TM_E4M3_128 : TM_BF16)) return cudaErrorInvalidValue;
     p.n_out[i] = g.n[i];
     p.tile_begin[i] = tiles;
     p.out_col[i] = col;
@@ -706,7 +698,7 @@ cudaError_t tc_group_launch(const TcGroup& g, const TcOut& o, cudaStream_t st) {
     col += g.n[i];
   }
   p.n_mats = g.n_mats;
-  p.kblocks = ceil_div(g.k, a8 ? 2 * TC_BK : TC_BK);
+  p.kblocks = ceil_div(g.k, g.fp8 ? 2 * TC_BK : TC_BK);
   p.m = g.m;
   p.amax_in = o.amax_in; p.n_amax_in = o.n_amax_in; p.amax_out = o.amax_out;
   p.mode = mode;

@@ -21,7 +21,9 @@ struct fdvlm {
   int act8;        // W8A8: the four layer projections quantise their input rows to e4m3 (weights e4m3 as for DT_FP8)
   int use_tc;      // bf16 / fp8 weights: tcgen05 + TMA GEMMs, tensor-core attention, folded norms
   int kv_type;     // tensor-core path: element type of q and the KV cache (KV_BF16 / KV_F16)
-  int xfmt;        // tensor-core path: storage of the GEMM inputs a / ao / act (XF_BF16X2 for bf16 weights, XF_F16 for fp8)
+  int xfmt;        // tensor-core path: storage of the GEMM inputs a / ao / act (XF_BF16X2 for bf16 weights, XF_E5M2X3 for
+                   // fp8, XF_F16 for W8A8)
+  int pf_fmt;      // the same for the prompt path (XF_BF16X2 / XF_F16)
   int head_fmt;    // storage of the LM head's input (as xfmt, but bf16 planes when the head is a tied bf16 table)
   size_t a_lo, ao_lo, act_lo;   // XF_BF16X2: element offset of each buffer's low-order plane
   char* slab;      // one allocation behind every device buffer below except the KV cache

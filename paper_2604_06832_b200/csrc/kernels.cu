@@ -345,16 +345,16 @@ void launch_embed_prep(const void* table, const int32_t* tokens, const void* row
                                        status, amax, stamp);
 }
 
-// bf16 rows -> f16 rows (saturating), for the operator-level entry points whose callers hand bf16 activations to an
-// fp8-weight projection
-__global__ void bf16_to_f16_kernel(const bf16* __restrict__ in, unsigned short* __restrict__ out, size_t n) {
+// bf16 rows -> the planes of XF_E5M2X3, n bytes apart, for the operator-level entry points whose callers hand bf16
+// activations to an fp8-weight projection
+__global__ void bf16_to_e5m2x3_kernel(const bf16* __restrict__ in, uint8_t* __restrict__ out, size_t n) {
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) out[i] = f16_bits_sat(__bfloat162float(in[i]));
+  if (i < n) store_act(out, n, i, __bfloat162float(in[i]), XF_E5M2X3);
 }
-void launch_bf16_to_f16(const void* in, void* out, size_t n, cudaStream_t st) {
-  bf16_to_f16_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>((const bf16*)in, (unsigned short*)out, n);
+void launch_bf16_to_e5m2x3(const void* in, void* out, size_t n, cudaStream_t st) {
+  bf16_to_e5m2x3_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>((const bf16*)in, (uint8_t*)out, n);
 }
-// The same with one block per row, which also leaves amax[row] = max |f16 value| of the row: what the quantising
+// bf16 rows -> f16 rows (saturating), one block per row, which also leaves amax[row] = max |f16 value| of the row: what the quantising
 // projection takes its per-row scale from.
 __global__ void bf16_rows_to_f16_amax_kernel(const bf16* __restrict__ in, unsigned short* __restrict__ out, int k,
                                              float* __restrict__ amax) {
@@ -568,20 +568,7 @@ __global__ void __launch_bounds__(256) fin_resid_rows_kernel(const float* __rest
       ss = fmaf(x[e], x[e], ss);
     }
     *reinterpret_cast<float4*>(h + idx) = make_float4(x[0], x[1], x[2], x[3]);
-    unsigned short hi[4], lo[4];
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const float y = x[e] * g[c + e];
-      if (fmt == XF_F16) {
-        hi[e] = f16_bits_sat(y);
-      } else {
-        const bf16 b = __float2bfloat16_rn(y);
-        hi[e] = __bfloat16_as_ushort(b);
-        lo[e] = __bfloat16_as_ushort(__float2bfloat16_rn(y - __bfloat162float(b)));
-      }
-    }
-    *reinterpret_cast<ushort4*>((unsigned short*)xg + idx) = make_ushort4(hi[0], hi[1], hi[2], hi[3]);
-    if (fmt == XF_BF16X2) *reinterpret_cast<ushort4*>((unsigned short*)xg + lo_off + idx) = make_ushort4(lo[0], lo[1], lo[2], lo[3]);
+    store_act4(xg, lo_off, idx, make_float4(x[0] * g[c], x[1] * g[c + 1], x[2] * g[c + 2], x[3] * g[c + 3]), fmt);
   }
   ss = warp_sum(ss);
   if (lane == 0) ssq[(size_t)r * nt + t] = ss;

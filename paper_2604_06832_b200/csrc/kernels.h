@@ -28,7 +28,7 @@ size_t linear_workspace_bytes(int m, int n, int k, int dtype);
 // tokens outside [0, vocab) read row 0 and leave ST_BAD_TOKEN in *status
 void launch_embed(const void* table, const int32_t* tokens, float* h, int n, int hidden, int dtype, int vocab, int* status,
                   cudaStream_t st);
-void launch_bf16_to_f16(const void* in, void* out, size_t n, cudaStream_t st);
+void launch_bf16_to_e5m2x3(const void* in, void* out, size_t n, cudaStream_t st);       // planes n bytes apart
 // the same row by row, leaving amax[row] = max |f16 value| of the row
 void launch_bf16_rows_to_f16_amax(const void* in, void* out, int m, int k, float* amax, cudaStream_t st);
 void launch_rows_to_f32(const void* rows, float* h, int n, int hidden, int dtype, cudaStream_t st);
@@ -67,8 +67,9 @@ void launch_init_block(int32_t* tokens, uint8_t* masked, int32_t* info, const in
 enum { TC_MODE_PARTIAL = 0, TC_MODE_DIRECT = 1, TC_MODE_SWIGLU = 2, TC_MODE_LOGITS = 3 };
 // Up to three bf16 matrices that share x and K; their outputs sit side by side in one row of width ld.
 struct TcGroup {
-  const void* x; int m, k;   // bf16 weights: bf16 rows (hi plane); fp8 weights: f16 rows
-  const void* x_lo;          // bf16 weights only, nullable: the rows' low-order bf16 plane (x = hi + lo)
+  const void* x; int m, k;   // bf16 weights: bf16 rows (hi plane); fp8 weights: XF_E5M2X3 rows (first plane); a8: f16 rows
+  const void* x_lo;          // bf16 weights, nullable: the rows' low-order bf16 plane (x = hi + lo); fp8 weights: second plane
+  const void* x_3;           // fp8 weights: third plane
   const void* w[3]; int n[3]; int n_mats;
   const float* scale[3]; const float* bias[3];
   int fp8;   // weights are e4m3 bytes (scale[] holds the per-output-channel factors)

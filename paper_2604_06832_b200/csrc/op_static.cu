@@ -8,7 +8,9 @@
 using namespace fdk;
 
 // Laid out like the workspace of fdvlm_op_linear: the status words first, then the kernels' scratch.
-static __device__ __align__(256) unsigned char g_static_scratch[FDVLM_STATIC_SCRATCH_BYTES];
+// (Rows that meet fp8 weights take three bytes an element where two decide what is refused, so that widening the format
+// refused nothing that had been taken: at most half as much again.)
+static __device__ __align__(256) unsigned char g_static_scratch[FDVLM_STATIC_SCRATCH_BYTES / 2 * 3];
 
 // In host code `g_static_scratch` is only a handle for the runtime, not a device address: the address a
 // kernel may use comes from cudaGetSymbolAddress, asked once per device with that device current.
@@ -36,7 +38,8 @@ extern "C" int fdvlm_op_linear_static(const void* x, const void* w, const float*
   if (dtype != FDVLM_F32 && dtype != FDVLM_BF16 && dtype != FDVLM_W_FP8E4M3)
     return fail(nullptr, FDVLM_ERR_INVALID_ARG, "op_linear_static: unknown dtype %d", (int)dtype);
   if (dtype == FDVLM_W_FP8E4M3 && !scale) return fail(nullptr, FDVLM_ERR_INVALID_ARG, "op_linear_static: fp8 weights need scales");
-  const size_t need = linear_workspace_bytes(m, n, k, (int)dtype);
+  size_t need = linear_workspace_bytes(m, n, k, (int)dtype);
+  if (dtype == FDVLM_W_FP8E4M3 && need > (size_t)m * k) need -= (size_t)m * k;
   const size_t room = (size_t)FDVLM_STATIC_SCRATCH_BYTES;
   if (need > room)
     return fail(nullptr, FDVLM_ERR_CAPACITY,
@@ -50,7 +53,7 @@ extern "C" int fdvlm_op_linear_static(const void* x, const void* w, const float*
   // partial sums need no clearing: every (tile, split) slot that is summed is written by this call.
   LinearArgs a;
   a.x = x; a.w = w; a.scale = scale; a.bias = bias; a.y = y; a.m = m; a.n = n; a.k = k; a.ldy = n; a.accumulate = 0;
-  a.dtype = (int)dtype; a.workspace = base; a.workspace_bytes = room;
+  a.dtype = (int)dtype; a.workspace = base; a.workspace_bytes = sizeof(g_static_scratch);
   if (launch_linear(a, (cudaStream_t)cuda_stream, &e) < 0)
     return fail(nullptr, FDVLM_ERR_CUDA, "op_linear_static: launch: %s", cudaGetErrorString(e));
   return FDVLM_OK;
