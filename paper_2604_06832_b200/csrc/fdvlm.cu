@@ -84,13 +84,14 @@ extern "C" int fdvlm_create(const fdvlm_config* cfg, const fdvlm_weights* w, voi
   h->launches = 0;
   h->prof_on = 0;
   h->prof_used = 0;
-  h->kv = nullptr; h->h = nullptr; h->a = h->ao = h->act = h->q = nullptr; h->y = nullptr; h->cs = nullptr; h->ssq = nullptr;
+  h->kv = nullptr; h->h = nullptr; h->a = h->ao = h->act = h->q = nullptr; h->cs = nullptr; h->ssq = nullptr;
   h->amax_a = h->amax_ao = h->amax_act = nullptr;
   h->stats = nullptr; h->logits = nullptr; h->conf = nullptr; h->pred = nullptr; h->unmask = nullptr; h->blk_tokens = nullptr;
   h->blk_masked = nullptr; h->info = nullptr; h->init_stage = nullptr; h->ws = nullptr; h->info_host = nullptr;
   h->host_stage = nullptr;
   h->slab = nullptr;
   h->dev_len = nullptr;
+  h->dev_len_set = -1;
   h->use_graphs = 0;
   h->stamps = nullptr;
   h->stamp_used = 0;
@@ -110,13 +111,9 @@ extern "C" int fdvlm_create(const fdvlm_config* cfg, const fdvlm_weights* w, voi
   if (wa > ws) ws = wa;
   h->use_tc = (h->dt == DT_BF16 || h->dt == DT_FP8) && tc_linear_supported(R, NQ, H, h->dt) && tc_linear_supported(R, H, I, h->dt);
   h->kv_type = (int)cfg->kv_dtype;
-  if (h->act8 && !h->use_tc) {
+  if (!h->use_tc && h->dt != DT_F32) {
     delete h;
-    return fail(nullptr, FDVLM_ERR_UNSUPPORTED, "W8A8 needs shapes the tensor-core kernels take");
-  }
-  if (!h->use_tc && h->dt != DT_F32 && h->kv_type != KV_BF16) {
-    delete h;
-    return fail(nullptr, FDVLM_ERR_UNSUPPORTED, "an f16 KV cache needs shapes the tensor-core kernels take");
+    return fail(nullptr, FDVLM_ERR_UNSUPPORTED, "16-bit and fp8 weights need the tensor-core kernels (no cuTensorMapEncodeTiled in this driver?)");
   }
   // GEMM inputs: bf16 hi + lo planes for bf16 weights; for fp8 weights e5m2 planes, or one f16 plane where the rows are
   // quantised (W8A8) or meet widened weights (prompts).  CUDA-core path: one plane.
@@ -135,7 +132,7 @@ extern "C" int fdvlm_create(const fdvlm_config* cfg, const fdvlm_weights* w, voi
   // Every buffer but the KV cache is carved out of one slab, the small hot ones first: with gigabytes of weights
   // streaming through the TLBs, each separately allocated buffer would cost its own page walk whenever it is touched.
   struct { void** p; size_t bytes; } allocs[] = {
-      {(void**)&h->info, 32},
+      {(void**)&h->info, 32},              // info .. blk_tokens: read back together, see sync_info
       {(void**)&h->dev_len, 16},
       {(void**)&h->conf, (size_t)R * 4},
       {(void**)&h->pred, (size_t)R * 4},
@@ -159,8 +156,7 @@ extern "C" int fdvlm_create(const fdvlm_config* cfg, const fdvlm_weights* w, voi
       {(void**)&h->ao, (size_t)R * NQ * h->act_sz * planes},
       {(void**)&h->q, (size_t)R * NQ * h->act_sz},
       {(void**)&h->act, (size_t)R * I * h->act_sz * planes},
-      {(void**)&h->stats, (size_t)((cfg->vocab + 127) / 128) * 4 * R * 16},
-      {(void**)&h->y, (size_t)R * (NQKV > 2 * I ? NQKV : 2 * I) * 4},
+      {(void**)&h->stats, (size_t)(h->use_tc ? (cfg->vocab + 127) / 128 * 4 : f32_logit_tiles(cfg->vocab)) * R * 16},
       {(void**)&h->ws, ws ? ws : 16},
       {(void**)&h->logits, (size_t)R * cfg->vocab * 4},
   };
@@ -199,7 +195,7 @@ extern "C" int fdvlm_create(const fdvlm_config* cfg, const fdvlm_weights* w, voi
     char* cur = h->slab;
     for (auto& a : allocs) { *a.p = cur; cur += (a.bytes + 255) / 256 * 256; }
   }
-  if (cudaMallocHost((void**)&h->info_host, 32) != cudaSuccess || cudaMallocHost((void**)&h->host_stage, 64 * 16) != cudaSuccess) {
+  if (cudaMallocHost((void**)&h->info_host, (char*)h->blk_tokens + 256 - (char*)h->info) != cudaSuccess || cudaMallocHost((void**)&h->host_stage, 64 * 16) != cudaSuccess) {
     fail(nullptr, FDVLM_ERR_OOM, "pinned host allocation failed");
     fdvlm_destroy(h);
     return FDVLM_ERR_OOM;
@@ -211,10 +207,10 @@ extern "C" int fdvlm_create(const fdvlm_config* cfg, const fdvlm_weights* w, voi
     fdvlm_destroy(h);
     return FDVLM_ERR_CUDA;
   }
-  // the tensor-core forward is replayed from captured CUDA graphs (FDVLM_NO_GRAPH=1: launch kernel by kernel)
+  // the forward is replayed from captured CUDA graphs (FDVLM_NO_GRAPH=1: launch kernel by kernel)
   const char* no_graph = getenv("FDVLM_NO_GRAPH");
   // (the legacy default stream cannot be captured: a handle created on it launches kernel by kernel)
-  h->use_graphs = h->use_tc && h->st != nullptr && !(no_graph && no_graph[0] == '1');
+  h->use_graphs = h->st != nullptr && !(no_graph && no_graph[0] == '1');
   *out = h;
   return FDVLM_OK;
 }
@@ -285,9 +281,11 @@ static int block_begin_common(fdvlm_t* h, int block_size) {
   return FDVLM_OK;
 }
 
-// Read the 16-byte device record back: counts for the state machine, and the kernels' timeout word.
-static int sync_info(fdvlm_t* h) {
-  CU(h, cudaMemcpyAsync(h->info_host, h->info, 32, cudaMemcpyDeviceToHost, h->st));
+// Read the device record back: counts for the state machine, and the kernels' timeout word.  step_results: with
+// confidences, predictions, reveal flags and block tokens, which lie behind it in the slab: one copy for all of them.
+static int sync_info(fdvlm_t* h, bool step_results = false) {
+  const size_t bytes = step_results ? (char*)h->blk_tokens + 256 - (char*)h->info : 32;
+  CU(h, cudaMemcpyAsync(h->info_host, h->info, bytes, cudaMemcpyDeviceToHost, h->st));
   CU(h, cudaStreamSynchronize(h->st));
   h->n_remaining = h->info_host[1];
   if (h->info_host[3] != 0) {
@@ -376,8 +374,8 @@ static int step_core(fdvlm_t* h, const fdvlm_step_params* p, int want_logits) {
   return FDVLM_OK;
 }
 
-static int finish_info(fdvlm_t* h, fdvlm_step_info* info) {
-  int rc = sync_info(h);
+static int finish_info(fdvlm_t* h, fdvlm_step_info* info, bool step_results = false) {
+  int rc = sync_info(h, step_results);
   if (rc) return rc;
   if (info) { info->n_unmasked = h->info_host[0]; info->n_remaining = h->info_host[1]; info->step_index = h->info_host[2]; }
   if (h->info_host[0] == 0 && h->info_host[1] > 0)
@@ -488,7 +486,7 @@ extern "C" int fdvlm_decode_block(fdvlm_t* h, int block_size, const int32_t* ini
   if (!info) return fail(h, FDVLM_ERR_INVALID_ARG, "decode_block needs the host info struct");
   int rc = check_step_params(h, p);
   if (rc) return rc;
-  if (!h->use_graphs) return fail(h, FDVLM_ERR_UNSUPPORTED, "decode_block needs the tensor-core path on a non-default stream");
+  if (!h->use_graphs || !h->use_tc) return fail(h, FDVLM_ERR_UNSUPPORTED, "decode_block needs the tensor-core path on a non-default stream");
   rc = fdvlm_block_begin(h, block_size, init_tokens);      // (reads the masked count back when tokens are given)
   if (rc) return rc;
   h->launches = 0;
@@ -509,7 +507,7 @@ static int decode_loop_rest(fdvlm_t* h, int block_size, const fdvlm_step_params*
       if (rc) rc = build_loop_graph(h, block_size, p, false);
       if (rc) return rc;
     }
-    launch_set_len(h->dev_len, h->cache_len, h->st);
+    set_dev_len(h);
     CU(h, cudaMemcpyAsync(h->info + 5, &steps_done, 4, cudaMemcpyHostToDevice, h->st));
     CU(h, cudaGraphLaunch(h->loop_exec, h->st));
   } else {
@@ -536,7 +534,7 @@ extern "C" int fdvlm_commit_decode_block(fdvlm_t* h, int block_size, const int32
   if (!info) return fail(h, FDVLM_ERR_INVALID_ARG, "commit_decode_block needs the host info struct");
   int rc = check_step_params(h, p);
   if (rc) return rc;
-  if (!h->use_graphs) return fail(h, FDVLM_ERR_UNSUPPORTED, "decode_block needs the tensor-core path on a non-default stream");
+  if (!h->use_graphs || !h->use_tc) return fail(h, FDVLM_ERR_UNSUPPORTED, "decode_block needs the tensor-core path on a non-default stream");
   rc = commit_step_core(h, block_size, init_tokens, p, 0);      // the finished block's commit + this block's first step
   if (rc) return rc;
   rc = sync_info(h);                                            // what the first step left masked decides whether the loop runs
@@ -544,24 +542,26 @@ extern "C" int fdvlm_commit_decode_block(fdvlm_t* h, int block_size, const int32
   return decode_loop_rest(h, block_size, p, block_tokens, info, 1);
 }
 
+// Wait for the step and hand its results out; row0: first row of the block within the forward.
+static int step_results_to_host(fdvlm_t* h, int row0, int B, float* conf, int32_t* pred, uint8_t* unmask, int32_t* tokens,
+                                fdvlm_step_info* info) {
+  int rc = finish_info(h, info, true);
+  if (rc) return rc;
+  auto copy = [&](void* dst, const void* dev, size_t bytes) {
+    if (dst) memcpy(dst, (const char*)h->info_host + ((const char*)dev - (const char*)h->info), bytes);
+  };
+  copy(conf, h->conf + row0, (size_t)B * 4);
+  copy(pred, h->pred + row0, (size_t)B * 4);
+  copy(unmask, h->unmask, (size_t)B);
+  copy(tokens, h->blk_tokens, (size_t)B * 4);
+  return FDVLM_OK;
+}
+
 extern "C" int fdvlm_block_step_host(fdvlm_t* h, const fdvlm_step_params* p, float* conf_host, int32_t* pred_host,
                                      uint8_t* unmask_host, int32_t* block_tokens_host, fdvlm_step_info* info) {
   int rc = step_core(h, p, 0);
   if (rc) return rc;
-  const int B = h->block_size;
-  char* s = h->host_stage;  // [conf 256 | pred 256 | tokens 256 | unmask 64]
-  const cudaMemcpyKind DH = cudaMemcpyDeviceToHost;
-  if (conf_host) CU(h, cudaMemcpyAsync(s, h->conf, (size_t)B * 4, DH, h->st));
-  if (pred_host) CU(h, cudaMemcpyAsync(s + 256, h->pred, (size_t)B * 4, DH, h->st));
-  if (block_tokens_host) CU(h, cudaMemcpyAsync(s + 512, h->blk_tokens, (size_t)B * 4, DH, h->st));
-  if (unmask_host) CU(h, cudaMemcpyAsync(s + 768, h->unmask, (size_t)B, DH, h->st));
-  rc = finish_info(h, info);
-  if (rc) return rc;
-  if (conf_host) memcpy(conf_host, s, (size_t)B * 4);
-  if (pred_host) memcpy(pred_host, s + 256, (size_t)B * 4);
-  if (block_tokens_host) memcpy(block_tokens_host, s + 512, (size_t)B * 4);
-  if (unmask_host) memcpy(unmask_host, s + 768, (size_t)B);
-  return FDVLM_OK;
+  return step_results_to_host(h, 0, h->block_size, conf_host, pred_host, unmask_host, block_tokens_host, info);
 }
 
 // Causal pass over the finished block with cache update.  all_rows: confidence / prediction of every row are left in
@@ -674,19 +674,7 @@ extern "C" int fdvlm_commit_begin_step_host(fdvlm_t* h, int next_block_size, con
   }
   int rc = commit_step_core(h, B, init_dev, p, 0);
   if (rc) return rc;
-  char* s = h->host_stage;  // [conf 256 | pred 256 | tokens 256 | unmask 64]
-  const cudaMemcpyKind DH = cudaMemcpyDeviceToHost;
-  if (conf_host) CU(h, cudaMemcpyAsync(s, h->conf + Bc, (size_t)B * 4, DH, h->st));
-  if (pred_host) CU(h, cudaMemcpyAsync(s + 256, h->pred + Bc, (size_t)B * 4, DH, h->st));
-  if (block_tokens_host) CU(h, cudaMemcpyAsync(s + 512, h->blk_tokens, (size_t)B * 4, DH, h->st));
-  if (unmask_host) CU(h, cudaMemcpyAsync(s + 768, h->unmask, (size_t)B, DH, h->st));
-  rc = finish_info(h, info);
-  if (rc) return rc;
-  if (conf_host) memcpy(conf_host, s, (size_t)B * 4);
-  if (pred_host) memcpy(pred_host, s + 256, (size_t)B * 4);
-  if (block_tokens_host) memcpy(block_tokens_host, s + 512, (size_t)B * 4);
-  if (unmask_host) memcpy(unmask_host, s + 768, (size_t)B);
-  return FDVLM_OK;
+  return step_results_to_host(h, Bc, B, conf_host, pred_host, unmask_host, block_tokens_host, info);
 }
 
 extern "C" int fdvlm_commit_decode_block_topk(fdvlm_t* h, int block_size, const int32_t* init_tokens, int k, int pred_shift,

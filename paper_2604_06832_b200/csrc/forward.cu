@@ -1,13 +1,13 @@
 // The decoder forward of one step as a launch sequence (Fast-dVLM Sec. 3.4; Appendix B Alg. 1 for the
-// two attention modes), in two flavours: the exact CUDA-core path (fp32 configuration, shapes the
-// tensor-core kernels do not take) and the tensor-core path (bf16 and fp8 weights).
+// two attention modes), in two flavours: the exact CUDA-core path (fp32 weights) and the tensor-core path (bf16 and fp8
+// weights).
 #include "handle.h"
 
 namespace fdk {
 
 int launch_linear_simt(const LinearArgs& a, cudaStream_t st, cudaError_t* err);
 size_t simt_workspace_bytes(int m, int n, int k);
-int launch_attention_simt(const AttnArgs& a, cudaStream_t st, cudaError_t* err);
+int launch_attention_f32(const AttnArgs& a, cudaStream_t st, cudaError_t* err);
 size_t attention_mma_workspace_bytes(int n, int hq, int hkv, int d);
 int launch_attention_mma(const AttnArgs& a, cudaStream_t st, cudaError_t* err);
 void launch_splitk_epilogue(const float* part, int S, int m, int n, const float* scale, const float* bias, float* y, int ldy,
@@ -79,7 +79,7 @@ int launch_linear(const LinearArgs& a, cudaStream_t st, cudaError_t* err) {
 size_t attention_workspace_bytes(int n, int hq, int hkv, int d) { return attention_mma_workspace_bytes(n, hq, hkv, d); }
 // 16-bit rows go to the split-KV tensor-core kernel, fp32 rows to the exact CUDA-core kernel.
 int launch_attention(const AttnArgs& a, cudaStream_t st, cudaError_t* err) {
-  return a.dtype == DT_F32 ? launch_attention_simt(a, st, err) : launch_attention_mma(a, st, err);
+  return a.dtype == DT_F32 ? launch_attention_f32(a, st, err) : launch_attention_mma(a, st, err);
 }
 
 int stage_rows(fdvlm_t* h, int row0, int n, const int32_t* tokens, const void* embeds) {
@@ -211,69 +211,63 @@ int forward_prefill(fdvlm_t* h, int n, int want_last_logits) {
   return FDVLM_OK;
 }
 
-// ---- exact CUDA-core path: one kernel per operator ---------------------------------------------------
-static int forward_rows_simt(fdvlm_t* h, int n, int mode, int logits_rows) {
+// ---- exact fp32 path ----------------------------------------------------------------------------------
+// per layer: [norm + QKV, bias, rotary, K/V rows] [attention] [O + residual] [norm + gate/up + SwiGLU] [down + residual]
+static int forward_rows_f32(fdvlm_t* h, int n, int mode, int logits_rows, int want_logits, const int* len_ptr) {
   const fdvlm_config& c = h->cfg;
-  const int H = c.hidden, I = c.intermediate, d = c.head_dim;
-  const int NQ = c.n_q_heads * d, NKV = c.n_kv_heads * d, NQKV = NQ + 2 * NKV;
+  const int H = c.hidden, I = c.intermediate, d = c.head_dim, NQ = c.n_q_heads * d, NKV = c.n_kv_heads * d;
   cudaError_t e = cudaSuccess;
-  auto lin = [&](const void* x, const void* w, const float* scale, const float* bias, float* y, int nn, int kk, int ldy,
-                 int accumulate, int m, int dt) -> int {
-    LinearArgs a;
-    a.x = x; a.w = w; a.scale = scale; a.bias = bias; a.y = y; a.m = m; a.n = nn; a.k = kk; a.ldy = ldy;
-    a.accumulate = accumulate; a.dtype = dt; a.workspace = h->ws; a.workspace_bytes = h->ws_bytes;
-    prof_begin(h, 0);
-    int r = launch_linear_simt(a, h->st, &e);
-    prof_end(h);
-    if (r < 0) return -1;
-    h->launches += r;
-    return 0;
+  auto lin = [&](int lm, const void* x, int m, int k, const float* gain, const void* w, int nn, float* out) {
+    F32Linear g;
+    memset(&g, 0, sizeof(g));
+    g.mode = lm; g.x = (const float*)x; g.m = m; g.k = k; g.gain = gain; g.inv_h = 1.f / (float)H; g.eps = c.rms_eps;
+    g.w[0] = (const float*)w; g.n[0] = nn; g.out = out;
+    return g;
   };
-  const int dt = h->dt;
-  launch_rope_table(h->cs, n, h->cache_len, d, c.rope_theta, h->st, nullptr, nullptr, mode == MODE_MASKED ? h->q_pos_off : nullptr);
+  auto run = [&](const F32Linear& g) {
+    prof_begin(h, 0);
+    e = launch_linear_f32(g, h->st);
+    prof_end(h);
+    h->launches++;
+    return e == cudaSuccess;
+  };
+  launch_rope_table(h->cs, n, h->cache_len, d, c.rope_theta, h->st, len_ptr, nullptr, mode == MODE_MASKED ? h->q_pos_off : nullptr);
   h->launches++;
   for (int l = 0; l < c.n_layers; ++l) {
     const fdvlm_layer_weights& lw = h->layers[l];
-    launch_rmsnorm(h->h, lw.g_attn, h->a, n, H, c.rms_eps, dt, h->st);
-    if (lin(h->a, lw.wq, lw.s_q, lw.bq, h->y, NQ, H, NQKV, 0, n, dt) || lin(h->a, lw.wk, lw.s_k, lw.bk, h->y + NQ, NKV, H, NQKV, 0, n, dt) ||
-        lin(h->a, lw.wv, lw.s_v, lw.bv, h->y + NQ + NKV, NKV, H, NQKV, 0, n, dt))
-      return fail(h, FDVLM_ERR_CUDA, "qkv projection launch: %s", cudaGetErrorString(e));
-    launch_qkv_post(h->y, h->cs, h->q, kv_ptr(h, l, 0), kv_ptr(h, l, 1), n, h->cache_len, c.n_q_heads, c.n_kv_heads, d,
-                    c.max_seq, dt, h->st);
+    F32Linear g = lin(FL_QKV, h->h, n, H, lw.g_attn, lw.wq, NQ, (float*)h->q);
+    g.w[1] = (const float*)lw.wk; g.w[2] = (const float*)lw.wv; g.n[1] = g.n[2] = NKV;
+    g.bias[0] = lw.bq; g.bias[1] = lw.bk; g.bias[2] = lw.bv;
+    g.kc = (float*)kv_ptr(h, l, 0); g.vc = (float*)kv_ptr(h, l, 1); g.cs = h->cs; g.len_ptr = len_ptr; g.pos0 = h->cache_len;
+    g.hq = c.n_q_heads; g.hkv = c.n_kv_heads; g.d = d; g.max_seq = c.max_seq;
+    if (!run(g)) return fail(h, FDVLM_ERR_CUDA, "qkv projection launch: %s", cudaGetErrorString(e));
     AttnArgs at;
     memset(&at, 0, sizeof(at));
-    at.q = h->q; at.kc = kv_ptr(h, l, 0); at.vc = kv_ptr(h, l, 1); at.out = h->ao; at.n = n; at.cache_len = h->cache_len;
-    at.max_seq = c.max_seq; at.hq = c.n_q_heads; at.hkv = c.n_kv_heads; at.d = d; at.causal = (mode == MODE_CAUSAL);
+    at.q = h->q; at.kc = kv_ptr(h, l, 0); at.vc = kv_ptr(h, l, 1); at.out = h->ao; at.n = n; at.cache_len = h->cache_len; at.len_ptr = len_ptr;
+    at.max_seq = c.max_seq; at.hq = c.n_q_heads; at.hkv = c.n_kv_heads; at.d = d; at.causal = (mode == MODE_CAUSAL); at.dtype = DT_F32;
     at.row_mask = (mode == MODE_MASKED) ? h->q_mask : (mode == MODE_FUSED ? h->f_mask : nullptr);
-    at.dtype = dt; at.workspace = h->ws; at.kv_type = KV_BF16; at.out_fmt = XF_BF16; at.long_cache = -1;
     prof_begin(h, 1);
-    int r = launch_attention(at, h->st, &e);
+    const int r = launch_attention(at, h->st, &e);
     prof_end(h);
     if (r < 0) return fail(h, FDVLM_ERR_CUDA, "attention launch: %s", cudaGetErrorString(e));
-    h->launches += r + 2;
-    if (lin(h->ao, lw.wo, lw.s_o, nullptr, h->h, H, NQ, H, 1, n, dt))
+    h->launches += r;
+    if (!run(lin(FL_RESID, h->ao, n, NQ, nullptr, lw.wo, H, h->h)))
       return fail(h, FDVLM_ERR_CUDA, "o projection launch: %s", cudaGetErrorString(e));
-    launch_rmsnorm(h->h, lw.g_mlp, h->a, n, H, c.rms_eps, dt, h->st);
-    if (lin(h->a, lw.w_gate, lw.s_gate, nullptr, h->y, I, H, 2 * I, 0, n, dt) || lin(h->a, lw.w_up, lw.s_up, nullptr, h->y + I, I, H, 2 * I, 0, n, dt))
-      return fail(h, FDVLM_ERR_CUDA, "gate/up projection launch: %s", cudaGetErrorString(e));
-    launch_swiglu(h->y, h->act, n, I, dt, h->st);
-    if (lin(h->act, lw.w_down, lw.s_down, nullptr, h->h, H, I, H, 1, n, dt))
+    g = lin(FL_SWIGLU, h->h, n, H, lw.g_mlp, lw.w_gate, I, (float*)h->act);
+    g.w[1] = (const float*)lw.w_up; g.n[1] = I;
+    if (!run(g)) return fail(h, FDVLM_ERR_CUDA, "gate/up projection launch: %s", cudaGetErrorString(e));
+    if (!run(lin(FL_RESID, h->act, n, I, nullptr, lw.w_down, H, h->h)))
       return fail(h, FDVLM_ERR_CUDA, "down projection launch: %s", cudaGetErrorString(e));
-    h->launches += 2;
   }
   if (logits_rows > 0) {
-    const int first = (logits_rows == n) ? 0 : n - 1;
-    const int m = n - first;
-    launch_rmsnorm(h->h + (size_t)first * H, h->w.g_final, h->a, m, H, c.rms_eps, dt, h->st);
-    h->launches++;
-    const void* table = c.tie_embeddings ? h->w.embed : h->w.lm_head;
-    const float* sc = c.tie_embeddings ? nullptr : h->w.s_lm_head;
-    // a tied table is stored in the embedding's type: fp32 for F32, bf16 otherwise (never fp8)
-    const int hdt = (c.tie_embeddings && dt == DT_FP8) ? DT_BF16 : dt;
-    if (lin(h->a, table, sc, nullptr, h->logits, c.vocab, H, c.vocab, 0, m, hdt))
-      return fail(h, FDVLM_ERR_CUDA, "lm head launch: %s", cudaGetErrorString(e));
-    if (logits_rows == n) {
-      launch_row_stats(h->logits, n, c.vocab, c.mask_id, h->conf, h->pred, h->st);
+    const bool all = logits_rows == n;
+    const int first = all ? 0 : n - 1;
+    F32Linear g = lin(FL_LOGITS, h->h + (size_t)first * H, n - first, H, h->w.g_final, c.tie_embeddings ? h->w.embed : h->w.lm_head, c.vocab,
+                      (!all || want_logits) ? h->logits : nullptr);
+    g.stats = all ? (float4*)h->stats : nullptr; g.mask_id = c.mask_id;
+    if (!run(g)) return fail(h, FDVLM_ERR_CUDA, "lm head launch: %s", cudaGetErrorString(e));
+    if (all) {
+      launch_stats_merge(h->stats, f32_logit_tiles(c.vocab), n, h->conf, h->pred, h->st);
       h->launches++;
     }
   }
@@ -408,14 +402,13 @@ static int forward_rows_tc(fdvlm_t* h, int n, int mode, int logits_rows, int wan
   return FDVLM_OK;
 }
 
-// The tensor-core forward as a replayed CUDA graph: every kernel takes the cache length from a device word, so one
+// The forward as a replayed CUDA graph: every kernel takes the cache length from a device word, so one
 // capture per (rows, mode, logits mode, stamped or not) serves every later call; the programmatic-dependent-launch
 // edges are kept.
 static int forward_rows_graph(fdvlm_t* h, int n, int mode, int logits_rows, int want_logits) {
   const int stamped = (h->prof_on == 2) ? 1 : 0;
   const int long_cache = attention_long_cache(h->cache_len + n) ? 1 : 0;
-  launch_set_len(h->dev_len, h->cache_len, h->st);
-  h->launches++;
+  set_dev_len(h);
   if (stamped) CU(h, cudaMemsetAsync(h->stamps, 0xFF, sizeof(KStamp) * FDVLM_MAX_STAMPS, h->st));
   for (auto& g : h->graphs) {
     if (g.n == n && g.mode == mode && g.logits_rows == logits_rows && g.want_logits == want_logits && g.stamped == stamped &&
@@ -431,7 +424,8 @@ static int forward_rows_graph(fdvlm_t* h, int n, int mode, int logits_rows, int 
   }
   const int before = h->launches;
   CU(h, cudaStreamBeginCapture(h->st, cudaStreamCaptureModeThreadLocal));
-  const int rc = forward_rows_tc(h, n, mode, logits_rows, want_logits, h->dev_len, stamped != 0, long_cache);
+  const int rc = h->use_tc ? forward_rows_tc(h, n, mode, logits_rows, want_logits, h->dev_len, stamped != 0, long_cache)
+                           : forward_rows_f32(h, n, mode, logits_rows, want_logits, h->dev_len);
   cudaGraph_t graph = nullptr;
   cudaError_t e = cudaStreamEndCapture(h->st, &graph);
   if (rc != FDVLM_OK) { if (graph) cudaGraphDestroy(graph); return rc; }
@@ -455,9 +449,9 @@ int forward_rows_enqueue(fdvlm_t* h, int n, int mode, int logits_rows, int want_
 }
 
 int forward_rows(fdvlm_t* h, int n, int mode, int logits_rows, int want_logits) {
-  if (!h->use_tc) return forward_rows_simt(h, n, mode, logits_rows);
   // event timing around each kernel needs the kernels launched one by one
   if (h->use_graphs && h->prof_on != 1) return forward_rows_graph(h, n, mode, logits_rows, want_logits);
+  if (!h->use_tc) return forward_rows_f32(h, n, mode, logits_rows, want_logits, nullptr);
   const bool stamped = h->prof_on == 2;
   if (stamped) CU(h, cudaMemsetAsync(h->stamps, 0xFF, sizeof(KStamp) * FDVLM_MAX_STAMPS, h->st));
   return forward_rows_tc(h, n, mode, logits_rows, want_logits, nullptr, stamped);

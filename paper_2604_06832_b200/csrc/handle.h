@@ -28,7 +28,8 @@ struct fdvlm {
   size_t a_lo, ao_lo, act_lo;   // XF_BF16X2: element offset of each buffer's low-order plane
   char* slab;      // one allocation behind every device buffer below except the KV cache
   int32_t* dev_len;   // device copy of cache_len, read by the captured forward graphs
-  int use_graphs;     // tensor-core path: replay one captured CUDA graph per (rows, mode, logits mode)
+  int dev_len_set;    // the value it was last given, in stream order (-1: none)
+  int use_graphs;     // replay one captured CUDA graph per (rows, mode, logits mode)
   struct FwdGraph { int n, mode, logits_rows, want_logits, stamped, long_cache, launches; cudaGraphExec_t exec; std::vector<int> kinds; };
   std::vector<FwdGraph> graphs;
   // on-device decode loop (fdvlm_decode_block): a graph whose conditional WHILE node repeats the denoise step
@@ -42,7 +43,6 @@ struct fdvlm {
   void* ao;        // [R, Hq*d] attention output
   void* act;       // [R, I]
   void* q;         // [R, Hq*d]
-  float* y;        // [R, max((Hq+2Hkv)d, 2I)] fp32 GEMM output (CUDA-core path)
   float* cs;       // [R, d/2] float2 rotary table
   float* ssq;      // [R, nt] partial sums of h^2 per 128 columns (tensor-core path)
   // W8A8: maxima of |value as stored| of the rows of a ([R, nt] partial maxima), ao ([R, Hq] partial maxima) and
@@ -130,6 +130,14 @@ inline void prof_end(fdvlm_t* h) {
   if (!h->prof_on) return;
   cudaEventRecord(h->prof_ev[h->prof_used * 2 + 1], h->st);
   h->prof_used++;
+}
+
+// the device copy of the cache length, brought up to date in stream order
+inline void set_dev_len(fdvlm_t* h) {
+  if (h->dev_len_set == h->cache_len) return;
+  launch_set_len(h->dev_len, h->cache_len, h->st);
+  h->launches++;
+  h->dev_len_set = h->cache_len;
 }
 
 // forward.cu

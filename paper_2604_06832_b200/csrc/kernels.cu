@@ -1,6 +1,5 @@
-// CUDA-core (SIMT) kernels of the denoise step: the exact-fp32 path of the fp32 configuration and
-// the small fused glue of every configuration (embedding gather, RMSNorm, rotary + KV staging,
-// SwiGLU, softmax-max confidence / argmax, unmask selection).
+// The small kernels of every configuration (embedding gather, rotary table, the glue of the tensor-core path, confidence
+// statistics, unmask selection, block state) and the stand-alone CUDA-core projection.
 #include "common.cuh"
 #include "kernels.h"
 
@@ -211,26 +210,6 @@ void launch_rows_to_f32(const void* rows, float* h, int n, int hidden, int dtype
 }
 
 // ================================================================================================
-// RMSNorm: out = x * rsqrt(mean(x^2) + eps) * g, fp32 math, output in the activation type
-// ================================================================================================
-template <typename AT>
-__global__ void rmsnorm_kernel(const float* __restrict__ h, const float* __restrict__ g, AT* __restrict__ out,
-                               int hidden, float eps) {
-  __shared__ float red[32];
-  const float* x = h + (size_t)blockIdx.x * hidden;
-  float ss = 0.f;
-  for (int c = threadIdx.x; c < hidden; c += blockDim.x) { float v = x[c]; ss = fmaf(v, v, ss); }
-  ss = block_sum(ss, red);
-  float r = rsqrtf(ss / (float)hidden + eps);
-  AT* o = out + (size_t)blockIdx.x * hidden;
-  for (int c = threadIdx.x; c < hidden; c += blockDim.x) o[c] = from_f32<AT>(x[c] * r * g[c]);
-}
-void launch_rmsnorm(const float* h, const float* g, void* out, int n, int hidden, float eps, int dtype, cudaStream_t st) {
-  if (dtype == DT_F32) rmsnorm_kernel<float><<<n, 256, 0, st>>>(h, g, (float*)out, hidden, eps);
-  else rmsnorm_kernel<bf16><<<n, 256, 0, st>>>(h, g, (bf16*)out, hidden, eps);
-}
-
-// ================================================================================================
 // rotary table: cs[r][j] = (cos, sin)(pos * theta^(-2j/d)), angles formed in fp64
 // ================================================================================================
 __global__ void set_len_kernel(int* len_ptr, int value) {
@@ -262,41 +241,6 @@ void launch_rope_table(float* cs, int n, int pos0, int head_dim, float theta, cu
   int half = head_dim / 2, total = n * half;
   launch_pdl(rope_table_kernel, dim3((total + 127) / 128), dim3(128), 0, st, (float2*)cs, n, pos0, half, (double)theta, len_ptr, pos_off,
              stamp);
-}
-
-// rotate-half pairing (j, j + d/2); q -> q buffer, k -> cache K plane, v -> cache V plane
-template <typename AT>
-__global__ void qkv_post_kernel(const float* __restrict__ qkv, const float2* __restrict__ cs, AT* __restrict__ q,
-                                AT* __restrict__ kc, AT* __restrict__ vc, int pos0, int hq, int hkv, int d, int max_seq) {
-  int r = blockIdx.x, half = d >> 1;
-  int width = (hq + 2 * hkv) * d;
-  const float* row = qkv + (size_t)r * width;
-  int pairs = (hq + hkv) * half;
-  for (int t = threadIdx.x; t < pairs; t += blockDim.x) {
-    int head = t / half, j = t % half;
-    float2 c = cs[r * half + j];
-    float a = row[head * d + j], b = row[head * d + j + half];
-    float ra = a * c.x - b * c.y, rb = b * c.x + a * c.y;
-    if (head < hq) {
-      AT* o = q + ((size_t)r * hq + head) * d;
-      o[j] = from_f32<AT>(ra); o[j + half] = from_f32<AT>(rb);
-    } else {
-      AT* o = kc + ((size_t)(head - hq) * max_seq + pos0 + r) * d;
-      o[j] = from_f32<AT>(ra); o[j + half] = from_f32<AT>(rb);
-    }
-  }
-  const float* vrow = row + (hq + hkv) * d;
-  for (int t = threadIdx.x; t < hkv * d; t += blockDim.x) {
-    int head = t / d, j = t % d;
-    vc[((size_t)head * max_seq + pos0 + r) * d + j] = from_f32<AT>(vrow[t]);
-  }
-}
-void launch_qkv_post(const float* qkv, const float* cs, void* q, void* kc, void* vc, int n, int pos0, int hq, int hkv,
-                     int d, int max_seq, int dtype, cudaStream_t st) {
-  if (dtype == DT_F32)
-    qkv_post_kernel<float><<<n, 256, 0, st>>>(qkv, (const float2*)cs, (float*)q, (float*)kc, (float*)vc, pos0, hq, hkv, d, max_seq);
-  else
-    qkv_post_kernel<bf16><<<n, 256, 0, st>>>(qkv, (const float2*)cs, (bf16*)q, (bf16*)kc, (bf16*)vc, pos0, hq, hkv, d, max_seq);
 }
 
 // ================================================================================================
@@ -638,73 +582,6 @@ void launch_stats_merge(const void* stats, int n_part, int m, float* conf, int32
 }
 
 // ================================================================================================
-// SwiGLU: act = silu(gate) * up, gu = [n, 2*inter] with gate in the first half of each row
-// ================================================================================================
-template <typename AT>
-__global__ void swiglu_kernel(const float* __restrict__ gu, AT* __restrict__ act, int n, int inter) {
-  size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= (size_t)n * inter) return;
-  int r = (int)(idx / inter), c = (int)(idx % inter);
-  float g = gu[(size_t)r * 2 * inter + c], u = gu[(size_t)r * 2 * inter + inter + c];
-  act[idx] = from_f32<AT>(g / (1.f + expf(-g)) * u);
-}
-void launch_swiglu(const float* gu, void* act, int n, int inter, int dtype, cudaStream_t st) {
-  size_t total = (size_t)n * inter;
-  unsigned blocks = (unsigned)((total + 255) / 256);
-  if (dtype == DT_F32) swiglu_kernel<float><<<blocks, 256, 0, st>>>(gu, (float*)act, n, inter);
-  else swiglu_kernel<bf16><<<blocks, 256, 0, st>>>(gu, (bf16*)act, n, inter);
-}
-
-// ================================================================================================
-// confidence and prediction of a row: pred = argmax_{v != mask_id} l_v (lowest id on a tie),
-// conf = 1 / sum_{v != mask_id} exp(l_v - l_pred)
-// ================================================================================================
-__global__ void __launch_bounds__(1024) row_stats_kernel(const float* __restrict__ logits, int vocab, int mask_id,
-                                                       float* __restrict__ conf, int32_t* __restrict__ pred) {
-  __shared__ float red[32];
-  __shared__ float smax[32];
-  __shared__ int sidx[32];
-  const float* l = logits + (size_t)blockIdx.x * vocab;
-  float best = -INFINITY;
-  int bi = 0x7fffffff;
-  for (int v = threadIdx.x; v < vocab; v += blockDim.x) {
-    if (v == mask_id) continue;
-    float x = l[v];
-    if (x > best) { best = x; bi = v; }
-  }
-  int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    float ob = __shfl_xor_sync(0xffffffffu, best, o);
-    int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-    if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
-  }
-  if (lane == 0) { smax[w] = best; sidx[w] = bi; }
-  __syncthreads();
-  if (w == 0) {
-    best = lane < nw ? smax[lane] : -INFINITY;
-    bi = lane < nw ? sidx[lane] : 0x7fffffff;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      float ob = __shfl_xor_sync(0xffffffffu, best, o);
-      int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-      if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
-    }
-    if (lane == 0) { smax[0] = best; sidx[0] = bi; }
-  }
-  __syncthreads();
-  best = smax[0];
-  float s = 0.f;
-  for (int v = threadIdx.x; v < vocab; v += blockDim.x)
-    if (v != mask_id) s += __expf(l[v] - best);
-  s = block_sum(s, red);
-  if (threadIdx.x == 0) { conf[blockIdx.x] = 1.f / s; pred[blockIdx.x] = sidx[0]; }
-}
-void launch_row_stats(const float* logits, int n, int vocab, int mask_id, float* conf, int32_t* pred, cudaStream_t st) {
-  row_stats_kernel<<<n, 1024, 0, st>>>(logits, vocab, mask_id, conf, pred);
-}
-
-// ================================================================================================
 // unmask selection (one CTA of 64 threads; n <= 64)
 // ================================================================================================
 __global__ void select_kernel(const float* __restrict__ conf, const int32_t* __restrict__ pred,
@@ -907,78 +784,6 @@ __global__ void init_block_kernel(int32_t* tokens, uint8_t* masked, int32_t* inf
 void launch_init_block(int32_t* tokens, uint8_t* masked, int32_t* info, const int32_t* init, int n, int mask_id, int step,
                        cudaStream_t st) {
   init_block_kernel<<<1, 64, 0, st>>>(tokens, masked, info, init, n, mask_id, step);
-}
-
-// ================================================================================================
-// attention, CUDA-core version: one CTA per (query head, row).  Exact-fp32 path of the fp32
-// configuration and the fallback where the tensor-core kernel does not apply.
-// ================================================================================================
-template <typename AT>
-__global__ void __launch_bounds__(128) attn_simt_kernel(const AT* __restrict__ q, const AT* __restrict__ kc,
-                                                        const AT* __restrict__ vc, AT* __restrict__ out, int n,
-                                                        int L, int max_seq, int hq, int hkv, int d, int causal,
-                                                        const unsigned long long* __restrict__ row_mask) {
-  extern __shared__ float smem[];
-  float* qs = smem;          // [d]
-  float* red = smem + d;     // [32]
-  float* ov = red + 32;      // [128]
-  float* sc = ov + 128;      // [T]
-  const int hqi = blockIdx.x, r = blockIdx.y;
-  const int hk = hqi / (hq / hkv);
-  const int T = causal ? (L + r + 1) : (L + n);
-  const float scale = rsqrtf((float)d);
-  const AT* qrow = q + ((size_t)r * hq + hqi) * d;
-  for (int t = threadIdx.x; t < d; t += blockDim.x) qs[t] = to_f32(qrow[t]) * scale;
-  __syncthreads();
-  const AT* kbase = kc + (size_t)hk * max_seq * d;
-  const AT* vbase = vc + (size_t)hk * max_seq * d;
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  const int epl = d / 32;
-  for (int j = w; j < T; j += nw) {
-    const AT* kr = kbase + (size_t)j * d + lane * epl;
-    float p = 0.f;
-    for (int e = 0; e < epl; ++e) p = fmaf(qs[lane * epl + e], to_f32(kr[e]), p);
-    p = warp_sum(p);
-    // explicit mask among the n rows: bit r' of row_mask[r] = row r reads row r' (the cache is always read)
-    if (row_mask && j >= L && !((row_mask[r] >> (j - L)) & 1ull)) p = -INFINITY;
-    if (lane == 0) sc[j] = p;
-  }
-  __syncthreads();
-  float mx = -INFINITY;
-  for (int j = threadIdx.x; j < T; j += blockDim.x) mx = fmaxf(mx, sc[j]);
-  mx = block_max(mx, red);
-  float sum = 0.f;
-  for (int j = threadIdx.x; j < T; j += blockDim.x) { float e = expf(sc[j] - mx); sc[j] = e; sum += e; }
-  sum = block_sum(sum, red);
-  __syncthreads();
-  const int dd = threadIdx.x % d, part = threadIdx.x / d, nparts = blockDim.x / d;
-  float acc = 0.f;
-  for (int j = part; j < T; j += nparts) acc = fmaf(sc[j], to_f32(vbase[(size_t)j * d + dd]), acc);
-  ov[threadIdx.x] = acc;
-  __syncthreads();
-  if (part == 0) {
-    for (int p2 = 1; p2 < nparts; ++p2) acc += ov[p2 * d + dd];
-    out[((size_t)r * hq + hqi) * d + dd] = from_f32<AT>(acc / sum);
-  }
-}
-
-int launch_attention_simt(const AttnArgs& a, cudaStream_t st, cudaError_t* err) {
-  size_t smem = (size_t)(a.d + 32 + 128 + a.cache_len + a.n) * sizeof(float);
-  dim3 grid(a.hq, a.n);
-  *err = cudaSuccess;
-  if (a.dtype == DT_F32) {
-    if (smem > 48 * 1024) *err = cudaFuncSetAttribute(attn_simt_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (*err != cudaSuccess) return -1;
-    attn_simt_kernel<float><<<grid, 128, smem, st>>>((const float*)a.q, (const float*)a.kc, (const float*)a.vc,
-                                                     (float*)a.out, a.n, a.cache_len, a.max_seq, a.hq, a.hkv, a.d, a.causal, a.row_mask);
-  } else {
-    if (smem > 48 * 1024) *err = cudaFuncSetAttribute(attn_simt_kernel<bf16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (*err != cudaSuccess) return -1;
-    attn_simt_kernel<bf16><<<grid, 128, smem, st>>>((const bf16*)a.q, (const bf16*)a.kc, (const bf16*)a.vc, (bf16*)a.out,
-                                                    a.n, a.cache_len, a.max_seq, a.hq, a.hkv, a.d, a.causal, a.row_mask);
-  }
-  *err = cudaGetLastError();
-  return *err == cudaSuccess ? 1 : -1;
 }
 
 }  // namespace fdk

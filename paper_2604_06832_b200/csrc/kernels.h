@@ -32,7 +32,6 @@ void launch_bf16_to_e5m2x3(const void* in, void* out, size_t n, cudaStream_t st)
 // the same row by row, leaving amax[row] = max |f16 value| of the row
 void launch_bf16_rows_to_f16_amax(const void* in, void* out, int m, int k, float* amax, cudaStream_t st);
 void launch_rows_to_f32(const void* rows, float* h, int n, int hidden, int dtype, cudaStream_t st);
-void launch_rmsnorm(const float* h, const float* g, void* out, int n, int hidden, float eps, int dtype, cudaStream_t st);
 void launch_rope_table(float* cs, int n, int pos0, int head_dim, float theta, cudaStream_t st, const int* len_ptr = nullptr,
                        KStamp* stamp = nullptr, const int* pos_off = nullptr);
 // quadratic self-speculative decoding (Appendix B, Alg. 2): row layout, input tokens, first draft, verify loop
@@ -46,12 +45,6 @@ void launch_quad_build(const int32_t* d, int B, int mask_id, int32_t* tokens, ui
 void launch_quad_first_draft(const int32_t* pred, int32_t first, int B, int32_t* d, cudaStream_t st);
 void launch_quad_accept(const int32_t* pred, int32_t* d, int B, int32_t* accepted, int32_t* out, cudaStream_t st);
 void launch_set_len(int* len_ptr, int value, cudaStream_t st);
-// qkv fp32 [n, (Hq + 2 Hkv) d] -> q (act type) [n, Hq, d] rotated; K (rotated) and V written into the
-// layer's cache planes [Hkv, max_seq, d] at positions pos0 .. pos0 + n - 1.
-void launch_qkv_post(const float* qkv, const float* cs, void* q, void* kc, void* vc, int n, int pos0,
-                     int hq, int hkv, int d, int max_seq, int dtype, cudaStream_t st);
-void launch_swiglu(const float* gu, void* act, int n, int inter, int dtype, cudaStream_t st);
-void launch_row_stats(const float* logits, int n, int vocab, int mask_id, float* conf, int32_t* pred, cudaStream_t st);
 // Unmask selection + block-state update.  info = {n_unmasked, n_remaining, step_index}.
 // loop = 1: the launch is the last node of a conditional WHILE body; it counts the iteration in info[5] and sets `cond`
 // to "masked positions remain".
@@ -62,6 +55,25 @@ void launch_select(const float* conf, const int32_t* pred, int32_t* tokens, uint
 void launch_accept(const int32_t* a, const int32_t* d, int n, int32_t* out, cudaStream_t st);
 void launch_init_block(int32_t* tokens, uint8_t* masked, int32_t* info, const int32_t* init, int n, int mask_id,
                        int step, cudaStream_t st);
+
+// ---- the exact fp32 path (exact_f32.cu) ---------------------------------------------------------------
+// One projection over m rows x [m, k], with the RMSNorm in front of it (gain set) and what follows it:
+//   QKV   : w = q, k, v; bias, rotary (cs); q rows into out, K / V rows into the cache planes kc, vc at pos0 (*len_ptr)
+//   RESID : out [m, n0] += x w^T
+//   SWIGLU: w = gate, up; out [m, n0] = silu(gate) * up
+//   LOGITS: out [m, n0] (nullable); stats[tile][m] (nullable): as TcOut's, one entry per 16 vocabulary ids
+enum { FL_QKV = 0, FL_RESID = 1, FL_SWIGLU = 2, FL_LOGITS = 3 };
+struct F32Linear {
+  int mode, m, k;
+  const float* x;
+  const float* gain; float inv_h, eps;
+  const float *w[3], *bias[3]; int n[3];
+  float *out, *kc, *vc;
+  const float* cs; const int* len_ptr; int pos0, hq, hkv, d, max_seq;
+  float4* stats; int mask_id;
+};
+int f32_logit_tiles(int vocab);
+cudaError_t launch_linear_f32(const F32Linear& p, cudaStream_t st);
 
 // ---- tensor-core (tcgen05 + TMA) small-M GEMM, bf16 ---------------------------------------------------
 enum { TC_MODE_PARTIAL = 0, TC_MODE_DIRECT = 1, TC_MODE_SWIGLU = 2, TC_MODE_LOGITS = 3 };
@@ -165,7 +177,7 @@ struct AttnArgs {
   int long_cache;       // tensor-core kernel: -1 pick the CTA shape from cache_len; 0 / 1 the short- / long-cache shape
                         // (a captured launch serves every later length of its class)
   void* workspace;
-  const int* len_ptr;   // nullable: device word holding the cache length (overrides cache_len; tensor-core kernel only)
+  const int* len_ptr;   // nullable: device word holding the cache length (overrides cache_len)
   int* status;          // nullable: device status words (see TcOut::status)
   float* amax_out;      // nullable (tensor-core kernel): [n][hq] maxima of |out| as stored, per row and head
   KStamp* stamp;        // nullable: two consecutive entries (attention, chunk merge)
