@@ -182,7 +182,7 @@ struct AttnArgs {
   float* amax_out;      // nullable (tensor-core kernel): [n][hq] maxima of |out| as stored, per row and head
   KStamp* stamp;        // nullable: two consecutive entries (attention, chunk merge)
 };
-// Prompt path: causal attention of any number of rows, one CTA per (128 rows, query head), no key split (prefill_attn.cu).
+// Prompt path: causal attention of any number of rows, one CTA per (256 rows, query head), no key split (prefill_attn.cu).
 cudaError_t launch_prefill_attention(const AttnArgs& a, cudaStream_t st);
 size_t attention_workspace_bytes(int n, int hq, int hkv, int d);
 bool attention_long_cache(int keys);   // whether the tensor-core kernel takes its long-cache shape for this many keys

@@ -1,233 +1,288 @@
 // Causal GQA attention of the prompt path: row i (position L + i) reads keys 0 .. L + i.
 //
-// One CTA = 128 consecutive rows of one query head; eight compute warps of 16 rows each, one producer warp that fetches
-// 64-key K and V tiles by 2-D TMA into a ring.  Hundreds of CTAs exist at any prompt length, so keys are not split and
-// the normalised result is written directly as the O projection's input.  CTAs with the most keys come first.
-// mma.sync m16n8k16, fp32 online softmax as in the decode kernel (attention.cu).
+// One CTA = two tiles of 128 consecutive rows of one query head.  S = Q K^T and O += P V run on the 5th-generation tensor
+// cores (tcgen05.mma, 128 keys at a time) with S, P and O in tensor memory: P replaces S in place and is the A operand of
+// the second product from there.  One softmax thread owns a row, so the online softmax needs no shuffles; O is rescaled
+// only when a row's maximum has grown by more than 2^8, until then P is taken relative to the old reference (values up to
+// 256, sums in fp32).  While the four warps of one row tile do their exponentials, the tensor cores work for the other
+// tile.  Bound by the exponentials: 2 x 128 x 128 of them per step at 16 per clock are 2048 clocks against 1024 of MMAs.
+// V stays as it lies in the cache ([key][dim], an MN-major operand).  Hundreds of CTAs exist at any prompt length, so keys
+// are not split and the normalised result is written directly as the O projection's input; CTAs with the most keys come
+// first.  (mma.sync with 16 rows per warp: %PA%.)
+// Every mbarrier wait is bounded as in gemm_tc.cu.
 #include "attn_plan.cuh"
 #include "kernels.h"
 #include "tc_ptx.cuh"
 
 namespace fdk {
 
+constexpr int PA_THREADS = 384;     // warp 0 TMA producer, warp 1 MMA issuer, warps 4..7 / 8..11 softmax of row tile 0 / 1
+constexpr int PA_KEYS = 128;
+constexpr int PA_ROWS = 256;        // per CTA
+
 template <int D>
 struct PaSmem {
-  static constexpr int ROWS = 128, NW = ROWS / 16, THREADS = NW * 32 + 32;
-  static constexpr int STAGES = D == 128 ? 4 : 8;
-  static constexpr int Q_BYTES = ROWS * D * 2;
-  static constexpr int TILE_BYTES = AT_KEYS * D * 2;
-  static constexpr int STAGE_BYTES = 2 * TILE_BYTES;
-  static constexpr int BAR_OFF = Q_BYTES + STAGES * STAGE_BYTES;
-  static constexpr int TOTAL = BAR_OFF + 8 * (2 * STAGES) + 16 + 1024;
+  static constexpr int TILE_BYTES = 128 * D * 2;        // a Q, K or V tile: D / 64 blocks of [128 rows][128 bytes], swizzled
+  static constexpr int K_OFF = 2 * TILE_BYTES, V_OFF = K_OFF + 2 * TILE_BYTES;
+  static constexpr int BAR_OFF = V_OFF + 2 * TILE_BYTES;
+  static constexpr int TOTAL = BAR_OFF + 256 + 1024;
 };
 
 struct PaParams {
-  CUtensorMap tm_k, tm_v;     // [Hkv * max_seq, D] planes, box {64, 64}
-  const void* q;              // [n, Hq, D]
+  CUtensorMap tm_q;           // [n, Hq * D], box {64, 128}
+  CUtensorMap tm_k, tm_v;     // [Hkv * max_seq, D] planes, box {64, 128}
   void* out; size_t lo_off; int fmt;
   int n, L, max_seq, hq, hkv;
   int* status;
 };
 
+__device__ __forceinline__ float ex2(float x) {
+  float r;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
 template <int D, typename E>
-__global__ void __launch_bounds__(PaSmem<D>::THREADS, 1) prefill_attn_kernel(const __grid_constant__ PaParams p) {
+__global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const __grid_constant__ PaParams p) {
   using S = PaSmem<D>;
-  constexpr int CH = D / 8, NW = S::NW, NCT = NW * 32;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
-  const uint32_t sQ = (raw + 1023u) & ~1023u;
-  uint8_t* sm = smem_raw + (sQ - raw);
-  const uint32_t sKV = sQ + S::Q_BYTES, bar0 = sQ + S::BAR_OFF;
-  auto full_bar = [&](int s) { return bar0 + 8u * s; };
-  auto empty_bar = [&](int s) { return bar0 + 8u * (S::STAGES + s); };
-  volatile int* abort_flag = (volatile int*)(sm + S::BAR_OFF + 8 * (2 * S::STAGES));
+  const uint32_t base = (raw + 1023u) & ~1023u;
+  uint8_t* sm = smem_raw + (base - raw);
+  const uint32_t bar0 = base + S::BAR_OFF;
+  const uint32_t q_full = bar0;
+  auto k_full = [&](int s) { return bar0 + 8u + 8u * s; };
+  auto k_empty = [&](int s) { return bar0 + 24u + 8u * s; };
+  auto v_full = [&](int s) { return bar0 + 40u + 8u * s; };
+  auto v_empty = [&](int s) { return bar0 + 56u + 8u * s; };
+  auto s_full = [&](int q) { return bar0 + 72u + 8u * q; };
+  auto p_full = [&](int q) { return bar0 + 88u + 8u * q; };
+  auto o_full = [&](int q) { return bar0 + 104u + 8u * q; };
+  volatile uint32_t* tmem_slot = (volatile uint32_t*)(sm + S::BAR_OFF + 120);
+  volatile int* abort_flag = (volatile int*)(sm + S::BAR_OFF + 124);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  pdl_trigger();
   if (tid == 0) {
-    for (int s = 0; s < S::STAGES; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), NW); }
+    mbar_init(q_full, 1);
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(k_full(i), 1); mbar_init(k_empty(i), 1); mbar_init(v_full(i), 1); mbar_init(v_empty(i), 1);
+      mbar_init(s_full(i), 1); mbar_init(p_full(i), 4); mbar_init(o_full(i), 1);
+    }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32((const void*)tmem_slot)), "r"(512) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = *tmem_slot;            // columns: S0 / P0 at 0, S1 / P1 at 128, O0 at 256, O1 at 384
+  pdl_trigger();            // (holding its tensor memory: see gemm_tc.cu)
   pdl_wait();
-  const int head = blockIdx.x, hk = head / (p.hq / p.hkv);
-  const int i0 = (int)(gridDim.y - 1 - blockIdx.y) * S::ROWS;
-  const int rows = min(S::ROWS, p.n - i0);
-  const int key_end = p.L + i0 + rows;                       // exclusive
-  const int n_tiles = (key_end + AT_KEYS - 1) / AT_KEYS;
 
-  if (warp == NW) {
+  const int head = blockIdx.x, hk = head / (p.hq / p.hkv);
+  const int i0 = (int)(gridDim.y - 1 - blockIdx.y) * PA_ROWS;
+  // key tiles of the two row tiles: up to the last row's own position (a row tile past the end of the prompt: none)
+  const int rows0 = min(128, p.n - i0), rows1 = min(128, p.n - i0 - 128);
+  const int n0 = (p.L + i0 + rows0 + PA_KEYS - 1) / PA_KEYS;
+  const int n1 = rows1 > 0 ? (p.L + i0 + 128 + rows1 + PA_KEYS - 1) / PA_KEYS : 0;
+  const int nt = max(n0, n1);
+
+  if (warp == 0) {
     if (lane == 0) {
       const bool poisoned = p.status && *reinterpret_cast<const volatile int*>(p.status + 1) != 0;   // host-set test hook
       if (poisoned) *abort_flag = 1;
       bool ok = !poisoned;
-      uint32_t armed = 0, armed_parity = 0;
-      for (int t = 0; t < n_tiles && ok; ++t) {
-        const int stage = t % S::STAGES;
-        const uint32_t phase = (uint32_t)(t / S::STAGES) & 1u;
-        if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag)) { ok = false; break; }
-        mbar_expect_tx(full_bar(stage), S::STAGE_BYTES);
-        armed |= 1u << stage;
-        armed_parity = (armed_parity & ~(1u << stage)) | (phase << stage);
-        const uint32_t dst = sKV + stage * S::STAGE_BYTES;
-        const int row = hk * p.max_seq + t * AT_KEYS;
-#pragma unroll
-        for (int hd = 0; hd < D / 64; ++hd) {
-          tma_load_2d_plain(dst + hd * (AT_KEYS * 128), &p.tm_k, full_bar(stage), hd * 64, row);
-          tma_load_2d_plain(dst + S::TILE_BYTES + hd * (AT_KEYS * 128), &p.tm_v, full_bar(stage), hd * 64, row);
-        }
+      uint32_t k_armed = 0, v_armed = 0, k_par = 0, v_par = 0;
+      if (ok) {
+        mbar_expect_tx(q_full, 2 * S::TILE_BYTES);
+        for (int q = 0; q < 2; ++q)
+          for (int b = 0; b < D / 64; ++b)
+            tma_load_2d_plain(base + q * S::TILE_BYTES + b * 16384, &p.tm_q, q_full, head * D + b * 64, i0 + q * 128);
+      }
+      for (int j = 0; j < nt && ok; ++j) {
+        const int s = j & 1;
+        const uint32_t ph = (uint32_t)(j >> 1) & 1u;
+        const int row = hk * p.max_seq + j * PA_KEYS;
+        if (!mbar_wait(k_empty(s), ph ^ 1u, abort_flag)) { ok = false; break; }
+        mbar_expect_tx(k_full(s), S::TILE_BYTES);
+        k_armed |= 1u << s; k_par = (k_par & ~(1u << s)) | (ph << s);
+        for (int b = 0; b < D / 64; ++b) tma_load_2d_plain(base + S::K_OFF + s * S::TILE_BYTES + b * 16384, &p.tm_k, k_full(s), b * 64, row);
+        if (!mbar_wait(v_empty(s), ph ^ 1u, abort_flag)) { ok = false; break; }
+        mbar_expect_tx(v_full(s), S::TILE_BYTES);
+        v_armed |= 1u << s; v_par = (v_par & ~(1u << s)) | (ph << s);
+        for (int b = 0; b < D / 64; ++b) tma_load_2d_plain(base + S::V_OFF + s * S::TILE_BYTES + b * 16384, &p.tm_v, v_full(s), b * 64, row);
       }
       if (!ok) {
         if (p.status) atomicCAS(p.status, 0, ST_ATTENTION);
-        for (int s = 0; s < S::STAGES; ++s) {
-          if (!(armed & (1u << s))) continue;
-          const uint32_t par = (armed_parity >> s) & 1u;
+        auto drain = [&](uint32_t bar, uint32_t par) {       // wait (bounded) for the copies in flight
           const long long t0 = clock64();
-          while (!mbar_try_wait(full_bar(s), par) && clock64() - t0 < TC_TIMEOUT) {}
+          while (!mbar_try_wait(bar, par) && clock64() - t0 < TC_TIMEOUT) {}
+        };
+        if (!poisoned) drain(q_full, 0);
+        for (int s = 0; s < 2; ++s) {
+          if (k_armed & (1u << s)) drain(k_full(s), (k_par >> s) & 1u);
+          if (v_armed & (1u << s)) drain(v_full(s), (v_par >> s) & 1u);
         }
       }
     }
-  } else {
-    const E* q = reinterpret_cast<const E*>(p.q);
-    for (int v = tid; v < S::ROWS * CH; v += NCT) {
-      const int r = v / CH, c = v % CH;
-      const bool live = r < rows;
-      cp_async16(sQ + swz_q<D>(r, c), live ? (const void*)(q + ((size_t)(i0 + r) * p.hq + head) * D + c * 8) : (const void*)q, live ? 16 : 0);
-    }
-    cp_async_commit();
-    cp_async_wait<0>();
-    asm volatile("bar.sync 1, %0;" ::"n"(NCT) : "memory");
-    const int row0 = warp * 16, g = lane >> 2, tq = lane & 3;
-    const int r_lo = row0 + g, r_hi = r_lo + 8;
-    // last visible key (exclusive); a row past the end of the prompt sees none
-    const int lim_lo = r_lo < rows ? p.L + i0 + r_lo + 1 : 0, lim_hi = r_hi < rows ? p.L + i0 + r_hi + 1 : 0;
-    const int warp_first = p.L + i0 + row0 + 1;               // keys that every row of the warp sees
-    const int warp_last = p.L + i0 + row0 + 16;               // keys beyond this are seen by none
-    const float sl2 = rsqrtf((float)D) * LOG2E;
-    uint32_t qf[D / 16][4];
+  } else if (warp == 1) {
+    if (lane == 0) {
+      constexpr bool F16 = sizeof(E) == 2 && !__is_same(E, bf16);
+      const uint32_t id_s = F16 ? umma_idesc_f16(PA_KEYS) : umma_idesc_bf16(PA_KEYS);
+      const uint32_t id_o = (F16 ? umma_idesc_f16(D) : umma_idesc_bf16(D)) | (1u << 16);      // (V: MN-major)
+      bool ok = mbar_wait(q_full, 0, abort_flag);
+      auto score = [&](int q, int j) {
+        const uint32_t qa = base + q * S::TILE_BYTES, ka = base + S::K_OFF + (j & 1) * S::TILE_BYTES;
 #pragma unroll
-    for (int kk = 0; kk < D / 16; ++kk)
-      ldsm_x4(sQ + swz_q<D>(row0 + (lane & 15), kk * 2 + (lane >> 4)), qf[kk][0], qf[kk][1], qf[kk][2], qf[kk][3]);
-    float o[D / 8][4];
+        for (int kk = 0; kk < D / 16; ++kk)
+          umma_bf16(tmem + q * 128, umma_desc_sw128(qa + (kk >> 2) * 16384) + 2u * (kk & 3), umma_desc_sw128(ka + (kk >> 2) * 16384) + 2u * (kk & 3),
+                    id_s, kk > 0 ? 1u : 0u);
+        umma_commit(s_full(q));
+      };
+      auto value = [&](int q, int j) {
+        if (!mbar_wait(p_full(q), (uint32_t)j & 1u, abort_flag)) { ok = false; return; }
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint64_t vd = umma_desc_sw128_mn(base + S::V_OFF + (j & 1) * S::TILE_BYTES, 16384);
 #pragma unroll
-    for (int i = 0; i < D / 8; ++i) { o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f; }
-    float m_lo = -INFINITY, m_hi = -INFINITY, l_lo = 0.f, l_hi = 0.f;
-    bool ok = true;
-    for (int t = 0; t < n_tiles && ok; ++t) {
-      const int stage = t % S::STAGES;
-      const uint32_t phase = (uint32_t)(t / S::STAGES) & 1u;
-      if (!mbar_wait(full_bar(stage), phase, abort_flag)) { ok = false; break; }
-      const uint32_t kt = sKV + stage * S::STAGE_BYTES, vt = kt + S::TILE_BYTES;
-      const int j0 = t * AT_KEYS;
-      if (j0 + AT_KEYS > key_end) {
-        // V rows past the last key hold whatever the cache holds there, and 0 x NaN would poison the product: every warp
-        // clears them (the same zeros) before it reads any
-        const int first = key_end - j0;
-        for (int v = lane; v < (AT_KEYS - first) * CH; v += 32) {
-          const int r = first + v / CH, c = v % CH;
-          asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(vt + swz_kv(r, c)), "r"(0u) : "memory");
+        for (int kk = 0; kk < PA_KEYS / 16; ++kk)
+          umma_f16_ta(tmem + 256 + q * 128, tmem + q * 128 + kk * 8, vd + (uint64_t)(kk * 128), id_o, (j > 0 || kk > 0) ? 1u : 0u);
+      };
+      auto wait_k = [&](int j) { if (ok && !mbar_wait(k_full(j & 1), (uint32_t)(j >> 1) & 1u, abort_flag)) ok = false; };
+      wait_k(0);
+      if (ok) {
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        score(0, 0);
+        if (n1 > 0) score(1, 0);
+        umma_commit(k_empty(0));
+      }
+      for (int j = 0; j < nt && ok; ++j) {
+        if (!mbar_wait(v_full(j & 1), (uint32_t)(j >> 1) & 1u, abort_flag)) { ok = false; break; }
+        if (j < n0) {
+          value(0, j);
+          if (!ok) break;
+          if (j + 1 == n0) umma_commit(o_full(0));
         }
+        if (j + 1 < nt) wait_k(j + 1);
+        if (!ok) break;
+        if (j + 1 < n0) score(0, j + 1);
+        if (j < n1) {
+          value(1, j);
+          if (!ok) break;
+          if (j + 1 == n1) umma_commit(o_full(1));
+        }
+        umma_commit(v_empty(j & 1));
+        if (j + 1 < n1) score(1, j + 1);
+        if (j + 1 < nt) umma_commit(k_empty((j + 1) & 1));
+      }
+      if (!ok && p.status) atomicCAS(p.status, 0, ST_ATTENTION);
+    }
+  } else if (warp >= 4) {
+    const int q = (warp - 4) >> 2, wq = warp & 3;
+    const int nq = q ? n1 : n0;
+    const int i = i0 + q * 128 + wq * 32 + lane;              // this thread's row
+    const int lim = p.L + min(i, p.n - 1) + 1;                // keys that it reads
+    const int lim_first = p.L + i0 + q * 128 + wq * 32 + 1;   // keys that every row of the warp reads
+    const int key_end = p.L + p.n;                            // (keys beyond this tile but before it are other rows' own)
+    const uint32_t ts = tmem + ((uint32_t)(wq * 32) << 16) + q * 128, to = ts + 256;
+    const float sl2 = rsqrtf((float)D) * LOG2E;               // scores in the log2 domain
+    float m_ref = -INFINITY, l = 0.f;
+    bool ok = true;
+    for (int j = 0; j < nq && ok; ++j) {
+      if (!mbar_wait(s_full(q), (uint32_t)j & 1u, abort_flag)) { ok = false; break; }
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      float s[PA_KEYS];
+#pragma unroll
+      for (int c = 0; c < PA_KEYS; c += 32) tmem_ld32(ts + c, s + c);
+      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+      const int j0 = j * PA_KEYS;
+      if (j0 + PA_KEYS > lim_first) {                         // the diagonal (uniform over the warp)
+#pragma unroll
+        for (int c = 0; c < PA_KEYS; ++c)
+          if (j0 + c >= lim) s[c] = -INFINITY;
+      }
+      float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+      for (int c = 0; c < PA_KEYS; c += 4) {
+        mx[0] = fmaxf(mx[0], s[c]); mx[1] = fmaxf(mx[1], s[c + 1]); mx[2] = fmaxf(mx[2], s[c + 2]); mx[3] = fmaxf(mx[3], s[c + 3]);
+      }
+      const float m = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * sl2;
+      const bool grow = m > m_ref + 8.f;                      // (always in the first tile: every row reads key 0)
+      if (j > 0 && __any_sync(0xffffffffu, grow)) {
+        // s_full also says that the product of the tile before is complete: O may be rewritten
+        const float f = grow ? ex2(m_ref - m) : 1.f;
+#pragma unroll 1
+        for (int c = 0; c < D; c += 16) {
+          float o[16];
+          tmem_ld16(to + c, o);
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+          for (int k = 0; k < 16; ++k) o[k] *= f;
+          tmem_st16(to + c, reinterpret_cast<const uint32_t*>(o));
+        }
+        l *= f;
+      }
+      if (grow) m_ref = m;
+      float sum[4] = {0.f, 0.f, 0.f, 0.f};
+      uint32_t pk[PA_KEYS / 2];
+#pragma unroll
+      for (int c = 0; c < PA_KEYS; c += 4) {
+        float e[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) { e[k] = ex2(fmaf(s[c + k], sl2, -m_ref)); sum[k] += e[k]; }
+        pk[c / 2] = pack2<E>(e[0], e[1]);
+        pk[c / 2 + 1] = pack2<E>(e[2], e[3]);
+      }
+      l += (sum[0] + sum[1]) + (sum[2] + sum[3]);
+#pragma unroll
+      for (int c = 0; c < PA_KEYS / 2; c += 16) tmem_st16(ts + c, pk + c);
+      if (j0 + PA_KEYS > key_end) {
+        // V rows past the last key hold whatever the cache holds there, and 0 x NaN would poison the product: cleared by
+        // both row tiles (the same zeros)
+        if (!mbar_wait(v_full(j & 1), (uint32_t)(j >> 1) & 1u, abort_flag)) ok = false;
+        const int first = key_end - j0;
+        for (int v = wq * 32 + lane; ok && v < (PA_KEYS - first) * (D / 8); v += 128) {
+          const int r = first + v / (D / 8), c = v % (D / 8);
+          const uint32_t a = base + S::V_OFF + (j & 1) * S::TILE_BYTES + (c >> 3) * 16384 + r * 128 + (((c & 7) ^ (r & 7)) << 4);
+          asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(a), "r"(0u) : "memory");
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncwarp();
       }
-      if (j0 < warp_last && row0 < rows) {
-        float s[AT_KEYS / 8][4];
+      asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) mbar_arrive(p_full(q));
+    }
+    if (nq > 0 && ok && !mbar_wait(o_full(q), 0, abort_flag)) ok = false;
+    if (nq > 0 && ok) {
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const float inv = 1.f / l;
+      const size_t idx = ((size_t)i * p.hq + head) * D;
+#pragma unroll 1
+      for (int c = 0; c < D; c += 32) {
+        float o[32];
+        __syncwarp();
+        tmem_ld32(to + c, o);
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        if (i < p.n) {
 #pragma unroll
-        for (int i = 0; i < AT_KEYS / 8; ++i) { s[i][0] = s[i][1] = s[i][2] = s[i][3] = 0.f; }
-#pragma unroll
-        for (int kk = 0; kk < D / 16; ++kk) {
-#pragma unroll
-          for (int np = 0; np < AT_KEYS / 16; ++np) {
-            uint32_t b0, b1, b2, b3;
-            ldsm_x4(kt + swz_kv(np * 16 + (lane & 7) + ((lane >> 4) << 3), kk * 2 + ((lane >> 3) & 1)), b0, b1, b2, b3);
-            mma_16816<E>(s[2 * np], qf[kk], b0, b1);
-            mma_16816<E>(s[2 * np + 1], qf[kk], b2, b3);
-          }
-        }
-        if (j0 + AT_KEYS > warp_first || row0 + 16 > rows) {   // the diagonal tiles (uniform over the warp)
-#pragma unroll
-          for (int nt = 0; nt < AT_KEYS / 8; ++nt) {
-            const int j = j0 + nt * 8 + tq * 2;
-            if (j >= lim_lo) s[nt][0] = -INFINITY;
-            if (j + 1 >= lim_lo) s[nt][1] = -INFINITY;
-            if (j >= lim_hi) s[nt][2] = -INFINITY;
-            if (j + 1 >= lim_hi) s[nt][3] = -INFINITY;
-          }
-        }
-        float mx_lo = -INFINITY, mx_hi = -INFINITY;
-#pragma unroll
-        for (int nt = 0; nt < AT_KEYS / 8; ++nt) {
-          mx_lo = fmaxf(mx_lo, fmaxf(s[nt][0], s[nt][1]));
-          mx_hi = fmaxf(mx_hi, fmaxf(s[nt][2], s[nt][3]));
-        }
-        mx_lo = fmaxf(mx_lo, __shfl_xor_sync(0xffffffffu, mx_lo, 1));
-        mx_lo = fmaxf(mx_lo, __shfl_xor_sync(0xffffffffu, mx_lo, 2));
-        mx_hi = fmaxf(mx_hi, __shfl_xor_sync(0xffffffffu, mx_hi, 1));
-        mx_hi = fmaxf(mx_hi, __shfl_xor_sync(0xffffffffu, mx_hi, 2));
-        const float mn_lo = fmaxf(m_lo, mx_lo * sl2), mn_hi = fmaxf(m_hi, mx_hi * sl2);
-        const float ref_lo = (mn_lo == -INFINITY) ? 0.f : mn_lo, ref_hi = (mn_hi == -INFINITY) ? 0.f : mn_hi;
-        const float al_lo = exp2f(m_lo - ref_lo), al_hi = exp2f(m_hi - ref_hi);
-        m_lo = mn_lo; m_hi = mn_hi;
-        float sum_lo = 0.f, sum_hi = 0.f;
-#pragma unroll
-        for (int nt = 0; nt < AT_KEYS / 8; ++nt) {
-          s[nt][0] = exp2f(fmaf(s[nt][0], sl2, -ref_lo)); s[nt][1] = exp2f(fmaf(s[nt][1], sl2, -ref_lo));
-          s[nt][2] = exp2f(fmaf(s[nt][2], sl2, -ref_hi)); s[nt][3] = exp2f(fmaf(s[nt][3], sl2, -ref_hi));
-          sum_lo += s[nt][0] + s[nt][1];
-          sum_hi += s[nt][2] + s[nt][3];
-        }
-        l_lo = l_lo * al_lo + sum_lo;
-        l_hi = l_hi * al_hi + sum_hi;
-#pragma unroll
-        for (int i = 0; i < D / 8; ++i) { o[i][0] *= al_lo; o[i][1] *= al_lo; o[i][2] *= al_hi; o[i][3] *= al_hi; }
-#pragma unroll
-        for (int kk = 0; kk < AT_KEYS / 16; ++kk) {
-          uint32_t pa[4];
-          pa[0] = pack2<E>(s[2 * kk][0], s[2 * kk][1]);
-          pa[1] = pack2<E>(s[2 * kk][2], s[2 * kk][3]);
-          pa[2] = pack2<E>(s[2 * kk + 1][0], s[2 * kk + 1][1]);
-          pa[3] = pack2<E>(s[2 * kk + 1][2], s[2 * kk + 1][3]);
-#pragma unroll
-          for (int dp = 0; dp < D / 16; ++dp) {
-            uint32_t b0, b1, b2, b3;
-            ldsm_x4_t(vt + swz_kv(kk * 16 + (lane & 7) + (((lane >> 3) & 1) << 3), dp * 2 + (lane >> 4)), b0, b1, b2, b3);
-            mma_16816<E>(o[2 * dp], pa, b0, b1);
-            mma_16816<E>(o[2 * dp + 1], pa, b2, b3);
-          }
+          for (int k = 0; k < 32; k += 4)
+            store_act4(p.out, p.lo_off, idx + c + k, make_float4(o[k] * inv, o[k + 1] * inv, o[k + 2] * inv, o[k + 3] * inv), p.fmt);
         }
       }
-      __syncwarp();
-      if (lane == 0) mbar_arrive(empty_bar(stage));
     }
     if (!ok && lane == 0 && p.status) atomicCAS(p.status, 0, ST_ATTENTION);
-    l_lo += __shfl_xor_sync(0xffffffffu, l_lo, 1);
-    l_lo += __shfl_xor_sync(0xffffffffu, l_lo, 2);
-    l_hi += __shfl_xor_sync(0xffffffffu, l_hi, 1);
-    l_hi += __shfl_xor_sync(0xffffffffu, l_hi, 2);
-#pragma unroll
-    for (int half = 0; half < 2; ++half) {
-      const int r = half ? r_hi : r_lo;
-      if (r >= rows || !ok) continue;
-      const float inv = 1.f / (half ? l_hi : l_lo);
-      const size_t idx = ((size_t)(i0 + r) * p.hq + head) * D + tq * 2;
-#pragma unroll
-      for (int dt = 0; dt < D / 8; ++dt) {
-        const float v0 = o[dt][2 * half] * inv, v1 = o[dt][2 * half + 1] * inv;
-        uint32_t* dst = reinterpret_cast<uint32_t*>(reinterpret_cast<unsigned short*>(p.out) + idx + dt * 8);
-        if (p.fmt == XF_F16) {
-          *dst = (uint32_t)f16_bits_sat(v0) | ((uint32_t)f16_bits_sat(v1) << 16);
-        } else {
-          const __nv_bfloat162 h = __floats2bfloat162_rn(v0, v1);
-          *dst = *reinterpret_cast<const uint32_t*>(&h);
-          if (p.fmt == XF_BF16X2) {
-            const __nv_bfloat162 l = __floats2bfloat162_rn(v0 - __low2float(h), v1 - __high2float(h));
-            *reinterpret_cast<uint32_t*>(reinterpret_cast<unsigned short*>(p.out) + p.lo_off + idx + dt * 8) = *reinterpret_cast<const uint32_t*>(&l);
-          }
-        }
-      }
-    }
   }
+  __syncwarp();
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();     // the producer's copies have all been consumed (or drained) before any thread leaves
+  if (warp == 1) {
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+  }
 }
 
 template <int D, typename E>
@@ -236,16 +291,17 @@ static cudaError_t pa_launch_t(const PaParams& p, cudaStream_t st) {
   static bool attr_set[MAX_DEVICES] = {};
   cudaError_t e = ensure_dynamic_smem(prefill_attn_kernel<D, E>, S::TOTAL, attr_set);
   if (e != cudaSuccess) return e;
-  return launch_pdl(prefill_attn_kernel<D, E>, dim3(p.hq, ceil_div(p.n, S::ROWS)), dim3(S::THREADS), (size_t)S::TOTAL, st, p);
+  return launch_pdl(prefill_attn_kernel<D, E>, dim3(p.hq, ceil_div(p.n, PA_ROWS)), dim3(PA_THREADS), (size_t)S::TOTAL, st, p);
 }
 
 cudaError_t launch_prefill_attention(const AttnArgs& a, cudaStream_t st) {
   PaParams p;
   memset(&p, 0, sizeof(p));
   const int kind = a.kv_type == KV_F16 ? TM_F16 : TM_BF16;
-  if (!make_tmap(&p.tm_k, a.kc, a.hkv * a.max_seq, a.d, AT_KEYS, kind) || !make_tmap(&p.tm_v, a.vc, a.hkv * a.max_seq, a.d, AT_KEYS, kind))
+  if (!make_tmap(&p.tm_q, a.q, a.n, a.hq * a.d, 128, kind) || !make_tmap(&p.tm_k, a.kc, a.hkv * a.max_seq, a.d, PA_KEYS, kind) ||
+      !make_tmap(&p.tm_v, a.vc, a.hkv * a.max_seq, a.d, PA_KEYS, kind))
     return cudaErrorInvalidValue;
-  p.q = a.q; p.out = a.out; p.lo_off = a.out_lo_off; p.fmt = a.out_fmt;
+  p.out = a.out; p.lo_off = a.out_lo_off; p.fmt = a.out_fmt;
   p.n = a.n; p.L = a.cache_len; p.max_seq = a.max_seq; p.hq = a.hq; p.hkv = a.hkv; p.status = a.status;
   if (a.kv_type == KV_F16) return a.d == 128 ? pa_launch_t<128, __half>(p, st) : pa_launch_t<64, __half>(p, st);
   return a.d == 128 ? pa_launch_t<128, bf16>(p, st) : pa_launch_t<64, bf16>(p, st);
