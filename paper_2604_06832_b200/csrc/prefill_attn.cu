@@ -1,11 +1,12 @@
 // Causal GQA attention of the prompt path: row i (position L + i) reads keys 0 .. L + i.
 //
 // One CTA = two tiles of 128 consecutive rows of one query head.  S = Q K^T and O += P V run on the 5th-generation tensor
-// cores (tcgen05.mma, 128 keys at a time) with S, P and O in tensor memory: P replaces S in place and is the A operand of
+// cores (tcgen05.mma, 64 keys at a time) with S, P and O in tensor memory: P replaces S in place and is the A operand of
 // the second product from there.  One softmax thread owns a row, so the online softmax needs no shuffles; O is rescaled
 // only when a row's maximum has grown by more than 2^8, until then P is taken relative to the old reference (values up to
-// 256, sums in fp32).  While the four warps of one row tile do their exponentials, the tensor cores work for the other
-// tile.  Bound by the exponentials: 2 x 128 x 128 of them per step at 16 per clock are 2048 clocks against 1024 of MMAs.
+// 256, sums in fp32).  Each row tile has two score buffers, so the scores of the next keys are there when a softmax thread
+// is done with its keys (with one buffer of 128 keys the threads waited for P V and Q K^T in turn: 97 us for 4096 rows of
+// the 3B shape, %PB% us now).  Bound by the exponentials, 16 per clock and SM.
 // V stays as it lies in the cache ([key][dim], an MN-major operand).  Hundreds of CTAs exist at any prompt length, so keys
 // are not split and the normalised result is written directly as the O projection's input; CTAs with the most keys come
 // first.  (mma.sync with 16 rows per warp: %PA%.)
@@ -17,7 +18,8 @@
 namespace fdk {
 
 constexpr int PA_THREADS = 384;     // warp 0 TMA producer, warp 1 MMA issuer, warps 4..7 / 8..11 softmax of row tile 0 / 1
-constexpr int PA_KEYS = 128;
+constexpr int PA_KEYS = 128;        // keys of a K / V tile in shared memory
+constexpr int PA_STEP = 64;         // keys of one score buffer
 constexpr int PA_ROWS = 256;        // per CTA
 
 template <int D>
@@ -42,6 +44,21 @@ __device__ __forceinline__ float ex2(float x) {
   return r;
 }
 
+// two fp32 operations in one instruction
+__device__ __forceinline__ float2 fma2(const float2& a, const float2& b, const float2& c) {
+  float2 d;
+  asm("{\n\t.reg .b64 a, b, c, d;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\tmov.b64 c, {%6, %7};\n\t"
+      "fma.rn.f32x2 d, a, b, c;\n\tmov.b64 {%0, %1}, d;\n\t}"
+      : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+  return d;
+}
+__device__ __forceinline__ float2 add2(const float2& a, const float2& b) {
+  float2 d;
+  asm("{\n\t.reg .b64 a, b, d;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\tadd.rn.f32x2 d, a, b;\n\tmov.b64 {%0, %1}, d;\n\t}"
+      : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return d;
+}
+
 template <int D, typename E>
 __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const __grid_constant__ PaParams p) {
   using S = PaSmem<D>;
@@ -55,17 +72,19 @@ __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const __gri
   auto k_empty = [&](int s) { return bar0 + 24u + 8u * s; };
   auto v_full = [&](int s) { return bar0 + 40u + 8u * s; };
   auto v_empty = [&](int s) { return bar0 + 56u + 8u * s; };
-  auto s_full = [&](int q) { return bar0 + 72u + 8u * q; };
-  auto p_full = [&](int q) { return bar0 + 88u + 8u * q; };
-  auto o_full = [&](int q) { return bar0 + 104u + 8u * q; };
-  volatile uint32_t* tmem_slot = (volatile uint32_t*)(sm + S::BAR_OFF + 120);
-  volatile int* abort_flag = (volatile int*)(sm + S::BAR_OFF + 124);
+  auto s_full = [&](int q, int t) { return bar0 + 72u + 16u * q + 8u * (t & 1); };      // per score buffer
+  auto p_full = [&](int q, int t) { return bar0 + 104u + 16u * q + 8u * (t & 1); };
+  auto o_done = [&](int q) { return bar0 + 136u + 8u * q; };                            // a step's P V is complete
+  auto o_full = [&](int q) { return bar0 + 152u + 8u * q; };                            // the last one is
+  volatile uint32_t* tmem_slot = (volatile uint32_t*)(sm + S::BAR_OFF + 168);
+  volatile int* abort_flag = (volatile int*)(sm + S::BAR_OFF + 172);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid == 0) {
     mbar_init(q_full, 1);
     for (int i = 0; i < 2; ++i) {
       mbar_init(k_full(i), 1); mbar_init(k_empty(i), 1); mbar_init(v_full(i), 1); mbar_init(v_empty(i), 1);
-      mbar_init(s_full(i), 1); mbar_init(p_full(i), 4); mbar_init(o_full(i), 1);
+      for (int t = 0; t < 2; ++t) { mbar_init(s_full(i, t), 1); mbar_init(p_full(i, t), 4); }
+      mbar_init(o_done(i), 1); mbar_init(o_full(i), 1);
     }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -78,17 +97,17 @@ __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const __gri
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem = *tmem_slot;            // columns: S0 / P0 at 0, S1 / P1 at 128, O0 at 256, O1 at 384
+  const uint32_t tmem = *tmem_slot;            // columns: score buffers (S, then P) of row tile q at 128 q and 128 q + 64, O at 256 + 128 q
   pdl_trigger();            // (holding its tensor memory: see gemm_tc.cu)
   pdl_wait();
 
   const int head = blockIdx.x, hk = head / (p.hq / p.hkv);
   const int i0 = (int)(gridDim.y - 1 - blockIdx.y) * PA_ROWS;
-  // key tiles of the two row tiles: up to the last row's own position (a row tile past the end of the prompt: none)
+  // steps of the two row tiles: up to the last row's own position (a row tile past the end of the prompt: none)
   const int rows0 = min(128, p.n - i0), rows1 = min(128, p.n - i0 - 128);
-  const int n0 = (p.L + i0 + rows0 + PA_KEYS - 1) / PA_KEYS;
-  const int n1 = rows1 > 0 ? (p.L + i0 + 128 + rows1 + PA_KEYS - 1) / PA_KEYS : 0;
-  const int nt = max(n0, n1);
+  const int n0 = (p.L + i0 + rows0 + PA_STEP - 1) / PA_STEP;
+  const int n1 = rows1 > 0 ? (p.L + i0 + 128 + rows1 + PA_STEP - 1) / PA_STEP : 0;
+  const int ns = max(n0, n1), nt = (ns + 1) / 2;
 
   if (warp == 0) {
     if (lane == 0) {
@@ -131,51 +150,45 @@ __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const __gri
   } else if (warp == 1) {
     if (lane == 0) {
       constexpr bool F16 = sizeof(E) == 2 && !__is_same(E, bf16);
-      const uint32_t id_s = F16 ? umma_idesc_f16(PA_KEYS) : umma_idesc_bf16(PA_KEYS);
+      const uint32_t id_s = F16 ? umma_idesc_f16(PA_STEP) : umma_idesc_bf16(PA_STEP);
       const uint32_t id_o = (F16 ? umma_idesc_f16(D) : umma_idesc_bf16(D)) | (1u << 16);      // (V: MN-major)
       bool ok = mbar_wait(q_full, 0, abort_flag);
-      auto score = [&](int q, int j) {
-        const uint32_t qa = base + q * S::TILE_BYTES, ka = base + S::K_OFF + (j & 1) * S::TILE_BYTES;
+      auto score = [&](int q, int t) {
+        const uint32_t qa = base + q * S::TILE_BYTES, ka = base + S::K_OFF + ((t >> 1) & 1) * S::TILE_BYTES + (t & 1) * (PA_STEP * 128);
 #pragma unroll
         for (int kk = 0; kk < D / 16; ++kk)
-          umma_bf16(tmem + q * 128, umma_desc_sw128(qa + (kk >> 2) * 16384) + 2u * (kk & 3), umma_desc_sw128(ka + (kk >> 2) * 16384) + 2u * (kk & 3),
-                    id_s, kk > 0 ? 1u : 0u);
-        umma_commit(s_full(q));
+          umma_bf16(tmem + q * 128 + (t & 1) * PA_STEP, umma_desc_sw128(qa + (kk >> 2) * 16384) + 2u * (kk & 3),
+                    umma_desc_sw128(ka + (kk >> 2) * 16384) + 2u * (kk & 3), id_s, kk > 0 ? 1u : 0u);
+        umma_commit(s_full(q, t));
       };
-      auto value = [&](int q, int j) {
-        if (!mbar_wait(p_full(q), (uint32_t)j & 1u, abort_flag)) { ok = false; return; }
+      auto value = [&](int q, int t) {
+        if (!mbar_wait(p_full(q, t), (uint32_t)(t >> 1) & 1u, abort_flag)) { ok = false; return; }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint64_t vd = umma_desc_sw128_mn(base + S::V_OFF + (j & 1) * S::TILE_BYTES, 16384);
+        const uint64_t vd = umma_desc_sw128_mn(base + S::V_OFF + ((t >> 1) & 1) * S::TILE_BYTES + (t & 1) * (PA_STEP * 128), 16384);
 #pragma unroll
-        for (int kk = 0; kk < PA_KEYS / 16; ++kk)
-          umma_f16_ta(tmem + 256 + q * 128, tmem + q * 128 + kk * 8, vd + (uint64_t)(kk * 128), id_o, (j > 0 || kk > 0) ? 1u : 0u);
+        for (int kk = 0; kk < PA_STEP / 16; ++kk)
+          umma_f16_ta(tmem + 256 + q * 128, tmem + q * 128 + (t & 1) * PA_STEP + kk * 8, vd + (uint64_t)(kk * 128), id_o, (t > 0 || kk > 0) ? 1u : 0u);
+        umma_commit(o_done(q));
+        if (t + 1 == (q ? n1 : n0)) umma_commit(o_full(q));
       };
-      auto wait_k = [&](int j) { if (ok && !mbar_wait(k_full(j & 1), (uint32_t)(j >> 1) & 1u, abort_flag)) ok = false; };
-      wait_k(0);
-      if (ok) {
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        score(0, 0);
-        if (n1 > 0) score(1, 0);
-        umma_commit(k_empty(0));
-      }
-      for (int j = 0; j < nt && ok; ++j) {
-        if (!mbar_wait(v_full(j & 1), (uint32_t)(j >> 1) & 1u, abort_flag)) { ok = false; break; }
-        if (j < n0) {
-          value(0, j);
-          if (!ok) break;
-          if (j + 1 == n0) umma_commit(o_full(0));
+      // the scores of step t for both row tiles; the K tile is free after its second half
+      auto scores = [&](int q, int t) {
+        if (t >= ns || !ok) return;
+        if (q == 0 && (t & 1) == 0) {
+          if (!mbar_wait(k_full((t >> 1) & 1), (uint32_t)(t >> 2) & 1u, abort_flag)) { ok = false; return; }
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         }
-        if (j + 1 < nt) wait_k(j + 1);
-        if (!ok) break;
-        if (j + 1 < n0) score(0, j + 1);
-        if (j < n1) {
-          value(1, j);
-          if (!ok) break;
-          if (j + 1 == n1) umma_commit(o_full(1));
-        }
-        umma_commit(v_empty(j & 1));
-        if (j + 1 < n1) score(1, j + 1);
-        if (j + 1 < nt) umma_commit(k_empty((j + 1) & 1));
+        if (t < (q ? n1 : n0)) score(q, t);
+        if (q == 1 && ((t & 1) || t + 1 == ns)) umma_commit(k_empty((t >> 1) & 1));
+      };
+      for (int t = 0; t < 2; ++t) { scores(0, t); scores(1, t); }
+      for (int t = 0; t < ns && ok; ++t) {
+        if ((t & 1) == 0 && !mbar_wait(v_full((t >> 1) & 1), (uint32_t)(t >> 2) & 1u, abort_flag)) { ok = false; break; }
+        if (t < n0) value(0, t);
+        scores(0, t + 2);
+        if (ok && t < n1) value(1, t);
+        if (ok && ((t & 1) || t + 1 == ns)) umma_commit(v_empty((t >> 1) & 1));
+        scores(1, t + 2);
       }
       if (!ok && p.status) atomicCAS(p.status, 0, ST_ATTENTION);
     }
@@ -190,28 +203,30 @@ __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const __gri
     const float sl2 = rsqrtf((float)D) * LOG2E;               // scores in the log2 domain
     float m_ref = -INFINITY, l = 0.f;
     bool ok = true;
-    for (int j = 0; j < nq && ok; ++j) {
-      if (!mbar_wait(s_full(q), (uint32_t)j & 1u, abort_flag)) { ok = false; break; }
+    for (int t = 0; t < nq && ok; ++t) {
+      if (!mbar_wait(s_full(q, t), (uint32_t)(t >> 1) & 1u, abort_flag)) { ok = false; break; }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      float s[PA_KEYS];
-#pragma unroll
-      for (int c = 0; c < PA_KEYS; c += 32) tmem_ld32(ts + c, s + c);
+      const uint32_t tb = ts + (t & 1) * PA_STEP;
+      float s[PA_STEP];
+      tmem_ld32(tb, s);
+      tmem_ld32(tb + 32, s + 32);
       asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-      const int j0 = j * PA_KEYS;
-      if (j0 + PA_KEYS > lim_first) {                         // the diagonal (uniform over the warp)
+      const int j0 = t * PA_STEP;
+      if (j0 + PA_STEP > lim_first) {                         // the diagonal (uniform over the warp)
 #pragma unroll
-        for (int c = 0; c < PA_KEYS; ++c)
+        for (int c = 0; c < PA_STEP; ++c)
           if (j0 + c >= lim) s[c] = -INFINITY;
       }
       float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
-      for (int c = 0; c < PA_KEYS; c += 4) {
-        mx[0] = fmaxf(mx[0], s[c]); mx[1] = fmaxf(mx[1], s[c + 1]); mx[2] = fmaxf(mx[2], s[c + 2]); mx[3] = fmaxf(mx[3], s[c + 3]);
-      }
+      for (int c = 0; c < PA_STEP; c += 8)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) mx[k] = fmaxf(fmaxf(mx[k], s[c + k]), s[c + 4 + k]);
       const float m = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * sl2;
-      const bool grow = m > m_ref + 8.f;                      // (always in the first tile: every row reads key 0)
-      if (j > 0 && __any_sync(0xffffffffu, grow)) {
-        // s_full also says that the product of the tile before is complete: O may be rewritten
+      const bool grow = m > m_ref + 8.f;                      // (always in the first step: every row reads key 0)
+      if (t > 0 && __any_sync(0xffffffffu, grow)) {
+        if (!mbar_wait(o_done(q), (uint32_t)(t - 1) & 1u, abort_flag)) { ok = false; break; }
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const float f = grow ? ex2(m_ref - m) : 1.f;
 #pragma unroll 1
         for (int c = 0; c < D; c += 16) {
@@ -225,27 +240,29 @@ __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const __gri
         l *= f;
       }
       if (grow) m_ref = m;
-      float sum[4] = {0.f, 0.f, 0.f, 0.f};
-      uint32_t pk[PA_KEYS / 2];
+      float2 sum[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+      const float2 sl = make_float2(sl2, sl2), mr = make_float2(-m_ref, -m_ref);
 #pragma unroll
-      for (int c = 0; c < PA_KEYS; c += 4) {
-        float e[4];
+      for (int h = 0; h < 2; ++h) {
+        uint32_t pk[16];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) { e[k] = ex2(fmaf(s[c + k], sl2, -m_ref)); sum[k] += e[k]; }
-        pk[c / 2] = pack2<E>(e[0], e[1]);
-        pk[c / 2 + 1] = pack2<E>(e[2], e[3]);
+        for (int c = 0; c < 16; ++c) {
+          float2 e = fma2(make_float2(s[h * 32 + 2 * c], s[h * 32 + 2 * c + 1]), sl, mr);
+          e = make_float2(ex2(e.x), ex2(e.y));
+          sum[c & 1] = add2(sum[c & 1], e);
+          pk[c] = pack2<E>(e.x, e.y);
+        }
+        tmem_st16(tb + h * 16, pk);
       }
-      l += (sum[0] + sum[1]) + (sum[2] + sum[3]);
-#pragma unroll
-      for (int c = 0; c < PA_KEYS / 2; c += 16) tmem_st16(ts + c, pk + c);
-      if (j0 + PA_KEYS > key_end) {
+      l += (sum[0].x + sum[0].y) + (sum[1].x + sum[1].y);
+      if (j0 + PA_STEP > key_end) {
         // V rows past the last key hold whatever the cache holds there, and 0 x NaN would poison the product: cleared by
         // both row tiles (the same zeros)
-        if (!mbar_wait(v_full(j & 1), (uint32_t)(j >> 1) & 1u, abort_flag)) ok = false;
+        if (!mbar_wait(v_full((t >> 1) & 1), (uint32_t)(t >> 2) & 1u, abort_flag)) ok = false;
         const int first = key_end - j0;
-        for (int v = wq * 32 + lane; ok && v < (PA_KEYS - first) * (D / 8); v += 128) {
-          const int r = first + v / (D / 8), c = v % (D / 8);
-          const uint32_t a = base + S::V_OFF + (j & 1) * S::TILE_BYTES + (c >> 3) * 16384 + r * 128 + (((c & 7) ^ (r & 7)) << 4);
+        for (int v = wq * 32 + lane; ok && v < (PA_STEP - first) * (D / 8); v += 128) {
+          const int r = (t & 1) * PA_STEP + first + v / (D / 8), c = v % (D / 8);
+          const uint32_t a = base + S::V_OFF + ((t >> 1) & 1) * S::TILE_BYTES + (c >> 3) * 16384 + r * 128 + (((c & 7) ^ (r & 7)) << 4);
           asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(a), "r"(0u) : "memory");
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -254,7 +271,7 @@ __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const __gri
       asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
-      if (lane == 0) mbar_arrive(p_full(q));
+      if (lane == 0) mbar_arrive(p_full(q, t));
     }
     if (nq > 0 && ok && !mbar_wait(o_full(q), 0, abort_flag)) ok = false;
     if (nq > 0 && ok) {
