@@ -304,7 +304,7 @@ __global__ void __launch_bounds__(KIND == TC_KIND_A8 ? TC_THREADS_A8 : TC_THREAD
     }
   } else if (warp == 1) {
     // ------------------------------------------------ MMA issuer --------------------------------------------------
-    if (lane == 0) {
+    {
       const uint32_t idesc = A8 ? umma_idesc_e4m3(M_PAD) : (X3 ? umma_idesc_e4m3_e5m2(3 * M_PAD) : umma_idesc_bf16(p.has_lo ? 2 * M_PAD : M_PAD));
       int stage = 0, cbuf = 0;
       uint32_t phase = 0, cphase = 0;
@@ -329,6 +329,7 @@ __global__ void __launch_bounds__(KIND == TC_KIND_A8 ? TC_THREADS_A8 : TC_THREAD
           const uint32_t c_addr = base + L::CONV_OFF + cbuf * L::CONV_BYTES;
           const uint64_t adesc = umma_desc_sw128(a_addr);
           const uint64_t bdesc = umma_desc_sw128(A8 ? c_addr : a_addr + L::W_BYTES);
+          if (elect_one()) {
           if (W8) {
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk)      // 32 bytes of k per instruction
@@ -339,15 +340,16 @@ __global__ void __launch_bounds__(KIND == TC_KIND_A8 ? TC_THREADS_A8 : TC_THREAD
               umma_bf16(d_tmem, adesc + 2u * kk, bdesc + 2u * kk, idesc, (kb > kb0 || kk > 0) ? 1u : 0u);
           }
           umma_commit(empty_bar(stage));
+          if (A8) umma_commit(cempty_bar(cbuf));
+          }
           if (A8) {
-            umma_commit(cempty_bar(cbuf));
             if (++cbuf == TC_NCONV) { cbuf = 0; cphase ^= 1u; }
           }
           if (++stage == TC_STAGES) { stage = 0; phase ^= 1u; }
         }
-        if (ok) umma_commit(tfull_bar(acc));
+        if (ok && elect_one()) umma_commit(tfull_bar(acc));
       }
-      if (!ok) atomicCAS(p.status, 0, TC_ERR_MMA);
+      if (!ok && lane == 0) atomicCAS(p.status, 0, TC_ERR_MMA);
     }
   } else if (A8 && warp >= 6) {
     // ------------------------------------------------ quantising warps (W8A8) ---------------------------------------

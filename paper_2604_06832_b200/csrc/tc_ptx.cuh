@@ -73,6 +73,14 @@ __device__ __forceinline__ uint64_t policy_evict_last() {
   asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(p));
   return p;
 }
+// True in one lane of a converged warp.  MMAs and commits are issued inside `if (elect_one())` by warps that wait together:
+// the operands are then known to be the same for all that execute the instruction.  Issued inside `if (lane == 0)` each
+// cost some 100 clocks of the issuing thread.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t r;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r));
+  return r != 0;
+}
 // Shared-memory matrix descriptor: K-major operand, 128-byte swizzle, rows 128 bytes apart, groups
 // of 8 rows 1024 bytes apart (stride-dimension byte offset), descriptor version 1 (sm_100).
 __device__ __forceinline__ uint64_t umma_desc_sw128(uint32_t saddr) {
