@@ -97,7 +97,8 @@ struct TcSmem {
   static constexpr int EX_BYTES = (M_PAD / EX_ROUNDS) * 256;
   static constexpr int BAR_OFF = EX_OFF + EX_BYTES;
   static constexpr int ROWSC_OFF = BAR_OFF + 256;                      // A8: the rows' quantisation scales and their reciprocals
-  static constexpr int TOTAL = ROWSC_OFF + 512 + 1024;  // + alignment slack
+  static constexpr int RS_OFF = ROWSC_OFF + (A8 ? 512 : 0);            // the rows' folded norm factors
+  static constexpr int TOTAL = RS_OFF + 256 + 1024;                    // + alignment slack
 };
 
 // Quantise NP 16-byte pieces (tid, tid + stride, ...) of the activation tile of one stage -- two 128-byte-swizzled f16
@@ -138,7 +139,7 @@ __device__ __forceinline__ void quantize_pieces(const uint8_t* x_tile, uint32_t 
 }
 
 template <int M_PAD, int KIND>
-__global__ void __launch_bounds__(KIND == TC_KIND_A8 ? TC_THREADS_A8 : TC_THREADS, 1) gemm_tc_kernel(const __grid_constant__ TcParams p) {
+__global__ void __launch_bounds__(KIND == TC_KIND_A8 ? TC_THREADS_A8 : TC_THREADS, (KIND == TC_KIND_A8 && M_PAD <= 32) ? 2 : 1) gemm_tc_kernel(const __grid_constant__ TcParams p) {
   extern __shared__ uint8_t smem_raw[];
   using L = TcSmem<M_PAD, KIND>;
   constexpr bool A8 = KIND == TC_KIND_A8;
@@ -385,19 +386,31 @@ __global__ void __launch_bounds__(KIND == TC_KIND_A8 ? TC_THREADS_A8 : TC_THREAD
     int local = 0;
     bool ok = true;
     pdl_wait();   // the epilogue reads the predecessor's row statistics and overwrites buffers it may still be reading
-    // folded RMSNorm: lane l keeps the factor of rows l and l + 32; broadcast by shuffle where needed
+    // folded RMSNorm: lane l keeps the factor of rows l and l + 32; broadcast by shuffle where needed.  Two threads add up a
+    // row's partial sums, so that the CTA asks for each of them once (they are the same few lines of L2 for every CTA of the
+    // launch), and leave the factor in shared memory.
     float rs0 = 1.f, rs1 = 1.f;
     if (p.ssq_in) {
-      if (lane < p.m) {
-        float s = 0.f;
-        for (int t = 0; t < p.nt_in; ++t) s += p.ssq_in[(size_t)lane * p.nt_in + t];
-        rs0 = rsqrtf(s * p.inv_h + p.eps);
+      float* row_rs = reinterpret_cast<float*>(sm + L::RS_OFF);
+      const int t = (int)threadIdx.x - 64, r = t >> 1;
+      float s = 0.f;
+      if (r < p.m) {
+        const float* src = p.ssq_in + (size_t)r * p.nt_in;
+        if ((p.nt_in & 3) == 0) {
+#pragma unroll 4
+          for (int i = t & 1; i < p.nt_in / 4; i += 2) {
+            const float4 x = __ldcg(reinterpret_cast<const float4*>(src) + i);
+            s += (x.x + x.y) + (x.z + x.w);
+          }
+        } else {
+          for (int i = t & 1; i < p.nt_in; i += 2) s += __ldcg(src + i);
+        }
       }
-      if (lane + 32 < p.m) {
-        float s = 0.f;
-        for (int t = 0; t < p.nt_in; ++t) s += p.ssq_in[(size_t)(lane + 32) * p.nt_in + t];
-        rs1 = rsqrtf(s * p.inv_h + p.eps);
-      }
+      s += __shfl_xor_sync(0xffffffffu, s, 1);
+      if ((t & 1) == 0) row_rs[r] = rsqrtf(s * p.inv_h + p.eps);
+      asm volatile("bar.sync 1, 128;" ::: "memory");
+      rs0 = row_rs[lane];
+      rs1 = row_rs[lane + 32];
     }
     for (int it = blockIdx.x; it < n_items && ok; it += gridDim.x, ++local) {
       const int tile = it % total_tiles, split = it / total_tiles;
@@ -476,7 +489,7 @@ __global__ void __launch_bounds__(KIND == TC_KIND_A8 ? TC_THREADS_A8 : TC_THREAD
             const float mine = side ? v[hi] * sc * rs_hi : v[lo] * sc * rs_lo;
             const float g = side ? other : mine, u = side ? mine : other;
             const int row = side ? hi : lo;
-            const float val = g / (1.f + __expf(-g)) * u;
+            const float val = silu_mul(g, u);
             if (live && row < p.m) store_act(p.act, p.act_lo_off, (size_t)row * p.inter + col, val, p.act_fmt);
             if (A8 && p.amax_out) {
               // maximum of |act| as stored (f16) over this warp's 32 features, for the consumer's quantiser; values
@@ -497,23 +510,34 @@ __global__ void __launch_bounds__(KIND == TC_KIND_A8 ? TC_THREADS_A8 : TC_THREAD
         const bool in_range = n < p.n_out[0];
         const bool counted = in_range && n != p.mask_id;
         const float sc = (in_range && p.scale[0]) ? p.scale[0][n] : 1.f;
+        // G rows at a time: their maxima and sums over the lanes are formed together (one row at a time, 15 shuffles each, made
+        // this epilogue longer than the main loop at 64 rows: LM head of the 3B shape 160 us, 112 us now)
+        constexpr int G = M_PAD % 32 == 0 ? 32 : 16;
 #pragma unroll
-        for (int b = 0; b < M_PAD; ++b) {
-          if (b >= p.m) break;                                // uniform across the warp
-          const float rs = __shfl_sync(0xffffffffu, (b < 32) ? rs0 : rs1, b & 31);
-          const float l = v[b] * sc * rs;
-          if (p.write_logits && in_range) p.y[(size_t)b * p.ldy + n] = l;
-          float mx = counted ? l : -INFINITY;
-          int ix = counted ? n : 0x7fffffff;
+        for (int b0 = 0; b0 < M_PAD; b0 += G) {
+          if (b0 >= p.m) break;                               // uniform across the warp
+          float w[G];
 #pragma unroll
-          for (int o = 16; o > 0; o >>= 1) {
-            const float omx = __shfl_xor_sync(0xffffffffu, mx, o);
-            const int oix = __shfl_xor_sync(0xffffffffu, ix, o);
-            if (omx > mx || (omx == mx && oix < ix)) { mx = omx; ix = oix; }
+          for (int b = 0; b < G; ++b) {
+            const float rs = __shfl_sync(0xffffffffu, (b0 + b < 32) ? rs0 : rs1, (b0 + b) & 31);
+            const float l = v[b0 + b] * sc * rs;
+            if (p.write_logits && in_range && b0 + b < p.m) p.y[(size_t)(b0 + b) * p.ldy + n] = l;
+            v[b0 + b] = counted ? l : -INFINITY;
+            w[b] = v[b0 + b];
           }
-          float e = (counted && mx > -INFINITY) ? __expf(l - mx) : 0.f;
-          e = warp_sum(e);
-          if (lane == 0) p.stats[(size_t)(tile * 4 + q) * p.m + b] = make_float4(mx, e, __int_as_float(ix), 0.f);
+          const float mx = warp_reduce_transposed<true, G>(w, lane);         // of row b0 + lane mod G
+          int first = 0;
+#pragma unroll
+          for (int b = 0; b < G; ++b) {
+            const float m = __shfl_sync(0xffffffffu, mx, b);
+            const unsigned at = __ballot_sync(0xffffffffu, v[b0 + b] == m);  // ids ascend with the lane: the lowest holds the argmax
+            if ((lane & (G - 1)) == b) first = __ffs(at) - 1;
+            w[b] = m > -INFINITY ? __expf(v[b0 + b] - m) : 0.f;
+          }
+          const float sum = warp_reduce_transposed<false, G>(w, lane);
+          if (lane < G && b0 + lane < p.m)
+            p.stats[(size_t)(tile * 4 + q) * p.m + b0 + lane] =
+                make_float4(mx, sum, __int_as_float(mx > -INFINITY ? tile * TC_BM + q * 32 + first : 0x7fffffff), 0.f);
         }
       } else {
         int mi = 0;
