@@ -1,15 +1,15 @@
-// Split-KV, block-masked GQA attention for the tensor-core path (Sec. 3.3 masks; Alg. 1 draft / verify).
+// Split-KV, block-masked GQA attention of the decode path (Sec. 3.3 masks; Alg. 1 draft / verify).
 //
-// One CTA = (KV head, group of query heads that share it, chunk of keys).  The CTA's rows are the block's n rows of
-// each of its query heads (ROWS = 64 or 128 in all, 16 per compute warp).  The K and V tiles of the chunk (64 keys
-// each) are fetched by one producer thread with 2-D TMA loads (128-byte swizzle) into a ring of shared-memory stages
-// guarded by full / empty mbarriers; tiles that lie wholly in the committed cache are requested before the wait for
-// the predecessor kernel.  Scores and P.V run on mma.sync m16n8k16 (bf16 or f16 operands, fp32 accumulate) with an
-// online softmax in fp32; each CTA leaves an unnormalised partial (O, running max, running sum) and a small second
-// kernel merges the chunks.  The in-block mask is applied by key index: denoise rows see all L + n keys, commit /
-// prefill rows see keys <= L + i.  Two shapes of CTA: 64 rows with a two-stage ring, two CTAs per SM (short caches:
-// one or two tiles per CTA); 128 rows with up to six tiles resident at once, one CTA per SM (long caches: every K/V
-// byte crosses from L2 half as often and the whole chunk is in flight from the start).
+// One CTA = (KV head, group of query heads that share it, chunk of keys).  Its rows, at most 128, are the block's n rows of
+// each of its query heads.  S = Q K^T and O += P V run on the 5th-generation tensor cores with S, P and O in tensor memory,
+// as in the prompt path's kernel (prefill_attn.cu): one softmax thread owns a row, P replaces S in place, O is rescaled only
+// when a row's maximum has grown by more than 2^8.  Here the two softmax warpgroups share the rows and take alternate
+// 64-key steps (every 128-key tile is one step of each), with accumulators of their own that are added at the end: a short
+// chunk is one step deep however it is cut.  K and V tiles are fetched by one producer warp with 2-D TMA loads; tiles that
+// lie wholly in the committed cache are requested before the wait for the predecessor kernel.  Each CTA leaves an
+// unnormalised partial (O, maximum, sum) and a small second kernel merges the chunks.  The in-block mask is applied by key
+// index: denoise rows see all L + n keys, commit / prefill rows see keys <= L + i, or the caller gives bit masks.
+// What bounds it is the chain through one CTA: rows to shared memory 1.5 us, S, softmax, P V, store (with mma.sync on 64-row CTAs: 13.4 us a layer at 8224 keys and 32 rows, 8.6 now; 5.5 both at 2052 keys and 4 rows).
 // Every mbarrier wait is bounded; a wait that gives up records ST_ATTENTION in the status word and the CTA drains its
 // copies in flight and returns.
 #include "attn_plan.cuh"
@@ -18,19 +18,22 @@
 
 namespace fdk {
 
-template <int D, int ROWS>
+constexpr int AT_THREADS = 384;     // warp 0 TMA producer, warp 1 MMA issuer, warps 4..7 / 8..11 softmax of even / odd steps
+constexpr int AT_ROWS = 128, AT_STEP = 64;
+
+template <int D>
 struct AtSmem {
-  static constexpr int STAGES = ROWS == 64 ? 2 : (D == 128 ? 6 : 12);
-  static constexpr int Q_BYTES = ROWS * D * 2;
-  static constexpr int TILE_BYTES = AT_KEYS * D * 2;          // one K or one V tile
-  static constexpr int STAGE_BYTES = 2 * TILE_BYTES;          // K then V
-  static constexpr int BAR_OFF = Q_BYTES + STAGES * STAGE_BYTES;
-  static constexpr int TOTAL = BAR_OFF + 8 * (2 * STAGES) + 16 + 1024;   // barriers, abort flag, alignment slack
-  static constexpr int THREADS = (ROWS / 16) * 32 + 32;       // compute warps + the producer warp
+  static constexpr int STAGES = 3;
+  static constexpr int TILE_BYTES = 128 * D * 2;             // a Q, K or V tile: D / 64 blocks of [128 rows][128 bytes], swizzled
+  static constexpr int KV_OFF = TILE_BYTES;                  // stage: K, then V
+  static constexpr int BAR_OFF = KV_OFF + STAGES * 2 * TILE_BYTES;
+  static constexpr int TOTAL = BAR_OFF + 256 + 1024;         // + alignment slack
+  // the K / V ring doubles as the exchange of the epilogue: the rows' (m, l) of both warpgroups, 4 KB per warp to turn
+  static constexpr int ML_OFF = KV_OFF, TURN_OFF = KV_OFF + 2048;
 };
 
 struct AttnParams {
-  CUtensorMap tm_k, tm_v;     // [Hkv * max_seq, D] views of the layer's K and V planes, box {64, 64}
+  CUtensorMap tm_k, tm_v;     // [Hkv * max_seq, D] views of the layer's K and V planes, box {64, 128}
   const void* q;              // [n, Hq, D]
   float* part_o;              // [Hq][n][chunks][D]
   float2* part_ml;            // [Hq][n][chunks]
@@ -41,32 +44,25 @@ struct AttnParams {
   KStamp* stamp;
 };
 
-template <int D, typename E, int ROWS>
-__global__ void __launch_bounds__(AtSmem<D, ROWS>::THREADS, ROWS == 64 ? 2 : 1) attn_mma_kernel(const __grid_constant__ AttnParams p) {
-  using S = AtSmem<D, ROWS>;
+template <int D, typename E>
+__global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_constant__ AttnParams p) {
+  using S = AtSmem<D>;
   constexpr int CH = D / 8;                 // 16-byte chunks per row
-  constexpr int NW = ROWS / 16;             // compute warps
-  constexpr int NCT = NW * 32;              // compute threads
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
-  const uint32_t sQ = (raw + 1023u) & ~1023u;
-  uint8_t* sm = smem_raw + (sQ - raw);
-  const uint32_t sKV = sQ + S::Q_BYTES;
-  const uint32_t bar0 = sQ + S::BAR_OFF;
-  auto full_bar = [&](int s) { return bar0 + 8u * s; };
-  auto empty_bar = [&](int s) { return bar0 + 8u * (S::STAGES + s); };
-  volatile int* abort_flag = (volatile int*)(sm + S::BAR_OFF + 8 * (2 * S::STAGES));
+  const uint32_t base = (raw + 1023u) & ~1023u;
+  uint8_t* sm = smem_raw + (base - raw);
+  const uint32_t bar0 = base + S::BAR_OFF;
+  const uint32_t q_full = bar0;
+  auto k_full = [&](int s) { return bar0 + 8u + 8u * s; };
+  auto v_full = [&](int s) { return bar0 + 32u + 8u * s; };
+  auto kv_empty = [&](int s) { return bar0 + 56u + 8u * s; };
+  auto s_full = [&](int w) { return bar0 + 80u + 8u * w; };
+  auto p_full = [&](int w) { return bar0 + 96u + 8u * w; };
+  auto o_full = [&](int w) { return bar0 + 112u + 8u * w; };     // the last P V of a warpgroup's steps is complete
+  volatile uint32_t* tmem_slot = (volatile uint32_t*)(sm + S::BAR_OFF + 128);
+  volatile int* abort_flag = (volatile int*)(sm + S::BAR_OFF + 132);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-
-  pdl_trigger();       // first thing: the successor's prologue overlaps this whole kernel
-  if (tid == 0) {
-    stamp_start(p.stamp);
-    for (int s = 0; s < S::STAGES; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), NW); }
-    *abort_flag = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  }
-  __syncthreads();
 
   int L = p.L, chunk_keys = p.chunk_keys, n_chunks = p.n_chunks;
   if (p.len_ptr) {   // the length word is written before the forward starts, not by a predecessor kernel
@@ -75,213 +71,251 @@ __global__ void __launch_bounds__(AtSmem<D, ROWS>::THREADS, ROWS == 64 ? 2 : 1) 
   }
   const int n = p.n, hq = p.hq, hkv = p.hkv, qh = p.qh;
   const int chunk = blockIdx.x, grp = blockIdx.y, hk = blockIdx.z;
-  if (chunk >= n_chunks) { pdl_wait(); return; }
+  if (chunk >= n_chunks) { pdl_trigger(); pdl_wait(); return; }
+  if (tid == 0) {
+    stamp_start(p.stamp);
+    mbar_init(q_full, 8);
+    for (int i = 0; i < S::STAGES; ++i) { mbar_init(k_full(i), 1); mbar_init(v_full(i), 1); mbar_init(kv_empty(i), 1); }
+    for (int w = 0; w < 2; ++w) { mbar_init(s_full(w), 1); mbar_init(p_full(w), 4); mbar_init(o_full(w), 1); }
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32((const void*)tmem_slot)), "r"(512) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = *tmem_slot;     // columns: S (then P) of warpgroup w at 64 w, O at 256 + 128 w
+  pdl_trigger();                        // (holding its tensor memory: see gemm_tc.cu)
+
   const int G = hq / hkv;
   const int head0 = hk * G + grp * qh;                 // first query head of this CTA
-  const int heads_here = min(qh, G - grp * qh);
-  const int m_valid = heads_here * n;
-  const int T = L + n;
+  const int m_valid = min(qh, G - grp * qh) * n;
   const int key_begin = chunk * chunk_keys;
-  const int key_end = min(T, key_begin + chunk_keys);
+  const int key_end = min(L + n, key_begin + chunk_keys);
   const int n_tiles = (key_end - key_begin + AT_KEYS - 1) / AT_KEYS;
+  // steps of warpgroup w: the w-th half of every tile that begins before the chunk's end
+  const int steps0 = n_tiles, steps1 = key_begin + (n_tiles - 1) * AT_KEYS + AT_STEP < key_end ? n_tiles : n_tiles - 1;
 
-  if (warp == NW) {
-    // ------------------------------------------------ TMA producer ------------------------------------------------
+  if (warp == 0) {
     if (lane == 0) {
       const uint64_t pol = policy_evict_last();     // the cache is read again by the other head groups and by the next step
-      // The host-set test hook (status[1], never written by a kernel): the producer issues nothing and raises the
-      // abort flag, so every wait of the compute warps gives up.  Only this thread pays for the read, off the
-      // critical path of the others.
+      // The host-set test hook (status[1], never written by a kernel): the producer issues nothing and raises the abort
+      // flag, so every other wait gives up.
       const bool poisoned = p.status && *reinterpret_cast<const volatile int*>(p.status + 1) != 0;
       if (poisoned) *abort_flag = 1;
       bool ok = !poisoned, waited = false;
-      uint32_t armed = 0, armed_parity = 0;
+      uint32_t armed = 0, parity = 0;
       for (int t = 0; t < n_tiles && ok; ++t) {
-        const int stage = t % S::STAGES;
-        const uint32_t phase = (uint32_t)(t / S::STAGES) & 1u;
+        const int s = t % S::STAGES;
+        const uint32_t ph = (uint32_t)(t / S::STAGES) & 1u;
         const int j0 = key_begin + t * AT_KEYS;
         // rows >= L are written by the predecessor kernel (the block's own K / V)
         if (!waited && j0 + AT_KEYS > L) { pdl_wait(); waited = true; }
-        if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag)) { ok = false; break; }
-        mbar_expect_tx(full_bar(stage), S::STAGE_BYTES);
-        armed |= 1u << stage;
-        armed_parity = (armed_parity & ~(1u << stage)) | (phase << stage);
-        const uint32_t dst = sKV + stage * S::STAGE_BYTES;
+        if (!mbar_wait(kv_empty(s), ph ^ 1u, abort_flag)) { ok = false; break; }
+        armed |= 1u << s; parity = (parity & ~(1u << s)) | (ph << s);
+        const uint32_t dst = base + S::KV_OFF + s * 2 * S::TILE_BYTES;
         const int row = hk * p.max_seq + j0;
+        mbar_expect_tx(k_full(s), S::TILE_BYTES);
 #pragma unroll
-        for (int hd = 0; hd < D / 64; ++hd) {
-          tma_load_2d(dst + hd * (AT_KEYS * 128), &p.tm_k, full_bar(stage), hd * 64, row, pol);
-          tma_load_2d(dst + S::TILE_BYTES + hd * (AT_KEYS * 128), &p.tm_v, full_bar(stage), hd * 64, row, pol);
-        }
+        for (int b = 0; b < D / 64; ++b) tma_load_2d(dst + b * 16384, &p.tm_k, k_full(s), b * 64, row, pol);
+        mbar_expect_tx(v_full(s), S::TILE_BYTES);
+#pragma unroll
+        for (int b = 0; b < D / 64; ++b) tma_load_2d(dst + S::TILE_BYTES + b * 16384, &p.tm_v, v_full(s), b * 64, row, pol);
       }
       if (!waited) pdl_wait();
       if (!ok) {
         if (p.status) atomicCAS(p.status, 0, ST_ATTENTION);
         for (int s = 0; s < S::STAGES; ++s) {      // drain: wait (bounded) for every bulk copy in flight
           if (!(armed & (1u << s))) continue;
-          const uint32_t par = (armed_parity >> s) & 1u;
-          const long long t0 = clock64();
-          while (!mbar_try_wait(full_bar(s), par) && clock64() - t0 < TC_TIMEOUT) {}
+          for (int v = 0; v < 2; ++v) {
+            const long long t0 = clock64();
+            while (!mbar_try_wait(v ? v_full(s) : k_full(s), (parity >> s) & 1u) && clock64() - t0 < TC_TIMEOUT) {}
+          }
         }
       }
     }
-  } else {
-    // ------------------------------------------------ compute warps -----------------------------------------------
-    // stage Q (rows = heads_here x n; row r -> head r / n, token r % n): written by the predecessor kernel
-    const E* q = reinterpret_cast<const E*>(p.q);
-    pdl_wait();
-    if (tid == 0) stamp_released(p.stamp);
-    for (int v = tid; v < ROWS * CH; v += NCT) {
-      const int r = v / CH, c = v % CH;
-      const bool live = r < m_valid;
-      const int hl = live ? r / n : 0, i = live ? r % n : 0;
-      cp_async16(sQ + swz_q<D>(r, c), live ? (const void*)(q + ((size_t)i * hq + head0 + hl) * D + c * 8) : (const void*)q, live ? 16 : 0);
-    }
-    cp_async_commit();
-    cp_async_wait<0>();
-    asm volatile("bar.sync 1, %0;" ::"n"(NCT) : "memory");
-
-    const int row0 = warp * 16;                       // this warp's rows of the CTA tile
-    const bool warp_live = row0 < m_valid;
-    const int g = lane >> 2, tq = lane & 3;
-    const int r_lo = row0 + g, r_hi = r_lo + 8;       // the two rows this thread owns
-    // last visible key (exclusive) of each row
-    const int lim_lo = (r_lo < m_valid) ? (p.causal ? L + (r_lo % n) + 1 : T) : 0;
-    const int lim_hi = (r_hi < m_valid) ? (p.causal ? L + (r_hi % n) + 1 : T) : 0;
-    const float sl2 = rsqrtf((float)D) * LOG2E;       // scores kept in the log2 domain
-
-    uint32_t qf[D / 16][4];
+  } else if (warp == 1) {
+    constexpr bool F16 = !__is_same(E, bf16);
+    const uint32_t id_s = F16 ? umma_idesc_f16(AT_STEP) : umma_idesc_bf16(AT_STEP);
+    const uint32_t id_o = (F16 ? umma_idesc_f16(D) : umma_idesc_bf16(D)) | (1u << 16);      // (V: MN-major)
+    bool ok = mbar_wait(q_full, 0, abort_flag);
+    auto score = [&](int w, int t) {
+      if (!ok || t >= (w ? steps1 : steps0)) return;
+      const int s = t % S::STAGES;
+      if (!mbar_wait(k_full(s), (uint32_t)(t / S::STAGES) & 1u, abort_flag)) { ok = false; return; }
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint32_t ka = base + S::KV_OFF + s * 2 * S::TILE_BYTES + w * (AT_STEP * 128);
+      if (elect_one()) {
 #pragma unroll
-    for (int kk = 0; kk < D / 16; ++kk)
-      ldsm_x4(sQ + swz_q<D>(row0 + (lane & 15), kk * 2 + (lane >> 4)), qf[kk][0], qf[kk][1], qf[kk][2], qf[kk][3]);
-    float o[D / 8][4];
+        for (int kk = 0; kk < D / 16; ++kk)
+          umma_bf16(tmem + w * AT_STEP, umma_desc_sw128(base + (kk >> 2) * 16384) + 2u * (kk & 3), umma_desc_sw128(ka + (kk >> 2) * 16384) + 2u * (kk & 3),
+                    id_s, kk > 0 ? 1u : 0u);
+        umma_commit(s_full(w));
+      }
+    };
+    auto value = [&](int w, int t) {
+      const int steps = w ? steps1 : steps0;
+      if (!ok || t >= steps) return;
+      const int s = t % S::STAGES;
+      if (!mbar_wait(p_full(w), (uint32_t)t & 1u, abort_flag) || !mbar_wait(v_full(s), (uint32_t)(t / S::STAGES) & 1u, abort_flag)) { ok = false; return; }
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint64_t vd = umma_desc_sw128_mn(base + S::KV_OFF + (s * 2 + 1) * S::TILE_BYTES + w * (AT_STEP * 128), 16384);
+      if (elect_one()) {
 #pragma unroll
-    for (int i = 0; i < D / 8; ++i) { o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f; }
-    float m_lo = -INFINITY, m_hi = -INFINITY, l_lo = 0.f, l_hi = 0.f;
-    bool ok = true;
-
+        for (int kk = 0; kk < AT_STEP / 16; ++kk)
+          umma_f16_ta(tmem + 256 + w * 128, tmem + w * AT_STEP + kk * 8, vd + (uint64_t)(kk * 128), id_o, (t > 0 || kk > 0) ? 1u : 0u);
+        if (t + 1 == steps) umma_commit(o_full(w));
+      }
+    };
+    score(0, 0);
+    score(1, 0);
     for (int t = 0; t < n_tiles && ok; ++t) {
-      const int stage = t % S::STAGES;
-      const uint32_t phase = (uint32_t)(t / S::STAGES) & 1u;
-      if (!mbar_wait(full_bar(stage), phase, abort_flag)) { ok = false; break; }
-      const uint32_t kt = sKV + stage * S::STAGE_BYTES;
-      const uint32_t vt = kt + S::TILE_BYTES;
-      const int j0 = key_begin + t * AT_KEYS;
-      if (j0 + AT_KEYS > key_end) {
-        // The box reaches past the last key: those V rows hold whatever the cache holds there, and 0 x NaN would
-        // poison the P.V product.  Clear them (only ever the last tile of the last chunk, which is never refilled).
-        // Every warp clears all of them itself before it reads any: the warps write the same zeros, so no barrier
-        // between the warps is needed.
-        const int first = key_end - j0;
-        for (int v = lane; v < (AT_KEYS - first) * CH; v += 32) {
-          const int r = first + v / CH, c = v % CH;
-          asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(vt + swz_kv(r, c)), "r"(0u) : "memory");
-        }
-        __syncwarp();
-      }
-      if (warp_live) {
-        float s[AT_KEYS / 8][4];
-#pragma unroll
-        for (int i = 0; i < AT_KEYS / 8; ++i) { s[i][0] = s[i][1] = s[i][2] = s[i][3] = 0.f; }
-#pragma unroll
-        for (int kk = 0; kk < D / 16; ++kk) {
-#pragma unroll
-          for (int np = 0; np < AT_KEYS / 16; ++np) {
-            uint32_t b0, b1, b2, b3;
-            ldsm_x4(kt + swz_kv(np * 16 + (lane & 7) + ((lane >> 4) << 3), kk * 2 + ((lane >> 3) & 1)), b0, b1, b2, b3);
-            mma_16816<E>(s[2 * np], qf[kk], b0, b1);
-            mma_16816<E>(s[2 * np + 1], qf[kk], b2, b3);
-          }
-        }
-        // explicit mask among the forward's own rows (keys L .. L+n-1; the words are set up before the chain, not by a
-        // kernel of it).  Only the last tile or two hold such keys, so the words are fetched there and kept out of the
-        // main loop's registers.
-        if (p.row_mask && j0 + AT_KEYS > L) {                // uniform over the warp
-          const unsigned long long msk_lo = (r_lo < m_valid) ? p.row_mask[r_lo % n] : 0ull;
-          const unsigned long long msk_hi = (r_hi < m_valid) ? p.row_mask[r_hi % n] : 0ull;
-#pragma unroll
-          for (int nt = 0; nt < AT_KEYS / 8; ++nt) {
-            const int j = j0 + nt * 8 + tq * 2;
-            if (j >= L && !((msk_lo >> ((j - L) & 63)) & 1ull)) s[nt][0] = -INFINITY;
-            if (j + 1 >= L && !((msk_lo >> ((j + 1 - L) & 63)) & 1ull)) s[nt][1] = -INFINITY;
-            if (j >= L && !((msk_hi >> ((j - L) & 63)) & 1ull)) s[nt][2] = -INFINITY;
-            if (j + 1 >= L && !((msk_hi >> ((j + 1 - L) & 63)) & 1ull)) s[nt][3] = -INFINITY;
-          }
-        }
-        // mask + running max
-        float mx_lo = -INFINITY, mx_hi = -INFINITY;
-#pragma unroll
-        for (int nt = 0; nt < AT_KEYS / 8; ++nt) {
-          const int j = j0 + nt * 8 + tq * 2;
-          s[nt][0] = (j < lim_lo) ? s[nt][0] * sl2 : -INFINITY;
-          s[nt][1] = (j + 1 < lim_lo) ? s[nt][1] * sl2 : -INFINITY;
-          s[nt][2] = (j < lim_hi) ? s[nt][2] * sl2 : -INFINITY;
-          s[nt][3] = (j + 1 < lim_hi) ? s[nt][3] * sl2 : -INFINITY;
-          mx_lo = fmaxf(mx_lo, fmaxf(s[nt][0], s[nt][1]));
-          mx_hi = fmaxf(mx_hi, fmaxf(s[nt][2], s[nt][3]));
-        }
-        mx_lo = fmaxf(mx_lo, __shfl_xor_sync(0xffffffffu, mx_lo, 1));
-        mx_lo = fmaxf(mx_lo, __shfl_xor_sync(0xffffffffu, mx_lo, 2));
-        mx_hi = fmaxf(mx_hi, __shfl_xor_sync(0xffffffffu, mx_hi, 1));
-        mx_hi = fmaxf(mx_hi, __shfl_xor_sync(0xffffffffu, mx_hi, 2));
-        const float mn_lo = fmaxf(m_lo, mx_lo), mn_hi = fmaxf(m_hi, mx_hi);
-        const float ref_lo = (mn_lo == -INFINITY) ? 0.f : mn_lo, ref_hi = (mn_hi == -INFINITY) ? 0.f : mn_hi;
-        const float al_lo = exp2f(m_lo - ref_lo), al_hi = exp2f(m_hi - ref_hi);   // exp2(-inf) = 0 on the first tile
-        m_lo = mn_lo; m_hi = mn_hi;
-        float sum_lo = 0.f, sum_hi = 0.f;
-#pragma unroll
-        for (int nt = 0; nt < AT_KEYS / 8; ++nt) {
-          s[nt][0] = exp2f(s[nt][0] - ref_lo); s[nt][1] = exp2f(s[nt][1] - ref_lo);
-          s[nt][2] = exp2f(s[nt][2] - ref_hi); s[nt][3] = exp2f(s[nt][3] - ref_hi);
-          sum_lo += s[nt][0] + s[nt][1];
-          sum_hi += s[nt][2] + s[nt][3];
-        }
-        l_lo = l_lo * al_lo + sum_lo;
-        l_hi = l_hi * al_hi + sum_hi;
-#pragma unroll
-        for (int i = 0; i < D / 8; ++i) { o[i][0] *= al_lo; o[i][1] *= al_lo; o[i][2] *= al_hi; o[i][3] *= al_hi; }
-#pragma unroll
-        for (int kk = 0; kk < AT_KEYS / 16; ++kk) {
-          uint32_t pa[4];
-          pa[0] = pack2<E>(s[2 * kk][0], s[2 * kk][1]);
-          pa[1] = pack2<E>(s[2 * kk][2], s[2 * kk][3]);
-          pa[2] = pack2<E>(s[2 * kk + 1][0], s[2 * kk + 1][1]);
-          pa[3] = pack2<E>(s[2 * kk + 1][2], s[2 * kk + 1][3]);
-#pragma unroll
-          for (int dp = 0; dp < D / 16; ++dp) {
-            uint32_t b0, b1, b2, b3;
-            ldsm_x4_t(vt + swz_kv(kk * 16 + (lane & 7) + (((lane >> 3) & 1) << 3), dp * 2 + (lane >> 4)), b0, b1, b2, b3);
-            mma_16816<E>(o[2 * dp], pa, b0, b1);
-            mma_16816<E>(o[2 * dp + 1], pa, b2, b3);
-          }
-        }
-      }
+      value(0, t);
+      score(0, t + 1);
+      value(1, t);
+      if (ok && elect_one()) umma_commit(kv_empty(t % S::STAGES));
       __syncwarp();
-      if (lane == 0) mbar_arrive(empty_bar(stage));
+      score(1, t + 1);
     }
     if (!ok && lane == 0 && p.status) atomicCAS(p.status, 0, ST_ATTENTION);
-
-    // ---- partial results: the quad's four lanes hold the row sums in pieces ----
-    l_lo += __shfl_xor_sync(0xffffffffu, l_lo, 1);
-    l_lo += __shfl_xor_sync(0xffffffffu, l_lo, 2);
-    l_hi += __shfl_xor_sync(0xffffffffu, l_hi, 1);
-    l_hi += __shfl_xor_sync(0xffffffffu, l_hi, 2);
+  } else if (warp >= 4) {
+    // Where this thread's pieces of Q come from and its rows of the result go is worked out before the wait: rows = heads x n,
+    // row r -> head r / n, token r % n.
+    const int wt = tid - 128;
+    const int w = (warp - 4) >> 2, wq = warp & 3;
+    constexpr int NQ = AT_ROWS * CH / 256, RS = 256 / CH;     // 16-byte pieces per thread, rows between them
+    int q_off[NQ], out_row[8];
 #pragma unroll
-    for (int half = 0; half < 2; ++half) {
-      const int r = half ? r_hi : r_lo;
-      if (r >= m_valid || !ok) continue;
-      const int head = head0 + r / n, i = r % n;
-      const size_t slot = ((size_t)head * n + i) * n_chunks + chunk;
-      float* dst = p.part_o + slot * D;
-#pragma unroll
-      for (int dt = 0; dt < D / 8; ++dt) {
-        float2 v = half ? make_float2(o[dt][2], o[dt][3]) : make_float2(o[dt][0], o[dt][1]);
-        *reinterpret_cast<float2*>(dst + dt * 8 + tq * 2) = v;
-      }
-      if (tq == 0) p.part_ml[slot] = half ? make_float2(m_hi, l_hi) : make_float2(m_lo, l_lo);
+    for (int i = 0; i < NQ; ++i) {
+      const int r = wt / CH + i * RS;
+      q_off[i] = r < m_valid ? ((r % n) * hq + head0 + r / n) * D + (wt % CH) * 8 : -1;
     }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int r = wq * 32 + (lane >> 3) + 4 * i;
+      out_row[i] = r < m_valid ? ((head0 + r / n) * n + r % n) * n_chunks + chunk : -1;
+    }
+    const int row = wq * 32 + lane;                           // this thread's row; the other warpgroup has it too
+    const bool row_live = row < m_valid;
+    const int tok = row % n, slot = ((head0 + row / n) * n + tok) * n_chunks + chunk;
+    const int lim = row_live && !p.causal ? L + n : L + tok + 1;      // keys it may read
+    const unsigned long long mask = p.row_mask ? p.row_mask[tok] : ~0ull;      // (set up before the chain)
+    // stage Q: written by the predecessor kernel
+    pdl_wait();
+    if (wt == 0) stamp_released(p.stamp);
+    const E* q = reinterpret_cast<const E*>(p.q);
+#pragma unroll
+    for (int i = 0; i < NQ; ++i) {
+      const int r = wt / CH + i * RS, c = wt % CH;
+      cp_async16(base + (c >> 3) * 16384 + r * 128 + (((c & 7) ^ (r & 7)) << 4), q + max(q_off[i], 0), q_off[i] >= 0 ? 16 : 0);
+    }
+    cp_async_commit();
+    const uint32_t ts = tmem + ((uint32_t)(wq * 32) << 16) + w * AT_STEP;
+    const uint32_t to = tmem + ((uint32_t)(wq * 32) << 16) + 256;
+    const float sl2 = rsqrtf((float)D) * LOG2E;               // scores in the log2 domain
+    float m_ref = -INFINITY, l = 0.f;
+    bool ok = true;
+    const int steps = w ? steps1 : steps0;
+    cp_async_wait<0>();
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");      // generic writes -> the MMA's async-proxy reads
+    __syncwarp();
+    if (lane == 0) mbar_arrive(q_full);
+    for (int t = 0; t < steps && ok; ++t) {
+      if (!mbar_wait(s_full(w), (uint32_t)t & 1u, abort_flag)) { ok = false; break; }
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      float s[AT_STEP];
+      tmem_ld32(ts, s);
+      tmem_ld32(ts + 32, s + 32);
+      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+      const int j0 = key_begin + t * AT_KEYS + w * AT_STEP;
+      if (j0 + AT_STEP > L) {               // keys of the forward's own rows (uniform)
+        // bit c: this row reads key j0 + c
+        unsigned long long vis = j0 <= L ? (mask << (L - j0)) | ((1ull << (L - j0)) - 1ull) : (j0 - L < 64 ? mask >> (j0 - L) : 0ull);
+        if (lim - j0 < 64) vis &= lim > j0 ? (1ull << (lim - j0)) - 1ull : 0ull;
+        const uint32_t v0 = (uint32_t)vis, v1 = (uint32_t)(vis >> 32);
+#pragma unroll
+        for (int c = 0; c < 32; ++c) {
+          if (!(v0 & (1u << c))) s[c] = -INFINITY;
+          if (!(v1 & (1u << c))) s[32 + c] = -INFINITY;
+        }
+      }
+      const float m = row_max64(s) * sl2;
+      const bool grow = m > m_ref + 8.f;
+      if (t > 0 && __any_sync(0xffffffffu, grow)) {
+        // (s_full also says that this warpgroup's product of the step before is complete: O may be rewritten)
+        const float f = grow ? ex2(m_ref - m) : 1.f;
+        scale_acc<D>(to + w * 128, f);
+        l *= f;
+      }
+      if (grow) m_ref = m;
+      l += exp_pack64<E>(s, sl2, m_ref == -INFINITY ? 0.f : m_ref, ts);
+      if (j0 + AT_STEP > key_end) {
+        // V rows past the last key hold whatever the cache holds there, and 0 x NaN would poison the product
+        const int sg = t % S::STAGES, first = max(0, key_end - j0);
+        if (!mbar_wait(v_full(sg), (uint32_t)(t / S::STAGES) & 1u, abort_flag)) ok = false;
+        for (int v = wq * 32 + lane; ok && v < (AT_STEP - first) * CH; v += 128) {
+          const int r = w * AT_STEP + first + v / CH, c = v % CH;
+          const uint32_t a = base + S::KV_OFF + (sg * 2 + 1) * S::TILE_BYTES + (c >> 3) * 16384 + r * 128 + (((c & 7) ^ (r & 7)) << 4);
+          asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(a), "r"(0u) : "memory");
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      }
+      asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) mbar_arrive(p_full(w));
+    }
+    for (int x = 0; x < 2; ++x)
+      if (ok && (x ? steps1 : steps0) > 0 && !mbar_wait(o_full(x), 0, abort_flag)) ok = false;
+    // every load has been used up and every product is complete: the ring is free.  Each warpgroup stores half of the
+    // columns of the sum of both accumulators.
+    ok = named_barrier_and<256>(ok);
+    if (ok) {
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      float2* ml = reinterpret_cast<float2*>(sm + S::ML_OFF);
+      ml[w * 128 + row] = make_float2(m_ref, l);
+      asm volatile("bar.sync 1, 256;" ::: "memory");
+      const float2 other = ml[(1 - w) * 128 + row];
+      const float m = fmaxf(m_ref, other.x), ref = m == -INFINITY ? 0.f : m;
+      const float fm = ex2(m_ref - ref), fo = ex2(other.x - ref);
+      const float f0 = w ? fo : fm, f1 = w ? fm : fo;
+      if (w == 0 && row_live) p.part_ml[slot] = make_float2(m, l * fm + other.y * fo);
+      // rows of a turned block: lane / 8 + 4 i, four columns each
+      const uint32_t buf = base + S::TURN_OFF + (warp - 4) * 4096;
+      const int lc = (lane & 7) * 4;
+#pragma unroll 1
+      for (int c = w * (D / 2); c < (w + 1) * (D / 2); c += 32) {
+        float a[32], b[32];
+        float4 o[8];
+        __syncwarp();
+        tmem_ld32(to + c, a);
+        tmem_ld32(to + 128 + c, b);
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+        for (int k = 0; k < 32; ++k) a[k] = (f0 > 0.f ? a[k] * f0 : 0.f) + (f1 > 0.f ? b[k] * f1 : 0.f);   // (an accumulator that was never written holds anything)
+        turn<32>(buf, lane, a, o);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          if (out_row[i] >= 0) *reinterpret_cast<float4*>(p.part_o + (size_t)out_row[i] * D + c + lc) = o[i];
+        }
+      }
+    } else if (lane == 0 && p.status) {
+      atomicCAS(p.status, 0, ST_ATTENTION);
+    }
+  } else {
+    pdl_wait();
   }
+  __syncwarp();
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();     // the producer's copies have all been consumed (or drained) before any thread leaves
+  if (warp == 1) {
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+  }
   if (tid == 0) stamp_end(p.stamp);
 }
 
@@ -394,53 +428,34 @@ cudaError_t launch_attn_combine(const float* part_o, const float2* part_ml, cons
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-// CTAs of 128 rows once the keys make more than this many tiles per 64-row CTA (all SMs busy either way)
-constexpr int AT_LONG_KEYS = 3072;
+struct AttnPlan { int qh, groups, chunk_keys, n_chunks, bound; };
 
-struct AttnPlan { int rows, qh, groups, chunk_keys, n_chunks, bound; };
-
-static int attn_sm_count() {
-  int dev = 0, v = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v <= 0) return 148;
-  return v;
-}
-
-// rows per CTA: the most query heads of one KV head whose n rows fit
-static void attn_rows(int n, int hq, int hkv, int rows_cap, int* qh, int* groups) {
-  const int G = hq / hkv;
-  *qh = 1;
-  for (int c = G; c >= 1; --c)
-    if (c * n <= rows_cap) { *qh = c; break; }
-  *groups = ceil_div(G, *qh);
-}
-
-static AttnPlan attn_plan(int n, int T, int hq, int hkv, bool long_cache) {
+// heads per CTA: the most query heads of one KV head whose n rows fit; chunks: one CTA per SM
+static AttnPlan attn_plan(int n, int T, int hq, int hkv) {
   AttnPlan p;
-  p.rows = (long_cache && (hq / hkv) * n > 64) ? 128 : 64;
-  attn_rows(n, hq, hkv, p.rows, &p.qh, &p.groups);
-  // 64-row CTAs sit two to an SM, 128-row CTAs one
-  p.bound = ceil_div((p.rows == 64 ? 2 : 1) * attn_sm_count(), hkv * p.groups);
+  const int G = hq / hkv;
+  p.qh = 1;
+  for (int c = G; c >= 1; --c)
+    if (c * n <= AT_ROWS) { p.qh = c; break; }
+  p.groups = ceil_div(G, p.qh);
+  p.bound = sm_count() / (hkv * p.groups);
+  if (p.bound < 1) p.bound = 1;
   attn_chunking(T, p.bound, &p.chunk_keys, &p.n_chunks);
   return p;
 }
 
-size_t attention_mma_workspace_bytes(int n, int hq, int hkv, int d) {
+size_t attention_tc_workspace_bytes(int n, int hq, int hkv, int d) {
   size_t worst = 0;
   for (int m = 1; m <= n; ++m) {
-    const int row_caps[2] = {64, 128};
-    for (int rows : row_caps) {
-      int qh, groups;
-      attn_rows(m, hq, hkv, rows, &qh, &groups);
-      const size_t slots = (size_t)hq * m * ceil_div(2 * 148, hkv * groups);
-      if (slots > worst) worst = slots;
-    }
+    const size_t slots = (size_t)hq * m * attn_plan(m, 1, hq, hkv).bound;
+    if (slots > worst) worst = slots;
   }
   return worst * ((size_t)d * 4 + 8) + 256;
 }
 
-template <int D, typename E, int ROWS>
+template <int D, typename E>
 static cudaError_t attn_launch_t(const AttnArgs& a, const AttnPlan& pl, cudaStream_t st) {
-  using S = AtSmem<D, ROWS>;
+  using S = AtSmem<D>;
   // with the length on the device the grid is sized for the most chunks any length can give
   int grid_x = pl.n_chunks;
   if (a.len_ptr) { grid_x = pl.bound; const int tmax = ceil_div(a.max_seq, AT_KEYS); if (grid_x > tmax) grid_x = tmax; }
@@ -456,27 +471,18 @@ static cudaError_t attn_launch_t(const AttnArgs& a, const AttnPlan& pl, cudaStre
   p.n = a.n; p.L = a.cache_len; p.max_seq = a.max_seq; p.hq = a.hq; p.hkv = a.hkv; p.qh = pl.qh;
   p.chunk_keys = pl.chunk_keys; p.n_chunks = pl.n_chunks; p.causal = a.row_mask ? 0 : a.causal; p.row_mask = a.row_mask; p.len_ptr = a.len_ptr; p.status = a.status; p.stamp = a.stamp;
   static bool attr_set[MAX_DEVICES] = {};
-  cudaError_t e = ensure_dynamic_smem(attn_mma_kernel<D, E, ROWS>, S::TOTAL, attr_set);
+  cudaError_t e = ensure_dynamic_smem(attn_tc_kernel<D, E>, S::TOTAL, attr_set);
   if (e != cudaSuccess) return e;
-  dim3 grid(grid_x, pl.groups, a.hkv);
-  e = launch_pdl(attn_mma_kernel<D, E, ROWS>, grid, dim3(S::THREADS), (size_t)S::TOTAL, st, p);
+  e = launch_pdl(attn_tc_kernel<D, E>, dim3(grid_x, pl.groups, a.hkv), dim3(AT_THREADS), (size_t)S::TOTAL, st, p);
   if (e != cudaSuccess) return e;
   return launch_attn_combine(p.part_o, p.part_ml, a, pl.n_chunks, grid_x, a.stamp ? a.stamp + 1 : nullptr, st);
 }
 
-template <int D, typename E>
-static cudaError_t attn_launch_r(const AttnArgs& a, const AttnPlan& pl, cudaStream_t st) {
-  return pl.rows == 128 ? attn_launch_t<D, E, 128>(a, pl, st) : attn_launch_t<D, E, 64>(a, pl, st);
-}
-
-bool attention_long_cache(int keys) { return keys > AT_LONG_KEYS; }
-
-int launch_attention_mma(const AttnArgs& a, cudaStream_t st, cudaError_t* err) {
-  const bool long_cache = a.long_cache >= 0 ? a.long_cache != 0 : attention_long_cache(a.cache_len + a.n);
+int launch_attention_tc(const AttnArgs& a, cudaStream_t st, cudaError_t* err) {
   if (!a.workspace) { *err = cudaErrorInvalidValue; return -1; }
-  const AttnPlan pl = attn_plan(a.n, a.cache_len + a.n, a.hq, a.hkv, long_cache);
-  if (a.kv_type == KV_F16) *err = (a.d == 128) ? attn_launch_r<128, __half>(a, pl, st) : attn_launch_r<64, __half>(a, pl, st);
-  else *err = (a.d == 128) ? attn_launch_r<128, bf16>(a, pl, st) : attn_launch_r<64, bf16>(a, pl, st);
+  const AttnPlan pl = attn_plan(a.n, a.cache_len + a.n, a.hq, a.hkv);
+  if (a.kv_type == KV_F16) *err = (a.d == 128) ? attn_launch_t<128, __half>(a, pl, st) : attn_launch_t<64, __half>(a, pl, st);
+  else *err = (a.d == 128) ? attn_launch_t<128, bf16>(a, pl, st) : attn_launch_t<64, bf16>(a, pl, st);
   return *err == cudaSuccess ? 2 : -1;
 }
 

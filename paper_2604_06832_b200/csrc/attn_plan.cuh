@@ -1,10 +1,10 @@
 // What the attention kernels of the decode and the prompt path share.
 #pragma once
-#include "common.cuh"
+#include "tc_ptx.cuh"
 
 namespace fdk {
 
-constexpr int AT_KEYS = 64;    // keys per shared-memory tile
+constexpr int AT_KEYS = 128;   // keys per shared-memory tile
 constexpr float LOG2E = 1.4426950408889634f;
 
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, int src_bytes) {
@@ -13,7 +13,7 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, int sr
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-// Split of T keys into chunks of whole 64-key tiles, at most `bound` chunks (the same on host and device, so a launch
+// Split of T keys into chunks of whole AT_KEYS-key tiles, at most `bound` chunks (the same on host and device, so a launch
 // whose grid was sized for `bound` can take the sequence length from device memory).
 __host__ __device__ inline void attn_chunking(int T, int bound, int* chunk_keys, int* n_chunks) {
   const int tiles = (T + AT_KEYS - 1) / AT_KEYS;
@@ -23,23 +23,6 @@ __host__ __device__ inline void attn_chunking(int T, int bound, int* chunk_keys,
   *n_chunks = (T + *chunk_keys - 1) / *chunk_keys;
 }
 
-__device__ __forceinline__ void ldsm_x4(uint32_t addr, uint32_t& r0, uint32_t& r1, uint32_t& r2, uint32_t& r3) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];" : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3) : "r"(addr));
-}
-__device__ __forceinline__ void ldsm_x4_t(uint32_t addr, uint32_t& r0, uint32_t& r1, uint32_t& r2, uint32_t& r3) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];" : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3) : "r"(addr));
-}
-template <typename T> __device__ __forceinline__ void mma_16816(float* c, const uint32_t* a, uint32_t b0, uint32_t b1);
-template <> __device__ __forceinline__ void mma_16816<bf16>(float* c, const uint32_t* a, uint32_t b0, uint32_t b1) {
-  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
-               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-               : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-template <> __device__ __forceinline__ void mma_16816<__half>(float* c, const uint32_t* a, uint32_t b0, uint32_t b1) {
-  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
-               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-               : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
 template <typename T> __device__ __forceinline__ uint32_t pack2(float lo, float hi);
 template <> __device__ __forceinline__ uint32_t pack2<bf16>(float lo, float hi) {
   __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
@@ -50,15 +33,67 @@ template <> __device__ __forceinline__ uint32_t pack2<__half>(float lo, float hi
   return *reinterpret_cast<uint32_t*>(&v);
 }
 
-// byte offset of 16-byte chunk `chunk` of row `row` in the Q tile: rows of D * 2 bytes, chunks XOR-swizzled by row
-template <int D>
-__device__ __forceinline__ uint32_t swz_q(int row, int chunk) {
-  return (uint32_t)(row * (D * 2) + ((chunk ^ (row & 7)) << 4));
+__device__ __forceinline__ float ex2(float x) {
+  float r;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
 }
-// the same for a K or V tile as the TMA leaves it: one [64 keys][128 bytes] sub-tile per 64 head dimensions, 16-byte
-// chunks XOR-swizzled by the key's row (the 128-byte swizzle of the tensor map)
-__device__ __forceinline__ uint32_t swz_kv(int row, int chunk) {
-  return (uint32_t)((chunk >> 3) * (AT_KEYS * 128) + row * 128 + (((chunk & 7) ^ (row & 7)) << 4));
+
+// two fp32 operations in one instruction
+__device__ __forceinline__ float2 fma2(const float2& a, const float2& b, const float2& c) {
+  float2 d;
+  asm("{\n\t.reg .b64 a, b, c, d;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\tmov.b64 c, {%6, %7};\n\t"
+      "fma.rn.f32x2 d, a, b, c;\n\tmov.b64 {%0, %1}, d;\n\t}"
+      : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+  return d;
+}
+__device__ __forceinline__ float2 add2(const float2& a, const float2& b) {
+  float2 d;
+  asm("{\n\t.reg .b64 a, b, d;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\tadd.rn.f32x2 d, a, b;\n\tmov.b64 {%0, %1}, d;\n\t}"
+      : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return d;
+}
+
+// ---- steps of the online softmax, one thread per row, 64 scores ------------------------------------------------
+__device__ __forceinline__ float row_max64(const float* s) {
+  float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+  for (int c = 0; c < 64; c += 8)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) mx[k] = fmaxf(fmaxf(mx[k], s[c + k]), s[c + 4 + k]);
+  return fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
+}
+// P = 2^(s sl2 - ref) as 16-bit values into the columns of S at tensor-memory address ts; returns the row's sum
+template <typename E>
+__device__ __forceinline__ float exp_pack64(const float* s, float sl2, float ref, uint32_t ts) {
+  float2 sum[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+  const float2 sl = make_float2(sl2, sl2), mr = make_float2(-ref, -ref);
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    uint32_t pk[16];
+#pragma unroll
+    for (int c = 0; c < 16; ++c) {
+      float2 e = fma2(make_float2(s[h * 32 + 2 * c], s[h * 32 + 2 * c + 1]), sl, mr);
+      e = make_float2(ex2(e.x), ex2(e.y));
+      sum[c & 1] = add2(sum[c & 1], e);
+      pk[c] = pack2<E>(e.x, e.y);
+    }
+    tmem_st16(ts + h * 16, pk);
+  }
+  return (sum[0].x + sum[0].y) + (sum[1].x + sum[1].y);
+}
+// the row's accumulator (D columns at `to`) times f
+template <int D>
+__device__ __forceinline__ void scale_acc(uint32_t to, float f) {
+#pragma unroll 1
+  for (int c = 0; c < D; c += 16) {
+    float o[16];
+    tmem_ld16(to + c, o);
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int k = 0; k < 16; ++k) o[k] *= f;
+    tmem_st16(to + c, reinterpret_cast<const uint32_t*>(o));
+  }
 }
 
 }  // namespace fdk

@@ -8,8 +8,8 @@ namespace fdk {
 int launch_linear_simt(const LinearArgs& a, cudaStream_t st, cudaError_t* err);
 size_t simt_workspace_bytes(int m, int n, int k);
 int launch_attention_f32(const AttnArgs& a, cudaStream_t st, cudaError_t* err);
-size_t attention_mma_workspace_bytes(int n, int hq, int hkv, int d);
-int launch_attention_mma(const AttnArgs& a, cudaStream_t st, cudaError_t* err);
+size_t attention_tc_workspace_bytes(int n, int hq, int hkv, int d);
+int launch_attention_tc(const AttnArgs& a, cudaStream_t st, cudaError_t* err);
 void launch_splitk_epilogue(const float* part, int S, int m, int n, const float* scale, const float* bias, float* y, int ldy,
                             int accumulate, cudaStream_t st, const float* row_amax = nullptr);
 
@@ -76,10 +76,10 @@ int launch_linear(const LinearArgs& a, cudaStream_t st, cudaError_t* err) {
   return *err == cudaSuccess ? launched : -1;
 }
 
-size_t attention_workspace_bytes(int n, int hq, int hkv, int d) { return attention_mma_workspace_bytes(n, hq, hkv, d); }
+size_t attention_workspace_bytes(int n, int hq, int hkv, int d) { return attention_tc_workspace_bytes(n, hq, hkv, d); }
 // 16-bit rows go to the split-KV tensor-core kernel, fp32 rows to the exact CUDA-core kernel.
 int launch_attention(const AttnArgs& a, cudaStream_t st, cudaError_t* err) {
-  return a.dtype == DT_F32 ? launch_attention_f32(a, st, err) : launch_attention_mma(a, st, err);
+  return a.dtype == DT_F32 ? launch_attention_f32(a, st, err) : launch_attention_tc(a, st, err);
 }
 
 int stage_rows(fdvlm_t* h, int row0, int n, const int32_t* tokens, const void* embeds) {
@@ -282,8 +282,7 @@ static int forward_rows_f32(fdvlm_t* h, int n, int mode, int logits_rows, int wa
 //            [down GEMM -> partials] [sum + residual + gain + ssq]
 // head:      [LM-head GEMM, folded final norm, logits + softmax statistics epilogue] [statistics merge]
 // stamped: every launch gets the next record of h->stamps (in-chain timing, fdvlm_profile_enable(h, 2)).
-static int forward_rows_tc(fdvlm_t* h, int n, int mode, int logits_rows, int want_logits, const int* len_ptr, bool stamped,
-                           int long_cache = -1) {
+static int forward_rows_tc(fdvlm_t* h, int n, int mode, int logits_rows, int want_logits, const int* len_ptr, bool stamped) {
   const fdvlm_config& c = h->cfg;
   const int H = c.hidden, I = c.intermediate, d = c.head_dim, nt = h->nt;
   const int NQ = c.n_q_heads * d, NKV = c.n_kv_heads * d, NQKV = NQ + 2 * NKV;
@@ -343,7 +342,6 @@ static int forward_rows_tc(fdvlm_t* h, int n, int mode, int logits_rows, int wan
     at.dtype = h->dt; at.workspace = h->ws; at.kv_type = h->kv_type; at.out_fmt = h->xfmt; at.out_lo_off = h->ao_lo;
     at.status = h->info + 3;
     at.amax_out = a8 ? h->amax_ao : nullptr;
-    at.long_cache = long_cache;
     at.stamp = stamp(FDVLM_K_ATTENTION);
     if (at.stamp && !stamp(FDVLM_K_ATTN_MERGE)) at.stamp = nullptr;     // the launcher uses two consecutive records
     prof_begin(h, 1);
@@ -407,12 +405,10 @@ static int forward_rows_tc(fdvlm_t* h, int n, int mode, int logits_rows, int wan
 // edges are kept.
 static int forward_rows_graph(fdvlm_t* h, int n, int mode, int logits_rows, int want_logits) {
   const int stamped = (h->prof_on == 2) ? 1 : 0;
-  const int long_cache = attention_long_cache(h->cache_len + n) ? 1 : 0;
   set_dev_len(h);
   if (stamped) CU(h, cudaMemsetAsync(h->stamps, 0xFF, sizeof(KStamp) * FDVLM_MAX_STAMPS, h->st));
   for (auto& g : h->graphs) {
-    if (g.n == n && g.mode == mode && g.logits_rows == logits_rows && g.want_logits == want_logits && g.stamped == stamped &&
-        g.long_cache == long_cache) {
+    if (g.n == n && g.mode == mode && g.logits_rows == logits_rows && g.want_logits == want_logits && g.stamped == stamped) {
       if (stamped) {      // the records' kinds are those of the capture: replay the bookkeeping only
         h->stamp_kind = g.kinds;
         h->stamp_used = (int)g.kinds.size();
@@ -424,14 +420,14 @@ static int forward_rows_graph(fdvlm_t* h, int n, int mode, int logits_rows, int 
   }
   const int before = h->launches;
   CU(h, cudaStreamBeginCapture(h->st, cudaStreamCaptureModeThreadLocal));
-  const int rc = h->use_tc ? forward_rows_tc(h, n, mode, logits_rows, want_logits, h->dev_len, stamped != 0, long_cache)
+  const int rc = h->use_tc ? forward_rows_tc(h, n, mode, logits_rows, want_logits, h->dev_len, stamped != 0)
                            : forward_rows_f32(h, n, mode, logits_rows, want_logits, h->dev_len);
   cudaGraph_t graph = nullptr;
   cudaError_t e = cudaStreamEndCapture(h->st, &graph);
   if (rc != FDVLM_OK) { if (graph) cudaGraphDestroy(graph); return rc; }
   if (e != cudaSuccess) return fail(h, FDVLM_ERR_CUDA, "graph capture: %s", cudaGetErrorString(e));
   fdvlm::FwdGraph g;
-  g.n = n; g.mode = mode; g.logits_rows = logits_rows; g.want_logits = want_logits; g.stamped = stamped; g.long_cache = long_cache;
+  g.n = n; g.mode = mode; g.logits_rows = logits_rows; g.want_logits = want_logits; g.stamped = stamped;
   g.launches = h->launches - before; g.exec = nullptr;
   if (stamped) g.kinds = h->stamp_kind;
   e = cudaGraphInstantiate(&g.exec, graph, 0);
@@ -445,7 +441,7 @@ static int forward_rows_graph(fdvlm_t* h, int n, int mode, int logits_rows, int 
 // The kernels of one tensor-core forward enqueued on the handle's stream, cache length taken from the device word:
 // what a caller that is itself capturing the stream (the on-device decode loop) records.
 int forward_rows_enqueue(fdvlm_t* h, int n, int mode, int logits_rows, int want_logits) {
-  return forward_rows_tc(h, n, mode, logits_rows, want_logits, h->dev_len, false, attention_long_cache(h->cache_len + n) ? 1 : 0);
+  return forward_rows_tc(h, n, mode, logits_rows, want_logits, h->dev_len, false);
 }
 
 int forward_rows(fdvlm_t* h, int n, int mode, int logits_rows, int want_logits) {

@@ -174,8 +174,6 @@ struct AttnArgs {
   size_t out_lo_off;
   const unsigned long long* row_mask;   // nullable, n <= 64 words: bit r' of word r = row r reads row r' of this forward
                                         // (the cached keys are always read); overrides `causal`
-  int long_cache;       // tensor-core kernel: -1 pick the CTA shape from cache_len; 0 / 1 the short- / long-cache shape
-                        // (a captured launch serves every later length of its class)
   void* workspace;
   const int* len_ptr;   // nullable: device word holding the cache length (overrides cache_len)
   int* status;          // nullable: device status words (see TcOut::status)
@@ -185,6 +183,5 @@ struct AttnArgs {
 // Prompt path: causal attention of any number of rows, one CTA per (256 rows, query head), no key split (prefill_attn.cu).
 cudaError_t launch_prefill_attention(const AttnArgs& a, cudaStream_t st);
 size_t attention_workspace_bytes(int n, int hq, int hkv, int d);
-bool attention_long_cache(int keys);   // whether the tensor-core kernel takes its long-cache shape for this many keys
 
 }  // namespace fdk

@@ -6,10 +6,10 @@
 // only when a row's maximum has grown by more than 2^8, until then P is taken relative to the old reference (values up to
 // 256, sums in fp32).  Each row tile has two score buffers, so the scores of the next keys are there when a softmax thread
 // is done with its keys (with one buffer of 128 keys the threads waited for P V and Q K^T in turn: 97 us for 4096 rows of
-// the 3B shape, %PB% us now).  Bound by the exponentials, 16 per clock and SM.
+// the 3B shape, 96 us by the same clock now that the issue of MMAs does not bound it).  Bound by the exponentials, 16 per clock and SM.
 // V stays as it lies in the cache ([key][dim], an MN-major operand).  Hundreds of CTAs exist at any prompt length, so keys
 // are not split and the normalised result is written directly as the O projection's input; CTAs with the most keys come
-// first.  (mma.sync with 16 rows per warp: %PA%.)
+// first. 
 // Every mbarrier wait is bounded as in gemm_tc.cu.
 #include "attn_plan.cuh"
 #include "kernels.h"
@@ -37,27 +37,6 @@ struct PaParams {
   int n, L, max_seq, hq, hkv;
   int* status;
 };
-
-__device__ __forceinline__ float ex2(float x) {
-  float r;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
-}
-
-// two fp32 operations in one instruction
-__device__ __forceinline__ float2 fma2(const float2& a, const float2& b, const float2& c) {
-  float2 d;
-  asm("{\n\t.reg .b64 a, b, c, d;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\tmov.b64 c, {%6, %7};\n\t"
-      "fma.rn.f32x2 d, a, b, c;\n\tmov.b64 {%0, %1}, d;\n\t}"
-      : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
-  return d;
-}
-__device__ __forceinline__ float2 add2(const float2& a, const float2& b) {
-  float2 d;
-  asm("{\n\t.reg .b64 a, b, d;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\tadd.rn.f32x2 d, a, b;\n\tmov.b64 {%0, %1}, d;\n\t}"
-      : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
-  return d;
-}
 
 template <int D, typename E>
 __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const __grid_constant__ PaParams p) {
@@ -221,44 +200,17 @@ __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const __gri
         for (int c = 0; c < PA_STEP; ++c)
           if (j0 + c >= lim) s[c] = -INFINITY;
       }
-      float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-#pragma unroll
-      for (int c = 0; c < PA_STEP; c += 8)
-#pragma unroll
-        for (int k = 0; k < 4; ++k) mx[k] = fmaxf(fmaxf(mx[k], s[c + k]), s[c + 4 + k]);
-      const float m = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * sl2;
+      const float m = row_max64(s) * sl2;
       const bool grow = m > m_ref + 8.f;                      // (always in the first step: every row reads key 0)
       if (t > 0 && __any_sync(0xffffffffu, grow)) {
         if (!mbar_wait(o_done(q), (uint32_t)(t - 1) & 1u, abort_flag)) { ok = false; break; }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const float f = grow ? ex2(m_ref - m) : 1.f;
-#pragma unroll 1
-        for (int c = 0; c < D; c += 16) {
-          float o[16];
-          tmem_ld16(to + c, o);
-          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-          for (int k = 0; k < 16; ++k) o[k] *= f;
-          tmem_st16(to + c, reinterpret_cast<const uint32_t*>(o));
-        }
+        scale_acc<D>(to, f);
         l *= f;
       }
       if (grow) m_ref = m;
-      float2 sum[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-      const float2 sl = make_float2(sl2, sl2), mr = make_float2(-m_ref, -m_ref);
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        uint32_t pk[16];
-#pragma unroll
-        for (int c = 0; c < 16; ++c) {
-          float2 e = fma2(make_float2(s[h * 32 + 2 * c], s[h * 32 + 2 * c + 1]), sl, mr);
-          e = make_float2(ex2(e.x), ex2(e.y));
-          sum[c & 1] = add2(sum[c & 1], e);
-          pk[c] = pack2<E>(e.x, e.y);
-        }
-        tmem_st16(tb + h * 16, pk);
-      }
-      l += (sum[0].x + sum[0].y) + (sum[1].x + sum[1].y);
+      l += exp_pack64<E>(s, sl2, m_ref, tb);
       if (j0 + PA_STEP > key_end) {
         // V rows past the last key hold whatever the cache holds there, and 0 x NaN would poison the product: cleared by
         // both row tiles (the same zeros)

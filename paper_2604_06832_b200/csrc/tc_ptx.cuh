@@ -52,6 +52,13 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     if (clock64() - t0 > TC_TIMEOUT) { *abort_flag = 1; return false; }
   }
 }
+// Barrier 1 of N threads that also tells every thread whether all of them came with `ok`.
+template <int N>
+__device__ __forceinline__ bool named_barrier_and(bool ok) {
+  uint32_t r;
+  asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbar.red.and.pred q, 1, %2, p;\n\tselp.u32 %0, 1, 0, q;\n\t}" : "=r"(r) : "r"((uint32_t)ok), "n"(N) : "memory");
+  return r != 0;
+}
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* tm, uint32_t bar, int c0, int c1, uint64_t pol) {
   asm volatile(
       "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%3, %4}], [%2], %5;"
@@ -220,4 +227,21 @@ __device__ __forceinline__ void e4m3x16_to_f16(const uint4& in, uint4& lo, uint4
   hi = make_uint4(o[4], o[5], o[6], o[7]);
 }
 
+// A warp's 32 x W block of values, thread = row, turned round through shared memory (32 * W floats of the warp's own,
+// 16-byte pieces XOR-swizzled, no bank conflicts either way): lane l gets columns 4 (l % (W/4)) .. + 3 of the rows
+// l / (W/4) + i * 128 / W, so that the warp's accesses to global memory are whole sectors of few rows instead of 16 bytes
+// of 32 rows (which made the epilogue as long as the main loop of a 2048-deep tile).
+template <int W>
+__device__ __forceinline__ void turn(uint32_t buf, int lane, const float* v, float4* w) {
+  constexpr int PR = W / 4, RI = 32 / PR;       // 16-byte pieces per row, rows per step
+  auto at = [&](int r, int c) { return buf + (uint32_t)((r * PR + (c ^ (W == 32 ? (r & 7) : ((r >> 1) & 3)))) << 4); };
+  __syncwarp();
+#pragma unroll
+  for (int c = 0; c < PR; ++c)
+    asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(at(lane, c)), "f"(v[4 * c]), "f"(v[4 * c + 1]), "f"(v[4 * c + 2]), "f"(v[4 * c + 3]) : "memory");
+  __syncwarp();
+#pragma unroll
+  for (int i = 0; i < W / 4; ++i)
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(w[i].x), "=f"(w[i].y), "=f"(w[i].z), "=f"(w[i].w) : "r"(at(lane / PR + i * RI, lane % PR)) : "memory");
+}
 }  // namespace fdk
