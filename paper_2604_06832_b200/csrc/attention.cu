@@ -28,7 +28,7 @@ struct AtSmem {
   static constexpr int KV_OFF = TILE_BYTES;                  // stage: K, then V
   static constexpr int BAR_OFF = KV_OFF + STAGES * 2 * TILE_BYTES;
   static constexpr int TOTAL = BAR_OFF + 256 + 1024;         // + alignment slack
-  // the K / V ring doubles as the exchange of the epilogue: the rows' (m, l) of both warpgroups, 4 KB per warp to turn
+  // the K / V ring doubles as the exchange of the epilogue: the rows' (m, l) of both warpgroups, 2 KB per warp to turn
   static constexpr int ML_OFF = KV_OFF, TURN_OFF = KV_OFF + 2048;
 };
 
@@ -188,15 +188,15 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
     const int wt = tid - 128;
     const int w = (warp - 4) >> 2, wq = warp & 3;
     constexpr int NQ = AT_ROWS * CH / 256, RS = 256 / CH;     // 16-byte pieces per thread, rows between them
-    int q_off[NQ], out_row[8];
+    int q_off[NQ], out_row[4];
 #pragma unroll
     for (int i = 0; i < NQ; ++i) {
       const int r = wt / CH + i * RS;
       q_off[i] = r < m_valid ? ((r % n) * hq + head0 + r / n) * D + (wt % CH) * 8 : -1;
     }
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int r = wq * 32 + (lane >> 3) + 4 * i;
+    for (int i = 0; i < 4; ++i) {
+      const int r = wq * 32 + (lane >> 2) + 8 * i;
       out_row[i] = r < m_valid ? ((head0 + r / n) * n + r % n) * n_chunks + chunk : -1;
     }
     const int row = wq * 32 + lane;                           // this thread's row; the other warpgroup has it too
@@ -284,24 +284,28 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
       const float fm = ex2(m_ref - ref), fo = ex2(other.x - ref);
       const float f0 = w ? fo : fm, f1 = w ? fm : fo;
       if (w == 0 && row_live) p.part_ml[slot] = make_float2(m, l * fm + other.y * fo);
-      // rows of a turned block: lane / 8 + 4 i, four columns each
-      const uint32_t buf = base + S::TURN_OFF + (warp - 4) * 4096;
-      const int lc = (lane & 7) * 4;
+      // rows of a turned block: lane / 4 + 8 i, four columns each.  (16 columns at a time: this code runs once, and half the
+      // instructions are fetched in half the time)
+      const uint32_t buf = base + S::TURN_OFF + (warp - 4) * 2048;
+      const int lc = (lane & 3) * 4;
 #pragma unroll 1
-      for (int c = w * (D / 2); c < (w + 1) * (D / 2); c += 32) {
-        float a[32], b[32];
-        float4 o[8];
+      for (int c = w * (D / 2); c < (w + 1) * (D / 2); c += 16) {
+        float a[16], b[16];
+        float4 o[4];
         __syncwarp();
-        tmem_ld32(to + c, a);
-        tmem_ld32(to + 128 + c, b);
+        tmem_ld16(to + c, a);
+        tmem_ld16(to + 128 + c, b);
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        if (steps1 == 0) {       // (the second accumulator was never written and holds anything)
 #pragma unroll
-        for (int k = 0; k < 32; ++k) a[k] = (f0 > 0.f ? a[k] * f0 : 0.f) + (f1 > 0.f ? b[k] * f1 : 0.f);   // (an accumulator that was never written holds anything)
-        turn<32>(buf, lane, a, o);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          if (out_row[i] >= 0) *reinterpret_cast<float4*>(p.part_o + (size_t)out_row[i] * D + c + lc) = o[i];
+          for (int k = 0; k < 16; ++k) b[k] = 0.f;
         }
+#pragma unroll
+        for (int k = 0; k < 16; ++k) a[k] = fmaf(a[k], f0, b[k] * f1);
+        turn<16>(buf, lane, a, o);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          if (out_row[i] >= 0) *reinterpret_cast<float4*>(p.part_o + (size_t)out_row[i] * D + c + lc) = o[i];
       }
     } else if (lane == 0 && p.status) {
       atomicCAS(p.status, 0, ST_ATTENTION);
@@ -319,112 +323,121 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
   if (tid == 0) stamp_end(p.stamp);
 }
 
-// Merge of the key chunks of one (row, head) by one warp: out = sum_c w_c O_c / sum_c w_c l_c, w_c = 2^(m_c - max m).
-// Lane j owns D / 32 consecutive output features; the chunk statistics are spread over the lanes.
-// The result is stored as `fmt` (XF_*) at element offset out_idx of `out`.
-template <int D>
-__device__ __forceinline__ void attn_merge_warp(const float* att_o, const float2* att_ml, void* out, size_t out_idx, size_t lo_off,
-                                                int fmt, size_t slot0, int n_chunks, int lane, float* amax_out = nullptr) {
-  constexpr int VPL = D / 32;
-  constexpr int CB = 32;     // chunks whose partial outputs are in flight together
-  // The statistics and the first CB partial outputs are requested together: one L2 round trip for up to 32 chunks.
-  float2 ml0 = make_float2(-INFINITY, 0.f);
-  if (lane < n_chunks) ml0 = __ldcg(&att_ml[slot0 + lane]);
-  float ov[CB][VPL];
-  auto issue = [&](int c0) {
-#pragma unroll
-    for (int cc = 0; cc < CB; ++cc) {
-      const float* src = att_o + (slot0 + c0 + cc) * D + lane * VPL;
-      if (c0 + cc < n_chunks) {
-        if (VPL == 4) {
-          const float4 o = __ldcg(reinterpret_cast<const float4*>(src));
-          ov[cc][0] = o.x; ov[cc][1] = o.y; ov[cc][2] = o.z; ov[cc][VPL - 1] = o.w;
-        } else {
-          const float2 o = __ldcg(reinterpret_cast<const float2*>(src));
-          ov[cc][0] = o.x; ov[cc][VPL - 1] = o.y;
-        }
-      } else {
-#pragma unroll
-        for (int i = 0; i < VPL; ++i) ov[cc][i] = 0.f;
-      }
-    }
-  };
-  issue(0);
-  float mx = ml0.x;
-  for (int c = lane + 32; c < n_chunks; c += 32) mx = fmaxf(mx, __ldcg(&att_ml[slot0 + c]).x);
-  mx = warp_max(mx);
-  float den = 0.f, acc[VPL];
-#pragma unroll
-  for (int i = 0; i < VPL; ++i) acc[i] = 0.f;
-  for (int c0 = 0; c0 < n_chunks; c0 += 32) {
-    const int c = c0 + lane;
-    float w = 0.f;
-    if (c < n_chunks) {
-      const float2 ml = (c0 == 0) ? ml0 : __ldcg(&att_ml[slot0 + c]);
-      if (ml.y != 0.f) { w = exp2f(ml.x - mx); den = fmaf(w, ml.y, den); }
-    }
-    for (int h0 = 0; h0 < 32 && c0 + h0 < n_chunks; h0 += CB) {
-      if (c0 + h0 > 0) issue(c0 + h0);
-#pragma unroll
-      for (int cc = 0; cc < CB; ++cc) {
-        const float wc = __shfl_sync(0xffffffffu, w, h0 + cc);     // zero for chunks past the end
-#pragma unroll
-        for (int i = 0; i < VPL; ++i) acc[i] = fmaf(wc, ov[cc][i], acc[i]);
-      }
-    }
-  }
-  den = warp_sum(den);
-  const float inv = 1.f / den;
-  if (VPL == 4) {
-    store_act4(out, lo_off, out_idx + lane * VPL, make_float4(acc[0] * inv, acc[1] * inv, acc[VPL - 2] * inv, acc[VPL - 1] * inv), fmt);
-  } else {
-#pragma unroll
-    for (int i = 0; i < VPL; ++i) store_act(out, lo_off, out_idx + lane * VPL + i, acc[i] * inv, fmt);
-  }
-  if (amax_out) {     // W8A8: the O projection quantises this row; its maximum as stored (f16) over this head
-    float am = 0.f;
-#pragma unroll
-    for (int i = 0; i < VPL; ++i) am = fmaxf(am, fabsf(__half2float(__ushort_as_half(f16_bits_sat(acc[i] * inv)))));
-    am = warp_max(am);
-    if (lane == 0) *amax_out = am;
-  }
-}
-
-// out[i][head] = sum_c w_c O_c / sum_c w_c l_c, w_c = 2^(m_c - max_c m_c): one warp per (row, head), four per CTA
-template <int D>
+// Merge of the key chunks: out[i][head] = sum_c w_c O_c / sum_c w_c l_c, w_c = 2^(m_c - max_c m_c).  WPP warps per
+// (row, head): warp w takes the chunks w, w + WPP, ..., CB of them in flight at once; with WPP = 4 warp 0 adds up the four.
+// Four where that is at most four CTAs per SM (one warp per pair took 5.4 us a layer for the 33 chunks of 8224 keys and 32
+// rows of the 3B shape, four take 3.6), one beyond (64 rows: 3.4 against 4.1).  Lane j owns D / 32 consecutive output
+// features.  The result is stored as `fmt` (XF_*).
+template <int D, int WPP>
 __global__ void __launch_bounds__(128) attn_combine_kernel(const float* __restrict__ part_o, const float2* __restrict__ part_ml,
-                                                          void* __restrict__ out, size_t lo_off, int fmt, int n, int hq, int n_chunks,
-                                                          const int* __restrict__ len_ptr, int bound, float* __restrict__ amax_out,
-                                                          KStamp* stamp) {
+                                                             void* __restrict__ out, size_t lo_off, int fmt, int n, int hq, int n_chunks,
+                                                             const int* __restrict__ len_ptr, int bound, float* __restrict__ amax_out,
+                                                             KStamp* stamp) {
+  constexpr int VPL = D / 32, CB = WPP == 4 ? 10 : 20;
   if (threadIdx.x == 0) stamp_start(stamp);
   pdl_trigger();
   if (len_ptr) {
     int ck;
     attn_chunking(*len_ptr + n, bound, &ck, &n_chunks);
   }
+  __shared__ float s_m[4], s_l[4];
+  __shared__ __align__(16) float s_o[4][D];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int pair = WPP == 4 ? blockIdx.x : blockIdx.x * 4 + warp;
+  const bool live = pair < n * hq;
+  const int i = pair / hq, head = pair - i * hq;
+  const size_t slot0 = ((size_t)head * n + i) * n_chunks;
+  const float* src = part_o + slot0 * D + lane * VPL;
   pdl_wait();
   if (threadIdx.x == 0) stamp_released(stamp);
-  const int p = blockIdx.x * 4 + (threadIdx.x >> 5);
-  if (p < n * hq) {
-    const int i = p / hq, head = p % hq;
-    attn_merge_warp<D>(part_o, part_ml, out, ((size_t)i * hq + head) * D, lo_off, fmt, ((size_t)head * n + i) * n_chunks, n_chunks,
-                       threadIdx.x & 31, amax_out ? amax_out + (size_t)i * hq + head : nullptr);
+  float m = -INFINITY, l = 0.f, acc[VPL];
+#pragma unroll
+  for (int k = 0; k < VPL; ++k) acc[k] = 0.f;
+  for (int c0 = WPP == 4 ? warp : 0; live && c0 < n_chunks; c0 += WPP * CB) {
+    float2 ml[CB];
+    float o[CB][VPL];
+#pragma unroll
+    for (int u = 0; u < CB; ++u) {
+      const int c = c0 + WPP * u;
+      ml[u] = make_float2(-INFINITY, 0.f);
+      if (c < n_chunks) {
+        ml[u] = __ldcg(&part_ml[slot0 + c]);
+        if (VPL == 4) {
+          const float4 x = __ldcg(reinterpret_cast<const float4*>(src + (size_t)c * D));
+          o[u][0] = x.x; o[u][1] = x.y; o[u][VPL - 2] = x.z; o[u][VPL - 1] = x.w;
+        } else {
+          const float2 x = __ldcg(reinterpret_cast<const float2*>(src + (size_t)c * D));
+          o[u][0] = x.x; o[u][VPL - 1] = x.y;
+        }
+      }
+    }
+    float mn = m;
+#pragma unroll
+    for (int u = 0; u < CB; ++u) mn = fmaxf(mn, ml[u].x);
+    if (mn == -INFINITY) continue;                 // (nothing visible so far; uniform over the warp)
+    const float keep = exp2f(m - mn);
+    m = mn;
+    l *= keep;
+#pragma unroll
+    for (int k = 0; k < VPL; ++k) acc[k] *= keep;
+#pragma unroll
+    for (int u = 0; u < CB; ++u) {
+      if (ml[u].y != 0.f) {
+        const float w = exp2f(ml[u].x - m);
+        l = fmaf(w, ml[u].y, l);
+#pragma unroll
+        for (int k = 0; k < VPL; ++k) acc[k] = fmaf(w, o[u][k], acc[k]);
+      }
+    }
   }
-  __syncthreads();
-  if (threadIdx.x == 0) stamp_end(stamp, true);
+  if (WPP == 4) {
+    if (lane == 0) { s_m[warp] = m; s_l[warp] = l; }
+#pragma unroll
+    for (int k = 0; k < VPL; ++k) s_o[warp][lane * VPL + k] = acc[k];
+    __syncthreads();
+  }
+  if (WPP == 4 ? warp == 0 : live) {
+    if (WPP == 4) {
+      m = fmaxf(fmaxf(s_m[0], s_m[1]), fmaxf(s_m[2], s_m[3]));
+      l = 0.f;
+#pragma unroll
+      for (int k = 0; k < VPL; ++k) acc[k] = 0.f;
+#pragma unroll
+      for (int w = 0; w < 4; ++w) {
+        const float f = exp2f(s_m[w] - m);
+        l = fmaf(f, s_l[w], l);
+#pragma unroll
+        for (int k = 0; k < VPL; ++k) acc[k] = fmaf(f, s_o[w][lane * VPL + k], acc[k]);
+      }
+    }
+    const float inv = 1.f / l;
+    const size_t idx = ((size_t)i * hq + head) * D + lane * VPL;
+    if (VPL == 4) {
+      store_act4(out, lo_off, idx, make_float4(acc[0] * inv, acc[1] * inv, acc[VPL - 2] * inv, acc[VPL - 1] * inv), fmt);
+    } else {
+#pragma unroll
+      for (int k = 0; k < VPL; ++k) store_act(out, lo_off, idx + k, acc[k] * inv, fmt);
+    }
+    if (amax_out) {     // W8A8: the O projection quantises this row; its maximum as stored (f16) over this head
+      float am = 0.f;
+#pragma unroll
+      for (int k = 0; k < VPL; ++k) am = fmaxf(am, fabsf(__half2float(__ushort_as_half(f16_bits_sat(acc[k] * inv)))));
+      am = warp_max(am);
+      if (lane == 0) amax_out[(size_t)i * hq + head] = am;
+    }
+    if (lane == 0 && warp == 0) stamp_end(stamp, true);
+  }
 }
 
 // ---- host side -------------------------------------------------------------------------------------
 // The chunk merge that follows either attention kernel.  grid_x: the chunk slots the partials were laid out for.
 cudaError_t launch_attn_combine(const float* part_o, const float2* part_ml, const AttnArgs& a, int n_chunks, int grid_x,
                                 KStamp* stamp, cudaStream_t st) {
-  cudaError_t e;
-  if (a.d == 128)
-    e = launch_pdl(attn_combine_kernel<128>, dim3((a.n * a.hq + 3) / 4), dim3(128), 0, st, part_o, part_ml, a.out, a.out_lo_off, a.out_fmt,
-                   a.n, a.hq, n_chunks, a.len_ptr, grid_x, a.amax_out, stamp);
-  else
-    e = launch_pdl(attn_combine_kernel<64>, dim3((a.n * a.hq + 3) / 4), dim3(128), 0, st, part_o, part_ml, a.out, a.out_lo_off, a.out_fmt,
-                   a.n, a.hq, n_chunks, a.len_ptr, grid_x, a.amax_out, stamp);
+  const int pairs = a.n * a.hq;
+  const bool four = pairs <= 4 * sm_count();
+  auto kern = a.d == 128 ? (four ? attn_combine_kernel<128, 4> : attn_combine_kernel<128, 1>) : (four ? attn_combine_kernel<64, 4> : attn_combine_kernel<64, 1>);
+  const cudaError_t e = launch_pdl(kern, dim3(four ? pairs : (pairs + 3) / 4), dim3(128), 0, st, part_o, part_ml, a.out, a.out_lo_off, a.out_fmt,
+                                   a.n, a.hq, n_chunks, a.len_ptr, grid_x, a.amax_out, stamp);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
