@@ -92,6 +92,8 @@ extern "C" int fdvlm_create(const fdvlm_config* cfg, const fdvlm_weights* w, voi
   h->slab = nullptr;
   h->dev_len = nullptr;
   h->dev_len_set = -1;
+  h->dev_step = nullptr;
+  h->step_set.rule = -1;
   h->use_graphs = 0;
   h->stamps = nullptr;
   h->stamp_used = 0;
@@ -140,6 +142,7 @@ extern "C" int fdvlm_create(const fdvlm_config* cfg, const fdvlm_weights* w, voi
       {(void**)&h->blk_tokens, 64 * 4},
       {(void**)&h->blk_masked, 64},
       {(void**)&h->init_stage, 64 * 4},
+      {(void**)&h->dev_step, sizeof(StepDev)},
       {(void**)&h->q_d, 64 * 4},
       {(void**)&h->q_mask, 64 * 8},
       {(void**)&h->q_pos_off, 64 * 4},
@@ -246,7 +249,9 @@ extern "C" int fdvlm_prefill(fdvlm_t* h, const void* embeds, int n_embeds, const
     const int parts = (total + h->pf_rows - 1) / h->pf_rows;
     R = ((total + parts - 1) / parts + 127) / 128 * 128;
   }
-  auto stage = large ? stage_prefill_rows : stage_rows;
+  auto stage = [&](int r0, int rows, const int32_t* t, const void* e) {
+    return large ? stage_prefill_rows(h, r0, rows, t, e) : stage_rows(h, r0, rows, t, e);
+  };
   int done = 0;
   while (done < total) {
     const int n = total - done < R ? total - done : R;
@@ -254,11 +259,11 @@ extern "C" int fdvlm_prefill(fdvlm_t* h, const void* embeds, int n_embeds, const
     int rc;
     if (done < n_embeds) {
       ne = n_embeds - done < n ? n_embeds - done : n;
-      rc = stage(h, 0, ne, nullptr, (const char*)embeds + (size_t)done * H * h->act_sz);
+      rc = stage(0, ne, nullptr, (const char*)embeds + (size_t)done * H * h->act_sz);
       if (rc) return rc;
     }
     if (ne < n) {
-      rc = stage(h, ne, n - ne, tokens + (done + ne - n_embeds), nullptr);
+      rc = stage(ne, n - ne, tokens + (done + ne - n_embeds), nullptr);
       if (rc) return rc;
     }
     const bool last = (done + n == total);
@@ -362,14 +367,10 @@ static int step_core(fdvlm_t* h, const fdvlm_step_params* p, int want_logits) {
   if (h->n_remaining == 0) return fail(h, FDVLM_ERR_STATE, "block_step with no masked position left");
   const int B = h->block_size;
   h->launches = 0;
-  int rc = stage_rows(h, 0, B, h->blk_tokens, nullptr);
+  StepEnds ends;
+  ends.tokens = h->blk_tokens; ends.sel = p;
+  int rc = forward_rows(h, B, MODE_BIDIR, B, want_logits, ends);
   if (rc) return rc;
-  rc = forward_rows(h, B, MODE_BIDIR, B, want_logits);
-  if (rc) return rc;
-  launch_select(h->conf, h->pred, h->blk_tokens, h->blk_masked, h->unmask, h->info, B, (int)p->rule, p->threshold, p->k, h->st,
-                p->pred_shift);
-  h->launches++;
-  CU(h, cudaGetLastError());
   h->step_index++;
   return FDVLM_OK;
 }
@@ -570,9 +571,9 @@ static int commit_core(fdvlm_t* h, int all_rows, int want_logits) {
   if (h->n_remaining != 0) return fail(h, FDVLM_ERR_STATE, "commit with %d masked positions left", h->n_remaining);
   const int B = h->block_size;
   h->launches = 0;
-  int rc = stage_rows(h, 0, B, h->blk_tokens, nullptr);
-  if (rc) return rc;
-  rc = forward_rows(h, B, MODE_CAUSAL, all_rows ? B : (want_logits ? 1 : 0), all_rows ? want_logits : 1);
+  StepEnds ends;
+  ends.tokens = h->blk_tokens;
+  int rc = forward_rows(h, B, MODE_CAUSAL, all_rows ? B : (want_logits ? 1 : 0), all_rows ? want_logits : 1, ends);
   if (rc) return rc;
   h->cache_len += B;
   h->block_open = 0;
@@ -625,14 +626,11 @@ static int commit_step_core(fdvlm_t* h, int Bn, const int32_t* init_dev, const f
   } else {
     h->n_remaining = Bn;
   }
-  int rc = stage_rows(h, 0, n, h->f_rows, nullptr);
+  StepEnds ends;
+  ends.tokens = h->f_rows; ends.sel = p; ends.sel_row0 = Bc;
+  int rc = forward_rows(h, n, MODE_FUSED, n, want_logits, ends);
   if (rc) return rc;
-  rc = forward_rows(h, n, MODE_FUSED, n, want_logits);
-  if (rc) return rc;
-  launch_select(h->conf + Bc, h->pred + Bc, h->blk_tokens, h->blk_masked, h->unmask, h->info, Bn, (int)p->rule, p->threshold, p->k,
-                h->st, p->pred_shift);
-  h->launches += 2;
-  CU(h, cudaGetLastError());
+  h->launches++;
   h->cache_len += Bc;
   h->block_size = Bn;
   h->block_open = 1;
@@ -772,9 +770,9 @@ extern "C" int fdvlm_quad_begin(fdvlm_t* h, int block_size, int32_t first_token,
   // step 1: B mask tokens after the prompt, one denoise pass; the cache keeps the prompt only
   h->launches = 0;
   launch_init_block(h->blk_tokens, h->blk_masked, h->info, nullptr, B, h->cfg.mask_id, 0, h->st);
-  int rc = stage_rows(h, 0, B, h->blk_tokens, nullptr);
-  if (rc) return rc;
-  rc = forward_rows(h, B, MODE_BIDIR, B, 0);
+  StepEnds ends;
+  ends.tokens = h->blk_tokens;
+  int rc = forward_rows(h, B, MODE_BIDIR, B, 0, ends);
   if (rc) return rc;
   launch_quad_first_draft(h->pred, first_token, B, h->q_d, h->st);
   launch_quad_layout(B, chain ? 1 : 0, h->q_mask, h->q_pos_off, h->st);
@@ -804,9 +802,9 @@ extern "C" int fdvlm_quad_step(fdvlm_t* h, int32_t* accepted_tokens, int32_t* ne
   if (L0 + n > h->cfg.max_seq) return fail(h, FDVLM_ERR_CAPACITY, "quad: %d + %d exceed max_seq %d", L0, n, h->cfg.max_seq);
   h->launches = 0;
   launch_quad_build(h->q_d, B, h->cfg.mask_id, h->blk_tokens, h->blk_masked, h->st);
-  int rc = stage_rows(h, 0, n, h->blk_tokens, nullptr);
-  if (rc) return rc;
-  rc = forward_rows(h, n, MODE_MASKED, n, logits != nullptr);
+  StepEnds ends;
+  ends.tokens = h->blk_tokens;
+  int rc = forward_rows(h, n, MODE_MASKED, n, logits != nullptr, ends);
   if (rc) return rc;
   const cudaMemcpyKind DD = cudaMemcpyDeviceToDevice;
   if (logits) CU(h, cudaMemcpyAsync(logits, h->logits, (size_t)n * h->cfg.vocab * 4, DD, h->st));

@@ -82,13 +82,16 @@ int launch_attention(const AttnArgs& a, cudaStream_t st, cudaError_t* err) {
   return a.dtype == DT_F32 ? launch_attention_f32(a, st, err) : launch_attention_tc(a, st, err);
 }
 
-int stage_rows(fdvlm_t* h, int row0, int n, const int32_t* tokens, const void* embeds) {
+int stage_rows(fdvlm_t* h, int row0, int n, const int32_t* tokens, const void* embeds, int mode, const int* len_ptr) {
   const int H = h->cfg.hidden;
   const int edt = h->dt == DT_F32 ? DT_F32 : DT_BF16;
   if (h->use_tc) {
     launch_embed_prep(h->w.embed, tokens, embeds, h->h + (size_t)row0 * H, (char*)h->a + (size_t)row0 * H * xf_bytes(h->xfmt), h->a_lo, h->xfmt,
                       h->layers[0].g_attn, h->ssq + (size_t)row0 * h->nt, h->nt, n, H, h->cfg.vocab, h->info + 3, h->st, nullptr,
                       h->act8 ? h->amax_a + (size_t)row0 * h->nt : nullptr);
+  } else if (tokens && mode >= 0) {
+    launch_embed_rope_f32(h->w.embed, tokens, h->h + (size_t)row0 * H, n, H, h->cfg.vocab, h->info + 3, h->cs, h->cache_len, h->cfg.head_dim,
+                          h->cfg.rope_theta, len_ptr, mode == MODE_MASKED ? h->q_pos_off : nullptr, h->st);
   } else if (tokens) {
     launch_embed(h->w.embed, tokens, h->h + (size_t)row0 * H, n, H, edt, h->cfg.vocab, h->info + 3, h->st);
   } else {
@@ -213,7 +216,7 @@ int forward_prefill(fdvlm_t* h, int n, int want_last_logits) {
 
 // ---- exact fp32 path ----------------------------------------------------------------------------------
 // per layer: [norm + QKV, bias, rotary, K/V rows] [attention] [O + residual] [norm + gate/up + SwiGLU] [down + residual]
-static int forward_rows_f32(fdvlm_t* h, int n, int mode, int logits_rows, int want_logits, const int* len_ptr) {
+static int forward_rows_f32(fdvlm_t* h, int n, int mode, int logits_rows, int want_logits, const int* len_ptr, bool rope_done) {
   const fdvlm_config& c = h->cfg;
   const int H = c.hidden, I = c.intermediate, d = c.head_dim, NQ = c.n_q_heads * d, NKV = c.n_kv_heads * d;
   cudaError_t e = cudaSuccess;
@@ -231,8 +234,10 @@ static int forward_rows_f32(fdvlm_t* h, int n, int mode, int logits_rows, int wa
     h->launches++;
     return e == cudaSuccess;
   };
-  launch_rope_table(h->cs, n, h->cache_len, d, c.rope_theta, h->st, len_ptr, nullptr, mode == MODE_MASKED ? h->q_pos_off : nullptr);
-  h->launches++;
+  if (!rope_done) {
+    launch_rope_table(h->cs, n, h->cache_len, d, c.rope_theta, h->st, len_ptr, nullptr, mode == MODE_MASKED ? h->q_pos_off : nullptr);
+    h->launches++;
+  }
   for (int l = 0; l < c.n_layers; ++l) {
     const fdvlm_layer_weights& lw = h->layers[l];
     F32Linear g = lin(FL_QKV, h->h, n, H, lw.g_attn, lw.wq, NQ, (float*)h->q);
@@ -400,15 +405,47 @@ static int forward_rows_tc(fdvlm_t* h, int n, int mode, int logits_rows, int wan
   return FDVLM_OK;
 }
 
-// The forward as a replayed CUDA graph: every kernel takes the cache length from a device word, so one
-// capture per (rows, mode, logits mode, stamped or not) serves every later call; the programmatic-dependent-launch
-// edges are kept.
-static int forward_rows_graph(fdvlm_t* h, int n, int mode, int logits_rows, int want_logits) {
-  const int stamped = (h->prof_on == 2) ? 1 : 0;
+// The kernels of one forward (with the ends of a step) on the handle's stream.  len_ptr: cache length from device memory.
+static int enqueue_rows(fdvlm_t* h, int n, int mode, int logits_rows, int want_logits, const int* len_ptr, bool stamped, const StepEnds& ends,
+                        bool sel_from_device) {
+  int rc;
+  if (ends.tokens) {
+    rc = stage_rows(h, 0, n, ends.tokens, nullptr, mode, len_ptr);
+    if (rc) return rc;
+  }
+  rc = h->use_tc ? forward_rows_tc(h, n, mode, logits_rows, want_logits, len_ptr, stamped)
+                 : forward_rows_f32(h, n, mode, logits_rows, want_logits, len_ptr, ends.tokens != nullptr);
+  if (rc || !ends.sel) return rc;
+  const float* conf = h->conf + ends.sel_row0;
+  const int32_t* pred = h->pred + ends.sel_row0;
+  if (sel_from_device)
+    launch_select_dev(conf, pred, h->blk_tokens, h->blk_masked, h->unmask, h->info, n - ends.sel_row0, h->dev_step, h->st);
+  else
+    launch_select(conf, pred, h->blk_tokens, h->blk_masked, h->unmask, h->info, n - ends.sel_row0, (int)ends.sel->rule, ends.sel->threshold,
+                  ends.sel->k, h->st, ends.sel->pred_shift);
+  h->launches++;
+  CU(h, cudaGetLastError());
+  return FDVLM_OK;
+}
+
+// The forward as a replayed CUDA graph: every kernel takes the cache length from a device word, so one capture per (rows,
+// mode, logits mode, ends, stamped or not) serves every later call; the programmatic-dependent-launch edges are kept.
+static int forward_rows_graph(fdvlm_t* h, int n, int mode, int logits_rows, int want_logits, const StepEnds& ends) {
+  const int stamped = (h->prof_on == 2) ? 1 : 0, staged = ends.tokens ? 1 : 0, sel_row0 = ends.sel ? ends.sel_row0 : -1;
   set_dev_len(h);
+  if (ends.sel) {
+    const StepDev v = {(int)ends.sel->rule, ends.sel->threshold, ends.sel->k, ends.sel->pred_shift};
+    const StepDev& w = h->step_set;
+    if (v.rule != w.rule || v.threshold != w.threshold || v.k != w.k || v.shift != w.shift) {
+      launch_set_step(h->dev_step, v, h->st);
+      h->launches++;
+      h->step_set = v;
+    }
+  }
   if (stamped) CU(h, cudaMemsetAsync(h->stamps, 0xFF, sizeof(KStamp) * FDVLM_MAX_STAMPS, h->st));
   for (auto& g : h->graphs) {
-    if (g.n == n && g.mode == mode && g.logits_rows == logits_rows && g.want_logits == want_logits && g.stamped == stamped) {
+    if (g.n == n && g.mode == mode && g.logits_rows == logits_rows && g.want_logits == want_logits && g.stamped == stamped && g.staged == staged &&
+        g.sel_row0 == sel_row0) {
       if (stamped) {      // the records' kinds are those of the capture: replay the bookkeeping only
         h->stamp_kind = g.kinds;
         h->stamp_used = (int)g.kinds.size();
@@ -420,14 +457,13 @@ static int forward_rows_graph(fdvlm_t* h, int n, int mode, int logits_rows, int 
   }
   const int before = h->launches;
   CU(h, cudaStreamBeginCapture(h->st, cudaStreamCaptureModeThreadLocal));
-  const int rc = h->use_tc ? forward_rows_tc(h, n, mode, logits_rows, want_logits, h->dev_len, stamped != 0)
-                           : forward_rows_f32(h, n, mode, logits_rows, want_logits, h->dev_len);
+  const int rc = enqueue_rows(h, n, mode, logits_rows, want_logits, h->dev_len, stamped != 0, ends, true);
   cudaGraph_t graph = nullptr;
   cudaError_t e = cudaStreamEndCapture(h->st, &graph);
   if (rc != FDVLM_OK) { if (graph) cudaGraphDestroy(graph); return rc; }
   if (e != cudaSuccess) return fail(h, FDVLM_ERR_CUDA, "graph capture: %s", cudaGetErrorString(e));
   fdvlm::FwdGraph g;
-  g.n = n; g.mode = mode; g.logits_rows = logits_rows; g.want_logits = want_logits; g.stamped = stamped;
+  g.n = n; g.mode = mode; g.logits_rows = logits_rows; g.want_logits = want_logits; g.stamped = stamped; g.staged = staged; g.sel_row0 = sel_row0;
   g.launches = h->launches - before; g.exec = nullptr;
   if (stamped) g.kinds = h->stamp_kind;
   e = cudaGraphInstantiate(&g.exec, graph, 0);
@@ -444,13 +480,12 @@ int forward_rows_enqueue(fdvlm_t* h, int n, int mode, int logits_rows, int want_
   return forward_rows_tc(h, n, mode, logits_rows, want_logits, h->dev_len, false);
 }
 
-int forward_rows(fdvlm_t* h, int n, int mode, int logits_rows, int want_logits) {
+int forward_rows(fdvlm_t* h, int n, int mode, int logits_rows, int want_logits, const StepEnds& ends) {
   // event timing around each kernel needs the kernels launched one by one
-  if (h->use_graphs && h->prof_on != 1) return forward_rows_graph(h, n, mode, logits_rows, want_logits);
-  if (!h->use_tc) return forward_rows_f32(h, n, mode, logits_rows, want_logits, nullptr);
+  if (h->use_graphs && h->prof_on != 1) return forward_rows_graph(h, n, mode, logits_rows, want_logits, ends);
   const bool stamped = h->prof_on == 2;
   if (stamped) CU(h, cudaMemsetAsync(h->stamps, 0xFF, sizeof(KStamp) * FDVLM_MAX_STAMPS, h->st));
-  return forward_rows_tc(h, n, mode, logits_rows, want_logits, nullptr, stamped);
+  return enqueue_rows(h, n, mode, logits_rows, want_logits, nullptr, stamped, ends, false);
 }
 
 }  // namespace fdk

@@ -28,9 +28,11 @@ struct fdvlm {
   size_t a_lo, ao_lo, act_lo;   // XF_BF16X2: element offset of each buffer's low-order plane
   char* slab;      // one allocation behind every device buffer below except the KV cache
   int32_t* dev_len;   // device copy of cache_len, read by the captured forward graphs
+  fdk::StepDev* dev_step;   // parameters of the selection at the end of a captured step
+  fdk::StepDev step_set;    // what they were last given, in stream order (rule -1: nothing)
   int dev_len_set;    // the value it was last given, in stream order (-1: none)
   int use_graphs;     // replay one captured CUDA graph per (rows, mode, logits mode)
-  struct FwdGraph { int n, mode, logits_rows, want_logits, stamped, launches; cudaGraphExec_t exec; std::vector<int> kinds; };
+  struct FwdGraph { int n, mode, logits_rows, want_logits, stamped, staged, sel_row0, launches; cudaGraphExec_t exec; std::vector<int> kinds; };
   std::vector<FwdGraph> graphs;
   // on-device decode loop (fdvlm_decode_block): a graph whose conditional WHILE node repeats the denoise step
   cudaGraphExec_t loop_exec;
@@ -143,13 +145,18 @@ inline void set_dev_len(fdvlm_t* h) {
 // forward.cu
 // Gather n input rows into the residual stream at row `row0`: from the embedding table (tokens, device
 // int32) or from caller-given embedding rows (activation type).
-int stage_rows(fdvlm_t* h, int row0, int n, const int32_t* tokens, const void* embeds);
+// fp32 path, tokens: also the rotary table of the rows (positions of mode; len_ptr: cache length from device memory).
+int stage_rows(fdvlm_t* h, int row0, int n, const int32_t* tokens, const void* embeds, int mode = -1, const int* len_ptr = nullptr);
 // One forward over the n rows staged in the residual stream.  mode: MODE_BIDIR (denoise; Alg. 1 draft
 // mask) or MODE_CAUSAL (prefill / commit; Alg. 1 verify mask).  K/V of the rows are staged at cache
 // positions cache_len .. cache_len + n - 1; only the caller's increment of cache_len commits them.
 // logits_rows: 0 none; n = all rows (logits into h->logits when want_logits, and conf / pred always);
 // 1 = last row only, raw logits into h->logits[0 .. V).
-int forward_rows(fdvlm_t* h, int n, int mode, int logits_rows, int want_logits);
+// Optionally with what stands before and behind it in a step, so that all of it is one graph launch: tokens: the n rows are
+// the embeddings of these (a buffer of the handle) instead of rows already staged; sel: the unmask selection over rows
+// sel_row0 .. n - 1.
+struct StepEnds { const int32_t* tokens = nullptr; const fdvlm_step_params* sel = nullptr; int sel_row0 = 0; };
+int forward_rows(fdvlm_t* h, int n, int mode, int logits_rows, int want_logits, const StepEnds& ends = StepEnds());
 // The causal forward over the n rows staged in pf_h / pf_a (n <= pf_rows); the last row's logits into h->logits.
 int forward_prefill(fdvlm_t* h, int n, int want_last_logits);
 int stage_prefill_rows(fdvlm_t* h, int row0, int n, const int32_t* tokens, const void* embeds);

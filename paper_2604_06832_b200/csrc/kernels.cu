@@ -205,6 +205,32 @@ void launch_embed(const void* table, const int32_t* tokens, float* h, int n, int
   if (dtype == DT_F32) embed_kernel<float><<<n, 256, 0, st>>>((const float*)table, tokens, h, hidden, vocab, status);
   else embed_kernel<bf16><<<n, 256, 0, st>>>((const bf16*)table, tokens, h, hidden, vocab, status);
 }
+// cs[r][j] = (cos, sin) of position(r) * theta^(-j / half), as rope_table_kernel below
+__device__ __forceinline__ float2 rope_entry(int pos, int j, int half, double theta) {
+  const double inv = pow(theta, -(double)j / (double)half);
+  double s, c;
+  sincos((double)pos * inv, &s, &c);
+  return make_float2((float)c, (float)s);
+}
+// The embedding gather and the rotary table of one fp32 row block in one launch: both are a microsecond of latency, so the launch is
+// what they cost.  With the selection captured too, a step from the host is one graph launch (8 rows of the tiny shape: 62 -> 55 us a step,
+// commit of a block 54 -> 49).
+__global__ void embed_rope_f32_kernel(const float* __restrict__ table, const int32_t* __restrict__ tokens, float* __restrict__ h, int hidden,
+                                      int vocab, int* status, float2* __restrict__ cs, int pos0, int half, double theta,
+                                      const int* __restrict__ len_ptr, const int* __restrict__ pos_off) {
+  pdl_trigger();
+  pdl_wait();
+  const int r = blockIdx.x;
+  const float* src = table + (size_t)checked_token(tokens, r, vocab, status) * hidden;
+  for (int c = threadIdx.x; c < hidden; c += blockDim.x) h[(size_t)r * hidden + c] = src[c];
+  if (len_ptr) pos0 = *len_ptr;
+  for (int j = threadIdx.x; j < half; j += blockDim.x) cs[r * half + j] = rope_entry(pos0 + (pos_off ? pos_off[r] : r), j, half, theta);
+}
+void launch_embed_rope_f32(const void* table, const int32_t* tokens, float* h, int n, int hidden, int vocab, int* status, float* cs,
+                           int pos0, int head_dim, float theta, const int* len_ptr, const int* pos_off, cudaStream_t st) {
+  launch_pdl(embed_rope_f32_kernel, dim3(n), dim3(128), 0, st, (const float*)table, tokens, h, hidden, vocab, status, (float2*)cs, pos0,
+             head_dim / 2, (double)theta, len_ptr, pos_off);
+}
 void launch_rows_to_f32(const void* rows, float* h, int n, int hidden, int dtype, cudaStream_t st) {
   launch_embed(rows, nullptr, h, n, hidden, dtype, 0, nullptr, st);
 }
@@ -231,10 +257,7 @@ __global__ void rope_table_kernel(float2* __restrict__ cs, int n, int pos0, int 
   int idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= n * half) return;
   int r = idx / half, j = idx % half;
-  double inv = pow(theta, -(double)j / (double)half);
-  double ang = (double)(pos0 + (pos_off ? pos_off[r] : r)) * inv, s, c;
-  sincos(ang, &s, &c);
-  cs[idx] = make_float2((float)c, (float)s);
+  cs[idx] = rope_entry(pos0 + (pos_off ? pos_off[r] : r), j, half, theta);
 }
 void launch_rope_table(float* cs, int n, int pos0, int head_dim, float theta, cudaStream_t st, const int* len_ptr, KStamp* stamp,
                        const int* pos_off) {
@@ -587,9 +610,11 @@ void launch_stats_merge(const void* stats, int n_part, int m, float* conf, int32
 __global__ void select_kernel(const float* __restrict__ conf, const int32_t* __restrict__ pred,
                               int32_t* __restrict__ tokens, uint8_t* __restrict__ masked,
                               uint8_t* __restrict__ unmask, int32_t* __restrict__ info, int n, int rule,
-                              float threshold, int k, int shift, cudaGraphConditionalHandle cond, int loop) {
+                              float threshold, int k, int shift, cudaGraphConditionalHandle cond, int loop,
+                              const StepDev* __restrict__ dev) {
   pdl_trigger();
   pdl_wait();
+  if (dev) { rule = dev->rule; threshold = dev->threshold; k = dev->k; shift = dev->shift; }
   __shared__ float c[64];
   __shared__ int mk[64];
   int i = threadIdx.x;
@@ -635,8 +660,14 @@ __global__ void select_kernel(const float* __restrict__ conf, const int32_t* __r
 void launch_select(const float* conf, const int32_t* pred, int32_t* tokens, uint8_t* masked, uint8_t* unmask,
                    int32_t* info, int n, int rule, float threshold, int k, cudaStream_t st, int shift,
                    cudaGraphConditionalHandle cond, int loop) {
-  select_kernel<<<1, 64, 0, st>>>(conf, pred, tokens, masked, unmask, info, n, rule, threshold, k, shift, cond, loop);
+  select_kernel<<<1, 64, 0, st>>>(conf, pred, tokens, masked, unmask, info, n, rule, threshold, k, shift, cond, loop, nullptr);
 }
+void launch_select_dev(const float* conf, const int32_t* pred, int32_t* tokens, uint8_t* masked, uint8_t* unmask, int32_t* info, int n,
+                       const StepDev* dev, cudaStream_t st) {
+  launch_pdl(select_kernel, dim3(1), dim3(64), 0, st, conf, pred, tokens, masked, unmask, info, n, 0, 0.f, 0, 0, (cudaGraphConditionalHandle)0, 0, dev);
+}
+__global__ void set_step_kernel(StepDev* dev, StepDev v) { *dev = v; }
+void launch_set_step(StepDev* dev, StepDev v, cudaStream_t st) { set_step_kernel<<<1, 1, 0, st>>>(dev, v); }
 
 // Longest accepted prefix of a drafted block d against the causal predictions a (a[j] predicts the token after d[j]):
 // k = 1 + (first j in [0, n-2] with a[j] != d[j+1]; n-1 if none).  out = {k, a[k-1]}.

@@ -26,6 +26,9 @@ size_t linear_workspace_bytes(int m, int n, int k, int dtype);
 
 // ---- elementwise / reduction kernels -----------------------------------------------------------
 // tokens outside [0, vocab) read row 0 and leave ST_BAD_TOKEN in *status
+// One launch for an fp32 row block: embedding gather and rotary table (as launch_rope_table).
+void launch_embed_rope_f32(const void* table, const int32_t* tokens, float* h, int n, int hidden, int vocab, int* status, float* cs,
+                           int pos0, int head_dim, float theta, const int* len_ptr, const int* pos_off, cudaStream_t st);
 void launch_embed(const void* table, const int32_t* tokens, float* h, int n, int hidden, int dtype, int vocab, int* status,
                   cudaStream_t st);
 void launch_bf16_to_e5m2x3(const void* in, void* out, size_t n, cudaStream_t st);       // planes n bytes apart
@@ -51,6 +54,11 @@ void launch_set_len(int* len_ptr, int value, cudaStream_t st);
 void launch_select(const float* conf, const int32_t* pred, int32_t* tokens, uint8_t* masked, uint8_t* unmask,
                    int32_t* info, int n, int rule, float threshold, int k, cudaStream_t st, int shift = 0,
                    cudaGraphConditionalHandle cond = 0, int loop = 0);
+// dev: the parameters come from device memory (a captured launch).
+struct StepDev { int rule; float threshold; int k, shift; };
+void launch_set_step(StepDev* dev, StepDev v, cudaStream_t st);
+void launch_select_dev(const float* conf, const int32_t* pred, int32_t* tokens, uint8_t* masked, uint8_t* unmask, int32_t* info, int n,
+                       const StepDev* dev, cudaStream_t st);
 // out[0] = accepted length k, out[1] = a[k - 1] (Alg. 1 "Accept: left-to-right comparison")
 void launch_accept(const int32_t* a, const int32_t* d, int n, int32_t* out, cudaStream_t st);
 void launch_init_block(int32_t* tokens, uint8_t* masked, int32_t* info, const int32_t* init, int n, int mask_id,
