@@ -85,7 +85,8 @@ extern "C" int fdvlm_create(const fdvlm_config* cfg, const fdvlm_weights* w, voi
   h->prof_on = 0;
   h->prof_used = 0;
   h->kv = nullptr; h->h = nullptr; h->a = h->ao = h->act = h->q = nullptr; h->cs = nullptr; h->ssq = nullptr;
-  h->amax_a = h->amax_ao = h->amax_act = nullptr;
+  h->amax_a = h->amax_ao = h->amax_act = h->xscale = nullptr;
+  h->codes = nullptr;
   h->stats = nullptr; h->logits = nullptr; h->conf = nullptr; h->pred = nullptr; h->unmask = nullptr; h->blk_tokens = nullptr;
   h->blk_masked = nullptr; h->info = nullptr; h->init_stage = nullptr; h->ws = nullptr; h->info_host = nullptr;
   h->host_stage = nullptr;
@@ -152,6 +153,8 @@ extern "C" int fdvlm_create(const fdvlm_config* cfg, const fdvlm_weights* w, voi
       {(void**)&h->amax_a, h->act8 ? (size_t)R * h->nt * 4 : 16},
       {(void**)&h->amax_ao, h->act8 ? (size_t)R * cfg->n_q_heads * 4 : 16},
       {(void**)&h->amax_act, h->act8 ? (size_t)R * 4 : 16},
+      {(void**)&h->codes, h->act8 ? (size_t)R * std::max(H, std::max(NQ, I)) : 16},
+      {(void**)&h->xscale, h->act8 ? (size_t)R * 4 : 16},
       {(void**)&h->cs, (size_t)R * d * 4},
       {(void**)&h->stamps, h->use_tc ? sizeof(KStamp) * FDVLM_MAX_STAMPS : 16},
       {(void**)&h->h, (size_t)R * H * 4},
@@ -166,7 +169,7 @@ extern "C" int fdvlm_create(const fdvlm_config* cfg, const fdvlm_weights* w, voi
   size_t slab_bytes = 0;
   for (auto& a : allocs) slab_bytes += (a.bytes + 255) / 256 * 256;
   // Prompt path: as many rows as one forward of it takes (PF_MAX_ROWS: above that its tiles fill the GPU many times over
-  // and more rows only cost memory).  W8A8 prompts run through the decode path's quantising GEMM.
+  // and more rows only cost memory).  W8A8 prompts run through the decode path.
   size_t pf_bytes = 0;
   if (h->use_tc && !h->act8 && cfg->max_seq > PF_MIN_ROWS) {
     const int max_rows = (cfg->max_seq + 127) / 128 * 128;

@@ -11,17 +11,17 @@ int launch_attention_f32(const AttnArgs& a, cudaStream_t st, cudaError_t* err);
 size_t attention_tc_workspace_bytes(int n, int hq, int hkv, int d);
 int launch_attention_tc(const AttnArgs& a, cudaStream_t st, cudaError_t* err);
 void launch_splitk_epilogue(const float* part, int S, int m, int n, const float* scale, const float* bias, float* y, int ldy,
-                            int accumulate, cudaStream_t st, const float* row_amax = nullptr);
+                            int accumulate, cudaStream_t st, const float* x_scale = nullptr);
 
 thread_local char g_create_error[512] = "";
 
 // Stand-alone projection.  The caller's workspace starts with OP_HEAD bytes for the two status words (see
-// TcOut::status; cleared here on the stream), then -- fp8 weights only -- the bf16 rows as XF_E5M2X3 planes (W8A8: as f16 rows,
-// followed by one 256-byte-rounded array of per-row maxima), then the split-K partial sums.
-static size_t op_amax_bytes(int m, int dtype) { return dtype == DT_A8 ? (((size_t)m * 4 + 255) / 256) * 256 : 0; }
+// TcOut::status; cleared here on the stream), then -- fp8 weights only -- the bf16 rows as XF_E5M2X3 planes (W8A8: as e4m3
+// codes, followed by one 256-byte-rounded array of per-row factors), then the split-K partial sums.
+static size_t op_scale_bytes(int m, int dtype) { return dtype == DT_A8 ? (((size_t)m * 4 + 255) / 256) * 256 : 0; }
 static size_t op_x16_bytes(int m, int k, int dtype) {
   if (dtype == DT_FP8) return (((size_t)m * k * 3 + 255) / 256) * 256;
-  return dtype == DT_A8 ? (((size_t)m * k * 2 + 255) / 256) * 256 + op_amax_bytes(m, dtype) : 0;
+  return dtype == DT_A8 ? (((size_t)m * k + 255) / 256) * 256 + op_scale_bytes(m, dtype) : 0;
 }
 size_t linear_workspace_bytes(int m, int n, int k, int dtype) {
   const int wdt = dtype == DT_A8 ? DT_FP8 : dtype;
@@ -50,10 +50,10 @@ int launch_linear(const LinearArgs& a, cudaStream_t st, cudaError_t* err) {
   g.fp8 = (a.dtype == DT_FP8 || a8); g.a8 = a8;
   const size_t x16 = op_x16_bytes(a.m, a.k, a.dtype);
   if (b.workspace_bytes < x16) { *err = cudaErrorInvalidValue; return -1; }
-  float* row_amax = a8 ? (float*)((char*)b.workspace + x16 - op_amax_bytes(a.m, a.dtype)) : nullptr;
+  float* x_scale = a8 ? (float*)((char*)b.workspace + x16 - op_scale_bytes(a.m, a.dtype)) : nullptr;
   int launched = 2;
-  if (a8) {        // f16 rows and each row's maximum: the kernel quantises the rows to e4m3 itself
-    launch_bf16_rows_to_f16_amax(a.x, b.workspace, a.m, a.k, row_amax, st);
+  if (a8) {
+    launch_quantize_bf16_rows(a.x, a.m, a.k, b.workspace, x_scale, st);
     g.x = b.workspace;
     ++launched;
   } else if (g.fp8) {
@@ -68,10 +68,9 @@ int launch_linear(const LinearArgs& a, cudaStream_t st, cudaError_t* err) {
   memset(&o, 0, sizeof(o));
   o.mode = TC_MODE_PARTIAL; o.part = part; o.part_bytes = b.workspace_bytes - x16; o.splits_out = &splits;
   o.ld = a.n; o.status = (int*)a.workspace;
-  o.amax_in = row_amax; o.n_amax_in = 1;
   *err = tc_group_launch(g, o, st);
   if (*err != cudaSuccess) return -1;
-  launch_splitk_epilogue(part, splits, a.m, a.n, a.scale, a.bias, a.y, a.ldy, a.accumulate, st, row_amax);
+  launch_splitk_epilogue(part, splits, a.m, a.n, a.scale, a.bias, a.y, a.ldy, a.accumulate, st, x_scale);
   *err = cudaGetLastError();
   return *err == cudaSuccess ? launched : -1;
 }
@@ -308,7 +307,15 @@ static int forward_rows_tc(fdvlm_t* h, int n, int mode, int logits_rows, int wan
     set_rows(&g, x, lo_off, row0_elems, h->xfmt);
     g.m = m; g.k = k; g.n_mats = nm;
     g.w[0] = w0; g.n[0] = n0; g.w[1] = w1; g.n[1] = n1; g.w[2] = w2; g.n[2] = n2;
-    g.a8 = a8;
+    return g;
+  };
+  // W8A8: a projection's input rows as e4m3 codes, from the partial maxima that whoever wrote them left
+  const float* xs = a8 ? h->xscale : nullptr;
+  auto quantised = [&](TcGroup g, const float* amax, int n_amax) {
+    if (!a8) return g;
+    launch_quantize_rows(g.x, g.m, g.k, amax, n_amax, h->codes, h->xscale, h->st);
+    h->launches++;
+    g.x = h->codes; g.x_lo = g.x_3 = nullptr; g.a8 = 1;
     return g;
   };
   auto out = [&](int tc_mode, int kind) {
@@ -332,12 +339,11 @@ static int forward_rows_tc(fdvlm_t* h, int n, int mode, int logits_rows, int wan
     int S = 0;
     TcOut o = out(TC_MODE_PARTIAL, FDVLM_K_GEMM_QKV);
     o.ld = NQKV; o.splits_out = &S;
-    o.amax_in = a8 ? h->amax_a : nullptr; o.n_amax_in = nt;
-    if (!gemm(group(h->a, h->a_lo, 0, n, H, 3, lw.wq, NQ, lw.wk, NKV, lw.wv, NKV), o))
+    if (!gemm(quantised(group(h->a, h->a_lo, 0, n, H, 3, lw.wq, NQ, lw.wk, NKV, lw.wv, NKV), h->amax_a, nt), o))
       return fail(h, FDVLM_ERR_CUDA, "qkv projection launch: %s", cudaGetErrorString(e));
     launch_fin_qkv(part, S, n, h->cs, h->ssq, nt, H, c.rms_eps, lw.bq, lw.bk, lw.bv, lw.s_q, lw.s_k, lw.s_v, h->q, kv_ptr(h, l, 0), kv_ptr(h, l, 1),
                    h->cache_len, c.n_q_heads, c.n_kv_heads, d, c.max_seq, h->kv_type, h->st, len_ptr, stamp(FDVLM_K_FIN_QKV),
-                   a8 ? h->amax_a : nullptr, a8 ? h->amax_act : nullptr);
+                   xs, a8 ? h->amax_act : nullptr);
     AttnArgs at;
     memset(&at, 0, sizeof(at));
     at.len_ptr = len_ptr;
@@ -356,29 +362,27 @@ static int forward_rows_tc(fdvlm_t* h, int n, int mode, int logits_rows, int wan
     h->launches += r + 1;
     o = out(TC_MODE_PARTIAL, FDVLM_K_GEMM_O);
     o.ld = H; o.splits_out = &S;
-    o.amax_in = a8 ? h->amax_ao : nullptr; o.n_amax_in = c.n_q_heads;
-    if (!gemm(group(h->ao, h->ao_lo, 0, n, NQ, 1, lw.wo, H, nullptr, 0, nullptr, 0), o))
+    if (!gemm(quantised(group(h->ao, h->ao_lo, 0, n, NQ, 1, lw.wo, H, nullptr, 0, nullptr, 0), h->amax_ao, c.n_q_heads), o))
       return fail(h, FDVLM_ERR_CUDA, "o projection launch: %s", cudaGetErrorString(e));
     launch_fin_resid(part, S, n, H, h->h, lw.g_mlp, h->a, h->a_lo, h->xfmt, h->ssq, nt, lw.s_o, h->st, stamp(FDVLM_K_FIN_RESID),
-                     a8 ? h->amax_ao : nullptr, c.n_q_heads, a8 ? h->amax_a : nullptr);
+                     xs, a8 ? h->amax_a : nullptr);
     o = out(TC_MODE_SWIGLU, FDVLM_K_GEMM_GATE_UP);
     o.act = h->act; o.act_lo_off = h->act_lo; o.act_fmt = h->xfmt;
     o.ssq_in = h->ssq; o.nt_in = nt; o.hidden = H; o.eps = c.rms_eps;
-    o.amax_in = a8 ? h->amax_a : nullptr; o.n_amax_in = nt; o.amax_out = a8 ? h->amax_act : nullptr;
+    o.x_scale = xs; o.amax_out = a8 ? h->amax_act : nullptr;
     TcGroup gu = group(h->a, h->a_lo, 0, n, H, 2, lw.w_gate, I, lw.w_up, I, nullptr, 0);
     gu.scale[0] = lw.s_gate; gu.scale[1] = lw.s_up;
-    if (!gemm(gu, o))
+    if (!gemm(quantised(gu, h->amax_a, nt), o))
       return fail(h, FDVLM_ERR_CUDA, "gate/up projection launch: %s", cudaGetErrorString(e));
     o = out(TC_MODE_PARTIAL, FDVLM_K_GEMM_DOWN);
     o.ld = H; o.splits_out = &S;
-    o.amax_in = a8 ? h->amax_act : nullptr; o.n_amax_in = 1;
-    if (!gemm(group(h->act, h->act_lo, 0, n, I, 1, lw.w_down, H, nullptr, 0, nullptr, 0), o))
+    if (!gemm(quantised(group(h->act, h->act_lo, 0, n, I, 1, lw.w_down, H, nullptr, 0, nullptr, 0), h->amax_act, 1), o))
       return fail(h, FDVLM_ERR_CUDA, "down projection launch: %s", cudaGetErrorString(e));
     // the last layer feeds the LM head, whose table (a tied bf16 embedding under fp8 layer weights) may want another format
     const bool last = (l + 1 == c.n_layers);
     const float* g_next = last ? h->w.g_final : h->layers[l + 1].g_attn;
     launch_fin_resid(part, S, n, H, h->h, g_next, h->a, h->a_lo, last ? h->head_fmt : h->xfmt, h->ssq, nt, lw.s_down, h->st,
-                     stamp(FDVLM_K_FIN_RESID), a8 ? h->amax_act : nullptr, 1, (a8 && !last) ? h->amax_a : nullptr);
+                     stamp(FDVLM_K_FIN_RESID), xs, (a8 && !last) ? h->amax_a : nullptr);
     h->launches += 2;
   }
   if (logits_rows > 0) {
@@ -391,7 +395,6 @@ static int forward_rows_tc(fdvlm_t* h, int n, int mode, int logits_rows, int wan
     o.stats = h->stats; o.mask_id = c.mask_id;
     TcGroup lm = group(h->a, h->a_lo, (size_t)first * H, m, H, 1, table, c.vocab, nullptr, 0, nullptr, 0);
     set_rows(&lm, h->a, h->a_lo, (size_t)first * H, h->head_fmt);
-    lm.a8 = 0;                                       // the LM head keeps 16-bit input rows
     if (!c.tie_embeddings) lm.scale[0] = h->w.s_lm_head;
     if (!gemm(lm, o))
       return fail(h, FDVLM_ERR_CUDA, "lm head launch: %s", cudaGetErrorString(e));

@@ -29,9 +29,7 @@
 namespace fdk {
 
 constexpr int TC_THREADS = 192;       // warp 0 TMA producer, warp 1 MMA issuer, warps 2..5 epilogue
-constexpr int TC_THREADS_A8 = 320;    // + warps 6..9: quantise the rows (W8A8)
 constexpr int TC_A_BYTES = TC_BM * TC_BK * 2;   // a bf16 weight tile
-constexpr int TC_NCONV = 2;           // quantised-tile buffers (W8A8 only)
 
 enum { TC_ERR_PRODUCER = ST_PRODUCER, TC_ERR_MMA = ST_MMA, TC_ERR_EPILOGUE = ST_EPILOGUE };
 
@@ -66,80 +64,41 @@ struct TcParams {
   int* status;          // device words: [0] set non-zero when a wait timed out; [1] read at start: non-zero makes
                         // every role take its give-up path at once (a host-set test hook for that path)
   KStamp* stamp;        // in-chain timing of this launch (null: off)
-  // TC_KIND_A8: amax_in[row][n_amax_in] = partial maxima of |x[row]| left by the producer of x; the row's quantisation
-  // scale is their maximum / 448.  SWIGLU mode also raises amax_out[row] (atomic maximum; zero before the launch) to
-  // the maximum of |act[row]| as stored, for the consumer of `act`.
-  const float* amax_in; int n_amax_in;
+  // TC_KIND_A8: x_scale[row] = the factor of the row's e4m3 codes.  SWIGLU mode also raises amax_out[row] (atomic maximum;
+  // zero before the launch) to the maximum of |act[row]| as stored, for whoever quantises `act`.
+  const float* x_scale;
   float* amax_out;
 };
 
 // Operand kinds of the kernel:
 //   TC_KIND_BF16: bf16 weights x bf16 hi/lo activation planes
 //   TC_KIND_FP8 : e4m3 weights x three e5m2 planes of the activations; a k-block is 128 elements
-//   TC_KIND_A8  : e4m3 weights x activations quantised to e4m3 per row inside the kernel (W8A8, Sec. 3.4 "System
-//                 integration"); a k-block is 128 elements, the byte tile of the weights is the MMA operand as it lands
+//   TC_KIND_A8  : e4m3 weights x rows of e4m3 codes with one factor per row (W8A8, Sec. 3.4 "System integration"); a k-block
+//                 is 128 elements, both byte tiles are MMA operands as they land.  (Quantising the rows in warps of this kernel,
+//                 which had to wait for the row maxima first and then stood between every stage and its MMA, cost 4 us in each of
+//                 a layer's four projections.)
 enum { TC_KIND_BF16 = 0, TC_KIND_FP8 = 1, TC_KIND_A8 = 2 };
 
 template <int M_PAD, int KIND>
 struct TcSmem {
   static constexpr bool FP8 = KIND == TC_KIND_FP8, A8 = KIND == TC_KIND_A8;
-  static constexpr int STAGES = FP8 ? (M_PAD <= 16 ? 4 : (M_PAD <= 48 ? 3 : 2)) : (M_PAD <= 32 ? 4 : 3);   // two CTAs per SM must fit (A8, M_PAD > 32: one)
+  static constexpr int STAGES = A8 ? (M_PAD <= 32 ? 5 : 4) : (FP8 ? (M_PAD <= 16 ? 4 : (M_PAD <= 48 ? 3 : 2)) : (M_PAD <= 32 ? 4 : 3));   // two CTAs per SM must fit
   static constexpr int KB_ELEMS = (A8 || FP8) ? 2 * TC_BK : TC_BK;     // k per stage
   static constexpr int W_BYTES = TC_A_BYTES;                           // weight tile
-  static constexpr int B_BYTES = M_PAD * 128;                          // one activation plane (A8: one 64-k half, f16)
-  static constexpr int X_PLANES = FP8 ? 3 : 2;                         // e5m2 planes; bf16 hi + lo; A8: two 64-k halves
+  static constexpr int B_BYTES = M_PAD * 128;                          // one activation plane
+  static constexpr int X_PLANES = FP8 ? 3 : (A8 ? 1 : 2);              // e5m2 planes; bf16 hi + lo; codes
   static constexpr int STAGE_BYTES = W_BYTES + X_PLANES * B_BYTES;
-  static constexpr int CONV_OFF = STAGES * STAGE_BYTES;                // tiles made by the quantising warps
-  static constexpr int CONV_BYTES = A8 ? M_PAD * 128 : 0;              // e4m3 activation tile
-  static constexpr int EX_OFF = CONV_OFF + TC_NCONV * CONV_BYTES;      // SwiGLU epilogue: gate/up exchange
+  static constexpr int EX_OFF = STAGES * STAGE_BYTES;                  // SwiGLU epilogue: gate/up exchange
   static constexpr int EX_ROWS = KIND != TC_KIND_BF16 ? 16 : 32;       // rows that pass through it per round
   static constexpr int EX_ROUNDS = (M_PAD + EX_ROWS - 1) / EX_ROWS;
   static constexpr int EX_BYTES = (M_PAD / EX_ROUNDS) * 256;
   static constexpr int BAR_OFF = EX_OFF + EX_BYTES;
-  static constexpr int ROWSC_OFF = BAR_OFF + 256;                      // A8: the rows' quantisation scales and their reciprocals
-  static constexpr int RS_OFF = ROWSC_OFF + (A8 ? 512 : 0);            // the rows' folded norm factors
+  static constexpr int RS_OFF = BAR_OFF + 256;                         // the rows' folded norm factors
   static constexpr int TOTAL = RS_OFF + 256 + 1024;                    // + alignment slack
 };
 
-// Quantise NP 16-byte pieces (tid, tid + stride, ...) of the activation tile of one stage -- two 128-byte-swizzled f16
-// halves of 64 k each -- into the 128-byte-swizzled e4m3 tile [M_PAD rows][128 k] the MMA reads: code = e4m3(x / scale
-// of the row), float32 quotient, round to nearest even, saturating.  The quotient is formed without the division
-// routine: with y = RN(1 / scale), q0 = RN(x y) and the exact remainder r = x - q0 scale (one FMA), RN(q0 + r y) is the
-// correctly rounded x / scale (Markstein's correction step; no operand here is zero, infinite or subnormal except
-// x = 0, which gives 0 either way).
-template <int M_PAD, int NP>
-__device__ __forceinline__ void quantize_pieces(const uint8_t* x_tile, uint32_t dst, const volatile float2* row_scale, int tid, int stride) {
-#pragma unroll
-  for (int i = 0; i < NP; ++i) {
-    const int piece = tid + stride * i;
-    if (piece >= M_PAD * 8) break;
-    const int r = piece >> 3, j = piece & 7;                 // row, 16-byte piece (16 k) of the output row
-    const uint8_t* half = x_tile + (j >> 2) * (M_PAD * 128) + r * 128;
-    const int c0 = 2 * (j & 3);
-    const uint4 a = *reinterpret_cast<const uint4*>(half + ((c0 ^ (r & 7)) << 4));
-    const uint4 b = *reinterpret_cast<const uint4*>(half + (((c0 + 1) ^ (r & 7)) << 4));
-    const float sc = row_scale[r].x, rinv = row_scale[r].y;
-    const uint32_t in[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-    uint32_t out[4];
-#pragma unroll
-    for (int w = 0; w < 4; ++w) {
-      unsigned short pair[2];
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const __half2 hv = *reinterpret_cast<const __half2*>(&in[2 * w + h]);
-        const float a0 = __low2float(hv), a1 = __high2float(hv);
-        const float q0 = a0 * rinv, q1 = a1 * rinv;
-        const float x0 = fmaf(fmaf(-q0, sc, a0), rinv, q0), x1 = fmaf(fmaf(-q1, sc, a1), rinv, q1);
-        asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(pair[h]) : "f"(x1), "f"(x0));   // first source -> upper byte
-      }
-      out[w] = (uint32_t)pair[0] | ((uint32_t)pair[1] << 16);
-    }
-    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst + r * 128 + ((j ^ (r & 7)) << 4)), "r"(out[0]), "r"(out[1]), "r"(out[2]), "r"(out[3]) : "memory");
-  }
-}
-
 template <int M_PAD, int KIND>
-__global__ void __launch_bounds__(KIND == TC_KIND_A8 ? TC_THREADS_A8 : TC_THREADS, (KIND == TC_KIND_A8 && M_PAD <= 32) ? 2 : 1) gemm_tc_kernel(const __grid_constant__ TcParams p) {
+__global__ void __launch_bounds__(TC_THREADS) gemm_tc_kernel(const __grid_constant__ TcParams p) {
   extern __shared__ uint8_t smem_raw[];
   using L = TcSmem<M_PAD, KIND>;
   constexpr bool A8 = KIND == TC_KIND_A8;
@@ -150,23 +109,20 @@ __global__ void __launch_bounds__(KIND == TC_KIND_A8 ? TC_THREADS_A8 : TC_THREAD
   const uint32_t base = (raw + 1023u) & ~1023u;
   uint8_t* sm = smem_raw + (base - raw);
   const uint32_t bar0 = base + L::BAR_OFF;
-  // barrier slots (8 bytes each): full[S], empty[S], tmem_full[2], tmem_empty[2], conv_full[2], conv_empty[2]
+  // barrier slots (8 bytes each): full[S], empty[S], tmem_full[2], tmem_empty[2]
   auto full_bar = [&](int s) { return bar0 + 8u * s; };
   auto empty_bar = [&](int s) { return bar0 + 8u * (TC_STAGES + s); };
   auto tfull_bar = [&](int a) { return bar0 + 8u * (2 * TC_STAGES + a); };
   auto tempty_bar = [&](int a) { return bar0 + 8u * (2 * TC_STAGES + 2 + a); };
-  auto cfull_bar = [&](int c) { return bar0 + 8u * (2 * TC_STAGES + 4 + c); };
-  auto cempty_bar = [&](int c) { return bar0 + 8u * (2 * TC_STAGES + 6 + c); };
   // SwiGLU epilogue, per warp pair pr: exchange buffer written (exw) / read (exr), two arrivals each
-  auto exw_bar = [&](int pr) { return bar0 + 8u * (2 * TC_STAGES + 10 + pr); };
-  auto exr_bar = [&](int pr) { return bar0 + 8u * (2 * TC_STAGES + 12 + pr); };
-  volatile uint32_t* tmem_slot = (volatile uint32_t*)(sm + L::BAR_OFF + 8 * (2 * TC_STAGES + 8));
-  volatile int* abort_flag = (volatile int*)(sm + L::BAR_OFF + 8 * (2 * TC_STAGES + 8) + 8);
-  volatile float2* row_scale = reinterpret_cast<volatile float2*>(sm + L::ROWSC_OFF);   // A8 only: (scale, RN(1 / scale))
+  auto exw_bar = [&](int pr) { return bar0 + 8u * (2 * TC_STAGES + 6 + pr); };
+  auto exr_bar = [&](int pr) { return bar0 + 8u * (2 * TC_STAGES + 8 + pr); };
+  volatile uint32_t* tmem_slot = (volatile uint32_t*)(sm + L::BAR_OFF + 8 * (2 * TC_STAGES + 4));
+  volatile int* abort_flag = (volatile int*)(sm + L::BAR_OFF + 8 * (2 * TC_STAGES + 4) + 8);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // two accumulator buffers; each holds the products of plane i in columns [i M_PAD, (i + 1) M_PAD)
-  constexpr int ACC_COLS = A8 ? M_PAD : L::X_PLANES * M_PAD;
+  constexpr int ACC_COLS = L::X_PLANES * M_PAD;
   // (one buffer where two would leave no tensor memory for a second CTA on the SM)
   constexpr int NACC = 2 * ACC_COLS <= 256 ? 2 : 1;
   constexpr int TMEM_COLS = (NACC * ACC_COLS <= 32) ? 32 : ((NACC * ACC_COLS <= 64) ? 64 : ((NACC * ACC_COLS <= 128) ? 128 : 256));
@@ -174,7 +130,6 @@ __global__ void __launch_bounds__(KIND == TC_KIND_A8 ? TC_THREADS_A8 : TC_THREAD
   if (threadIdx.x == 0) {
     for (int s = 0; s < TC_STAGES; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
     for (int a = 0; a < 2; ++a) { mbar_init(tfull_bar(a), 1); mbar_init(tempty_bar(a), 4); }
-    for (int c = 0; c < TC_NCONV; ++c) { mbar_init(cfull_bar(c), 4); mbar_init(cempty_bar(c), 1); }
     for (int pr = 0; pr < 2; ++pr) { mbar_init(exw_bar(pr), 2); mbar_init(exr_bar(pr), 2); }
     stamp_start(p.stamp);
     *abort_flag = 0;
@@ -196,29 +151,6 @@ __global__ void __launch_bounds__(KIND == TC_KIND_A8 ? TC_THREADS_A8 : TC_THREAD
   const int total_tiles = p.tile_begin[p.n_mats];
   const int n_items = total_tiles * p.splits;
 
-  const int kbps = p.kb_per_split, kblocks = p.kblocks;
-  auto quantize_all = [&](int cvt_tid) -> bool {
-    int stage = 0, cbuf = 0;
-    uint32_t phase = 0, cphase = 0;
-    for (int it = blockIdx.x; it < n_items; it += gridDim.x) {
-      const int split = it / total_tiles;
-      const int kb0 = split * kbps;
-      const int kb1 = min(kblocks, kb0 + kbps);
-      for (int kb = kb0; kb < kb1; ++kb) {
-        if (!mbar_wait(full_bar(stage), phase, abort_flag) || !mbar_wait(cempty_bar(cbuf), cphase ^ 1u, abort_flag)) return false;
-        const uint8_t* src = sm + stage * L::STAGE_BYTES;
-        const uint32_t dst = base + L::CONV_OFF + cbuf * L::CONV_BYTES;
-        quantize_pieces<M_PAD, (M_PAD * 8 + 127) / 128>(src + L::W_BYTES, dst, row_scale, cvt_tid, 128);
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic writes -> the MMA's async-proxy reads
-        __syncwarp();
-        if (lane == 0) mbar_arrive(cfull_bar(cbuf));
-        if (++cbuf == TC_NCONV) { cbuf = 0; cphase ^= 1u; }
-        if (++stage == TC_STAGES) { stage = 0; phase ^= 1u; }
-      }
-    }
-    return true;
-  };
-
   if (warp == 0) {
     // ------------------------------------------------ TMA producer ------------------------------------------------
     if (lane == 0) {
@@ -235,12 +167,11 @@ __global__ void __launch_bounds__(KIND == TC_KIND_A8 ? TC_THREADS_A8 : TC_THREAD
       bool ok = !poisoned;
       bool waited = false;
       int n_pend = 0, pend_stage[TC_STAGES], pend_kb[TC_STAGES];
-      const uint32_t stage_tx = L::W_BYTES + (X3 ? 3 : ((A8 || p.has_lo) ? 2 : 1)) * L::B_BYTES;
+      const uint32_t stage_tx = L::W_BYTES + (X3 ? 3 : (p.has_lo ? 2 : 1)) * L::B_BYTES;
       auto load_x = [&](int st_, int kb_) {
         const uint32_t dst = base + st_ * L::STAGE_BYTES + L::W_BYTES;
         tma_load_2d(dst, &p.tm_x, full_bar(st_), kb_ * L::KB_ELEMS, 0, pol_x);
-        if (A8) tma_load_2d(dst + L::B_BYTES, &p.tm_x, full_bar(st_), kb_ * L::KB_ELEMS + TC_BK, 0, pol_x);   // second 64 k
-        if (!A8 && (X3 || p.has_lo)) tma_load_2d(dst + L::B_BYTES, &p.tm_xl, full_bar(st_), kb_ * L::KB_ELEMS, 0, pol_x);
+        if (X3 || p.has_lo) tma_load_2d(dst + L::B_BYTES, &p.tm_xl, full_bar(st_), kb_ * L::KB_ELEMS, 0, pol_x);
         if (X3) tma_load_2d(dst + 2 * L::B_BYTES, &p.tm_x3, full_bar(st_), kb_ * L::KB_ELEMS, 0, pol_x);
       };
       for (int it = blockIdx.x; it < n_items && ok; it += gridDim.x) {
@@ -307,8 +238,8 @@ __global__ void __launch_bounds__(KIND == TC_KIND_A8 ? TC_THREADS_A8 : TC_THREAD
     // ------------------------------------------------ MMA issuer --------------------------------------------------
     {
       const uint32_t idesc = A8 ? umma_idesc_e4m3(M_PAD) : (X3 ? umma_idesc_e4m3_e5m2(3 * M_PAD) : umma_idesc_bf16(p.has_lo ? 2 * M_PAD : M_PAD));
-      int stage = 0, cbuf = 0;
-      uint32_t phase = 0, cphase = 0;
+      int stage = 0;
+      uint32_t phase = 0;
       int local = 0;
       bool ok = true;
       for (int it = blockIdx.x; it < n_items && ok; it += gridDim.x, ++local) {
@@ -321,15 +252,11 @@ __global__ void __launch_bounds__(KIND == TC_KIND_A8 ? TC_THREADS_A8 : TC_THREAD
         const int kb0 = split * p.kb_per_split;
         const int kb1 = min(p.kblocks, kb0 + p.kb_per_split);
         for (int kb = kb0; kb < kb1; ++kb) {
-          // A8: the quantising warps have waited for the stage and left the activations in buffer cbuf; the weight bytes
-          // are read from the stage itself, whose barrier this thread then observes too
-          if (!mbar_wait(A8 ? cfull_bar(cbuf) : full_bar(stage), A8 ? cphase : phase, abort_flag)) { ok = false; break; }
-          if (A8 && !mbar_wait(full_bar(stage), phase, abort_flag)) { ok = false; break; }
+          if (!mbar_wait(full_bar(stage), phase, abort_flag)) { ok = false; break; }
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           const uint32_t a_addr = base + stage * L::STAGE_BYTES;
-          const uint32_t c_addr = base + L::CONV_OFF + cbuf * L::CONV_BYTES;
           const uint64_t adesc = umma_desc_sw128(a_addr);
-          const uint64_t bdesc = umma_desc_sw128(A8 ? c_addr : a_addr + L::W_BYTES);
+          const uint64_t bdesc = umma_desc_sw128(a_addr + L::W_BYTES);
           if (elect_one()) {
           if (W8) {
 #pragma unroll
@@ -341,10 +268,6 @@ __global__ void __launch_bounds__(KIND == TC_KIND_A8 ? TC_THREADS_A8 : TC_THREAD
               umma_bf16(d_tmem, adesc + 2u * kk, bdesc + 2u * kk, idesc, (kb > kb0 || kk > 0) ? 1u : 0u);
           }
           umma_commit(empty_bar(stage));
-          if (A8) umma_commit(cempty_bar(cbuf));
-          }
-          if (A8) {
-            if (++cbuf == TC_NCONV) { cbuf = 0; cphase ^= 1u; }
           }
           if (++stage == TC_STAGES) { stage = 0; phase ^= 1u; }
         }
@@ -352,34 +275,6 @@ __global__ void __launch_bounds__(KIND == TC_KIND_A8 ? TC_THREADS_A8 : TC_THREAD
       }
       if (!ok && lane == 0) atomicCAS(p.status, 0, TC_ERR_MMA);
     }
-  } else if (A8 && warp >= 6) {
-    // ------------------------------------------------ quantising warps (W8A8) ---------------------------------------
-    // First every row's scale = max of the producer's partial maxima / 448 (two threads per row; 1 for an all-zero row),
-    // then the activation tile of each stage, thread t taking the 16-byte pieces t, t + 128, ...
-    {
-      const int t = (int)threadIdx.x - 192, r = t >> 1;
-      pdl_wait();                      // the partial maxima are the predecessor's
-      float mx = 0.f;
-      if (r < p.m && p.amax_in) {
-        // sixteen loads in flight per thread: the usual counts (a few dozen partial maxima) cost one round trip
-        const float* src = p.amax_in + (size_t)r * p.n_amax_in;
-        for (int i0 = (t & 1); i0 < p.n_amax_in; i0 += 32) {
-          float v[16];
-#pragma unroll
-          for (int u = 0; u < 16; ++u) v[u] = (i0 + 2 * u < p.n_amax_in) ? __ldcg(src + i0 + 2 * u) : 0.f;
-#pragma unroll
-          for (int u = 0; u < 16; ++u) mx = fmaxf(mx, v[u]);
-        }
-      }
-      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-      if ((t & 1) == 0) {
-        const float sc = mx > 0.f ? __fdiv_rn(mx, 448.f) : 1.f;
-        row_scale[r].x = sc;
-        row_scale[r].y = __frcp_rn(sc);
-      }
-      asm volatile("bar.sync 2, 128;" ::: "memory");
-    }
-    if (!quantize_all(threadIdx.x - 192) && threadIdx.x == 192) atomicCAS(p.status, 0, TC_ERR_MMA);
   } else {
     // ------------------------------------------------ epilogue warps ----------------------------------------------
     const int q = warp & 3;  // TMEM lane quarter this warp may read
@@ -407,7 +302,7 @@ __global__ void __launch_bounds__(KIND == TC_KIND_A8 ? TC_THREADS_A8 : TC_THREAD
         }
       }
       s += __shfl_xor_sync(0xffffffffu, s, 1);
-      if ((t & 1) == 0) row_rs[r] = rsqrtf(s * p.inv_h + p.eps);
+      if ((t & 1) == 0) row_rs[r] = rsqrtf(s * p.inv_h + p.eps) * (A8 && r < p.m ? __ldcg(p.x_scale + r) : 1.f);
       asm volatile("bar.sync 1, 128;" ::: "memory");
       rs0 = row_rs[lane];
       rs1 = row_rs[lane + 32];
@@ -418,12 +313,6 @@ __global__ void __launch_bounds__(KIND == TC_KIND_A8 ? TC_THREADS_A8 : TC_THREAD
       const uint32_t acc_phase = (uint32_t)(local / NACC) & 1u;
       if (!mbar_wait(tfull_bar(acc), acc_phase, abort_flag)) { ok = false; break; }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      if (A8 && local == 0) {
-        // the converters left every row's quantisation scale in shared memory before the first tile they made; the
-        // accumulator holds sums of code products, so the scale multiplies the folded norm factor
-        rs0 *= row_scale[lane].x;
-        rs1 *= row_scale[lane + 32].x;
-      }
       float v[M_PAD];
       const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * ACC_COLS);
 #pragma unroll
@@ -438,7 +327,7 @@ __global__ void __launch_bounds__(KIND == TC_KIND_A8 ? TC_THREADS_A8 : TC_THREAD
 #pragma unroll
           for (int i = 0; i < 16; ++i) v[c + i] += fmaf(b2[i], 0.0078125f, b1[i] * 0.25f);
         }
-      } else if (!A8 && p.has_lo) {      // the low-order plane's product sits M_PAD columns further on
+      } else if (p.has_lo) {      // the low-order plane's product sits M_PAD columns further on
 #pragma unroll
         for (int c = 0; c < M_PAD; c += 16) {
           float lo[16];
@@ -480,6 +369,7 @@ __global__ void __launch_bounds__(KIND == TC_KIND_A8 ? TC_THREADS_A8 : TC_THREAD
           __syncwarp();
           if (lane == 0) mbar_arrive(exw_bar(pr));
           if (!mbar_wait(exw_bar(pr), par, abort_flag)) { ok = false; break; }
+          float am[HR];
 #pragma unroll
           for (int b = 0; b < HR; ++b) {
             const int lo = r * HR + b, hi = HALF + r * HR + b;
@@ -491,13 +381,14 @@ __global__ void __launch_bounds__(KIND == TC_KIND_A8 ? TC_THREADS_A8 : TC_THREAD
             const int row = side ? hi : lo;
             const float val = silu_mul(g, u);
             if (live && row < p.m) store_act(p.act, p.act_lo_off, (size_t)row * p.inter + col, val, p.act_fmt);
-            if (A8 && p.amax_out) {
-              // maximum of |act| as stored (f16) over this warp's 32 features, for the consumer's quantiser; values
-              // are non-negative, so their bit patterns order like integers (and the result does not depend on order)
-              float am = (live && row < p.m) ? fabsf(__half2float(__ushort_as_half(f16_bits_sat(val)))) : 0.f;
-              am = warp_max(am);
-              if (lane == 0 && row < p.m && am > 0.f) atomicMax(reinterpret_cast<int*>(p.amax_out) + row, __float_as_int(am));
-            }
+            if (A8) am[b] = (live && row < p.m) ? fabsf(__half2float(__ushort_as_half(f16_bits_sat(val)))) : 0.f;
+          }
+          if constexpr (A8) {
+            // maxima of |act| as stored (f16) over this warp's 32 features, for whoever quantises the rows: non-negative values,
+            // whose bit patterns order like integers (and the result does not depend on the order)
+            const float mx = warp_reduce_transposed<true, HR>(am, lane);
+            const int row = (side ? HALF : 0) + r * HR + lane;
+            if (lane < HR && row < p.m && mx > 0.f) atomicMax(reinterpret_cast<int*>(p.amax_out) + row, __float_as_int(mx));
           }
           __syncwarp();
           if (lane == 0) mbar_arrive(exr_bar(pr));
@@ -677,7 +568,7 @@ static cudaError_t tc_launch_t(const TcParams& p, int grid, cudaStream_t st) {
   static bool attr_set[MAX_DEVICES] = {};
   cudaError_t e = ensure_dynamic_smem(gemm_tc_kernel<M_PAD, KIND>, TcSmem<M_PAD, KIND>::TOTAL, attr_set);
   if (e != cudaSuccess) return e;
-  return launch_pdl(gemm_tc_kernel<M_PAD, KIND>, dim3(grid), dim3(KIND == TC_KIND_A8 ? TC_THREADS_A8 : TC_THREADS),
+  return launch_pdl(gemm_tc_kernel<M_PAD, KIND>, dim3(grid), dim3(TC_THREADS),
                     (size_t)TcSmem<M_PAD, KIND>::TOTAL, st, p);
 }
 
@@ -703,11 +594,11 @@ cudaError_t tc_group_launch(const TcGroup& g, const TcOut& o, cudaStream_t st) {
   memset(&p, 0, sizeof(p));
   const int mode = o.mode;
   const int mp = pad_m(g.m);
-  const bool a8 = g.fp8 && g.a8;                  // f16 rows that the kernel quantises to e4m3 itself
+  const bool a8 = g.fp8 && g.a8;                  // rows as e4m3 codes
   const bool x3 = g.fp8 && !a8;                   // rows as e5m2 planes
-  const int xkind = a8 ? TM_F16 : (x3 ? TM_E4M3_128 : TM_BF16);     // (bytes are bytes: e5m2 planes take the same map)
+  const int xkind = g.fp8 ? TM_E4M3_128 : TM_BF16;     // (bytes are bytes: e5m2 planes take the same map)
   if (a8 && (mode == TC_MODE_DIRECT || mode == TC_MODE_LOGITS)) return cudaErrorInvalidValue;
-  if (a8 && (!o.amax_in || o.n_amax_in < 1)) return cudaErrorInvalidValue;
+  if (a8 && mode == TC_MODE_SWIGLU && (!o.x_scale || !o.amax_out || !o.ssq_in)) return cudaErrorInvalidValue;
   if (!make_tmap(&p.tm_x, g.x, g.m, g.k, mp, xkind)) return cudaErrorInvalidValue;
   p.has_lo = (!g.fp8 && g.x_lo) ? 1 : 0;
   if ((x3 || p.has_lo) && !make_tmap(&p.tm_xl, g.x_lo, g.m, g.k, mp, xkind)) return cudaErrorInvalidValue;
@@ -726,7 +617,7 @@ cudaError_t tc_group_launch(const TcGroup& g, const TcOut& o, cudaStream_t st) {
   p.n_mats = g.n_mats;
   p.kblocks = ceil_div(g.k, g.fp8 ? 2 * TC_BK : TC_BK);
   p.m = g.m;
-  p.amax_in = o.amax_in; p.n_amax_in = o.n_amax_in; p.amax_out = o.amax_out;
+  p.x_scale = o.x_scale; p.amax_out = o.amax_out;
   p.mode = mode;
   p.status = o.status;
   p.stamp = o.stamp;

@@ -50,6 +50,7 @@ struct fdvlm {
   // W8A8: maxima of |value as stored| of the rows of a ([R, nt] partial maxima), ao ([R, Hq] partial maxima) and
   // act ([R], raised atomically by the gate/up epilogue, zeroed by the QKV finalisation of the same layer)
   float* amax_a; float* amax_ao; float* amax_act;
+  uint8_t* codes; float* xscale;   // W8A8: the input rows of the projection at hand as e4m3 codes, and their factors
   void* stats;     // [ceil(V/128)*4][R] float4 softmax statistics of the LM-head epilogue
   float* logits;   // [R, V]
   float* conf;     // [R]

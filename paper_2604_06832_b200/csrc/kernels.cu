@@ -115,7 +115,7 @@ linear_simt_kernel(const XT* __restrict__ x, const WT* __restrict__ w, float* __
 // y[r, n] = (accumulate ? y : 0) + (sum_s part[s][r][n]) * scale[n] + bias[n]; fixed summation order.
 __global__ void splitk_epilogue_kernel(const float* __restrict__ part, int S, int m, int N,
                                        const float* __restrict__ scale, const float* __restrict__ bias,
-                                       float* __restrict__ y, int ldy, int accumulate, const float* __restrict__ row_amax) {
+                                       float* __restrict__ y, int ldy, int accumulate, const float* __restrict__ x_scale) {
   pdl_trigger();
   pdl_wait();
   size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -125,16 +125,16 @@ __global__ void splitk_epilogue_kernel(const float* __restrict__ part, int S, in
   float s = 0.f;
   for (int i = 0; i < S; ++i) s += part[(size_t)i * total + idx];
   if (scale) s *= scale[n];
-  if (row_amax) s *= row_amax[r] > 0.f ? __fdiv_rn(row_amax[r], 448.f) : 1.f;   // sums of e4m3 code products: the row's scale
+  if (x_scale) s *= x_scale[r];   // sums of e4m3 code products
   if (bias) s += bias[n];
   float* o = y + (size_t)r * ldy + n;
   *o = accumulate ? (*o + s) : s;
 }
 
 void launch_splitk_epilogue(const float* part, int S, int m, int n, const float* scale, const float* bias, float* y, int ldy,
-                            int accumulate, cudaStream_t st, const float* row_amax) {
+                            int accumulate, cudaStream_t st, const float* x_scale) {
   size_t total = (size_t)m * n;
-  splitk_epilogue_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(part, S, m, n, scale, bias, y, ldy, accumulate, row_amax);
+  splitk_epilogue_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(part, S, m, n, scale, bias, y, ldy, accumulate, x_scale);
 }
 
 static void simt_plan(int m, int n, int k, int* bm, int* splits, int* kps) {
@@ -321,23 +321,60 @@ __global__ void bf16_to_e5m2x3_kernel(const bf16* __restrict__ in, uint8_t* __re
 void launch_bf16_to_e5m2x3(const void* in, void* out, size_t n, cudaStream_t st) {
   bf16_to_e5m2x3_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>((const bf16*)in, (uint8_t*)out, n);
 }
-// bf16 rows -> f16 rows (saturating), one block per row, which also leaves amax[row] = max |f16 value| of the row: what the quantising
-// projection takes its per-row scale from.
-__global__ void bf16_rows_to_f16_amax_kernel(const bf16* __restrict__ in, unsigned short* __restrict__ out, int k,
-                                             float* __restrict__ amax) {
+// Eight f16 values -> e4m3 codes of x / scale: float32 quotient, round to nearest even, saturating.  The quotient is formed
+// without the division routine: with y = RN(1 / scale), q0 = RN(x y) and the exact remainder r = x - q0 scale (one FMA),
+// RN(q0 + r y) is the correctly rounded x / scale (Markstein's correction step; no operand here is zero, infinite or
+// subnormal except x = 0, which gives 0 either way).
+__device__ __forceinline__ uint2 e4m3_codes8(uint4 x, float sc, float rinv) {
+  const uint32_t in[4] = {x.x, x.y, x.z, x.w};
+  unsigned short out[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&in[i]));
+    const float q0 = a.x * rinv, q1 = a.y * rinv;
+    const float x0 = fmaf(fmaf(-q0, sc, a.x), rinv, q0), x1 = fmaf(fmaf(-q1, sc, a.y), rinv, q1);
+    asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(out[i]) : "f"(x1), "f"(x0));   // first source -> upper byte
+  }
+  return make_uint2((uint32_t)out[0] | ((uint32_t)out[1] << 16), (uint32_t)out[2] | ((uint32_t)out[3] << 16));
+}
+// grid (ceil(k / 1024), rows), 128 threads, eight values each: two dependent L2 round trips, of which the maxima and the values share
+// the first, so the launch and those are what it costs (about 2 us) and more values a thread would only lengthen it.  Against quantising in the
+// projections' own warps: 8 layers of the 7B shape and the LM head 843 -> 731 us a step at 32 rows, 717 -> 657 at 8.
+__global__ void __launch_bounds__(128) quantize_rows_kernel(const unsigned short* __restrict__ x, int k, const float* __restrict__ amax,
+                                                            int n_amax, uint8_t* __restrict__ codes, float* __restrict__ scale) {
+  pdl_trigger();
+  pdl_wait();
+  const int r = blockIdx.y, c = (blockIdx.x * 128 + threadIdx.x) * 8, lane = threadIdx.x & 31;
+  uint4 v = make_uint4(0, 0, 0, 0);
+  if (c < k) v = __ldcg(reinterpret_cast<const uint4*>(x + (size_t)r * k + c));
+  float am = 0.f;
+  for (int i = lane; i < n_amax; i += 32) am = fmaxf(am, __ldcg(amax + (size_t)r * n_amax + i));
+  const float sc = scale_of_amax(warp_max(am));
+  if (c < k) *reinterpret_cast<uint2*>(codes + (size_t)r * k + c) = e4m3_codes8(v, sc, __frcp_rn(sc));
+  if (blockIdx.x == 0 && threadIdx.x == 0) scale[r] = sc;
+}
+void launch_quantize_rows(const void* x, int m, int k, const float* amax, int n_amax, void* codes, float* scale, cudaStream_t st) {
+  launch_pdl(quantize_rows_kernel, dim3((k + 1023) / 1024, m), dim3(128), 0, st, (const unsigned short*)x, k, amax, n_amax,
+             (uint8_t*)codes, scale);
+}
+__global__ void __launch_bounds__(256) quantize_bf16_rows_kernel(const bf16* __restrict__ in, int k, uint8_t* __restrict__ codes,
+                                                                 float* __restrict__ scale) {
   __shared__ float red[32];
   const size_t base = (size_t)blockIdx.x * k;
   float am = 0.f;
-  for (int c = threadIdx.x; c < k; c += blockDim.x) {
-    const unsigned short b = f16_bits_sat(__bfloat162float(in[base + c]));
-    out[base + c] = b;
-    am = fmaxf(am, fabsf(__half2float(__ushort_as_half(b))));
+  for (int c = threadIdx.x; c < k; c += blockDim.x) am = fmaxf(am, abs_as_f16(__bfloat162float(in[base + c])));
+  const float sc = scale_of_amax(block_max(am, red)), rinv = __frcp_rn(sc);
+  for (int c = threadIdx.x * 8; c < k; c += blockDim.x * 8) {
+    uint32_t w[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      w[i] = (uint32_t)f16_bits_sat(__bfloat162float(in[base + c + 2 * i])) | ((uint32_t)f16_bits_sat(__bfloat162float(in[base + c + 2 * i + 1])) << 16);
+    *reinterpret_cast<uint2*>(codes + base + c) = e4m3_codes8(make_uint4(w[0], w[1], w[2], w[3]), sc, rinv);
   }
-  am = block_max(am, red);
-  if (threadIdx.x == 0) amax[blockIdx.x] = am;
+  if (threadIdx.x == 0) scale[blockIdx.x] = sc;
 }
-void launch_bf16_rows_to_f16_amax(const void* in, void* out, int m, int k, float* amax, cudaStream_t st) {
-  bf16_rows_to_f16_amax_kernel<<<m, 256, 0, st>>>((const bf16*)in, (unsigned short*)out, k, amax);
+void launch_quantize_bf16_rows(const void* in, int m, int k, void* codes, float* scale, cudaStream_t st) {
+  quantize_bf16_rows_kernel<<<m, 256, 0, st>>>((const bf16*)in, k, (uint8_t*)codes, scale);
 }
 
 // Sum of S split-K partials p[i * stride].  These kernels are a handful of dependent L2 round trips long, so every
@@ -373,7 +410,7 @@ __global__ void fin_qkv_kernel(const float* __restrict__ part, int S, int m, con
                                const float* __restrict__ bq, const float* __restrict__ bk, const float* __restrict__ bv,
                                const float* __restrict__ sq, const float* __restrict__ sk, const float* __restrict__ sv,
                                T* __restrict__ q, T* __restrict__ kc, T* __restrict__ vc, int pos0, int hq, int hkv,
-                               int d, int max_seq, const int* __restrict__ len_ptr, const float* __restrict__ amax_in,
+                               int d, int max_seq, const int* __restrict__ len_ptr, const float* __restrict__ x_scale,
                                float* __restrict__ amax_zero, KStamp* stamp) {
   if (threadIdx.x == 0) stamp_start(stamp);
   pdl_trigger();
@@ -391,18 +428,17 @@ __global__ void fin_qkv_kernel(const float* __restrict__ part, int S, int m, con
   pdl_wait();
   if (threadIdx.x == 0) stamp_released(stamp);
   __shared__ float s_rstd;
-  // W8A8: the row's slot of the running maximum that this layer's gate/up epilogue raises; its last readers (the
-  // previous layer's down projection) are long done, its next writers start after this kernel
+  // W8A8: the row's slot of the running maximum that this layer's gate/up epilogue raises; its last reader (the
+  // quantisation in front of the previous layer's down projection) is long done, its next writers start after this kernel
   if (amax_zero && head == 0 && threadIdx.x == 0) amax_zero[r] = 0.f;
   // every load of this kernel is issued before the first result is needed
   const int width = (hq + 2 * hkv) * d;
   const size_t sstride = (size_t)m * width;
   const float* pa = part + (size_t)r * width + head * d + j;
-  float ssq_v = 0.f, am = 0.f;
+  float ssq_v = 0.f, xs = 1.f;
   if (threadIdx.x < 32) {
     for (int t = threadIdx.x; t < nt; t += 32) ssq_v += __ldcg(ssq + (size_t)r * nt + t);
-    if (amax_in)     // W8A8: the partial sums are sums of code products; the row's scale joins the norm factor
-      for (int t = threadIdx.x; t < nt; t += 32) am = fmaxf(am, __ldcg(amax_in + (size_t)r * nt + t));
+    if (x_scale) xs = __ldcg(x_scale + r);     // W8A8: the partial sums are sums of code products; the row's factor joins the norm's
   }
   const float2 c = (head < hq + hkv) ? __ldcg(&cs[r * half + j]) : make_float2(1.f, 0.f);
   Partials<16> va, vb;
@@ -411,8 +447,7 @@ __global__ void fin_qkv_kernel(const float* __restrict__ part, int S, int m, con
   if (threadIdx.x < 32) {
     // fixed order: lanes hold disjoint strided subsets, combined by the butterfly below
     const float t = warp_sum(ssq_v);
-    am = warp_max(am);
-    if (threadIdx.x == 0) s_rstd = rsqrtf(t * inv_h + eps) * (amax_in ? scale_of_amax(am) : 1.f);
+    if (threadIdx.x == 0) s_rstd = rsqrtf(t * inv_h + eps) * xs;
   }
   float a = add_partials(va, 0.f), b = add_partials(vb, 0.f);
   a = sum_partials_from(pa, sstride, 16, S, a);
@@ -440,14 +475,14 @@ __global__ void fin_qkv_kernel(const float* __restrict__ part, int S, int m, con
 }
 void launch_fin_qkv(const float* part, int S, int m, const float* cs, const float* ssq, int nt, int hidden, float eps,
                     const float* bq, const float* bk, const float* bv, const float* sq, const float* sk, const float* sv, void* q, void* kc, void* vc, int pos0, int hq,
-                    int hkv, int d, int max_seq, int kv_type, cudaStream_t st, const int* len_ptr, KStamp* stamp, const float* amax_in,
+                    int hkv, int d, int max_seq, int kv_type, cudaStream_t st, const int* len_ptr, KStamp* stamp, const float* x_scale,
                     float* amax_zero) {
   if (kv_type == KV_F16)
     launch_pdl(fin_qkv_kernel<__half>, dim3(hq + 2 * hkv, m), dim3(d / 2), 0, st, part, S, m, (const float2*)cs, ssq, nt, 1.f / (float)hidden,
-               eps, bq, bk, bv, sq, sk, sv, (__half*)q, (__half*)kc, (__half*)vc, pos0, hq, hkv, d, max_seq, len_ptr, amax_in, amax_zero, stamp);
+               eps, bq, bk, bv, sq, sk, sv, (__half*)q, (__half*)kc, (__half*)vc, pos0, hq, hkv, d, max_seq, len_ptr, x_scale, amax_zero, stamp);
   else
     launch_pdl(fin_qkv_kernel<bf16>, dim3(hq + 2 * hkv, m), dim3(d / 2), 0, st, part, S, m, (const float2*)cs, ssq, nt, 1.f / (float)hidden,
-               eps, bq, bk, bv, sq, sk, sv, (bf16*)q, (bf16*)kc, (bf16*)vc, pos0, hq, hkv, d, max_seq, len_ptr, amax_in, amax_zero, stamp);
+               eps, bq, bk, bv, sq, sk, sv, (bf16*)q, (bf16*)kc, (bf16*)vc, pos0, hq, hkv, d, max_seq, len_ptr, x_scale, amax_zero, stamp);
 }
 
 // Residual finalisation: h += sum of split-K partials; xg = h * gain of the next norm (stored as `fmt`);
@@ -455,24 +490,17 @@ void launch_fin_qkv(const float* part, int S, int m, const float* cs, const floa
 __global__ void __launch_bounds__(128) fin_resid_kernel(const float* __restrict__ part, int S, int m, int hidden,
                                                         float* __restrict__ h, const float* __restrict__ g,
                                                         void* __restrict__ xg, size_t lo_off, int fmt, float* __restrict__ ssq, int nt,
-                                                        const float* __restrict__ scale, const float* __restrict__ amax_in,
-                                                        int n_amax_in, float* __restrict__ amax_out, KStamp* stamp) {
+                                                        const float* __restrict__ scale, const float* __restrict__ x_scale,
+                                                        float* __restrict__ amax_out, KStamp* stamp) {
   if (threadIdx.x == 0) stamp_start(stamp);
   pdl_trigger();
-  __shared__ float red[32];
   const int t = blockIdx.x, r = blockIdx.y, c = t * 128 + threadIdx.x;
   // weights (gain, scale) do not depend on the predecessor
   const float gc = (c < hidden) ? g[c] : 0.f;
   float sc = (c < hidden && scale) ? scale[c] : 1.f;
   pdl_wait();
   if (threadIdx.x == 0) stamp_released(stamp);
-  // W8A8: the partial sums are sums of code products of a row quantised with the scale max / 448; the maxima are
-  // asked for first and reduced only after the other loads are on their way
-  float am_in = 0.f;
-  if (amax_in) {
-    if (n_amax_in == 1) am_in = __ldcg(amax_in + r);
-    else for (int i = threadIdx.x; i < n_amax_in; i += 128) am_in = fmaxf(am_in, __ldcg(amax_in + (size_t)r * n_amax_in + i));
-  }
+  const float xs = x_scale ? __ldcg(x_scale + r) : 1.f;     // W8A8: the partial sums are sums of code products
   float v = 0.f;
   Partials<32> pv;
   float hv = 0.f;
@@ -481,7 +509,7 @@ __global__ void __launch_bounds__(128) fin_resid_kernel(const float* __restrict_
     issue_partials(pv, part + idx, sstride, 0, S);
     hv = __ldcg(h + idx);
   }
-  if (amax_in) sc *= scale_of_amax(n_amax_in == 1 ? am_in : block_max(am_in, red));
+  sc *= xs;
   if (c < hidden) {
     v = hv + sum_partials_from(part + idx, sstride, 32, S, add_partials(pv, 0.f)) * sc;
     h[idx] = v;
@@ -545,10 +573,9 @@ void launch_fin_resid_rows(const float* part, int S, int m, int hidden, float* h
   launch_pdl(fin_resid_rows_kernel, dim3((m * nt + 7) / 8), dim3(256), 0, st, part, S, m, hidden, h, g, xg, lo_off, fmt, ssq, nt, scale);
 }
 void launch_fin_resid(const float* part, int S, int m, int hidden, float* h, const float* g, void* xg, size_t lo_off, int fmt,
-                      float* ssq, int nt, const float* scale, cudaStream_t st, KStamp* stamp, const float* amax_in, int n_amax_in,
-                      float* amax_out) {
-  launch_pdl(fin_resid_kernel, dim3(nt, m), dim3(128), 0, st, part, S, m, hidden, h, g, xg, lo_off, fmt, ssq, nt, scale, amax_in,
-             n_amax_in, amax_out, stamp);
+                      float* ssq, int nt, const float* scale, cudaStream_t st, KStamp* stamp, const float* x_scale, float* amax_out) {
+  launch_pdl(fin_resid_kernel, dim3(nt, m), dim3(128), 0, st, part, S, m, hidden, h, g, xg, lo_off, fmt, ssq, nt, scale, x_scale,
+             amax_out, stamp);
 }
 
 // Merge the per-warp softmax statistics of the LM-head epilogue into confidence and prediction per row.

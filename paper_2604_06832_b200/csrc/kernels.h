@@ -32,8 +32,10 @@ void launch_embed_rope_f32(const void* table, const int32_t* tokens, float* h, i
 void launch_embed(const void* table, const int32_t* tokens, float* h, int n, int hidden, int dtype, int vocab, int* status,
                   cudaStream_t st);
 void launch_bf16_to_e5m2x3(const void* in, void* out, size_t n, cudaStream_t st);       // planes n bytes apart
-// the same row by row, leaving amax[row] = max |f16 value| of the row
-void launch_bf16_rows_to_f16_amax(const void* in, void* out, int m, int k, float* amax, cudaStream_t st);
+// W8A8: rows of k f16 values (k a multiple of 8) -> e4m3 codes and scale[row] = max / 448, from amax[row][n_amax], partial maxima
+// of |value| left by whoever wrote the rows; and bf16 rows -> f16 (saturating) -> the same, maxima included.
+void launch_quantize_rows(const void* x, int m, int k, const float* amax, int n_amax, void* codes, float* scale, cudaStream_t st);
+void launch_quantize_bf16_rows(const void* in, int m, int k, void* codes, float* scale, cudaStream_t st);
 void launch_rows_to_f32(const void* rows, float* h, int n, int hidden, int dtype, cudaStream_t st);
 void launch_rope_table(float* cs, int n, int pos0, int head_dim, float theta, cudaStream_t st, const int* len_ptr = nullptr,
                        KStamp* stamp = nullptr, const int* pos_off = nullptr);
@@ -87,13 +89,13 @@ cudaError_t launch_linear_f32(const F32Linear& p, cudaStream_t st);
 enum { TC_MODE_PARTIAL = 0, TC_MODE_DIRECT = 1, TC_MODE_SWIGLU = 2, TC_MODE_LOGITS = 3 };
 // Up to three bf16 matrices that share x and K; their outputs sit side by side in one row of width ld.
 struct TcGroup {
-  const void* x; int m, k;   // bf16 weights: bf16 rows (hi plane); fp8 weights: XF_E5M2X3 rows (first plane); a8: f16 rows
+  const void* x; int m, k;   // bf16 weights: bf16 rows (hi plane); fp8 weights: XF_E5M2X3 rows (first plane); a8: rows of e4m3 codes
   const void* x_lo;          // bf16 weights, nullable: the rows' low-order bf16 plane (x = hi + lo); fp8 weights: second plane
   const void* x_3;           // fp8 weights: third plane
   const void* w[3]; int n[3]; int n_mats;
   const float* scale[3]; const float* bias[3];
   int fp8;   // weights are e4m3 bytes (scale[] holds the per-output-channel factors)
-  int a8;    // with fp8: the kernel quantises the f16 rows to e4m3, one scale per row (W8A8); PARTIAL and SWIGLU only
+  int a8;    // with fp8: the rows are e4m3 codes, one factor per row (W8A8); PARTIAL and SWIGLU only
 };
 // What the GEMM leaves behind.
 //   PARTIAL: part[split][m][ld] = split-K partial sums (*splits_out of them) for the caller's reduce kernel
@@ -112,10 +114,10 @@ struct TcOut {
   int* status;   // two device words: [0] set non-zero if a bounded wait inside the kernel gave up; [1] read at kernel
                  // start, non-zero sends every role down its give-up path at once
   KStamp* stamp; // in-chain timing of the launch, nullable
-  // a8 groups: amax_in[row][n_amax_in] = partial maxima of |x[row]| (as stored) left by whoever wrote x; the accumulators
-  // are sums of code products, so PARTIAL output still lacks the row's scale max / 448 (the reduce kernel applies it) while
-  // SWIGLU applies it itself and raises amax_out[row] (atomic maximum: zero before the launch) to max |act[row]|.
-  const float* amax_in; int n_amax_in;
+  // a8 groups: x_scale[row] = the factor of the row's codes.  The accumulators are sums of code products: PARTIAL output still
+  // lacks the factor (the reduce kernel applies it), SWIGLU applies it itself and raises amax_out[row] (atomic maximum: zero
+  // before the launch) to max |act[row]|.
+  const float* x_scale;
   float* amax_out;
 };
 // Tensor map of a 2-D row-major [rows, cols] tensor with box {64 columns, box_rows}, zero fill outside the tensor
@@ -162,10 +164,10 @@ void launch_fin_qkv(const float* part, int S, int m, const float* cs, const floa
                     const float* bq, const float* bk, const float* bv, const float* sq, const float* sk, const float* sv, void* q,
                     void* kc, void* vc, int pos0, int hq,
                     int hkv, int d, int max_seq, int kv_type, cudaStream_t st, const int* len_ptr = nullptr, KStamp* stamp = nullptr,
-                    const float* amax_in = nullptr, float* amax_zero = nullptr);
+                    const float* x_scale = nullptr, float* amax_zero = nullptr);
 void launch_fin_resid(const float* part, int S, int m, int hidden, float* h, const float* g, void* xg, size_t lo_off, int fmt,
                       float* ssq, int nt, const float* scale, cudaStream_t st, KStamp* stamp = nullptr,
-                      const float* amax_in = nullptr, int n_amax_in = 0, float* amax_out = nullptr);
+                      const float* x_scale = nullptr, float* amax_out = nullptr);
 void launch_fin_resid_rows(const float* part, int S, int m, int hidden, float* h, const float* g, void* xg, size_t lo_off, int fmt,
                            float* ssq, int nt, const float* scale, cudaStream_t st);
 void launch_stats_merge(const void* stats, int n_part, int m, float* conf, int32_t* pred, cudaStream_t st, KStamp* stamp = nullptr);
