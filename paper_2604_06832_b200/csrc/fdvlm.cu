@@ -181,6 +181,7 @@ extern "C" int fdvlm_create(const fdvlm_config* cfg, const fdvlm_weights* w, voi
         {(void**)&h->pf_ssq, P * h->nt * 4},  {(void**)&h->pf_a, P * H * 2 * a_planes},
         {(void**)&h->pf_q, P * NQ * 2},       {(void**)&h->pf_ao, P * NQ * 2 * planes},
         {(void**)&h->pf_act, P * I * 2 * planes}, {(void**)&h->pf_part, h->pf_part_bytes},
+        {(void**)&h->pf_arrived, (size_t)sm_count() * 4 * sizeof(unsigned)},
     };
     for (auto& a : pf) pf_bytes += (a.bytes + 255) / 256 * 256;
     e = cudaMalloc((void**)&h->pf_slab, pf_bytes);

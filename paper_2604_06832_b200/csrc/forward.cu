@@ -135,6 +135,7 @@ int forward_prefill(fdvlm_t* h, int n, int want_last_logits) {
     g.mode = mode; g.m = n; g.k = k; g.x_rows = (int)R; g.fp8 = fp8; g.n_mats = 1;
     g.x = x; g.x_lo = fp8 ? nullptr : (const char*)x + R * ld * 2;
     g.nt = nt; g.inv_h = 1.f / (float)H; g.eps = c.rms_eps; g.status = h->info + 3;
+    g.part = h->pf_part; g.arrived = h->pf_arrived;
     return g;
   };
   auto run = [&](const PfGemm& g) {
@@ -150,7 +151,7 @@ int forward_prefill(fdvlm_t* h, int n, int want_last_logits) {
     g.w[0] = w; g.n[0] = H;
     g.splits = prefill_splits(n, H, k);
     if (g.splits > 1 && (size_t)g.splits * n * H * sizeof(float) <= h->pf_part_bytes) {
-      g.mode = PF_PARTIAL; g.part = h->pf_part;
+      g.mode = PF_PARTIAL;
       if (!run(g)) return false;
       launch_fin_resid_rows(h->pf_part, g.splits, n, H, h->pf_h, gain, h->pf_a, R * H, fmt, h->pf_ssq, nt, scale, h->st);
       h->launches++;
@@ -159,6 +160,8 @@ int forward_prefill(fdvlm_t* h, int n, int want_last_logits) {
     g.scale[0] = scale; g.h = h->pf_h; g.gain = gain; g.out = h->pf_a; g.out_lo_off = R * H; g.out_fmt = fmt; g.ssq_out = h->pf_ssq;
     return run(g);
   };
+  // (a forward whose waits gave up may have left some)
+  CU(h, cudaMemsetAsync(h->pf_arrived, 0, (size_t)sm_count() * 4 * sizeof(unsigned), h->st));
   launch_rope_table(h->pf_cs, n, h->cache_len, d, c.rope_theta, h->st);
   h->launches++;
   for (int l = 0; l < c.n_layers; ++l) {

@@ -77,6 +77,7 @@ struct fdvlm {
   int pf_rows;
   char* pf_slab;
   float *pf_h, *pf_cs, *pf_ssq, *pf_part;
+  unsigned* pf_arrived;   // arrivals at tiles that several SM pairs work on (zero between forwards)
   void *pf_a, *pf_ao, *pf_act, *pf_q;
   size_t pf_part_bytes;
   int32_t* info_host;  // pinned

@@ -150,6 +150,7 @@ struct PfGemm {
   void *kc, *vc; const float* cs; int pos0, max_seq, d, kv_type;
   float* h; const float* gain; float* ssq_out;
   float* part; int splits;
+  unsigned* arrived;      // nullable: sm_count() * 4 zeroed words; with `part` (256 x 256 sums per two SMs) tiles may come in pieces
   int* status;
 };
 int prefill_splits(int m, int n, int k);
