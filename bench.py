@@ -500,7 +500,7 @@ def run_ours(args, wl, block):
                      "forward_ms_in_chain_timing": statistics.median(chain_total) / 1000.0 if chain_total else None,
                      "isolated": {"ms_per_forward": gemm_ms_isolated, "achieved": wbytes / (gemm_ms_isolated / 1000.0) / 1e9,
                                   "note": "the same launches timed one by one with CUDA events, without the chain's overlap"}},
-        "attention": {"kernel": "attn_mma_kernel + attn_combine_kernel, in-chain", "kv_bytes_per_forward": kv_bytes,
+        "attention": {"kernel": "attn_tc_kernel + attn_combine_kernel, in-chain", "kv_bytes_per_forward": kv_bytes,
                       "in_chain_ms_per_forward": attn_us_chain / 1000.0,
                       "achieved_gbs": kv_bytes / (attn_us_chain * 1e-6) / 1e9 if attn_us_chain > 0 else None},
         "chain_us_per_forward": {k_: round(v, 2) for k_, v in sorted(chain_us.items())},

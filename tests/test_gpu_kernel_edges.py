@@ -1,0 +1,85 @@
+"""GPU parity where a kernel's split of the work changes: the branches that the small models of the other files do not reach."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import fdvlm_oracle as orc
+from paper_2604_06832_b200 import inputs as I
+
+from helpers import make_pair, replay_decode, upload_prefix
+from test_gpu_prefill import BF16, FP8, check
+
+pytestmark = pytest.mark.gpu
+
+
+# ---- decode attention: one warp per (row, head) in the merge, more chunks than it takes at a time, chunks longer than the ring ----
+@pytest.mark.parametrize("elem", [torch.bfloat16, torch.float16], ids=["bf16", "f16"])
+@pytest.mark.parametrize("n,L,hq,hkv,d,causal", [(64, 3000, 16, 2, 128, 0), (64, 9000, 16, 2, 128, 1), (64, 4100, 32, 8, 64, 1),
+                                                 (8, 18000, 8, 1, 128, 0), (37, 2500, 28, 4, 128, 1)])
+def test_decode_attention_chunks_and_merge(elem, n, L, hq, hkv, d, causal):
+    from paper_2604_06832_b200 import binding as B
+    g = torch.Generator().manual_seed(n + L)
+    q, kc, vc = (torch.randn(*s, generator=g).to(elem) for s in ((n, hq, d), (hkv, L + n + 5, d), (hkv, L + n + 5, d)))
+    T = L + n
+    allowed = np.ones((n, T), dtype=bool)
+    if causal:
+        allowed[:, L:] = np.tril(np.ones((n, n), dtype=bool))
+    f = lambda t: t.double().numpy()
+    ref = orc.attend(f(q), f(kc)[:, :T].transpose(1, 0, 2), f(vc)[:, :T].transpose(1, 0, 2), allowed).reshape(n, hq * d)
+    out = B.op_attention(q.cuda(), kc.cuda(), vc.cuda(), L, bool(causal), dtype=B.DT_BF16)
+    torch.cuda.synchronize()
+    # P is rounded to the element type (relative 2^-9 or 2^-12): a sum of p v with sum p = 1 moves by at most that times max |v|,
+    # and the result is rounded once more
+    eps = 2.0 ** -9 if elem == torch.bfloat16 else 2.0 ** -12
+    bound = 2 * eps * float(vc.float().abs().max())
+    assert np.abs(out.double().cpu().numpy() - ref).max() <= bound
+
+
+# ---- exact fp32: depth beyond one shared-memory panel, ragged widths, every row tile, more keys than one pass holds ----
+WIDE_F32 = I.TINY.with_(n_layers=1, hidden=1096, intermediate=1112, vocab=1003, mask_id=1002)
+
+
+@pytest.mark.parametrize("n", [1, 7, 9, 17, 33])
+def test_exact_f32_row_tiles_and_ragged_widths(n):
+    check(WIDE_F32, [(0, n)])
+
+
+def test_exact_f32_attention_over_many_keys():
+    check(I.TINY.with_(n_layers=1), [(0, 2100), (0, 9)], max_seq=2200)
+
+
+# ---- prompts: tiles of the last wave in pieces along k, 256-row attention CTAs ----
+@pytest.mark.parametrize("shape,n", [
+    (BF16.with_(n_layers=1, hidden=1536, intermediate=2560, vocab=512, mask_id=511), 770),                        # gate/up
+    (BF16.with_(n_layers=1, hidden=2048, n_q_heads=16, intermediate=1536, vocab=512, mask_id=511), 2310),         # QKV, O, down
+    (FP8.with_(n_layers=1, hidden=2048, n_q_heads=32, n_kv_heads=4, intermediate=1792, vocab=512, mask_id=511), 1290)],
+    ids=["bf16-gate-up", "bf16-qkv-o-down", "fp8-gate-up"])
+def test_prompt_tiles_in_pieces(shape, n):
+    check(shape, [(n - 100, 100)])
+
+
+# ---- the captured step: rule and threshold change between replays of one graph ----
+@pytest.mark.parametrize("shape", [I.TINY, BF16], ids=["f32", "bf16"])
+def test_captured_step_follows_its_parameters(shape):
+    oracle, handle, _ = make_pair(shape, 5, max_seq=128, stream=torch.cuda.Stream())
+    emb, toks = I.make_prefix(shape, 30, 10, 3)
+    oracle.prefill(I.as_numpy_storage(emb), toks.numpy())
+    handle.prefill(*upload_prefix(emb, toks))
+    for rule, tau, k in ((orc.THRESHOLD, 0.9, 0), (orc.TOPK, 0.0, 3), (orc.TOPK, 0.0, 5), (orc.THRESHOLD, 1e-4, 0)):
+        replay_decode(oracle, handle, shape, 8, rule, tau, k)
+    handle.close()
+
+
+# ---- fp8 weights: the byte planes of rows whose values span the range of f16 ----
+def test_fp8_projection_of_rows_with_small_values():
+    from paper_2604_06832_b200 import binding as B
+    g = torch.Generator().manual_seed(3)
+    m, n, k = 40, 300, 640
+    x = (torch.randn(m, k, generator=g) * 10.0 ** (-7.0 * torch.rand(m, k, generator=g))).to(torch.bfloat16)
+    codes, scale = I.quantize_e4m3_rows(torch.randn(n, k, generator=g) * 0.02)
+    w = orc.to_f64(codes.numpy()) * scale.double().numpy()[:, None]
+    xv = x.double().numpy()
+    y = B.op_linear(x.cuda(), codes.cuda(), scale.cuda(), None, dtype=B.DT_FP8).double().cpu().numpy()
+    # f16 of a bf16 value and its planes are exact from 2^-13 up and off by at most 2^-24 below; fp32 sums of k products
+    bound = (2.0 ** -24 + 2.0 ** -25) * np.abs(w).sum(1)[None] + 2.0 ** -20 * (np.abs(xv) @ np.abs(w).T)
+    assert (np.abs(y - xv @ w.T) <= bound).all()
