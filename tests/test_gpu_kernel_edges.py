@@ -61,12 +61,15 @@ def test_prompt_tiles_in_pieces(shape, n):
 # ---- the captured step: rule and threshold change between replays of one graph ----
 @pytest.mark.parametrize("shape", [I.TINY, BF16], ids=["f32", "bf16"])
 def test_captured_step_follows_its_parameters(shape):
-    oracle, handle, _ = make_pair(shape, 5, max_seq=128, stream=torch.cuda.Stream())
+    stream = torch.cuda.Stream()
+    oracle, handle, _ = make_pair(shape, 5, max_seq=128, stream=stream)
     emb, toks = I.make_prefix(shape, 30, 10, 3)
     oracle.prefill(I.as_numpy_storage(emb), toks.numpy())
-    handle.prefill(*upload_prefix(emb, toks))
-    for rule, tau, k in ((orc.THRESHOLD, 0.9, 0), (orc.TOPK, 0.0, 3), (orc.TOPK, 0.0, 5), (orc.THRESHOLD, 1e-4, 0)):
-        replay_decode(oracle, handle, shape, 8, rule, tau, k)
+    with torch.cuda.stream(stream):       # (the commit is only enqueued: its logits are read back on the handle's own stream)
+        handle.prefill(*upload_prefix(emb, toks))
+        for rule, tau, k in ((orc.THRESHOLD, 0.9, 0), (orc.TOPK, 0.0, 3), (orc.TOPK, 0.0, 5), (orc.THRESHOLD, 1e-4, 0)):
+            replay_decode(oracle, handle, shape, 8, rule, tau, k)
+        handle.synchronize()
     handle.close()
 
 
