@@ -142,11 +142,11 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
     constexpr bool F16 = !__is_same(E, bf16);
     const uint32_t id_s = F16 ? umma_idesc_f16(AT_STEP) : umma_idesc_bf16(AT_STEP);
     const uint32_t id_o = (F16 ? umma_idesc_f16(D) : umma_idesc_bf16(D)) | (1u << 16);      // (V: MN-major)
-    bool ok = mbar_wait(q_full, 0, abort_flag);
+    bool ok = mbar_wait_warp(q_full, 0, abort_flag);
     auto score = [&](int w, int t) {
       if (!ok || t >= (w ? steps1 : steps0)) return;
       const int s = t % S::STAGES;
-      if (!mbar_wait(k_full(s), (uint32_t)(t / S::STAGES) & 1u, abort_flag)) { ok = false; return; }
+      if (!mbar_wait_warp(k_full(s), (uint32_t)(t / S::STAGES) & 1u, abort_flag)) { ok = false; return; }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint32_t ka = base + S::KV_OFF + s * 2 * S::TILE_BYTES + w * (AT_STEP * 128);
       if (elect_one()) {
@@ -161,7 +161,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
       const int steps = w ? steps1 : steps0;
       if (!ok || t >= steps) return;
       const int s = t % S::STAGES;
-      if (!mbar_wait(p_full(w), (uint32_t)t & 1u, abort_flag) || !mbar_wait(v_full(s), (uint32_t)(t / S::STAGES) & 1u, abort_flag)) { ok = false; return; }
+      if (!mbar_wait_warp(p_full(w), (uint32_t)t & 1u, abort_flag) || !mbar_wait_warp(v_full(s), (uint32_t)(t / S::STAGES) & 1u, abort_flag)) { ok = false; return; }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint64_t vd = umma_desc_sw128_mn(base + S::KV_OFF + (s * 2 + 1) * S::TILE_BYTES + w * (AT_STEP * 128), 16384);
       if (elect_one()) {
@@ -225,7 +225,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
     __syncwarp();
     if (lane == 0) mbar_arrive(q_full);
     for (int t = 0; t < steps && ok; ++t) {
-      if (!mbar_wait(s_full(w), (uint32_t)t & 1u, abort_flag)) { ok = false; break; }
+      if (!mbar_wait_warp(s_full(w), (uint32_t)t & 1u, abort_flag)) { ok = false; break; }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       float s[AT_STEP];
       tmem_ld32(ts, s);
@@ -256,7 +256,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
       if (j0 + AT_STEP > key_end) {
         // V rows past the last key hold whatever the cache holds there, and 0 x NaN would poison the product
         const int sg = t % S::STAGES, first = max(0, key_end - j0);
-        if (!mbar_wait(v_full(sg), (uint32_t)(t / S::STAGES) & 1u, abort_flag)) ok = false;
+        if (!mbar_wait_warp(v_full(sg), (uint32_t)(t / S::STAGES) & 1u, abort_flag)) ok = false;
         for (int v = wq * 32 + lane; ok && v < (AT_STEP - first) * CH; v += 128) {
           const int r = w * AT_STEP + first + v / CH, c = v % CH;
           const uint32_t a = base + S::KV_OFF + (sg * 2 + 1) * S::TILE_BYTES + (c >> 3) * 16384 + r * 128 + (((c & 7) ^ (r & 7)) << 4);
@@ -270,7 +270,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
       if (lane == 0) mbar_arrive(p_full(w));
     }
     for (int x = 0; x < 2; ++x)
-      if (ok && (x ? steps1 : steps0) > 0 && !mbar_wait(o_full(x), 0, abort_flag)) ok = false;
+      if (ok && (x ? steps1 : steps0) > 0 && !mbar_wait_warp(o_full(x), 0, abort_flag)) ok = false;
     // every load has been used up and every product is complete: the ring is free.  Each warpgroup stores half of the
     // columns of the sum of both accumulators.
     ok = named_barrier_and<256>(ok);

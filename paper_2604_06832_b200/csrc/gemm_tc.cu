@@ -246,13 +246,13 @@ __global__ void __launch_bounds__(TC_THREADS) gemm_tc_kernel(const __grid_consta
         const int split = it / total_tiles;
         const int acc = local % NACC;
         const uint32_t acc_phase = (uint32_t)(local / NACC) & 1u;
-        if (!mbar_wait(tempty_bar(acc), acc_phase ^ 1u, abort_flag)) { ok = false; break; }
+        if (!mbar_wait_warp(tempty_bar(acc), acc_phase ^ 1u, abort_flag)) { ok = false; break; }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const uint32_t d_tmem = tmem_base + (uint32_t)(acc * ACC_COLS);
         const int kb0 = split * p.kb_per_split;
         const int kb1 = min(p.kblocks, kb0 + p.kb_per_split);
         for (int kb = kb0; kb < kb1; ++kb) {
-          if (!mbar_wait(full_bar(stage), phase, abort_flag)) { ok = false; break; }
+          if (!mbar_wait_warp(full_bar(stage), phase, abort_flag)) { ok = false; break; }
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           const uint32_t a_addr = base + stage * L::STAGE_BYTES;
           const uint64_t adesc = umma_desc_sw128(a_addr);
@@ -311,7 +311,7 @@ __global__ void __launch_bounds__(TC_THREADS) gemm_tc_kernel(const __grid_consta
       const int tile = it % total_tiles, split = it / total_tiles;
       const int acc = local % NACC;
       const uint32_t acc_phase = (uint32_t)(local / NACC) & 1u;
-      if (!mbar_wait(tfull_bar(acc), acc_phase, abort_flag)) { ok = false; break; }
+      if (!mbar_wait_warp(tfull_bar(acc), acc_phase, abort_flag)) { ok = false; break; }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       float v[M_PAD];
       const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * ACC_COLS);
@@ -368,7 +368,7 @@ __global__ void __launch_bounds__(TC_THREADS) gemm_tc_kernel(const __grid_consta
           }
           __syncwarp();
           if (lane == 0) mbar_arrive(exw_bar(pr));
-          if (!mbar_wait(exw_bar(pr), par, abort_flag)) { ok = false; break; }
+          if (!mbar_wait_warp(exw_bar(pr), par, abort_flag)) { ok = false; break; }
           float am[HR];
 #pragma unroll
           for (int b = 0; b < HR; ++b) {
@@ -393,7 +393,7 @@ __global__ void __launch_bounds__(TC_THREADS) gemm_tc_kernel(const __grid_consta
           __syncwarp();
           if (lane == 0) mbar_arrive(exr_bar(pr));
           // the buffer may be rewritten once the partner has read it too
-          if (!mbar_wait(exr_bar(pr), par, abort_flag)) { ok = false; break; }
+          if (!mbar_wait_warp(exr_bar(pr), par, abort_flag)) { ok = false; break; }
         }
         if (!ok) break;
       } else if (p.mode == TC_MODE_LOGITS) {

@@ -130,7 +130,7 @@ __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const __gri
       constexpr bool F16 = sizeof(E) == 2 && !__is_same(E, bf16);
       const uint32_t id_s = F16 ? umma_idesc_f16(PA_STEP) : umma_idesc_bf16(PA_STEP);
       const uint32_t id_o = (F16 ? umma_idesc_f16(D) : umma_idesc_bf16(D)) | (1u << 16);      // (V: MN-major)
-      bool ok = mbar_wait(q_full, 0, abort_flag);
+      bool ok = mbar_wait_warp(q_full, 0, abort_flag);
       auto score = [&](int q, int t) {
         const uint32_t qa = base + q * S::TILE_BYTES, ka = base + S::K_OFF + ((t >> 1) & 1) * S::TILE_BYTES + (t & 1) * (PA_STEP * 128);
         if (elect_one()) {
@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const __gri
         }
       };
       auto value = [&](int q, int t) {
-        if (!mbar_wait(p_full(q, t), (uint32_t)(t >> 1) & 1u, abort_flag)) { ok = false; return; }
+        if (!mbar_wait_warp(p_full(q, t), (uint32_t)(t >> 1) & 1u, abort_flag)) { ok = false; return; }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const uint64_t vd = umma_desc_sw128_mn(base + S::V_OFF + ((t >> 1) & 1) * S::TILE_BYTES + (t & 1) * (PA_STEP * 128), 16384);
         if (elect_one()) {
@@ -157,7 +157,7 @@ __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const __gri
       auto scores = [&](int q, int t) {
         if (t >= ns || !ok) return;
         if (q == 0 && (t & 1) == 0) {
-          if (!mbar_wait(k_full((t >> 1) & 1), (uint32_t)(t >> 2) & 1u, abort_flag)) { ok = false; return; }
+          if (!mbar_wait_warp(k_full((t >> 1) & 1), (uint32_t)(t >> 2) & 1u, abort_flag)) { ok = false; return; }
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         }
         if (t < (q ? n1 : n0)) score(q, t);
@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const __gri
       };
       for (int t = 0; t < 2; ++t) { scores(0, t); scores(1, t); }
       for (int t = 0; t < ns && ok; ++t) {
-        if ((t & 1) == 0 && !mbar_wait(v_full((t >> 1) & 1), (uint32_t)(t >> 2) & 1u, abort_flag)) { ok = false; break; }
+        if ((t & 1) == 0 && !mbar_wait_warp(v_full((t >> 1) & 1), (uint32_t)(t >> 2) & 1u, abort_flag)) { ok = false; break; }
         if (t < n0) value(0, t);
         scores(0, t + 2);
         if (ok && t < n1) value(1, t);
@@ -186,7 +186,7 @@ __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const __gri
     float m_ref = -INFINITY, l = 0.f;
     bool ok = true;
     for (int t = 0; t < nq && ok; ++t) {
-      if (!mbar_wait(s_full(q, t), (uint32_t)(t >> 1) & 1u, abort_flag)) { ok = false; break; }
+      if (!mbar_wait_warp(s_full(q, t), (uint32_t)(t >> 1) & 1u, abort_flag)) { ok = false; break; }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint32_t tb = ts + (t & 1) * PA_STEP;
       float s[PA_STEP];
@@ -202,7 +202,7 @@ __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const __gri
       const float m = row_max64(s) * sl2;
       const bool grow = m > m_ref + 8.f;                      // (always in the first step: every row reads key 0)
       if (t > 0 && __any_sync(0xffffffffu, grow)) {
-        if (!mbar_wait(o_done(q), (uint32_t)(t - 1) & 1u, abort_flag)) { ok = false; break; }
+        if (!mbar_wait_warp(o_done(q), (uint32_t)(t - 1) & 1u, abort_flag)) { ok = false; break; }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const float f = grow ? ex2(m_ref - m) : 1.f;
         scale_acc<D>(to, f);
@@ -213,7 +213,7 @@ __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const __gri
       if (j0 + PA_STEP > key_end) {
         // V rows past the last key hold whatever the cache holds there, and 0 x NaN would poison the product: cleared by
         // both row tiles (the same zeros)
-        if (!mbar_wait(v_full((t >> 1) & 1), (uint32_t)(t >> 2) & 1u, abort_flag)) ok = false;
+        if (!mbar_wait_warp(v_full((t >> 1) & 1), (uint32_t)(t >> 2) & 1u, abort_flag)) ok = false;
         const int first = key_end - j0;
         for (int v = wq * 32 + lane; ok && v < (PA_STEP - first) * (D / 8); v += 128) {
           const int r = (t & 1) * PA_STEP + first + v / (D / 8), c = v % (D / 8);
@@ -228,7 +228,7 @@ __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const __gri
       __syncwarp();
       if (lane == 0) mbar_arrive(p_full(q, t));
     }
-    if (nq > 0 && ok && !mbar_wait(o_full(q), 0, abort_flag)) ok = false;
+    if (nq > 0 && ok && !mbar_wait_warp(o_full(q), 0, abort_flag)) ok = false;
     if (nq > 0 && ok) {
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const float inv = 1.f / l;

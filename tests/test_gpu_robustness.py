@@ -62,6 +62,41 @@ def test_give_up_path_of_the_bounded_waits(shape, on_stream):
     handle.close()
 
 
+@pytest.mark.parametrize("shape,n", [
+    (SMALL_BF16.with_(n_layers=2, hidden=1536, intermediate=2560, vocab=512, mask_id=511), 770),
+    (SMALL_FP8.with_(n_layers=2, hidden=2048, n_q_heads=32, n_kv_heads=4, intermediate=1792, vocab=512, mask_id=511), 1290)],
+    ids=["bf16", "fp8"])
+def test_give_up_path_of_the_prompt_kernels(shape, n):
+    """The same for the kernels of long prompts (CTA pairs, whose exit needs both CTAs; gate/up tiles that come in pieces along k,
+    whose arrival counters an abandoned forward may leave non-zero; attention of whole row blocks).  They are deterministic, so
+    after the flag is cleared the handle gives what it gave before, bit for bit."""
+    b = B()
+    stream = torch.cuda.Stream()
+    handle = b.Handle(shape, b.weights_to_device(I.make_weights(shape, 31)), max_seq=n + 64, stream=stream)
+    emb, toks = I.make_prefix(shape, n - 100, 100, 8)
+
+    def prompt():
+        last = torch.zeros(shape.vocab, dtype=torch.float32, device="cuda")
+        handle.reset()
+        handle.prefill(*upload_prefix(emb, toks), last)
+        handle.synchronize()
+        kv = [handle.cache_read(l, w, 0, n) for l in range(shape.n_layers) for w in (0, 1)]
+        torch.cuda.synchronize()
+        return [last] + kv
+
+    with torch.cuda.stream(stream):
+        before = prompt()
+        assert all(torch.isfinite(t.float()).all() for t in before) and before[0].any()
+        for _ in range(2):
+            handle.debug_poison(True)
+            with pytest.raises(b.FdvlmError) as e:
+                prompt()
+            assert e.value.code == b.ERR_TIMEOUT and "gave up" in str(e.value)
+            handle.debug_poison(False)
+            assert all(torch.equal(x, y) for x, y in zip(before, prompt()))
+    handle.close()
+
+
 def test_poisoned_operator_call_reports_through_its_status_query():
     b = B()
     m, n, k = 32, 1024, 512

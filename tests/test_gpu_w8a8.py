@@ -130,8 +130,8 @@ def test_w8a8_model_is_as_close_to_the_oracle_as_rounding_allows(shape, B_, L_e,
 
 
 def test_w8a8_give_up_path_and_recovery():
-    """The quantising GEMM kind under the poison flag: every role (the converter warps included) leaves by the branch a
-    timed-out wait takes, the call reports FDVLM_ERR_TIMEOUT, and after the flag is cleared the handle computes, bit for
+    """The quantising GEMM kind under the poison flag: every role leaves by the branch a timed-out wait
+    takes, the call reports FDVLM_ERR_TIMEOUT, and after the flag is cleared the handle computes, bit for
     bit, what it computed before (the path is deterministic)."""
     b = B()
     w = I.make_weights(SMALL, 7, gain_spread=0.5)
