@@ -486,9 +486,15 @@ int forward_rows_enqueue(fdvlm_t* h, int n, int mode, int logits_rows, int want_
   return forward_rows_tc(h, n, mode, logits_rows, want_logits, h->dev_len, false);
 }
 
+static bool being_captured(cudaStream_t st) {
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  return cudaStreamIsCapturing(st, &status) == cudaSuccess && status != cudaStreamCaptureStatusNone;
+}
+
 int forward_rows(fdvlm_t* h, int n, int mode, int logits_rows, int want_logits, const StepEnds& ends) {
-  // event timing around each kernel needs the kernels launched one by one
-  if (h->use_graphs && h->prof_on != 1) return forward_rows_graph(h, n, mode, logits_rows, want_logits, ends);
+  // Event timing around each kernel needs the kernels launched one by one.  So does a stream that the caller is capturing: it
+  // takes no second capture, and the caller's graph may be replayed when the device's length word holds something else.
+  if (h->use_graphs && h->prof_on != 1 && !being_captured(h->st)) return forward_rows_graph(h, n, mode, logits_rows, want_logits, ends);
   const bool stamped = h->prof_on == 2;
   if (stamped) CU(h, cudaMemsetAsync(h->stamps, 0xFF, sizeof(KStamp) * FDVLM_MAX_STAMPS, h->st));
   return enqueue_rows(h, n, mode, logits_rows, want_logits, nullptr, stamped, ends, false);

@@ -229,6 +229,54 @@ def test_in_chain_timing_records_are_consistent():
     handle.close()
 
 
+@pytest.mark.parametrize("shape,n", [(I.TINY, 20), (I.TINY, 150), (SMALL_BF16, 20), (SMALL_BF16, 150), (SMALL_FP8, 20)],
+                         ids=["f32-20", "f32-150", "bf16-20", "bf16-150", "fp8-20"])
+def test_prompt_and_commit_in_graphs_of_the_caller(shape, n):
+    """The asynchronous calls on a stream that the caller is capturing: the graphs run them at the cache lengths of the capture,
+    whatever the handle has done since, and its own later calls are what they were."""
+    b = B()
+    stream = torch.cuda.Stream()
+    handle = b.Handle(shape, b.weights_to_device(I.make_weights(shape, 13)), max_seq=256, stream=stream)
+    ids = [I.random_tokens(shape, n, s).cuda() for s in (1, 2)]
+    draft = I.random_tokens(shape, 8, 9).cuda()
+    vec = lambda: torch.zeros(shape.vocab, dtype=torch.float32, device="cuda")
+
+    def eager(toks):
+        last, nxt = vec(), vec()
+        handle.reset()
+        handle.prefill(None, toks, last)
+        handle.block_begin(8, draft)
+        handle.commit_block(nxt)
+        handle.synchronize()
+        return last, nxt
+
+    same = lambda x, y: all(torch.equal(p, q) for p, q in zip(x, y))
+    with torch.cuda.stream(stream):
+        want = [eager(t) for t in ids]
+        assert not same(*want)
+        toks, last, nxt = ids[0].clone(), vec(), vec()
+        prompt, commit = torch.cuda.CUDAGraph(), torch.cuda.CUDAGraph()
+        handle.reset()
+        handle.prefill(None, ids[0])              # (the device's length word already holds what the captured call needs)
+        handle.reset()
+        with torch.cuda.graph(prompt, stream=stream):
+            handle.prefill(None, toks, last)
+        handle.block_begin(8, draft)
+        with torch.cuda.graph(commit, stream=stream):
+            handle.commit_block(nxt)
+        assert handle.cache_len() == n + 8
+        assert same(eager(ids[1]), want[1])       # (nothing has run what was captured)
+        for i in (1, 0, 1):
+            toks.copy_(ids[i])
+            prompt.replay()
+            commit.replay()
+            handle.synchronize()
+            assert same((last, nxt), want[i])
+        handle.truncate(n)
+        assert same(eager(ids[0]), want[0])
+    handle.close()
+
+
 def test_two_handles_on_two_streams_in_one_process():
     shape = SMALL_BF16
     s1, s2 = torch.cuda.Stream(), torch.cuda.Stream()
