@@ -142,14 +142,14 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
     constexpr bool F16 = !__is_same(E, bf16);
     const uint32_t id_s = F16 ? umma_idesc_f16(AT_STEP) : umma_idesc_bf16(AT_STEP);
     const uint32_t id_o = (F16 ? umma_idesc_f16(D) : umma_idesc_bf16(D)) | (1u << 16);      // (V: MN-major)
-    bool ok = mbar_wait_warp(q_full, 0, abort_flag);
+    bool ok = mbar_wait(q_full, 0, abort_flag);
     auto score = [&](int w, int t) {
-      if (!ok || t >= (w ? steps1 : steps0)) return;
+      if (t >= (w ? steps1 : steps0)) return;
       const int s = t % S::STAGES;
-      if (!mbar_wait_warp(k_full(s), (uint32_t)(t / S::STAGES) & 1u, abort_flag)) { ok = false; return; }
+      ok = ok && mbar_wait(k_full(s), (uint32_t)(t / S::STAGES) & 1u, abort_flag);
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint32_t ka = base + S::KV_OFF + s * 2 * S::TILE_BYTES + w * (AT_STEP * 128);
-      if (elect_one()) {
+      if (elect_one() && ok) {
 #pragma unroll
         for (int kk = 0; kk < D / 16; ++kk)
           umma_bf16(tmem + w * AT_STEP, umma_desc_sw128(base + (kk >> 2) * 16384) + 2u * (kk & 3), umma_desc_sw128(ka + (kk >> 2) * 16384) + 2u * (kk & 3),
@@ -159,12 +159,12 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
     };
     auto value = [&](int w, int t) {
       const int steps = w ? steps1 : steps0;
-      if (!ok || t >= steps) return;
+      if (t >= steps) return;
       const int s = t % S::STAGES;
-      if (!mbar_wait_warp(p_full(w), (uint32_t)t & 1u, abort_flag) || !mbar_wait_warp(v_full(s), (uint32_t)(t / S::STAGES) & 1u, abort_flag)) { ok = false; return; }
+      ok = ok && mbar_wait(p_full(w), (uint32_t)t & 1u, abort_flag) && mbar_wait(v_full(s), (uint32_t)(t / S::STAGES) & 1u, abort_flag);
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint64_t vd = umma_desc_sw128_mn(base + S::KV_OFF + (s * 2 + 1) * S::TILE_BYTES + w * (AT_STEP * 128), 16384);
-      if (elect_one()) {
+      if (elect_one() && ok) {
 #pragma unroll
         for (int kk = 0; kk < AT_STEP / 16; ++kk)
           umma_f16_ta(tmem + 256 + w * 128, tmem + w * AT_STEP + kk * 8, vd + (uint64_t)(kk * 128), id_o, (t > 0 || kk > 0) ? 1u : 0u);
@@ -173,15 +173,15 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
     };
     score(0, 0);
     score(1, 0);
-    for (int t = 0; t < n_tiles && ok; ++t) {
+    for (int t = 0; t < n_tiles; ++t) {
       value(0, t);
       score(0, t + 1);
       value(1, t);
-      if (ok && elect_one()) umma_commit(kv_empty(t % S::STAGES));
+      if (elect_one() && ok) umma_commit(kv_empty(t % S::STAGES));
       __syncwarp();
       score(1, t + 1);
     }
-    if (!ok && lane == 0 && p.status) atomicCAS(p.status, 0, ST_ATTENTION);
+    if (!ok && p.status) atomicCAS(p.status, 0, ST_ATTENTION);
   } else if (warp >= 4) {
     // Where this thread's pieces of Q come from and its rows of the result go is worked out before the wait: rows = heads x n,
     // row r -> head r / n, token r % n.
@@ -224,8 +224,8 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");      // generic writes -> the MMA's async-proxy reads
     __syncwarp();
     if (lane == 0) mbar_arrive(q_full);
-    for (int t = 0; t < steps && ok; ++t) {
-      if (!mbar_wait_warp(s_full(w), (uint32_t)t & 1u, abort_flag)) { ok = false; break; }
+    for (int t = 0; t < steps; ++t) {
+      ok = ok && mbar_wait(s_full(w), (uint32_t)t & 1u, abort_flag);
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       float s[AT_STEP];
       tmem_ld32(ts, s);
@@ -256,7 +256,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
       if (j0 + AT_STEP > key_end) {
         // V rows past the last key hold whatever the cache holds there, and 0 x NaN would poison the product
         const int sg = t % S::STAGES, first = max(0, key_end - j0);
-        if (!mbar_wait_warp(v_full(sg), (uint32_t)(t / S::STAGES) & 1u, abort_flag)) ok = false;
+        ok = ok && mbar_wait(v_full(sg), (uint32_t)(t / S::STAGES) & 1u, abort_flag);
         for (int v = wq * 32 + lane; ok && v < (AT_STEP - first) * CH; v += 128) {
           const int r = w * AT_STEP + first + v / CH, c = v % CH;
           const uint32_t a = base + S::KV_OFF + (sg * 2 + 1) * S::TILE_BYTES + (c >> 3) * 16384 + r * 128 + (((c & 7) ^ (r & 7)) << 4);
@@ -267,10 +267,10 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
       asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
-      if (lane == 0) mbar_arrive(p_full(w));
+      if (lane == 0 && ok) mbar_arrive(p_full(w));
     }
     for (int x = 0; x < 2; ++x)
-      if (ok && (x ? steps1 : steps0) > 0 && !mbar_wait_warp(o_full(x), 0, abort_flag)) ok = false;
+      if ((x ? steps1 : steps0) > 0) ok = ok && mbar_wait(o_full(x), 0, abort_flag);
     // every load has been used up and every product is complete: the ring is free.  Each warpgroup stores half of the
     // columns of the sum of both accumulators.
     ok = named_barrier_and<256>(ok);

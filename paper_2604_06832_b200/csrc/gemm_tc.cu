@@ -242,22 +242,22 @@ __global__ void __launch_bounds__(TC_THREADS) gemm_tc_kernel(const __grid_consta
       uint32_t phase = 0;
       int local = 0;
       bool ok = true;
-      for (int it = blockIdx.x; it < n_items && ok; it += gridDim.x, ++local) {
+      for (int it = blockIdx.x; it < n_items; it += gridDim.x, ++local) {
         const int split = it / total_tiles;
         const int acc = local % NACC;
         const uint32_t acc_phase = (uint32_t)(local / NACC) & 1u;
-        if (!mbar_wait_warp(tempty_bar(acc), acc_phase ^ 1u, abort_flag)) { ok = false; break; }
+        ok = ok && mbar_wait(tempty_bar(acc), acc_phase ^ 1u, abort_flag);
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const uint32_t d_tmem = tmem_base + (uint32_t)(acc * ACC_COLS);
         const int kb0 = split * p.kb_per_split;
         const int kb1 = min(p.kblocks, kb0 + p.kb_per_split);
         for (int kb = kb0; kb < kb1; ++kb) {
-          if (!mbar_wait_warp(full_bar(stage), phase, abort_flag)) { ok = false; break; }
+          ok = ok && mbar_wait(full_bar(stage), phase, abort_flag);
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           const uint32_t a_addr = base + stage * L::STAGE_BYTES;
           const uint64_t adesc = umma_desc_sw128(a_addr);
           const uint64_t bdesc = umma_desc_sw128(a_addr + L::W_BYTES);
-          if (elect_one()) {
+          if (elect_one() && ok) {
           if (W8) {
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk)      // 32 bytes of k per instruction
@@ -271,9 +271,9 @@ __global__ void __launch_bounds__(TC_THREADS) gemm_tc_kernel(const __grid_consta
           }
           if (++stage == TC_STAGES) { stage = 0; phase ^= 1u; }
         }
-        if (ok && elect_one()) umma_commit(tfull_bar(acc));
+        if (elect_one() && ok) umma_commit(tfull_bar(acc));
       }
-      if (!ok && lane == 0) atomicCAS(p.status, 0, TC_ERR_MMA);
+      if (!ok) atomicCAS(p.status, 0, TC_ERR_MMA);
     }
   } else {
     // ------------------------------------------------ epilogue warps ----------------------------------------------
@@ -307,11 +307,11 @@ __global__ void __launch_bounds__(TC_THREADS) gemm_tc_kernel(const __grid_consta
       rs0 = row_rs[lane];
       rs1 = row_rs[lane + 32];
     }
-    for (int it = blockIdx.x; it < n_items && ok; it += gridDim.x, ++local) {
+    for (int it = blockIdx.x; it < n_items; it += gridDim.x, ++local) {
       const int tile = it % total_tiles, split = it / total_tiles;
       const int acc = local % NACC;
       const uint32_t acc_phase = (uint32_t)(local / NACC) & 1u;
-      if (!mbar_wait_warp(tfull_bar(acc), acc_phase, abort_flag)) { ok = false; break; }
+      ok = ok && mbar_wait(tfull_bar(acc), acc_phase, abort_flag);
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       float v[M_PAD];
       const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * ACC_COLS);
@@ -340,7 +340,7 @@ __global__ void __launch_bounds__(TC_THREADS) gemm_tc_kernel(const __grid_consta
       asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
-      if (lane == 0) mbar_arrive(tempty_bar(acc));
+      if (lane == 0 && ok) mbar_arrive(tempty_bar(acc));
 
       if (p.mode == TC_MODE_SWIGLU) {
         // Warps 0, 1 of the epilogue hold the gate values of features 32 pr + lane, warps 2, 3 the up values of the
@@ -367,8 +367,8 @@ __global__ void __launch_bounds__(TC_THREADS) gemm_tc_kernel(const __grid_consta
             ex[(side * HR + b) * 32 + lane] = side ? v[lo] * sc * rs_lo : v[hi] * sc * rs_hi;
           }
           __syncwarp();
-          if (lane == 0) mbar_arrive(exw_bar(pr));
-          if (!mbar_wait_warp(exw_bar(pr), par, abort_flag)) { ok = false; break; }
+          if (lane == 0 && ok) mbar_arrive(exw_bar(pr));
+          ok = ok && mbar_wait(exw_bar(pr), par, abort_flag);
           float am[HR];
 #pragma unroll
           for (int b = 0; b < HR; ++b) {
@@ -391,11 +391,10 @@ __global__ void __launch_bounds__(TC_THREADS) gemm_tc_kernel(const __grid_consta
             if (lane < HR && row < p.m && mx > 0.f) atomicMax(reinterpret_cast<int*>(p.amax_out) + row, __float_as_int(mx));
           }
           __syncwarp();
-          if (lane == 0) mbar_arrive(exr_bar(pr));
+          if (lane == 0 && ok) mbar_arrive(exr_bar(pr));
           // the buffer may be rewritten once the partner has read it too
-          if (!mbar_wait_warp(exr_bar(pr), par, abort_flag)) { ok = false; break; }
+          ok = ok && mbar_wait(exr_bar(pr), par, abort_flag);
         }
-        if (!ok) break;
       } else if (p.mode == TC_MODE_LOGITS) {
         const int n = tile * TC_BM + q * 32 + lane;          // vocabulary id held by this lane
         const bool in_range = n < p.n_out[0];
@@ -459,7 +458,7 @@ __global__ void __launch_bounds__(TC_THREADS) gemm_tc_kernel(const __grid_consta
         }
       }
     }
-    if (!ok && lane == 0) atomicCAS(p.status, 0, TC_ERR_EPILOGUE);
+    if (!ok) atomicCAS(p.status, 0, TC_ERR_EPILOGUE);
   }
 
   // ---- teardown: every thread arrives here, whatever happened ----

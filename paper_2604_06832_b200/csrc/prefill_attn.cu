@@ -130,10 +130,10 @@ __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const __gri
       constexpr bool F16 = sizeof(E) == 2 && !__is_same(E, bf16);
       const uint32_t id_s = F16 ? umma_idesc_f16(PA_STEP) : umma_idesc_bf16(PA_STEP);
       const uint32_t id_o = (F16 ? umma_idesc_f16(D) : umma_idesc_bf16(D)) | (1u << 16);      // (V: MN-major)
-      bool ok = mbar_wait_warp(q_full, 0, abort_flag);
+      bool ok = mbar_wait(q_full, 0, abort_flag);
       auto score = [&](int q, int t) {
         const uint32_t qa = base + q * S::TILE_BYTES, ka = base + S::K_OFF + ((t >> 1) & 1) * S::TILE_BYTES + (t & 1) * (PA_STEP * 128);
-        if (elect_one()) {
+        if (elect_one() && ok) {
 #pragma unroll
         for (int kk = 0; kk < D / 16; ++kk)
           umma_bf16(tmem + q * 128 + (t & 1) * PA_STEP, umma_desc_sw128(qa + (kk >> 2) * 16384) + 2u * (kk & 3),
@@ -142,10 +142,10 @@ __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const __gri
         }
       };
       auto value = [&](int q, int t) {
-        if (!mbar_wait_warp(p_full(q, t), (uint32_t)(t >> 1) & 1u, abort_flag)) { ok = false; return; }
+        ok = ok && mbar_wait(p_full(q, t), (uint32_t)(t >> 1) & 1u, abort_flag);
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const uint64_t vd = umma_desc_sw128_mn(base + S::V_OFF + ((t >> 1) & 1) * S::TILE_BYTES + (t & 1) * (PA_STEP * 128), 16384);
-        if (elect_one()) {
+        if (elect_one() && ok) {
 #pragma unroll
         for (int kk = 0; kk < PA_STEP / 16; ++kk)
           umma_f16_ta(tmem + 256 + q * 128, tmem + q * 128 + (t & 1) * PA_STEP + kk * 8, vd + (uint64_t)(kk * 128), id_o, (t > 0 || kk > 0) ? 1u : 0u);
@@ -155,24 +155,24 @@ __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const __gri
       };
       // the scores of step t for both row tiles; the K tile is free after its second half
       auto scores = [&](int q, int t) {
-        if (t >= ns || !ok) return;
+        if (t >= ns) return;
         if (q == 0 && (t & 1) == 0) {
-          if (!mbar_wait_warp(k_full((t >> 1) & 1), (uint32_t)(t >> 2) & 1u, abort_flag)) { ok = false; return; }
+          ok = ok && mbar_wait(k_full((t >> 1) & 1), (uint32_t)(t >> 2) & 1u, abort_flag);
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         }
         if (t < (q ? n1 : n0)) score(q, t);
-        if (q == 1 && ((t & 1) || t + 1 == ns)) { if (elect_one()) umma_commit(k_empty((t >> 1) & 1)); }
+        if (q == 1 && ((t & 1) || t + 1 == ns)) { if (elect_one() && ok) umma_commit(k_empty((t >> 1) & 1)); }
       };
       for (int t = 0; t < 2; ++t) { scores(0, t); scores(1, t); }
-      for (int t = 0; t < ns && ok; ++t) {
-        if ((t & 1) == 0 && !mbar_wait_warp(v_full((t >> 1) & 1), (uint32_t)(t >> 2) & 1u, abort_flag)) { ok = false; break; }
+      for (int t = 0; t < ns; ++t) {
+        if ((t & 1) == 0) ok = ok && mbar_wait(v_full((t >> 1) & 1), (uint32_t)(t >> 2) & 1u, abort_flag);
         if (t < n0) value(0, t);
         scores(0, t + 2);
-        if (ok && t < n1) value(1, t);
-        if (ok && ((t & 1) || t + 1 == ns)) { if (elect_one()) umma_commit(v_empty((t >> 1) & 1)); }
+        if (t < n1) value(1, t);
+        if ((t & 1) || t + 1 == ns) { if (elect_one() && ok) umma_commit(v_empty((t >> 1) & 1)); }
         scores(1, t + 2);
       }
-      if (!ok && lane == 0 && p.status) atomicCAS(p.status, 0, ST_ATTENTION);
+      if (!ok && p.status) atomicCAS(p.status, 0, ST_ATTENTION);
     }
   } else if (warp >= 4) {
     const int q = (warp - 4) >> 2, wq = warp & 3;
@@ -185,8 +185,8 @@ __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const __gri
     const float sl2 = rsqrtf((float)D) * LOG2E;               // scores in the log2 domain
     float m_ref = -INFINITY, l = 0.f;
     bool ok = true;
-    for (int t = 0; t < nq && ok; ++t) {
-      if (!mbar_wait_warp(s_full(q, t), (uint32_t)(t >> 1) & 1u, abort_flag)) { ok = false; break; }
+    for (int t = 0; t < nq; ++t) {
+      ok = ok && mbar_wait(s_full(q, t), (uint32_t)(t >> 1) & 1u, abort_flag);
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint32_t tb = ts + (t & 1) * PA_STEP;
       float s[PA_STEP];
@@ -202,7 +202,7 @@ __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const __gri
       const float m = row_max64(s) * sl2;
       const bool grow = m > m_ref + 8.f;                      // (always in the first step: every row reads key 0)
       if (t > 0 && __any_sync(0xffffffffu, grow)) {
-        if (!mbar_wait_warp(o_done(q), (uint32_t)(t - 1) & 1u, abort_flag)) { ok = false; break; }
+        ok = ok && mbar_wait(o_done(q), (uint32_t)(t - 1) & 1u, abort_flag);
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const float f = grow ? ex2(m_ref - m) : 1.f;
         scale_acc<D>(to, f);
@@ -213,7 +213,7 @@ __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const __gri
       if (j0 + PA_STEP > key_end) {
         // V rows past the last key hold whatever the cache holds there, and 0 x NaN would poison the product: cleared by
         // both row tiles (the same zeros)
-        if (!mbar_wait_warp(v_full((t >> 1) & 1), (uint32_t)(t >> 2) & 1u, abort_flag)) ok = false;
+        ok = ok && mbar_wait(v_full((t >> 1) & 1), (uint32_t)(t >> 2) & 1u, abort_flag);
         const int first = key_end - j0;
         for (int v = wq * 32 + lane; ok && v < (PA_STEP - first) * (D / 8); v += 128) {
           const int r = (t & 1) * PA_STEP + first + v / (D / 8), c = v % (D / 8);
@@ -226,10 +226,10 @@ __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const __gri
       asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
-      if (lane == 0) mbar_arrive(p_full(q, t));
+      if (lane == 0 && ok) mbar_arrive(p_full(q, t));
     }
-    if (nq > 0 && ok && !mbar_wait_warp(o_full(q), 0, abort_flag)) ok = false;
-    if (nq > 0 && ok) {
+    if (nq > 0) {
+      ok = ok && mbar_wait(o_full(q), 0, abort_flag);
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const float inv = 1.f / l;
       const size_t idx = ((size_t)i * p.hq + head) * D;
@@ -239,14 +239,14 @@ __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const __gri
         __syncwarp();
         tmem_ld32(to + c, o);
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-        if (i < p.n) {
+        if (ok && i < p.n) {
 #pragma unroll
           for (int k = 0; k < 32; k += 4)
             store_act4(p.out, p.lo_off, idx + c + k, make_float4(o[k] * inv, o[k + 1] * inv, o[k + 2] * inv, o[k + 3] * inv), p.fmt);
         }
       }
     }
-    if (!ok && lane == 0 && p.status) atomicCAS(p.status, 0, ST_ATTENTION);
+    if (!ok && p.status) atomicCAS(p.status, 0, ST_ATTENTION);
   }
   __syncwarp();
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
