@@ -118,6 +118,13 @@ int stage_prefill_rows(fdvlm_t* h, int row0, int n, const int32_t* tokens, const
   return FDVLM_OK;
 }
 
+// In-chain timing: the record of the next launch, null while it is off.
+static KStamp* next_stamp(fdvlm_t* h, bool stamped, int kind) {
+  if (!stamped || h->stamp_used >= FDVLM_MAX_STAMPS) return nullptr;
+  h->stamp_kind.push_back(kind);
+  return h->stamps + h->stamp_used++;
+}
+
 // ---- prompt path ---------------------------------------------------------------------------------------------------------
 // per layer: [QKV GEMM + norm factor, bias, rotary, K/V rows] [causal attention] [O GEMM + residual, gain, ssq]
 //            [gate/up GEMM + SwiGLU] [down GEMM + residual, gain, ssq]
@@ -127,15 +134,20 @@ int forward_prefill(fdvlm_t* h, int n, int want_last_logits) {
   const int H = c.hidden, I = c.intermediate, d = c.head_dim, nt = h->nt;
   const int NQ = c.n_q_heads * d, NKV = c.n_kv_heads * d;
   const size_t R = h->pf_rows;
-  const bool fp8 = h->dt == DT_FP8;
+  const bool fp8 = h->dt == DT_FP8, stamped = h->prof_on == 2;
   cudaError_t e = cudaSuccess;
-  auto gemm = [&](int mode, const void* x, size_t ld, int k) {
+  if (stamped) {
+    h->stamp_kind.clear();
+    h->stamp_used = 0;
+    CU(h, cudaMemsetAsync(h->stamps, 0xFF, sizeof(KStamp) * FDVLM_MAX_STAMPS, h->st));
+  }
+  auto gemm = [&](int mode, int kind, const void* x, size_t ld, int k) {
     PfGemm g;
     memset(&g, 0, sizeof(g));
     g.mode = mode; g.m = n; g.k = k; g.x_rows = (int)R; g.fp8 = fp8; g.n_mats = 1;
     g.x = x; g.x_lo = fp8 ? nullptr : (const char*)x + R * ld * 2;
     g.nt = nt; g.inv_h = 1.f / (float)H; g.eps = c.rms_eps; g.status = h->info + 3;
-    g.part = h->pf_part; g.arrived = h->pf_arrived;
+    g.part = h->pf_part; g.arrived = h->pf_arrived; g.stamp = next_stamp(h, stamped, kind);
     return g;
   };
   auto run = [&](const PfGemm& g) {
@@ -146,14 +158,15 @@ int forward_prefill(fdvlm_t* h, int n, int want_last_logits) {
     return e == cudaSuccess;
   };
   // residual add of x w^T, the next norm's gain and sums of squares
-  auto resid = [&](const void* x, size_t ld, int k, const void* w, const float* scale, const float* gain, int fmt) {
-    PfGemm g = gemm(PF_RESID, x, ld, k);
+  auto resid = [&](int kind, const void* x, size_t ld, int k, const void* w, const float* scale, const float* gain, int fmt) {
+    PfGemm g = gemm(PF_RESID, kind, x, ld, k);
     g.w[0] = w; g.n[0] = H;
     g.splits = prefill_splits(n, H, k);
     if (g.splits > 1 && (size_t)g.splits * n * H * sizeof(float) <= h->pf_part_bytes) {
       g.mode = PF_PARTIAL;
       if (!run(g)) return false;
-      launch_fin_resid_rows(h->pf_part, g.splits, n, H, h->pf_h, gain, h->pf_a, R * H, fmt, h->pf_ssq, nt, scale, h->st);
+      launch_fin_resid_rows(h->pf_part, g.splits, n, H, h->pf_h, gain, h->pf_a, R * H, fmt, h->pf_ssq, nt, scale, h->st,
+                            next_stamp(h, stamped, FDVLM_K_FIN_RESID));
       h->launches++;
       return true;
     }
@@ -162,11 +175,11 @@ int forward_prefill(fdvlm_t* h, int n, int want_last_logits) {
   };
   // (a forward whose waits gave up may have left some)
   CU(h, cudaMemsetAsync(h->pf_arrived, 0, (size_t)sm_count() * 4 * sizeof(unsigned), h->st));
-  launch_rope_table(h->pf_cs, n, h->cache_len, d, c.rope_theta, h->st);
+  launch_rope_table(h->pf_cs, n, h->cache_len, d, c.rope_theta, h->st, nullptr, next_stamp(h, stamped, FDVLM_K_ROPE_TABLE));
   h->launches++;
   for (int l = 0; l < c.n_layers; ++l) {
     const fdvlm_layer_weights& lw = h->layers[l];
-    PfGemm g = gemm(PF_QKV, h->pf_a, H, H);
+    PfGemm g = gemm(PF_QKV, FDVLM_K_GEMM_QKV, h->pf_a, H, H);
     g.n_mats = 3;
     g.w[0] = lw.wq; g.w[1] = lw.wk; g.w[2] = lw.wv; g.n[0] = NQ; g.n[1] = g.n[2] = NKV;
     g.scale[0] = lw.s_q; g.scale[1] = lw.s_k; g.scale[2] = lw.s_v; g.bias[0] = lw.bq; g.bias[1] = lw.bk; g.bias[2] = lw.bv;
@@ -178,26 +191,28 @@ int forward_prefill(fdvlm_t* h, int n, int want_last_logits) {
     at.q = h->pf_q; at.kc = kv_ptr(h, l, 0); at.vc = kv_ptr(h, l, 1); at.out = h->pf_ao; at.n = n; at.cache_len = h->cache_len;
     at.max_seq = c.max_seq; at.hq = c.n_q_heads; at.hkv = c.n_kv_heads; at.d = d; at.causal = 1; at.kv_type = h->kv_type;
     at.out_fmt = h->pf_fmt; at.out_lo_off = R * NQ; at.status = h->info + 3;
+    at.stamp = next_stamp(h, stamped, FDVLM_K_ATTENTION);
     prof_begin(h, 1);
     e = launch_prefill_attention(at, h->st);
     prof_end(h);
     h->launches++;
     if (e != cudaSuccess) return fail(h, FDVLM_ERR_CUDA, "attention launch: %s", cudaGetErrorString(e));
-    if (!resid(h->pf_ao, NQ, NQ, lw.wo, lw.s_o, lw.g_mlp, h->pf_fmt))
+    if (!resid(FDVLM_K_GEMM_O, h->pf_ao, NQ, NQ, lw.wo, lw.s_o, lw.g_mlp, h->pf_fmt))
       return fail(h, FDVLM_ERR_CUDA, "o projection launch: %s", cudaGetErrorString(e));
-    g = gemm(PF_SWIGLU, h->pf_a, H, H);
+    g = gemm(PF_SWIGLU, FDVLM_K_GEMM_GATE_UP, h->pf_a, H, H);
     g.n_mats = 2;
     g.w[0] = lw.w_gate; g.w[1] = lw.w_up; g.n[0] = g.n[1] = I; g.scale[0] = lw.s_gate; g.scale[1] = lw.s_up;
     g.ssq_in = h->pf_ssq; g.out = h->pf_act; g.out_lo_off = R * I; g.out_fmt = h->pf_fmt;
     if (!run(g)) return fail(h, FDVLM_ERR_CUDA, "gate/up projection launch: %s", cudaGetErrorString(e));
     const bool last = l + 1 == c.n_layers;
-    if (!resid(h->pf_act, I, I, lw.w_down, lw.s_down, last ? h->w.g_final : h->layers[l + 1].g_attn, last ? h->head_fmt : h->pf_fmt))
+    if (!resid(FDVLM_K_GEMM_DOWN, h->pf_act, I, I, lw.w_down, lw.s_down, last ? h->w.g_final : h->layers[l + 1].g_attn, last ? h->head_fmt : h->pf_fmt))
       return fail(h, FDVLM_ERR_CUDA, "down projection launch: %s", cudaGetErrorString(e));
   }
   if (want_last_logits) {
     TcOut o;
     memset(&o, 0, sizeof(o));
     o.mode = TC_MODE_LOGITS; o.status = h->info + 3; o.y = h->logits; o.ld = c.vocab; o.write_logits = 1;
+    o.stamp = next_stamp(h, stamped, FDVLM_K_GEMM_LM_HEAD);
     o.ssq_in = h->pf_ssq + (size_t)(n - 1) * nt; o.nt_in = nt; o.hidden = H; o.eps = c.rms_eps; o.stats = h->stats; o.mask_id = c.mask_id;
     TcGroup lm;
     memset(&lm, 0, sizeof(lm));
@@ -296,11 +311,7 @@ static int forward_rows_tc(fdvlm_t* h, int n, int mode, int logits_rows, int wan
   float* part = (float*)h->ws;
   cudaError_t e = cudaSuccess;
   if (stamped) { h->stamp_kind.clear(); h->stamp_used = 0; }
-  auto stamp = [&](int kind) -> KStamp* {
-    if (!stamped || h->stamp_used >= FDVLM_MAX_STAMPS) return nullptr;
-    h->stamp_kind.push_back(kind);
-    return h->stamps + h->stamp_used++;
-  };
+  auto stamp = [&](int kind) { return next_stamp(h, stamped, kind); };
   const bool a8 = h->act8 != 0;                      // W8A8: the four layer projections quantise their input rows
   // a GEMM input buffer: hi (or only) plane, and its lo plane when the format has one
   auto group = [&](const void* x, size_t lo_off, size_t row0_elems, int m, int k, int nm, const void* w0, int n0, const void* w1, int n1,

@@ -121,7 +121,7 @@ inline size_t kv_plane(const fdvlm_t* h) {
 inline char* kv_ptr(const fdvlm_t* h, int layer, int which) { return h->kv + ((size_t)layer * 2 + which) * kv_plane(h); }
 
 inline void prof_begin(fdvlm_t* h, int kind) {
-  if (!h->prof_on) return;
+  if (h->prof_on != 1) return;
   if (h->prof_used * 2 + 2 > h->prof_ev.size()) {
     cudaEvent_t a, b;
     if (cudaEventCreate(&a) != cudaSuccess || cudaEventCreate(&b) != cudaSuccess) { h->prof_on = 0; return; }
@@ -131,7 +131,7 @@ inline void prof_begin(fdvlm_t* h, int kind) {
   cudaEventRecord(h->prof_ev[h->prof_used * 2], h->st);
 }
 inline void prof_end(fdvlm_t* h) {
-  if (!h->prof_on) return;
+  if (h->prof_on != 1) return;
   cudaEventRecord(h->prof_ev[h->prof_used * 2 + 1], h->st);
   h->prof_used++;
 }

@@ -536,11 +536,13 @@ __global__ void __launch_bounds__(128) fin_resid_kernel(const float* __restrict_
 __global__ void __launch_bounds__(256) fin_resid_rows_kernel(const float* __restrict__ part, int S, int m, int hidden,
                                                              float* __restrict__ h, const float* __restrict__ g, void* __restrict__ xg,
                                                              size_t lo_off, int fmt, float* __restrict__ ssq, int nt,
-                                                             const float* __restrict__ scale) {
+                                                             const float* __restrict__ scale, KStamp* stamp) {
+  if (threadIdx.x == 0) stamp_start(stamp);
   pdl_trigger();
   const int idx_w = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   const int r = idx_w / nt, t = idx_w - r * nt, c = t * 128 + lane * 4;
   pdl_wait();
+  if (threadIdx.x == 0) stamp_released(stamp);
   if (r >= m) return;
   float ss = 0.f;
   if (c < hidden) {
@@ -567,10 +569,11 @@ __global__ void __launch_bounds__(256) fin_resid_rows_kernel(const float* __rest
   }
   ss = warp_sum(ss);
   if (lane == 0) ssq[(size_t)r * nt + t] = ss;
+  if (threadIdx.x == 0) stamp_end(stamp, true);
 }
 void launch_fin_resid_rows(const float* part, int S, int m, int hidden, float* h, const float* g, void* xg, size_t lo_off, int fmt,
-                           float* ssq, int nt, const float* scale, cudaStream_t st) {
-  launch_pdl(fin_resid_rows_kernel, dim3((m * nt + 7) / 8), dim3(256), 0, st, part, S, m, hidden, h, g, xg, lo_off, fmt, ssq, nt, scale);
+                           float* ssq, int nt, const float* scale, cudaStream_t st, KStamp* stamp) {
+  launch_pdl(fin_resid_rows_kernel, dim3((m * nt + 7) / 8), dim3(256), 0, st, part, S, m, hidden, h, g, xg, lo_off, fmt, ssq, nt, scale, stamp);
 }
 void launch_fin_resid(const float* part, int S, int m, int hidden, float* h, const float* g, void* xg, size_t lo_off, int fmt,
                       float* ssq, int nt, const float* scale, cudaStream_t st, KStamp* stamp, const float* x_scale, float* amax_out) {

@@ -152,6 +152,7 @@ struct PfGemm {
   float* part; int splits;
   unsigned* arrived;      // nullable: sm_count() * 4 zeroed words; with `part` (256 x 256 sums per two SMs) tiles may come in pieces
   int* status;
+  KStamp* stamp;          // in-chain timing of the launch, nullable
 };
 int prefill_splits(int m, int n, int k);
 cudaError_t prefill_gemm_launch(const PfGemm& g, cudaStream_t st);
@@ -170,7 +171,7 @@ void launch_fin_resid(const float* part, int S, int m, int hidden, float* h, con
                       float* ssq, int nt, const float* scale, cudaStream_t st, KStamp* stamp = nullptr,
                       const float* x_scale = nullptr, float* amax_out = nullptr);
 void launch_fin_resid_rows(const float* part, int S, int m, int hidden, float* h, const float* g, void* xg, size_t lo_off, int fmt,
-                           float* ssq, int nt, const float* scale, cudaStream_t st);
+                           float* ssq, int nt, const float* scale, cudaStream_t st, KStamp* stamp = nullptr);
 void launch_stats_merge(const void* stats, int n_part, int m, float* conf, int32_t* pred, cudaStream_t st, KStamp* stamp = nullptr);
 
 // ---- attention -----------------------------------------------------------------------------------
@@ -189,7 +190,7 @@ struct AttnArgs {
   const int* len_ptr;   // nullable: device word holding the cache length (overrides cache_len)
   int* status;          // nullable: device status words (see TcOut::status)
   float* amax_out;      // nullable (tensor-core kernel): [n][hq] maxima of |out| as stored, per row and head
-  KStamp* stamp;        // nullable: two consecutive entries (attention, chunk merge)
+  KStamp* stamp;        // nullable: decode: two consecutive entries (attention, chunk merge); prompt path: one
 };
 // Prompt path: causal attention of any number of rows, one CTA per (256 rows, query head), no key split (prefill_attn.cu).
 cudaError_t launch_prefill_attention(const AttnArgs& a, cudaStream_t st);

@@ -35,6 +35,7 @@ struct PaParams {
   void* out; size_t lo_off; int fmt;
   int n, L, max_seq, hq, hkv, rows;      // rows per CTA: 256 (both row tiles) or 128 (the first only)
   int* status;
+  KStamp* stamp;
 };
 
 template <int D, typename E>
@@ -58,6 +59,7 @@ __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const __gri
   volatile int* abort_flag = (volatile int*)(sm + S::BAR_OFF + 172);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid == 0) {
+    stamp_start(p.stamp);
     mbar_init(q_full, 1);
     for (int i = 0; i < 2; ++i) {
       mbar_init(k_full(i), 1); mbar_init(k_empty(i), 1); mbar_init(v_full(i), 1); mbar_init(v_empty(i), 1);
@@ -78,6 +80,7 @@ __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const __gri
   const uint32_t tmem = *tmem_slot;            // columns: score buffers (S, then P) of row tile q at 128 q and 128 q + 64, O at 256 + 128 q
   pdl_trigger();            // (holding its tensor memory: see gemm_tc.cu)
   pdl_wait();
+  if (tid == 0) stamp_released(p.stamp);
 
   const int head = blockIdx.x, hk = head / (p.hq / p.hkv);
   const int i0 = (int)(gridDim.y - 1 - blockIdx.y) * p.rows;
@@ -255,6 +258,7 @@ __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const __gri
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
   }
+  if (tid == 0) stamp_end(p.stamp);
 }
 
 template <int D, typename E>
@@ -277,7 +281,7 @@ cudaError_t launch_prefill_attention(const AttnArgs& a, cudaStream_t st) {
   // twice as many of one (1024 rows of the 3B shape 35 -> 25 us, 2048 rows 53 -> 43; 4096 rows 99 against 122).
   p.rows = a.hq * ceil_div(a.n, 256) <= sm_count() ? 128 : 256;
   p.out = a.out; p.lo_off = a.out_lo_off; p.fmt = a.out_fmt;
-  p.n = a.n; p.L = a.cache_len; p.max_seq = a.max_seq; p.hq = a.hq; p.hkv = a.hkv; p.status = a.status;
+  p.n = a.n; p.L = a.cache_len; p.max_seq = a.max_seq; p.hq = a.hq; p.hkv = a.hkv; p.status = a.status; p.stamp = a.stamp;
   if (a.kv_type == KV_F16) return a.d == 128 ? pa_launch_t<128, __half>(p, st) : pa_launch_t<64, __half>(p, st);
   return a.d == 128 ? pa_launch_t<128, bf16>(p, st) : pa_launch_t<64, bf16>(p, st);
 }

@@ -229,6 +229,37 @@ def test_in_chain_timing_records_are_consistent():
     handle.close()
 
 
+@pytest.mark.parametrize("shape,n", [(SMALL_BF16, 150), (SMALL_FP8, 150), (SMALL_BF16.with_(n_layers=1), 4200)], ids=["bf16", "fp8", "two-forwards"])
+def test_in_chain_timing_records_of_a_long_prompt(shape, n):
+    """The records are those of the last forward also where that is a prompt's, and the prompt is what it is without them."""
+    b = B()
+    stream = torch.cuda.Stream()
+    handle = b.Handle(shape, b.weights_to_device(I.make_weights(shape, 5)), max_seq=n + 32, stream=stream)
+    toks = I.random_tokens(shape, n, 2).cuda()
+    last = [torch.empty(shape.vocab, dtype=torch.float32, device="cuda") for _ in range(2)]
+    with torch.cuda.stream(stream):
+        handle.prefill(None, toks, last[0])
+        handle.block_begin(16)
+        handle.profile_enable(2)
+        handle.block_step(b.RULE_TOPK, 0.0, 16)
+        handle.commit_block()
+        handle.reset()
+        handle.prefill(None, toks, last[1])
+        recs = handle.profile_read_chain()
+        handle.profile_enable(0)
+        stream.synchronize()
+    assert torch.equal(*last)
+    kinds = [r["kind"] for r in recs if r["kind"] != "fin_resid"]      # (behind O and down only where their depth is split)
+    assert kinds == ["rope_table"] + ["gemm_qkv", "attention", "gemm_o", "gemm_gate_up", "gemm_down"] * shape.n_layers + ["gemm_lm_head"]
+    prev_end = None
+    for r in recs:
+        assert 0 <= r["start_us"] <= r["released_us"] <= r["end_us"], r
+        if prev_end is not None:
+            assert r["released_us"] >= prev_end - 0.5, (r, prev_end)     # half a microsecond for timer granularity
+        prev_end = r["end_us"]
+    handle.close()
+
+
 @pytest.mark.parametrize("shape,n", [(I.TINY, 20), (I.TINY, 150), (SMALL_BF16, 20), (SMALL_BF16, 150), (SMALL_FP8, 20)],
                          ids=["f32-20", "f32-150", "bf16-20", "bf16-150", "fp8-20"])
 def test_prompt_and_commit_in_graphs_of_the_caller(shape, n):
