@@ -412,7 +412,8 @@ __global__ void __launch_bounds__(128) attn_combine_kernel(const float* __restri
     }
     const float inv = 1.f / l;
     const size_t idx = ((size_t)i * hq + head) * D + lane * VPL;
-    if (VPL == 4) {
+    // (a caller's `out` may lie at any element: four of them in one store only where they are aligned)
+    if (VPL == 4 && (reinterpret_cast<uintptr_t>(out) & 7) == 0) {
       store_act4(out, lo_off, idx, make_float4(acc[0] * inv, acc[1] * inv, acc[VPL - 2] * inv, acc[VPL - 1] * inv), fmt);
     } else {
 #pragma unroll

@@ -18,10 +18,19 @@ __device__ __forceinline__ float dot4(const float4& a, const float4& b, float c)
   return fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, fmaf(a.x, b.x, c))));
 }
 
+// Four consecutive floats; `vec`: they are 16-byte aligned (callers' gains, queries and caches may lie at any float).
+__device__ __forceinline__ float4 ldg_f4(const float* p, bool vec) {
+  return vec ? __ldg(reinterpret_cast<const float4*>(p)) : make_float4(__ldg(p), __ldg(p + 1), __ldg(p + 2), __ldg(p + 3));
+}
+__device__ __forceinline__ float4 ldcg_f4(const float* p, bool vec) {
+  return vec ? __ldcg(reinterpret_cast<const float4*>(p)) : make_float4(__ldcg(p), __ldcg(p + 1), __ldcg(p + 2), __ldcg(p + 3));
+}
+static inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
+
 // One CTA: RM rows x 8 pairs of output features.  The pair is what the epilogue combines: (j, j + d/2) of a head for the
-// rotary embedding, (gate, up) for SwiGLU, else features f and f + 8.  A warp takes every eighth 16-wide slice of k; lane =
+// rotary embedding, (gate, up) for SwiGLU, else features f and f + 8.  GV: the gains are 16-byte aligned.  A warp takes every eighth 16-wide slice of k; lane =
 // (feature 0..7, quarter of the slice).
-template <int RM, int MODE>
+template <int RM, int MODE, bool GV>
 __global__ void __launch_bounds__(FL_WARPS * 32) linear_f32_kernel(const F32Linear p) {
   extern __shared__ float4 fl_smem[];
   float* xs = reinterpret_cast<float*>(fl_smem);                 // [RM][kc]
@@ -84,7 +93,7 @@ __global__ void __launch_bounds__(FL_WARPS * 32) linear_f32_kernel(const F32Line
         if (k >= cn) break;
         ssq[i] = dot4(v[j], v[j], ssq[i]);
         if (p.gain) {
-          const float4 g = __ldg(reinterpret_cast<const float4*>(p.gain + c0 + k));
+          const float4 g = ldg_f4(p.gain + c0 + k, GV);
           v[j] = make_float4(v[j].x * g.x, v[j].y * g.y, v[j].z * g.z, v[j].w * g.w);
         }
         *reinterpret_cast<float4*>(xs + rl * kc + k) = v[j];
@@ -183,13 +192,17 @@ __global__ void __launch_bounds__(FL_WARPS * 32) linear_f32_kernel(const F32Line
   }
 }
 
-template <int RM, int MODE>
-static cudaError_t fl_launch_t(const F32Linear& p, int tiles, cudaStream_t st) {
+template <int RM, int MODE, bool GV>
+static cudaError_t fl_launch_v(const F32Linear& p, int tiles, cudaStream_t st) {
   static bool attr_set[MAX_DEVICES] = {};
-  cudaError_t e = ensure_dynamic_smem(linear_f32_kernel<RM, MODE>, RM * FL_KC * 4, attr_set);
+  cudaError_t e = ensure_dynamic_smem(linear_f32_kernel<RM, MODE, GV>, RM * FL_KC * 4, attr_set);
   if (e != cudaSuccess) return e;
   const size_t smem = (size_t)RM * (p.k < FL_KC ? p.k : FL_KC) * 4;
-  return launch_pdl(linear_f32_kernel<RM, MODE>, dim3(tiles, ceil_div(p.m, RM)), dim3(FL_WARPS * 32), smem, st, p);
+  return launch_pdl(linear_f32_kernel<RM, MODE, GV>, dim3(tiles, ceil_div(p.m, RM)), dim3(FL_WARPS * 32), smem, st, p);
+}
+template <int RM, int MODE>
+static cudaError_t fl_launch_t(const F32Linear& p, int tiles, cudaStream_t st) {
+  return aligned16(p.gain) ? fl_launch_v<RM, MODE, true>(p, tiles, st) : fl_launch_v<RM, MODE, false>(p, tiles, st);
 }
 // rows per CTA: all of them up to 32, so that a weight is read once (64 rows: twice)
 template <int MODE>
@@ -213,7 +226,8 @@ cudaError_t launch_linear_f32(const F32Linear& p, cudaStream_t st) {
 // ================================================================================================
 constexpr int FA_THREADS = 256, FA_KEYS = 2048, FA_U = 8;      // FA_U: loads in flight per thread
 
-template <int D>
+// VEC: q and the caches are 16-byte aligned
+template <int D, bool VEC>
 __global__ void __launch_bounds__(FA_THREADS) attn_f32_kernel(const float* __restrict__ q, const float* __restrict__ kc,
                                                               const float* __restrict__ vc, float* __restrict__ out, int n, int L,
                                                               const int* __restrict__ len_ptr, int max_seq, int hq, int hkv, int causal,
@@ -228,11 +242,11 @@ __global__ void __launch_bounds__(FA_THREADS) attn_f32_kernel(const float* __res
   const int sub = lane / LPK, li = lane % LPK, part = threadIdx.x / LPK, col = threadIdx.x % LPK;
   if (len_ptr) L = *len_ptr;
   const int T = causal ? L + r + 1 : L + n;
-  const float4* kb = reinterpret_cast<const float4*>(kc + (size_t)hk * max_seq * D);
-  const float4* vb = reinterpret_cast<const float4*>(vc + (size_t)hk * max_seq * D);
+  const float* kb = kc + (size_t)hk * max_seq * D;
+  const float* vb = vc + (size_t)hk * max_seq * D;
   pdl_wait();
   const float scale = rsqrtf((float)D);
-  float4 qv = __ldcg(reinterpret_cast<const float4*>(q + ((size_t)r * hq + head) * D) + li);
+  float4 qv = ldcg_f4(q + ((size_t)r * hq + head) * D + li * 4, VEC);
   qv = make_float4(qv.x * scale, qv.y * scale, qv.z * scale, qv.w * scale);
   const unsigned long long mask = row_mask ? row_mask[r] : ~0ull;
   float m_run = -INFINITY, sum = 0.f;
@@ -243,7 +257,7 @@ __global__ void __launch_bounds__(FA_THREADS) attn_f32_kernel(const float* __res
     for (int b = warp * KPW * FA_U; b < cn; b += NW * KPW * FA_U) {
       float4 kv[FA_U];
 #pragma unroll
-      for (int u = 0; u < FA_U; ++u) kv[u] = __ldcg(kb + (size_t)(c0 + min(b + u * KPW + sub, cn - 1)) * LPK + li);
+      for (int u = 0; u < FA_U; ++u) kv[u] = ldcg_f4(kb + (size_t)(c0 + min(b + u * KPW + sub, cn - 1)) * D + li * 4, VEC);
 #pragma unroll
       for (int u = 0; u < FA_U; ++u) {
         float s = dot4(qv, kv[u], 0.f);
@@ -273,7 +287,7 @@ __global__ void __launch_bounds__(FA_THREADS) attn_f32_kernel(const float* __res
     for (int j0 = part; j0 < cn; j0 += PARTS * FA_U) {
       float4 vv[FA_U];
 #pragma unroll
-      for (int u = 0; u < FA_U; ++u) vv[u] = __ldcg(vb + (size_t)(c0 + min(j0 + u * PARTS, cn - 1)) * LPK + col);
+      for (int u = 0; u < FA_U; ++u) vv[u] = ldcg_f4(vb + (size_t)(c0 + min(j0 + u * PARTS, cn - 1)) * D + col * 4, VEC);
 #pragma unroll
       for (int u = 0; u < FA_U; ++u) {
         const int j = j0 + u * PARTS;
@@ -293,7 +307,8 @@ __global__ void __launch_bounds__(FA_THREADS) attn_f32_kernel(const float* __res
 }
 
 int launch_attention_f32(const AttnArgs& a, cudaStream_t st, cudaError_t* err) {
-  auto kern = a.d == 128 ? attn_f32_kernel<128> : attn_f32_kernel<64>;
+  const bool vec = aligned16(a.q) && aligned16(a.kc) && aligned16(a.vc);
+  auto kern = a.d == 128 ? (vec ? attn_f32_kernel<128, true> : attn_f32_kernel<128, false>) : (vec ? attn_f32_kernel<64, true> : attn_f32_kernel<64, false>);
   *err = launch_pdl(kern, dim3(a.hq, a.n), dim3(FA_THREADS), 0, st, (const float*)a.q, (const float*)a.kc, (const float*)a.vc, (float*)a.out,
                     a.n, a.cache_len, a.len_ptr, a.max_seq, a.hq, a.hkv, a.causal, a.row_mask);
   return *err == cudaSuccess ? 1 : -1;

@@ -35,6 +35,49 @@ def test_decode_attention_chunks_and_merge(elem, n, L, hq, hkv, d, causal):
     assert np.abs(out.double().cpu().numpy() - ref).max() <= bound
 
 
+# ---- callers' tensors need no more alignment than their elements where the loads and stores are no bulk copies ----
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("elem", [torch.float32, torch.bfloat16, torch.float16], ids=["f32", "bf16", "f16"])
+def test_attention_operator_on_tensors_at_any_element(elem, d):
+    from paper_2604_06832_b200 import binding as B
+    n, L, hq, hkv, seq = 5, 70, 4, 2, 80
+    g = torch.Generator().manual_seed(d)
+    q, kc, vc = (torch.randn(*s, generator=g).to(elem).cuda() for s in ((n, hq, d), (hkv, seq, d), (hkv, seq, d)))
+    f32 = elem == torch.float32
+    dt, kv = (B.DT_F32 if f32 else B.DT_BF16), (B.KV_BF16 if elem == torch.bfloat16 else B.KV_F16)
+    want = B.op_attention(q, kc, vc, L, True, dtype=dt)
+    ws = torch.zeros(B.lib().fdvlm_op_attention_workspace_bytes(n, hq, hkv, d), dtype=torch.uint8, device="cuda")
+    for off in (1, 2, 3):
+        out = torch.zeros(want.numel() + 4, dtype=elem, device="cuda")
+        args = [q, kc, vc]
+        if f32:       # (the 16-bit kernels fetch these with 16-byte copies)
+            args = [torch.zeros(t.numel() + 4, device="cuda")[off:off + t.numel()].copy_(t.flatten()) for t in args]
+        rc = B.lib().fdvlm_op_attention(*(t.data_ptr() for t in args), out[off:].data_ptr(), n, L, seq, hq, hkv, d, 1, dt, kv, ws.data_ptr(), None)
+        assert rc == 0
+        torch.cuda.synchronize()
+        assert torch.equal(out[off:off + want.numel()], want.flatten()) and not out[:off].any() and not out[off + want.numel():].any()
+
+
+@pytest.mark.parametrize("shape", [I.TINY, BF16, FP8], ids=["f32", "bf16", "fp8"])
+def test_norm_gains_at_any_element(shape):
+    from paper_2604_06832_b200 import binding as B
+    w = B.weights_to_device(I.make_weights(shape, 3, gain_spread=0.5))
+    toks = I.random_tokens(shape, 150, 4).cuda()
+    outs = []
+    for off in (0, 1):
+        for t in [w] + w["layers"]:
+            for name in ("g_final", "g_attn", "g_mlp"):
+                if name in t:
+                    t[name] = torch.zeros(shape.hidden + 4, device="cuda")[off:off + shape.hidden].copy_(t[name])
+        h = B.Handle(shape, w, max_seq=256)
+        last = torch.empty(shape.vocab, device="cuda")
+        h.prefill(None, toks, last)
+        h.synchronize()
+        outs.append(last)
+        h.close()
+    assert torch.equal(*outs)
+
+
 # ---- exact fp32: depth beyond one shared-memory panel, ragged widths, every row tile, more keys than one pass holds ----
 WIDE_F32 = I.TINY.with_(n_layers=1, hidden=1096, intermediate=1112, vocab=1003, mask_id=1002)
 
