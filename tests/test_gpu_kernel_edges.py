@@ -78,6 +78,30 @@ def test_norm_gains_at_any_element(shape):
     assert torch.equal(*outs)
 
 
+# ---- SwiGLU of gates outside the range of its arithmetic ----
+@pytest.mark.parametrize("n", [5, 150], ids=["decode", "prompt"])
+def test_an_infinite_gate_saturates_like_a_large_one(n):
+    """A gate of +inf gives an activation that is stored as +-65504, as one of 1e7 does.  (fp8 weights, whose activations are f16 values;
+    all entries of the embedding rows are positive and dominate the residual stream, so the gate of the feature is.)"""
+    from paper_2604_06832_b200 import binding as B
+    shape = FP8.with_(n_layers=1)
+    w = B.weights_to_device(I.make_weights(shape, 3))
+    lw, feature = w["layers"][0], 37
+    lw["w_gate"][feature] = 0x38                                  # e4m3 code of 1.0
+    lw["w_up"][feature] = 0x38                                    # (far above 65504 / 1e7 too)
+    emb = torch.ones(n, shape.hidden, dtype=torch.bfloat16, device="cuda")
+    outs = []
+    for scale in (1e7 / shape.hidden, 3e38):
+        lw["s_gate"][feature] = scale
+        h = B.Handle(shape, w, max_seq=256)
+        last = torch.empty(shape.vocab, device="cuda")
+        h.prefill(emb, None, last)
+        h.synchronize()
+        outs.append(last)
+        h.close()
+    assert torch.isfinite(outs[0]).all() and torch.equal(*outs)
+
+
 # ---- exact fp32: depth beyond one shared-memory panel, ragged widths, every row tile, more keys than one pass holds ----
 WIDE_F32 = I.TINY.with_(n_layers=1, hidden=1096, intermediate=1112, vocab=1003, mask_id=1002)
 
