@@ -154,8 +154,8 @@ __global__ void __launch_bounds__(FL_WARPS * 32) linear_f32_kernel(const F32Line
     if (!p.stats) return;
     // softmax statistics of the CTA's 16 vocabulary ids, the mask token excluded
     const float la = (in0 && f0 != p.mask_id) ? a : -INFINITY, lb = (in1 && f1 != p.mask_id) ? b : -INFINITY;
-    float mx = fmaxf(la, lb);
-    int ix = la >= lb ? f0 : f1;                      // (f0 < f1: a tie goes to the lower id)
+    float mx = fmaxf(fmaxf(la, lb), -INFINITY);       // (a NaN logit is no maximum; it does reach the sum)
+    int ix = (lb > la || la != la) ? f1 : f0;         // (f0 < f1: a tie goes to the lower id)
 #pragma unroll
     for (int o = 4; o > 0; o >>= 1) {
       const float omx = __shfl_xor_sync(0xffffffffu, mx, o);

@@ -102,6 +102,35 @@ def test_an_infinite_gate_saturates_like_a_large_one(n):
     assert torch.isfinite(outs[0]).all() and torch.equal(*outs)
 
 
+# ---- exact fp32: a NaN logit spoils the confidences and is never the prediction ----
+@pytest.mark.parametrize("step", [8, -8, 1], ids=["same-pair-above", "same-pair-below", "next-pair"])
+def test_exact_f32_prediction_beside_a_nan_logit(step):
+    from paper_2604_06832_b200 import binding as B
+    w = B.weights_to_device(I.make_weights(I.TINY, 6))
+    toks = torch.arange(40, dtype=torch.int32, device="cuda")
+    pred, conf = torch.empty(1, dtype=torch.int32, device="cuda"), torch.empty(1, device="cuda")
+
+    def predict():
+        h = B.Handle(I.TINY, w, max_seq=64)
+        h.prefill(None, toks)
+        h.block_begin(1)
+        h.block_step(B.RULE_TOPK, 0.0, 1, pred=pred, conf=conf)
+        h.close()
+        return int(pred), float(conf)
+
+    target = 304 + (8 if step == -8 else 0)                       # lane 0 of a tile of 16 ids, as its lower or upper one
+    mask_row = w["embed"][I.TINY.mask_id].clone()
+    for gain in (1.0, 4.0, 16.0, 64.0):                           # until the id wins: its row points along the mask row
+        w["embed"][target] = gain * mask_row
+        best, c = predict()
+        if best == target:
+            break
+    assert best == target and np.isfinite(c)
+    w["embed"][target + step] = float("nan")
+    best, c = predict()
+    assert best == target and np.isnan(c)
+
+
 # ---- exact fp32: depth beyond one shared-memory panel, ragged widths, every row tile, more keys than one pass holds ----
 WIDE_F32 = I.TINY.with_(n_layers=1, hidden=1096, intermediate=1112, vocab=1003, mask_id=1002)
 
