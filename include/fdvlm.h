@@ -121,7 +121,10 @@ typedef struct { int n_unmasked, n_remaining, step_index; } fdvlm_step_info;
 
 /* Create a handle on the current CUDA device.  `cuda_stream` is a cudaStream_t (NULL = default
  * stream).  Allocates the KV cache (n_layers * 2 * n_kv_heads * max_seq * head_dim elements) and a
- * workspace.  Requires: head_dim in {64, 128}; n_q_heads % n_kv_heads == 0; hidden, intermediate,
+ * workspace; for bf16 and fp8 weights with max_seq > 128 also, if they fit, the buffers of long prompts' forwards: for each
+ * of min(max_seq, 4096) rows about 10 (bf16) or 8 (fp8) bytes per hidden unit, 6 or 4 per query width, 4 or 2 per
+ * intermediate unit, and 39 MB (3B shape: 0.34 GB, 7B shape with fp8 weights: 0.37 GB).  Without them prompts run in forwards of
+ * max_block rows.  Requires: head_dim in {64, 128}; n_q_heads % n_kv_heads == 0; hidden, intermediate,
  * q/kv widths multiples of 8 (bf16/fp8: hidden and intermediate multiples of 16); 1 <= max_block <= 64. */
 int fdvlm_create(const fdvlm_config *cfg, const fdvlm_weights *w, void *cuda_stream, fdvlm_t **out);
 void fdvlm_destroy(fdvlm_t *h);

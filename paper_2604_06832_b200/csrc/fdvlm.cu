@@ -168,35 +168,41 @@ extern "C" int fdvlm_create(const fdvlm_config* cfg, const fdvlm_weights* w, voi
   };
   size_t slab_bytes = 0;
   for (auto& a : allocs) slab_bytes += (a.bytes + 255) / 256 * 256;
+  e = cudaMalloc((void**)&h->slab, slab_bytes);
+  const size_t kv_bytes = (size_t)cfg->n_layers * 2 * kv_plane(h);
+  if (e == cudaSuccess) e = cudaMalloc((void**)&h->kv, kv_bytes);
+  if (e != cudaSuccess) {
+    fail(nullptr, FDVLM_ERR_OOM, "cudaMalloc of the work buffers (%zu bytes) or the KV cache (%zu bytes) failed: %s", slab_bytes, kv_bytes,
+         cudaGetErrorString(e));
+    cudaGetLastError();
+    fdvlm_destroy(h);
+    return FDVLM_ERR_OOM;
+  }
   // Prompt path: as many rows as one forward of it takes (PF_MAX_ROWS: above that its tiles fill the GPU many times over
-  // and more rows only cost memory).  W8A8 prompts run through the decode path.
-  size_t pf_bytes = 0;
+  // and more rows only cost memory).  W8A8 prompts run through the decode path, and so do all prompts of a handle whose memory
+  // is taken up by what it cannot do without.
   if (h->use_tc && !h->act8 && cfg->max_seq > PF_MIN_ROWS) {
     const int max_rows = (cfg->max_seq + 127) / 128 * 128;
     const size_t P = max_rows < PF_MAX_ROWS ? max_rows : PF_MAX_ROWS;
-    h->pf_rows = (int)P;
+    const int pf_planes = h->pf_fmt == XF_BF16X2 ? 2 : 1;      // (pf_a also holds the LM head's input)
     h->pf_part_bytes = (size_t)sm_count() * 256 * 256 * sizeof(float);
     struct { void** p; size_t bytes; } pf[] = {
         {(void**)&h->pf_h, P * H * 4},        {(void**)&h->pf_cs, P * d * 4},
         {(void**)&h->pf_ssq, P * h->nt * 4},  {(void**)&h->pf_a, P * H * 2 * a_planes},
-        {(void**)&h->pf_q, P * NQ * 2},       {(void**)&h->pf_ao, P * NQ * 2 * planes},
-        {(void**)&h->pf_act, P * I * 2 * planes}, {(void**)&h->pf_part, h->pf_part_bytes},
+        {(void**)&h->pf_q, P * NQ * 2},       {(void**)&h->pf_ao, P * NQ * 2 * pf_planes},
+        {(void**)&h->pf_act, P * I * 2 * pf_planes}, {(void**)&h->pf_part, h->pf_part_bytes},
         {(void**)&h->pf_arrived, (size_t)sm_count() * 4 * sizeof(unsigned)},
     };
+    size_t pf_bytes = 0;
     for (auto& a : pf) pf_bytes += (a.bytes + 255) / 256 * 256;
-    e = cudaMalloc((void**)&h->pf_slab, pf_bytes);
-    if (e == cudaSuccess) {
+    if (cudaMalloc((void**)&h->pf_slab, pf_bytes) == cudaSuccess) {
+      h->pf_rows = (int)P;
       char* cur = h->pf_slab;
       for (auto& a : pf) { *a.p = cur; cur += (a.bytes + 255) / 256 * 256; }
+    } else {
+      h->pf_slab = nullptr;
+      cudaGetLastError();
     }
-  }
-  if (e == cudaSuccess) e = cudaMalloc((void**)&h->slab, slab_bytes);
-  if (e == cudaSuccess) e = cudaMalloc((void**)&h->kv, (size_t)cfg->n_layers * 2 * kv_plane(h));
-  if (e != cudaSuccess) {
-    fail(nullptr, FDVLM_ERR_OOM, "cudaMalloc of the work buffers (%zu bytes) or the KV cache failed: %s", slab_bytes, cudaGetErrorString(e));
-    cudaGetLastError();
-    fdvlm_destroy(h);
-    return FDVLM_ERR_OOM;
   }
   {
     char* cur = h->slab;

@@ -329,6 +329,41 @@ def test_two_handles_on_two_streams_in_one_process():
     h2.close()
 
 
+@pytest.mark.parametrize("shape", [SMALL_BF16, SMALL_FP8], ids=["bf16", "fp8"])
+def test_a_handle_where_only_the_buffers_of_long_prompts_do_not_fit(shape):
+    """Such a handle takes long prompts all the same, in forwards of max_block rows."""
+    b = B()
+    n = 300
+    oracle, roomy, w = make_pair(shape, 23, max_seq=4096)
+    emb, toks = I.make_prefix(shape, 200, n - 200, 4)
+    ref = oracle.prefill(I.as_numpy_storage(emb), toks.numpy())
+    wd = b.weights_to_device(w)
+    emb, toks = upload_prefix(emb, toks)
+    got = [torch.empty(shape.vocab, dtype=torch.float32, device="cuda") for _ in range(2)]
+    roomy.prefill(emb, toks, got[0])
+    roomy.synchronize()
+    launches = roomy.last_launch_count()
+    roomy.prefill(emb[:100], None)                # (the kernels of the other path are loaded)
+    roomy.synchronize()
+    roomy.close()
+    torch.cuda.empty_cache()
+    # all but 44 to 56 MB of the device's memory: more than the 25 MB that such a handle needs, less than the prompt buffers (66 MB
+    # and more)
+    taken = []
+    for chunk in (1 << 30, 12 << 20):
+        while torch.cuda.mem_get_info()[0] >= (44 << 20) + chunk:
+            taken.append(torch.empty(chunk, dtype=torch.uint8, device="cuda"))
+    handle = b.Handle(shape, wd, max_seq=4096)
+    handle.prefill(emb, toks, got[1])
+    handle.synchronize()
+    assert handle.last_launch_count() > 2 * launches
+    handle.close()
+    del taken
+    torch.cuda.empty_cache()
+    for g in got:
+        assert np.abs(g.double().cpu().numpy() - ref).max() <= TOL[shape.dtype]["logits"]
+
+
 def test_stream_read_yardstick_runs_and_rejects_bad_arguments():
     b = B()
     buf = torch.zeros(64 << 20, dtype=torch.uint8, device="cuda")
