@@ -19,14 +19,14 @@ thread_local char g_create_error[512] = "";
 // TcOut::status; cleared here on the stream), then -- fp8 weights only -- the bf16 rows as XF_E5M2X3 planes (W8A8: as e4m3
 // codes, followed by one 256-byte-rounded array of per-row factors), then the split-K partial sums.
 static size_t op_scale_bytes(int m, int dtype) { return dtype == DT_A8 ? (((size_t)m * 4 + 255) / 256) * 256 : 0; }
-static size_t op_x16_bytes(int m, int k, int dtype) {
-  if (dtype == DT_FP8) return (((size_t)m * k * 3 + 255) / 256) * 256;
+static size_t op_x16_bytes(int m, int k, int dtype, int fp8_row_bytes = 3) {
+  if (dtype == DT_FP8) return (((size_t)m * k * fp8_row_bytes + 255) / 256) * 256;
   return dtype == DT_A8 ? (((size_t)m * k + 255) / 256) * 256 + op_scale_bytes(m, dtype) : 0;
 }
-size_t linear_workspace_bytes(int m, int n, int k, int dtype) {
+size_t linear_workspace_bytes(int m, int n, int k, int dtype, int fp8_row_bytes) {
   const int wdt = dtype == DT_A8 ? DT_FP8 : dtype;
   size_t a = dtype == DT_A8 ? 0 : simt_workspace_bytes(m, n, k);
-  size_t b = tc_linear_supported(m, n, k, wdt) ? tc_workspace_bytes(m, n, (n + 127) / 128, k) + op_x16_bytes(m, k, dtype) : 0;
+  size_t b = tc_linear_supported(m, n, k, wdt) ? tc_workspace_bytes(m, n, (n + 127) / 128, k) + op_x16_bytes(m, k, dtype, fp8_row_bytes) : 0;
   return OP_HEAD + (a > b ? a : b);
 }
 

@@ -164,7 +164,8 @@ int forward_prefill(fdvlm_t* h, int n, int want_last_logits);
 int stage_prefill_rows(fdvlm_t* h, int row0, int n, const int32_t* tokens, const void* embeds);
 int forward_rows_enqueue(fdvlm_t* h, int n, int mode, int logits_rows, int want_logits);
 
-size_t linear_workspace_bytes(int m, int n, int k, int dtype);
+// (fp8_row_bytes: bytes that an element of the rows takes beside fp8 weights)
+size_t linear_workspace_bytes(int m, int n, int k, int dtype, int fp8_row_bytes = 3);
 size_t attention_workspace_bytes(int n, int hq, int hkv, int d);
 
 constexpr int PF_MIN_ROWS = 128;     // a prompt of at most this many rows is one forward of the decode path

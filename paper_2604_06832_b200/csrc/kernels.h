@@ -22,7 +22,6 @@ struct LinearArgs {
   void* workspace;      // split-K partial sums
   size_t workspace_bytes;
 };
-size_t linear_workspace_bytes(int m, int n, int k, int dtype);
 
 // ---- elementwise / reduction kernels -----------------------------------------------------------
 // tokens outside [0, vocab) read row 0 and leave ST_BAD_TOKEN in *status

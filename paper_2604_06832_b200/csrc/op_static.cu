@@ -38,8 +38,7 @@ extern "C" int fdvlm_op_linear_static(const void* x, const void* w, const float*
   if (dtype != FDVLM_F32 && dtype != FDVLM_BF16 && dtype != FDVLM_W_FP8E4M3)
     return fail(nullptr, FDVLM_ERR_INVALID_ARG, "op_linear_static: unknown dtype %d", (int)dtype);
   if (dtype == FDVLM_W_FP8E4M3 && !scale) return fail(nullptr, FDVLM_ERR_INVALID_ARG, "op_linear_static: fp8 weights need scales");
-  size_t need = linear_workspace_bytes(m, n, k, (int)dtype);
-  if (dtype == FDVLM_W_FP8E4M3 && need > (size_t)m * k) need -= (size_t)m * k;
+  const size_t need = linear_workspace_bytes(m, n, k, (int)dtype, 2);
   const size_t room = (size_t)FDVLM_STATIC_SCRATCH_BYTES;
   if (need > room)
     return fail(nullptr, FDVLM_ERR_CAPACITY,

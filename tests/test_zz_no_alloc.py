@@ -88,3 +88,17 @@ def test_static_scratch_variant_refuses_shapes_beyond_its_array():
     with pytest.raises(B.FdvlmError) as e:
         B.op_linear_static(x, w, dtype=B.DT_BF16)
     assert e.value.code == B.ERR_CAPACITY and "scratch" in str(e.value)
+
+
+@pytest.mark.parametrize("m,n,k,fits", [(49, 1365, 17344, True), (53, 12133, 6336, True), (49, 1365, 17360, False)])
+def test_static_scratch_limit_of_fp8_rows(m, n, k, fits):
+    """The limit counts two bytes an element of the rows, rounded up as one buffer: calls at the limit itself."""
+    from paper_2604_06832_b200 import binding as B
+    x = torch.zeros(m, k, dtype=torch.bfloat16, device="cuda")
+    w = torch.zeros(n, k, dtype=torch.uint8, device="cuda")
+    y = torch.ones(m, n, dtype=torch.float32, device="cuda")
+    scale = torch.ones(n, device="cuda")
+    rc = B.lib().fdvlm_op_linear_static(x.data_ptr(), w.data_ptr(), scale.data_ptr(), None, y.data_ptr(), m, n, k, B.DT_FP8, None)
+    assert rc == (0 if fits else B.ERR_CAPACITY)
+    assert B.lib().fdvlm_op_linear_status(None, None) == 0
+    assert not y.any() if fits else y.all()
