@@ -240,6 +240,28 @@ extern "C" int fdvlm_reset(fdvlm_t* h) {
 extern "C" int fdvlm_cache_len(const fdvlm_t* h) { return h ? h->cache_len : (int)FDVLM_ERR_INVALID_ARG; }
 extern "C" int fdvlm_last_launch_count(const fdvlm_t* h) { return h ? h->launches : (int)FDVLM_ERR_INVALID_ARG; }
 
+// Whether a prompt of `rows` rows takes the prompt path (forward_prefill): above PF_MIN_ROWS rows, unless it is a short turn behind a
+// long cache.  The prompt attention does not split the keys, so while its CTAs leave SMs idle each key costs a layer 12 ns; the decode path
+// splits them, but streams the weights once for every max_block rows.  Measured (us, decode path : prompt path, 64-row forwards):
+//   3B shape, 6 layers, 129 / 192 rows : 4000 keys 1163 : 1093 / 1293 : 1141, 6000 keys 1195 : 1201 / 1320 : 1248, 8000 keys 1226 : 1339 / 1353 : 1366
+//                       256 rows       : 12000 keys 1852 : 1704, 16000 keys 1911 : 2007; 400 rows: 24000 keys 3399 : 2847, 32000 keys 3573 : 3427
+//   7B shape, fp8, 4 layers, 192 rows  : 8000 keys 1308 : 1049, 16000 keys 1489 : 1515; 256 rows: 32000 keys 2340 : 2282
+//   512 wide, 8 heads, 3 layers, 192 rows : 6000 keys 461 : 416, 8000 keys 466 : 485; fp8: 8000 keys 491 : 461, 10000 keys 507 : 575
+// The times of a layer below (us; `mb` megabytes of weights) are those of these runs at an empty cache.
+static bool takes_prompt_path(const fdvlm_t* h, int rows) {
+  if (h->pf_rows <= 0 || rows <= PF_MIN_ROWS) return false;
+  const fdvlm_config& c = h->cfg;
+  const bool fp8 = h->dt == DT_FP8;
+  const double q = (double)c.n_q_heads * c.head_dim, kv = (double)c.n_kv_heads * c.head_dim, keys = (double)h->cache_len + rows;
+  const double mb = (double)c.hidden * (2 * q + 2 * kv + 3.0 * c.intermediate) * (fp8 ? 1e-6 : 2e-6);
+  const int full = (rows - 1) / c.max_block, more = (rows - 1) / 256;
+  const double forwards = full + 0.7 + 0.3 * (rows - full * c.max_block) / c.max_block;      // (of few rows: a little cheaper)
+  const double decode = forwards * (fp8 ? 52 + 0.19 * mb : 48 + 0.14 * mb);
+  const double prompt = fp8 ? 62 + (0.41 + 0.35 * more) * mb : 70 + (0.38 + 0.25 * more) * mb;
+  const double per_key = (c.head_dim == 128 ? 12.2e-3 : 10.5e-3) - 0.33e-6 * q * forwards;   // (more than in the decode path)
+  return prompt + per_key * keys <= decode;
+}
+
 extern "C" int fdvlm_prefill(fdvlm_t* h, const void* embeds, int n_embeds, const int32_t* tokens, int n_tokens,
                              float* last_logits) {
   if (!h) return FDVLM_ERR_INVALID_ARG;
@@ -252,8 +274,8 @@ extern "C" int fdvlm_prefill(fdvlm_t* h, const void* embeds, int n_embeds, const
     return fail(h, FDVLM_ERR_CAPACITY, "prefill: %d + %d rows exceed max_seq %d", h->cache_len, total, h->cfg.max_seq);
   h->launches = 0;
   const int H = h->cfg.hidden;
-  // Above PF_MIN_ROWS rows the prompt path; its forwards are of equal size (in whole 128-row tiles).
-  const bool large = h->pf_rows > 0 && total > PF_MIN_ROWS;
+  // The prompt path's forwards are of equal size (in whole 128-row tiles).
+  const bool large = takes_prompt_path(h, total);
   int R = h->cfg.max_block;
   if (large) {
     const int parts = (total + h->pf_rows - 1) / h->pf_rows;
