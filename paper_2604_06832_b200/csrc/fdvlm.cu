@@ -953,7 +953,7 @@ extern "C" int fdvlm_op_linear(const void* x, const void* w, const float* scale,
   if (dtype != FDVLM_F32 && dtype != FDVLM_BF16 && dtype != FDVLM_W_FP8E4M3 && dtype != FDVLM_W8A8_FP8E4M3) return FDVLM_ERR_INVALID_ARG;
   if ((dtype == FDVLM_W_FP8E4M3 || dtype == FDVLM_W8A8_FP8E4M3) && !scale) return FDVLM_ERR_INVALID_ARG;
   LinearArgs a;
-  a.x = x; a.w = w; a.scale = scale; a.bias = bias; a.y = y; a.m = m; a.n = n; a.k = k; a.ldy = n; a.accumulate = 0;
+  a.x = x; a.w = w; a.scale = scale; a.bias = bias; a.y = y; a.m = m; a.n = n; a.k = k;
   a.dtype = (int)dtype; a.workspace = workspace; a.workspace_bytes = linear_workspace_bytes(m, n, k, (int)dtype);
   if (!workspace) return FDVLM_ERR_INVALID_ARG;
   cudaError_t e;

@@ -10,8 +10,8 @@ size_t simt_workspace_bytes(int m, int n, int k);
 int launch_attention_f32(const AttnArgs& a, cudaStream_t st, cudaError_t* err);
 size_t attention_tc_workspace_bytes(int n, int hq, int hkv, int d);
 int launch_attention_tc(const AttnArgs& a, cudaStream_t st, cudaError_t* err);
-void launch_splitk_epilogue(const float* part, int S, int m, int n, const float* scale, const float* bias, float* y, int ldy,
-                            int accumulate, cudaStream_t st, const float* x_scale = nullptr);
+void launch_splitk_epilogue(const float* part, int S, int m, int n, const float* scale, const float* bias, float* y,
+                            cudaStream_t st, const float* x_scale = nullptr);
 
 thread_local char g_create_error[512] = "";
 
@@ -70,7 +70,7 @@ int launch_linear(const LinearArgs& a, cudaStream_t st, cudaError_t* err) {
   o.ld = a.n; o.status = (int*)a.workspace;
   *err = tc_group_launch(g, o, st);
   if (*err != cudaSuccess) return -1;
-  launch_splitk_epilogue(part, splits, a.m, a.n, a.scale, a.bias, a.y, a.ldy, a.accumulate, st, x_scale);
+  launch_splitk_epilogue(part, splits, a.m, a.n, a.scale, a.bias, a.y, st, x_scale);
   *err = cudaGetLastError();
   return *err == cudaSuccess ? launched : -1;
 }
@@ -83,7 +83,6 @@ int launch_attention(const AttnArgs& a, cudaStream_t st, cudaError_t* err) {
 
 int stage_rows(fdvlm_t* h, int row0, int n, const int32_t* tokens, const void* embeds, int mode, const int* len_ptr) {
   const int H = h->cfg.hidden;
-  const int edt = h->dt == DT_F32 ? DT_F32 : DT_BF16;
   if (h->use_tc) {
     launch_embed_prep(h->w.embed, tokens, embeds, h->h + (size_t)row0 * H, (char*)h->a + (size_t)row0 * H * xf_bytes(h->xfmt), h->a_lo, h->xfmt,
                       h->layers[0].g_attn, h->ssq + (size_t)row0 * h->nt, h->nt, n, H, h->cfg.vocab, h->info + 3, h->st, nullptr,
@@ -91,10 +90,8 @@ int stage_rows(fdvlm_t* h, int row0, int n, const int32_t* tokens, const void* e
   } else if (tokens && mode >= 0) {
     launch_embed_rope_f32(h->w.embed, tokens, h->h + (size_t)row0 * H, n, H, h->cfg.vocab, h->info + 3, h->cs, h->cache_len, h->cfg.head_dim,
                           h->cfg.rope_theta, len_ptr, mode == MODE_MASKED ? h->q_pos_off : nullptr, h->st);
-  } else if (tokens) {
-    launch_embed(h->w.embed, tokens, h->h + (size_t)row0 * H, n, H, edt, h->cfg.vocab, h->info + 3, h->st);
   } else {
-    launch_rows_to_f32(embeds, h->h + (size_t)row0 * H, n, H, edt, h->st);
+    launch_embed_f32(tokens ? h->w.embed : embeds, tokens, h->h + (size_t)row0 * H, n, H, h->cfg.vocab, h->info + 3, h->st);
   }
   h->launches++;
   CU(h, cudaGetLastError());

@@ -43,12 +43,11 @@ struct TcParams {
   int tile_begin[4];    // first tile of each matrix; [n_mats] = total tiles
   int out_col[3];       // column of each matrix's first feature in the output row
   const float* scale[3];
-  const float* bias[3];
   int n_mats, kblocks, splits, kb_per_split, m, mode;
   float* part;          // [splits][m][ldp]     (PARTIAL)
   int ldp;
-  float* y;             // [m][ldy]             (DIRECT)
-  int ldy, accumulate;
+  float* y;             // [m][ldy]             (LOGITS)
+  int ldy;
   void* act;            // [m][inter]           (SWIGLU), stored as act_fmt (XF_*), lo plane act_lo_off elements on
   size_t act_lo_off;
   int act_fmt, inter;
@@ -435,26 +434,11 @@ __global__ void __launch_bounds__(TC_THREADS) gemm_tc_kernel(const __grid_consta
         const int n = (tile - p.tile_begin[mi]) * TC_BM + q * 32 + lane;
         const bool in_range = n < p.n_out[mi];
         const int col = p.out_col[mi] + n;
-        if (p.mode == TC_MODE_PARTIAL) {
-          if (in_range) {
-            float* dst = p.part + (size_t)split * p.m * p.ldp + col;
+        if (in_range) {
+          float* dst = p.part + (size_t)split * p.m * p.ldp + col;
 #pragma unroll
-            for (int b = 0; b < M_PAD; ++b)
-              if (b < p.m) dst[(size_t)b * p.ldp] = v[b];
-          }
-        } else {
-          const float sc = (in_range && p.scale[mi]) ? p.scale[mi][n] : 1.f;
-          const float bi = (in_range && p.bias[mi]) ? p.bias[mi][n] : 0.f;
-#pragma unroll
-          for (int b = 0; b < M_PAD; ++b) {
-            const float rs = __shfl_sync(0xffffffffu, (b < 32) ? rs0 : rs1, b & 31);
-            if (in_range && b < p.m) {
-              float* dst = p.y + (size_t)b * p.ldy + col;
-              float r = v[b] * sc * rs + bi;
-              if (p.accumulate) r += *dst;
-              *dst = r;
-            }
-          }
+          for (int b = 0; b < M_PAD; ++b)
+            if (b < p.m) dst[(size_t)b * p.ldp] = v[b];
         }
       }
     }
@@ -585,7 +569,6 @@ static cudaError_t tc_launch_f(const TcParams& p, cudaStream_t st) {
 
 // A group of up to three bf16 matrices that share x and K, outputs side by side in one row of width ld.
 //   mode PARTIAL: part[split][m][ld] (split-K sums left to the caller's reduce kernel); *splits_out tells how many
-//   mode DIRECT : y[m][ld] = x w^T * scale + bias (+ y)   (forces one split)
 //   mode SWIGLU : act[m][inter] = silu(x wg^T * sg) * (x wu^T * su)  (w[0] = gate, w[1] = up; one split)
 
 cudaError_t tc_group_launch(const TcGroup& g, const TcOut& o, cudaStream_t st) {
@@ -596,7 +579,7 @@ cudaError_t tc_group_launch(const TcGroup& g, const TcOut& o, cudaStream_t st) {
   const bool a8 = g.fp8 && g.a8;                  // rows as e4m3 codes
   const bool x3 = g.fp8 && !a8;                   // rows as e5m2 planes
   const int xkind = g.fp8 ? TM_E4M3_128 : TM_BF16;     // (bytes are bytes: e5m2 planes take the same map)
-  if (a8 && (mode == TC_MODE_DIRECT || mode == TC_MODE_LOGITS)) return cudaErrorInvalidValue;
+  if (a8 && mode == TC_MODE_LOGITS) return cudaErrorInvalidValue;
   if (a8 && mode == TC_MODE_SWIGLU && (!o.x_scale || !o.amax_out || !o.ssq_in)) return cudaErrorInvalidValue;
   if (!make_tmap(&p.tm_x, g.x, g.m, g.k, mp, xkind)) return cudaErrorInvalidValue;
   p.has_lo = (!g.fp8 && g.x_lo) ? 1 : 0;
@@ -609,7 +592,6 @@ cudaError_t tc_group_launch(const TcGroup& g, const TcOut& o, cudaStream_t st) {
     p.tile_begin[i] = tiles;
     p.out_col[i] = col;
     p.scale[i] = g.scale[i];
-    p.bias[i] = g.bias[i];
     tiles += ceil_div(g.n[i], TC_BM);
     col += g.n[i];
   }
@@ -631,7 +613,7 @@ cudaError_t tc_group_launch(const TcGroup& g, const TcOut& o, cudaStream_t st) {
     p.tile_begin[g.n_mats] = tiles;
     if (mode == TC_MODE_PARTIAL) tc_plan(tiles, p.kblocks, &p.splits, &p.kb_per_split);
     else { p.splits = 1; p.kb_per_split = p.kblocks; }
-    p.part = o.part; p.ldp = o.ld; p.y = o.y; p.ldy = o.ld; p.accumulate = o.accumulate;
+    p.part = o.part; p.ldp = o.ld; p.y = o.y; p.ldy = o.ld;
     p.stats = (float4*)o.stats; p.mask_id = o.mask_id; p.write_logits = o.write_logits;
     if (mode == TC_MODE_PARTIAL && (size_t)p.splits * g.m * o.ld * sizeof(float) > o.part_bytes) return cudaErrorInvalidValue;
     if (mode == TC_MODE_LOGITS && (g.n_mats != 1 || !o.stats)) return cudaErrorInvalidValue;

@@ -112,10 +112,10 @@ linear_simt_kernel(const XT* __restrict__ x, const WT* __restrict__ w, float* __
   }
 }
 
-// y[r, n] = (accumulate ? y : 0) + (sum_s part[s][r][n]) * scale[n] + bias[n]; fixed summation order.
+// y[r, n] = (sum_s part[s][r][n]) * scale[n] + bias[n]; fixed summation order.
 __global__ void splitk_epilogue_kernel(const float* __restrict__ part, int S, int m, int N,
                                        const float* __restrict__ scale, const float* __restrict__ bias,
-                                       float* __restrict__ y, int ldy, int accumulate, const float* __restrict__ x_scale) {
+                                       float* __restrict__ y, const float* __restrict__ x_scale) {
   pdl_trigger();
   pdl_wait();
   size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -127,14 +127,13 @@ __global__ void splitk_epilogue_kernel(const float* __restrict__ part, int S, in
   if (scale) s *= scale[n];
   if (x_scale) s *= x_scale[r];   // sums of e4m3 code products
   if (bias) s += bias[n];
-  float* o = y + (size_t)r * ldy + n;
-  *o = accumulate ? (*o + s) : s;
+  y[idx] = s;
 }
 
-void launch_splitk_epilogue(const float* part, int S, int m, int n, const float* scale, const float* bias, float* y, int ldy,
-                            int accumulate, cudaStream_t st, const float* x_scale) {
+void launch_splitk_epilogue(const float* part, int S, int m, int n, const float* scale, const float* bias, float* y,
+                            cudaStream_t st, const float* x_scale) {
   size_t total = (size_t)m * n;
-  splitk_epilogue_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(part, S, m, n, scale, bias, y, ldy, accumulate, x_scale);
+  splitk_epilogue_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(part, S, m, n, scale, bias, y, x_scale);
 }
 
 static void simt_plan(int m, int n, int k, int* bm, int* splits, int* kps) {
@@ -178,7 +177,7 @@ int launch_linear_simt(const LinearArgs& a, cudaStream_t st, cudaError_t* err) {
   else simt_dispatch<fp8e4m3, bf16>(a, bm, grid, part, kps, st);
   size_t total = (size_t)a.m * a.n;
   splitk_epilogue_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(part, s, a.m, a.n, a.scale, a.bias, a.y,
-                                                                         a.ldy, a.accumulate, nullptr);
+                                                                         nullptr);
   *err = cudaGetLastError();
   return *err == cudaSuccess ? 2 : -1;
 }
@@ -193,17 +192,15 @@ __device__ __forceinline__ int checked_token(const int32_t* tokens, int r, int v
   if (threadIdx.x == 0 && status) atomicCAS(status, 0, ST_BAD_TOKEN);
   return 0;
 }
-template <typename ET>
-__global__ void embed_kernel(const ET* __restrict__ table, const int32_t* __restrict__ tokens,
-                             float* __restrict__ h, int hidden, int vocab, int* status) {
+// fp32 rows into the residual stream: those of `tokens`, or (null) the first n of the table
+__global__ void embed_f32_kernel(const float* __restrict__ table, const int32_t* __restrict__ tokens,
+                                 float* __restrict__ h, int hidden, int vocab, int* status) {
   int r = blockIdx.x;
-  const ET* src = table + (size_t)(tokens ? checked_token(tokens, r, vocab, status) : r) * hidden;
-  for (int c = threadIdx.x; c < hidden; c += blockDim.x) h[(size_t)r * hidden + c] = to_f32(src[c]);
+  const float* src = table + (size_t)(tokens ? checked_token(tokens, r, vocab, status) : r) * hidden;
+  for (int c = threadIdx.x; c < hidden; c += blockDim.x) h[(size_t)r * hidden + c] = src[c];
 }
-void launch_embed(const void* table, const int32_t* tokens, float* h, int n, int hidden, int dtype, int vocab, int* status,
-                  cudaStream_t st) {
-  if (dtype == DT_F32) embed_kernel<float><<<n, 256, 0, st>>>((const float*)table, tokens, h, hidden, vocab, status);
-  else embed_kernel<bf16><<<n, 256, 0, st>>>((const bf16*)table, tokens, h, hidden, vocab, status);
+void launch_embed_f32(const void* table, const int32_t* tokens, float* h, int n, int hidden, int vocab, int* status, cudaStream_t st) {
+  embed_f32_kernel<<<n, 256, 0, st>>>((const float*)table, tokens, h, hidden, vocab, status);
 }
 // cs[r][j] = (cos, sin) of position(r) * theta^(-j / half), as rope_table_kernel below
 __device__ __forceinline__ float2 rope_entry(int pos, int j, int half, double theta) {
@@ -230,9 +227,6 @@ void launch_embed_rope_f32(const void* table, const int32_t* tokens, float* h, i
                            int pos0, int head_dim, float theta, const int* len_ptr, const int* pos_off, cudaStream_t st) {
   launch_pdl(embed_rope_f32_kernel, dim3(n), dim3(128), 0, st, (const float*)table, tokens, h, hidden, vocab, status, (float2*)cs, pos0,
              head_dim / 2, (double)theta, len_ptr, pos_off);
-}
-void launch_rows_to_f32(const void* rows, float* h, int n, int hidden, int dtype, cudaStream_t st) {
-  launch_embed(rows, nullptr, h, n, hidden, dtype, 0, nullptr, st);
 }
 
 // ================================================================================================

@@ -15,9 +15,8 @@ struct LinearArgs {
   const void* w;        // [n, k]   per dtype
   const float* scale;   // [n] or null
   const float* bias;    // [n] or null
-  float* y;             // [m, ldy] fp32 result (written, or accumulated into when `accumulate`)
-  int m, n, k, ldy;
-  int accumulate;       // 1: y += result (residual add)
+  float* y;             // [m, n] fp32 result
+  int m, n, k;
   int dtype;            // DT_*
   void* workspace;      // split-K partial sums
   size_t workspace_bytes;
@@ -28,14 +27,12 @@ struct LinearArgs {
 // One launch for an fp32 row block: embedding gather and rotary table (as launch_rope_table).
 void launch_embed_rope_f32(const void* table, const int32_t* tokens, float* h, int n, int hidden, int vocab, int* status, float* cs,
                            int pos0, int head_dim, float theta, const int* len_ptr, const int* pos_off, cudaStream_t st);
-void launch_embed(const void* table, const int32_t* tokens, float* h, int n, int hidden, int dtype, int vocab, int* status,
-                  cudaStream_t st);
+void launch_embed_f32(const void* table, const int32_t* tokens, float* h, int n, int hidden, int vocab, int* status, cudaStream_t st);
 void launch_bf16_to_e5m2x3(const void* in, void* out, size_t n, cudaStream_t st);       // planes n bytes apart
 // W8A8: rows of k f16 values (k a multiple of 8) -> e4m3 codes and scale[row] = max / 448, from amax[row][n_amax], partial maxima
 // of |value| left by whoever wrote the rows; and bf16 rows -> f16 (saturating) -> the same, maxima included.
 void launch_quantize_rows(const void* x, int m, int k, const float* amax, int n_amax, void* codes, float* scale, cudaStream_t st);
 void launch_quantize_bf16_rows(const void* in, int m, int k, void* codes, float* scale, cudaStream_t st);
-void launch_rows_to_f32(const void* rows, float* h, int n, int hidden, int dtype, cudaStream_t st);
 void launch_rope_table(float* cs, int n, int pos0, int head_dim, float theta, cudaStream_t st, const int* len_ptr = nullptr,
                        KStamp* stamp = nullptr, const int* pos_off = nullptr);
 // quadratic self-speculative decoding (Appendix B, Alg. 2): row layout, input tokens, first draft, verify loop
@@ -85,28 +82,27 @@ int f32_logit_tiles(int vocab);
 cudaError_t launch_linear_f32(const F32Linear& p, cudaStream_t st);
 
 // ---- tensor-core (tcgen05 + TMA) small-M GEMM, bf16 ---------------------------------------------------
-enum { TC_MODE_PARTIAL = 0, TC_MODE_DIRECT = 1, TC_MODE_SWIGLU = 2, TC_MODE_LOGITS = 3 };
+enum { TC_MODE_PARTIAL = 0, TC_MODE_SWIGLU = 1, TC_MODE_LOGITS = 2 };
 // Up to three bf16 matrices that share x and K; their outputs sit side by side in one row of width ld.
 struct TcGroup {
   const void* x; int m, k;   // bf16 weights: bf16 rows (hi plane); fp8 weights: XF_E5M2X3 rows (first plane); a8: rows of e4m3 codes
   const void* x_lo;          // bf16 weights, nullable: the rows' low-order bf16 plane (x = hi + lo); fp8 weights: second plane
   const void* x_3;           // fp8 weights: third plane
   const void* w[3]; int n[3]; int n_mats;
-  const float* scale[3]; const float* bias[3];
+  const float* scale[3];
   int fp8;   // weights are e4m3 bytes (scale[] holds the per-output-channel factors)
   int a8;    // with fp8: the rows are e4m3 codes, one factor per row (W8A8); PARTIAL and SWIGLU only
 };
 // What the GEMM leaves behind.
 //   PARTIAL: part[split][m][ld] = split-K partial sums (*splits_out of them) for the caller's reduce kernel
-//   DIRECT : y[m][ld] = (x w^T) * rstd[row] * scale + bias (+ y when accumulate)
 //   SWIGLU : act[m][n0] = silu(x w0^T * rstd * s0) * (x w1^T * rstd * s1)   (w[0] = gate, w[1] = up)
-//   LOGITS : y (when write_logits) as DIRECT, and stats[tile * 4 + quarter][m] = (max, sum exp(l - max), argmax id)
+//   LOGITS : y[m][ld] = (x w^T) * rstd[row] * scale (when write_logits), and stats[tile * 4 + quarter][m] = (max, sum exp(l - max), argmax id)
 //            over the 32 vocabulary ids a warp holds, mask_id excluded
 // rstd[row] = rsqrt(sum_t ssq_in[row][t] / hidden + eps) when ssq_in is set (RMSNorm folded into the consumer), else 1.
 struct TcOut {
   int mode;
   float* part; size_t part_bytes; int* splits_out;
-  float* y; int ld; int accumulate;
+  float* y; int ld;
   void* act; size_t act_lo_off; int act_fmt;   // SWIGLU output, stored as XF_* (lo plane act_lo_off elements on)
   const float* ssq_in; int nt_in; int hidden; float eps;
   void* stats; int mask_id; int write_logits;

@@ -51,7 +51,7 @@ extern "C" int fdvlm_op_linear_static(const void* x, const void* w, const float*
   // The status words are cleared on the stream by the launcher (an earlier call may have left a report there); the
   // partial sums need no clearing: every (tile, split) slot that is summed is written by this call.
   LinearArgs a;
-  a.x = x; a.w = w; a.scale = scale; a.bias = bias; a.y = y; a.m = m; a.n = n; a.k = k; a.ldy = n; a.accumulate = 0;
+  a.x = x; a.w = w; a.scale = scale; a.bias = bias; a.y = y; a.m = m; a.n = n; a.k = k;
   a.dtype = (int)dtype; a.workspace = base; a.workspace_bytes = sizeof(g_static_scratch);
   if (launch_linear(a, (cudaStream_t)cuda_stream, &e) < 0)
     return fail(nullptr, FDVLM_ERR_CUDA, "op_linear_static: launch: %s", cudaGetErrorString(e));
