@@ -311,7 +311,7 @@ int fdvlm_profile_read_chain(fdvlm_t *h, fdvlm_kernel_record *records, int cap, 
 
 /* Test hook for the give-up path of the kernels' bounded waits.  While `on` is non-zero, every tensor-core GEMM of
  * this handle reads the flag when it starts and each of its roles (TMA producer, MMA issuer, converters, epilogue)
- * leaves at once by the path a timed-out wait takes -- nothing issued, nothing in flight, tensor memory freed -- and
+ * waits for nothing, as after a timed-out wait -- nothing issued, nothing in flight, tensor memory freed -- and
  * records its role in the status word, so the next synchronous call returns FDVLM_ERR_TIMEOUT.  Outputs of such
  * calls are undefined; committed cache positions are not written.  Takes effect in stream order. */
 int fdvlm_debug_poison(fdvlm_t *h, int on);
@@ -341,7 +341,7 @@ int fdvlm_util_stream_read(const void *device_buf, size_t bytes, void *device_si
  * undefined), else FDVLM_OK.  workspace = NULL asks about the built-in scratch of fdvlm_op_linear_static on the
  * current device.
  * dtype = FDVLM_W8A8_FP8E4M3: w and scale as for fp8 weights; the bf16 rows of x are first stored as f16 (saturating)
- * and each row is then quantised to e4m3 with its own scale max|row| / 448 inside the GEMM kernel, which multiplies
+ * and each row is then quantised to e4m3 with its own scale max|row| / 448 in front of the GEMM kernel, which multiplies
  * e4m3 by e4m3; FDVLM_ERR_UNSUPPORTED where the tensor-core kernel does not take the shape (k not a multiple of 16). */
 int fdvlm_op_linear(const void *x, const void *w, const float *scale, const float *bias, float *y,
                     int m, int n, int k, fdvlm_dtype dtype, void *workspace, void *cuda_stream);

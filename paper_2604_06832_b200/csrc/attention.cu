@@ -326,7 +326,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
 // Merge of the key chunks: out[i][head] = sum_c w_c O_c / sum_c w_c l_c, w_c = 2^(m_c - max_c m_c).  WPP warps per
 // (row, head): warp w takes the chunks w, w + WPP, ..., CB of them in flight at once; with WPP = 4 warp 0 adds up the four.
 // Four where that is at most four CTAs per SM (one warp per pair took 5.4 us a layer for the 33 chunks of 8224 keys and 32
-// rows of the 3B shape, four take 3.6), one beyond (64 rows: 3.4 against 4.1).  Lane j owns D / 32 consecutive output
+// rows of the 3B shape, four about 3.5), one beyond (64 rows: 3.4 against 4.1).  Lane j owns D / 32 consecutive output
 // features.  The result is stored as `fmt` (XF_*).
 template <int D, int WPP>
 __global__ void __launch_bounds__(128) attn_combine_kernel(const float* __restrict__ part_o, const float2* __restrict__ part_ml,

@@ -5,11 +5,12 @@
 // the second product from there.  One softmax thread owns a row, so the online softmax needs no shuffles; O is rescaled
 // only when a row's maximum has grown by more than 2^8, until then P is taken relative to the old reference (values up to
 // 256, sums in fp32).  Each row tile has two score buffers, so the scores of the next keys are there when a softmax thread
-// is done with its keys (with one buffer of 128 keys the threads waited for P V and Q K^T in turn: 97 us for 4096 rows of
-// the 3B shape, 96 us by the same clock now that the issue of MMAs does not bound it).  Bound by the exponentials, 16 per clock and SM.
-// V stays as it lies in the cache ([key][dim], an MN-major operand).  Hundreds of CTAs exist at any prompt length, so keys
-// are not split and the normalised result is written directly as the O projection's input; CTAs with the most keys come
-// first. 
+// is done with its keys (one buffer of 128 keys: 97 us instead of 96 for 4096 rows of the 3B shape).  Bound by the
+// exponentials, 16 per clock and SM.
+// V stays as it lies in the cache ([key][dim], an MN-major operand).  Keys are not split and the normalised result is written directly as
+// the O projection's input: 1024 rows of the 3B shape are 128 CTAs, one per SM (CTAs with the most keys come first).  A short turn
+// is few CTAs (200 rows: 32), each of which walks all keys at 0.8 us per 64, so behind a long cache such turns take the decode
+// path (takes_prompt_path).
 // Every mbarrier wait is bounded as in gemm_tc.cu.
 #include "attn_plan.cuh"
 #include "kernels.h"
