@@ -27,6 +27,32 @@ __device__ __forceinline__ float4 ldcg_f4(const float* p, bool vec) {
 }
 static inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
+// What follows the sums a, b of features f0, f1 of row r (not LOGITS)
+template <int MODE>
+__device__ __forceinline__ void fl_finish(const F32Linear& p, int r, int mi, int f0, int f1, float a, float b) {
+  if (MODE == FL_QKV) {
+    const int half = p.d >> 1, j = f0 % p.d, head = f0 / p.d;
+    const int pos0 = p.len_ptr ? *p.len_ptr : p.pos0;
+    if (p.bias[mi]) { a += p.bias[mi][f0]; b += p.bias[mi][f1]; }
+    if (mi < 2) {
+      const float2 c = reinterpret_cast<const float2*>(p.cs)[(size_t)r * half + j];
+      const float a0 = a, b0 = b;
+      a = a0 * c.x - b0 * c.y;
+      b = b0 * c.x + a0 * c.y;
+    }
+    float* dst = mi == 0 ? p.out + ((size_t)r * p.hq + head) * p.d + j
+                         : (mi == 1 ? p.kc : p.vc) + ((size_t)head * p.max_seq + pos0 + r) * p.d + j;
+    dst[0] = a;
+    dst[half] = b;
+  } else if (MODE == FL_SWIGLU) {
+    if (f0 < p.n[0]) p.out[(size_t)r * p.n[0] + f0] = a / (1.f + expf(-a)) * b;
+  } else {
+    float* o = p.out + (size_t)r * p.n[0];
+    if (f0 < p.n[0]) o[f0] += a;
+    if (f1 < p.n[0]) o[f1] += b;
+  }
+}
+
 // One CTA: RM rows x 8 pairs of output features.  The pair is what the epilogue combines: (j, j + d/2) of a head for the
 // rotary embedding, (gate, up) for SwiGLU, else features f and f + 8.  GV: the gains are 16-byte aligned.  A warp takes every eighth 16-wide slice of k; lane =
 // (feature 0..7, quarter of the slice).
@@ -169,55 +195,196 @@ __global__ void __launch_bounds__(FL_WARPS * 32) linear_f32_kernel(const F32Line
     return;
   }
   if (r >= p.m) return;
-  if (MODE == FL_QKV) {
-    const int half = p.d >> 1, j = f0 % p.d, head = f0 / p.d;
-    const int pos0 = p.len_ptr ? *p.len_ptr : p.pos0;
-    if (p.bias[mi]) { a += p.bias[mi][f0]; b += p.bias[mi][f1]; }
-    if (mi < 2) {
-      const float2 c = reinterpret_cast<const float2*>(p.cs)[(size_t)r * half + j];
-      const float a0 = a, b0 = b;
-      a = a0 * c.x - b0 * c.y;
-      b = b0 * c.x + a0 * c.y;
+  fl_finish<MODE>(p, r, mi, f0, f1, a, b);
+}
+
+// The same for 32 rows x 16 pairs, two pairs per lane, where those CTAs still fill the SMs: with 32 rows the reads of a row's values from shared
+// memory, one for every pair of a lane, bound the kernel above.  Step of 3 layers of the 3B shape in fp32, empty cache, one pair : two per lane:
+// 32 rows 1453 : 1234 us, 33 rows 2338 : 1967, 64 rows 2500 : 2076; 1024 wide, 4 layers, 64 rows 839 : 747.  (A kernel of its own: as one
+// source for both the kernels of 8 rows compiled to other register counts, and 1 row of the 3B shape went from 541 to 565 us.)
+constexpr int FLW_ROWS = 32, FLW_PAIRS = 16;
+template <int MODE, bool GV>
+__global__ void __launch_bounds__(FL_WARPS * 32) linear_f32_wide_kernel(const F32Linear p) {
+  extern __shared__ float4 fl_smem[];
+  float* xs = reinterpret_cast<float*>(fl_smem);                 // [rows][kc]
+  __shared__ float red[FL_WARPS][FLW_ROWS][2 * FLW_PAIRS];
+  __shared__ float rstd[FLW_ROWS];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, fl = lane >> 2, kq = lane & 3;
+  const int r0 = blockIdx.y * FLW_ROWS, K = p.k;
+  const int kc = K < FL_KC ? K : FL_KC;
+  pdl_trigger();
+  int mi = 0, f0, f1;
+  auto pair_of = [&](int i) {
+    if (MODE == FL_QKV) {
+      const int half = p.d >> 1, tph = half / FLW_PAIRS, head = blockIdx.x / tph;
+      mi = head < p.hq ? 0 : (head < p.hq + p.hkv ? 1 : 2);
+      const int hl = head - (mi == 0 ? 0 : (mi == 1 ? p.hq : p.hq + p.hkv));
+      f0 = hl * p.d + (blockIdx.x % tph) * FLW_PAIRS + i;
+      f1 = f0 + half;
+    } else if (MODE == FL_SWIGLU) {
+      f0 = f1 = blockIdx.x * FLW_PAIRS + i;
+    } else {
+      f0 = blockIdx.x * (2 * FLW_PAIRS) + i;
+      f1 = f0 + FLW_PAIRS;
     }
-    float* dst = mi == 0 ? p.out + ((size_t)r * p.hq + head) * p.d + j
-                         : (mi == 1 ? p.kc : p.vc) + ((size_t)head * p.max_seq + pos0 + r) * p.d + j;
-    dst[0] = a;
-    dst[half] = b;
-  } else if (MODE == FL_SWIGLU) {
-    if (f0 < p.n[0]) p.out[(size_t)r * p.n[0] + f0] = a / (1.f + expf(-a)) * b;
-  } else {
-    float* o = p.out + (size_t)r * p.n[0];
-    if (f0 < p.n[0]) o[f0] += a;
-    if (f1 < p.n[0]) o[f1] += b;
+  };
+  const float* wp[4];              // first and second feature of pairs fl and fl + 8
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    pair_of(fl + 8 * q);
+    wp[2 * q] = p.w[mi] + (size_t)min(f0, p.n[mi] - 1) * K;
+    wp[2 * q + 1] = (MODE == FL_SWIGLU ? p.w[1] : p.w[mi]) + (size_t)min(f1, p.n[mi] - 1) * K;
+  }
+  pdl_wait();
+  float acc[FLW_ROWS][4], ssq[FLW_ROWS / FL_WARPS];
+#pragma unroll
+  for (int r = 0; r < FLW_ROWS; ++r)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) acc[r][c] = 0.f;
+#pragma unroll
+  for (int i = 0; i < FLW_ROWS / FL_WARPS; ++i) ssq[i] = 0.f;
+  for (int c0 = 0; c0 < K; c0 += FL_KC) {
+    const int cn = min(FL_KC, K - c0);
+    if (c0) __syncthreads();
+#pragma unroll
+    for (int i = 0; i < FLW_ROWS / FL_WARPS; ++i) {
+      const int rl = warp + i * FL_WARPS, r = r0 + rl;
+      const float* src = p.x + (size_t)r * K + c0;
+      float4 v[FL_KC / 128];
+#pragma unroll
+      for (int j = 0; j < FL_KC / 128; ++j) {
+        const int k = lane * 4 + j * 128;
+        v[j] = (r < p.m && k < cn) ? __ldcg(reinterpret_cast<const float4*>(src + k)) : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+#pragma unroll
+      for (int j = 0; j < FL_KC / 128; ++j) {
+        const int k = lane * 4 + j * 128;
+        if (k >= cn) break;
+        ssq[i] = dot4(v[j], v[j], ssq[i]);
+        if (p.gain) {
+          const float4 g = ldg_f4(p.gain + c0 + k, GV);
+          v[j] = make_float4(v[j].x * g.x, v[j].y * g.y, v[j].z * g.z, v[j].w * g.w);
+        }
+        *reinterpret_cast<float4*>(xs + rl * kc + k) = v[j];
+      }
+    }
+    __syncthreads();
+#pragma unroll 2
+    for (int k = c0 + warp * 16 + kq * 4; k < c0 + cn; k += FL_STEP) {
+      float4 w[4];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) w[c] = __ldg(reinterpret_cast<const float4*>(wp[c] + k));
+      const float* xp = xs + (k - c0);
+#pragma unroll
+      for (int r = 0; r < FLW_ROWS; ++r) {
+        const float4 xv = *reinterpret_cast<const float4*>(xp + r * kc);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) acc[r][c] = dot4(w[c], xv, acc[r][c]);
+      }
+    }
+  }
+  if (p.gain) {
+#pragma unroll
+    for (int i = 0; i < FLW_ROWS / FL_WARPS; ++i) {
+      const float t = warp_sum(ssq[i]);
+      if (lane == 0) rstd[warp + i * FL_WARPS] = rsqrtf(t * p.inv_h + p.eps);
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < FLW_ROWS; ++r)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      float t = acc[r][c];
+      t += __shfl_xor_sync(0xffffffffu, t, 1);
+      t += __shfl_xor_sync(0xffffffffu, t, 2);
+      if (kq == 0) red[warp][r][(c & 1) * FLW_PAIRS + (c >> 1) * 8 + fl] = t;
+    }
+  __syncthreads();
+  // thread: row t / 8, pairs t % 8 and 8 further on
+  const int rl = threadIdx.x >> 3, i = threadIdx.x & 7, r = r0 + rl;
+  [[maybe_unused]] float lv[4], mx = -INFINITY;       // LOGITS: this thread's logits that count, their maximum (a NaN is none) and its id
+  [[maybe_unused]] int ix = 0x7fffffff;
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    pair_of(i + 8 * q);
+    float v[2] = {0.f, 0.f};
+#pragma unroll
+    for (int w = 0; w < FL_WARPS; ++w)
+#pragma unroll
+      for (int c = 0; c < 2; ++c) v[c] += red[w][rl][c * FLW_PAIRS + 8 * q + i];
+    if (p.gain) { v[0] *= rstd[rl]; v[1] *= rstd[rl]; }
+    if constexpr (MODE != FL_LOGITS) {
+      if (r < p.m) fl_finish<MODE>(p, r, mi, f0, f1, v[0], v[1]);
+    } else {
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        const int f = c ? f1 : f0;
+        const bool in = f < p.n[0];
+        if (p.out && in && r < p.m) p.out[(size_t)r * p.n[0] + f] = v[c];
+        const float l = (in && f != p.mask_id) ? v[c] : -INFINITY;
+        lv[2 * q + c] = l;
+        if (l > mx || (l == mx && f < ix)) { mx = l; ix = f; }      // (a tie goes to the lower id)
+      }
+    }
+  }
+  if constexpr (MODE == FL_LOGITS) {
+    if (!p.stats) return;
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) {
+      const float omx = __shfl_xor_sync(0xffffffffu, mx, o);
+      const int oix = __shfl_xor_sync(0xffffffffu, ix, o);
+      if (omx > mx || (omx == mx && oix < ix)) { mx = omx; ix = oix; }
+    }
+    float e = 0.f;
+    if (mx > -INFINITY) {
+#pragma unroll
+      for (int c = 0; c < 4; ++c) e += __expf(lv[c] - mx);
+    }
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
+    if (i == 0 && r < p.m) p.stats[(size_t)blockIdx.x * p.m + r] = make_float4(mx, e, __int_as_float(ix), 0.f);
   }
 }
 
-template <int RM, int MODE, bool GV>
-static cudaError_t fl_launch_v(const F32Linear& p, int tiles, cudaStream_t st) {
-  static bool attr_set[MAX_DEVICES] = {};
-  cudaError_t e = ensure_dynamic_smem(linear_f32_kernel<RM, MODE, GV>, RM * FL_KC * 4, attr_set);
+template <int RM>
+static cudaError_t fl_launch(void (*kern)(F32Linear), bool* attr_set, const F32Linear& p, int tiles, cudaStream_t st) {
+  cudaError_t e = ensure_dynamic_smem(kern, RM * FL_KC * 4, attr_set);
   if (e != cudaSuccess) return e;
   const size_t smem = (size_t)RM * (p.k < FL_KC ? p.k : FL_KC) * 4;
-  return launch_pdl(linear_f32_kernel<RM, MODE, GV>, dim3(tiles, ceil_div(p.m, RM)), dim3(FL_WARPS * 32), smem, st, p);
+  return launch_pdl(kern, dim3(tiles, ceil_div(p.m, RM)), dim3(FL_WARPS * 32), smem, st, p);
 }
 template <int RM, int MODE>
 static cudaError_t fl_launch_t(const F32Linear& p, int tiles, cudaStream_t st) {
-  return aligned16(p.gain) ? fl_launch_v<RM, MODE, true>(p, tiles, st) : fl_launch_v<RM, MODE, false>(p, tiles, st);
+  static bool attr_set[2][MAX_DEVICES] = {};
+  return aligned16(p.gain) ? fl_launch<RM>(linear_f32_kernel<RM, MODE, true>, attr_set[0], p, tiles, st)
+                           : fl_launch<RM>(linear_f32_kernel<RM, MODE, false>, attr_set[1], p, tiles, st);
+}
+template <int MODE>
+static cudaError_t fl_launch_wide(const F32Linear& p, int tiles, cudaStream_t st) {
+  static bool attr_set[2][MAX_DEVICES] = {};
+  return aligned16(p.gain) ? fl_launch<FLW_ROWS>(linear_f32_wide_kernel<MODE, true>, attr_set[0], p, tiles, st)
+                           : fl_launch<FLW_ROWS>(linear_f32_wide_kernel<MODE, false>, attr_set[1], p, tiles, st);
+}
+// whether m rows of `features` output features take the wide kernel
+static bool fl_wide(int m, int features) {
+  return m > 16 && ceil_div(features, 2 * FLW_PAIRS) * ceil_div(m, FLW_ROWS) >= sm_count();
 }
 // rows per CTA: all of them up to 32, so that a weight is read once (64 rows: twice)
 template <int MODE>
-static cudaError_t fl_launch_m(const F32Linear& p, int tiles, cudaStream_t st) {
+static cudaError_t fl_launch_m(const F32Linear& p, int features, cudaStream_t st) {
+  if (fl_wide(p.m, features)) return fl_launch_wide<MODE>(p, ceil_div(features, 2 * FLW_PAIRS), st);
+  const int tiles = ceil_div(features, 16);
   if (p.m <= 8) return fl_launch_t<8, MODE>(p, tiles, st);
   if (p.m <= 16) return fl_launch_t<16, MODE>(p, tiles, st);
   return fl_launch_t<32, MODE>(p, tiles, st);
 }
-int f32_logit_tiles(int vocab) { return ceil_div(vocab, 16); }
+int f32_logit_tiles(int vocab, int m) { return ceil_div(vocab, fl_wide(m, vocab) ? 2 * FLW_PAIRS : 16); }
 cudaError_t launch_linear_f32(const F32Linear& p, cudaStream_t st) {
   switch (p.mode) {
-    case FL_QKV: return fl_launch_m<FL_QKV>(p, (p.hq + 2 * p.hkv) * (p.d / 16), st);
-    case FL_SWIGLU: return fl_launch_m<FL_SWIGLU>(p, ceil_div(p.n[0], 8), st);
-    case FL_RESID: return fl_launch_m<FL_RESID>(p, ceil_div(p.n[0], 16), st);
-    default: return fl_launch_m<FL_LOGITS>(p, f32_logit_tiles(p.n[0]), st);
+    case FL_QKV: return fl_launch_m<FL_QKV>(p, (p.hq + 2 * p.hkv) * p.d, st);
+    case FL_SWIGLU: return fl_launch_m<FL_SWIGLU>(p, 2 * p.n[0], st);
+    case FL_RESID: return fl_launch_m<FL_RESID>(p, p.n[0], st);
+    default: return fl_launch_m<FL_LOGITS>(p, p.n[0], st);
   }
 }
 

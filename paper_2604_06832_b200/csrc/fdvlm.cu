@@ -162,7 +162,7 @@ extern "C" int fdvlm_create(const fdvlm_config* cfg, const fdvlm_weights* w, voi
       {(void**)&h->ao, (size_t)R * NQ * h->act_sz * planes},
       {(void**)&h->q, (size_t)R * NQ * h->act_sz},
       {(void**)&h->act, (size_t)R * I * h->act_sz * planes},
-      {(void**)&h->stats, (size_t)(h->use_tc ? (cfg->vocab + 127) / 128 * 4 : f32_logit_tiles(cfg->vocab)) * R * 16},
+      {(void**)&h->stats, (size_t)(h->use_tc ? (cfg->vocab + 127) / 128 * 4 : (cfg->vocab + 15) / 16) * R * 16},
       {(void**)&h->ws, ws ? ws : 16},
       {(void**)&h->logits, (size_t)R * cfg->vocab * 4},
   };

@@ -286,7 +286,7 @@ static int forward_rows_f32(fdvlm_t* h, int n, int mode, int logits_rows, int wa
     g.stats = all ? (float4*)h->stats : nullptr; g.mask_id = c.mask_id;
     if (!run(g)) return fail(h, FDVLM_ERR_CUDA, "lm head launch: %s", cudaGetErrorString(e));
     if (all) {
-      launch_stats_merge(h->stats, f32_logit_tiles(c.vocab), n, h->conf, h->pred, h->st);
+      launch_stats_merge(h->stats, f32_logit_tiles(c.vocab, n), n, h->conf, h->pred, h->st);
       h->launches++;
     }
   }

@@ -67,7 +67,7 @@ void launch_init_block(int32_t* tokens, uint8_t* masked, int32_t* info, const in
 //   QKV   : w = q, k, v; bias, rotary (cs); q rows into out, K / V rows into the cache planes kc, vc at pos0 (*len_ptr)
 //   RESID : out [m, n0] += x w^T
 //   SWIGLU: w = gate, up; out [m, n0] = silu(gate) * up
-//   LOGITS: out [m, n0] (nullable); stats[tile][m] (nullable): as TcOut's, one entry per 16 vocabulary ids
+//   LOGITS: out [m, n0] (nullable); stats[tile][m] (nullable): as TcOut's, f32_logit_tiles entries
 enum { FL_QKV = 0, FL_RESID = 1, FL_SWIGLU = 2, FL_LOGITS = 3 };
 struct F32Linear {
   int mode, m, k;
@@ -78,7 +78,7 @@ struct F32Linear {
   const float* cs; const int* len_ptr; int pos0, hq, hkv, d, max_seq;
   float4* stats; int mask_id;
 };
-int f32_logit_tiles(int vocab);
+int f32_logit_tiles(int vocab, int m);      // entries of `stats` for each of m rows, at most ceil(vocab / 16)
 cudaError_t launch_linear_f32(const F32Linear& p, cudaStream_t st);
 
 // ---- tensor-core (tcgen05 + TMA) small-M GEMM, bf16 ---------------------------------------------------

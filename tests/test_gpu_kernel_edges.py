@@ -140,6 +140,19 @@ def test_exact_f32_row_tiles_and_ragged_widths(n):
     check(WIDE_F32, [(0, n)])
 
 
+@pytest.mark.parametrize("n", [33, 64])
+def test_exact_f32_wide_layers(n):
+    """Widths from which 32 rows take two pairs of features a lane, the last tile of each ragged: every projection, and the statistics."""
+    shape = I.TINY.with_(n_layers=1, hidden=2376, n_q_heads=32, n_kv_heads=4, intermediate=1192, vocab=2399, mask_id=1200)
+    oracle, handle, _ = make_pair(shape, 5, max_seq=128, qkv_bias=True)
+    emb, toks = I.make_prefix(shape, 20, 20, 3)
+    oracle.prefill(I.as_numpy_storage(emb), toks.numpy())
+    handle.prefill(*upload_prefix(emb, toks))
+    stats = replay_decode(oracle, handle, shape, n, orc.TOPK, 0.0, n)
+    assert stats["steps"] == 1 and stats["rows_sure"] > 0
+    handle.close()
+
+
 def test_exact_f32_attention_over_many_keys():
     check(I.TINY.with_(n_layers=1), [(0, 2100), (0, 9)], max_seq=2200)
 
