@@ -383,7 +383,13 @@ static int forward_rows_tc(fdvlm_t* h, int n, int mode, int logits_rows, int wan
     o.x_scale = xs; o.amax_out = a8 ? h->amax_act : nullptr;
     TcGroup gu = group(h->a, h->a_lo, 0, n, H, 2, lw.w_gate, I, lw.w_up, I, nullptr, 0);
     gu.scale[0] = lw.s_gate; gu.scale[1] = lw.s_up;
-    if (!gemm(quantised(gu, h->amax_a, nt), o))
+    gu = quantised(gu, h->amax_a, nt);
+    prof_begin(h, 0);
+    e = gemm_gu_launch(gu, o, lw.w_down, H, I, h->st);
+    if (e == cudaErrorNotSupported) e = tc_group_launch(gu, o, h->st);
+    prof_end(h);
+    h->launches++;
+    if (e != cudaSuccess)
       return fail(h, FDVLM_ERR_CUDA, "gate/up projection launch: %s", cudaGetErrorString(e));
     o = out(TC_MODE_PARTIAL, FDVLM_K_GEMM_DOWN);
     o.ld = H; o.splits_out = &S;

@@ -504,6 +504,18 @@ bool make_tmap(CUtensorMap* tm, const void* ptr, int rows, int cols, int box_row
   return true;
 }
 
+// The planes of a GEMM input, equally far apart, as one 3-D tensor [planes, rows, cols]: one box fetches a k-block of all of them.
+bool make_tmap_planes(CUtensorMap* tm, const void* ptr, int rows, int cols, int planes, size_t plane_bytes, int box_rows, bool bytes) {
+  EncodeTiledFn fn = encode_fn();
+  if (!fn) return false;
+  cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)rows, (cuuint64_t)planes};
+  cuuint64_t strides[2] = {(cuuint64_t)cols * (bytes ? 1 : 2), (cuuint64_t)plane_bytes};
+  cuuint32_t box[3] = {(cuuint32_t)(bytes ? 2 * TC_BK : TC_BK), (cuuint32_t)box_rows, (cuuint32_t)planes};
+  cuuint32_t estr[3] = {1, 1, 1};
+  return fn(tm, bytes ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), dims, strides, box, estr,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 // SM count of the current device (cached per device: one process may drive several GPUs)
 int sm_count() {
   static int n[MAX_DEVICES] = {};

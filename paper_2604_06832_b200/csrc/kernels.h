@@ -120,9 +120,13 @@ struct TcOut {
 // TM_E4M3_128: bytes, box of 128 columns, 128-byte swizzle.  False when the driver entry point is missing or the encode fails.
 enum { TM_BF16 = 0, TM_E4M3 = 1, TM_F16 = 2, TM_E4M3_128 = 3 };
 bool make_tmap(CUtensorMap* tm, const void* ptr, int rows, int cols, int box_rows, int kind = TM_BF16);
+bool make_tmap_planes(CUtensorMap* tm, const void* ptr, int rows, int cols, int planes, size_t plane_bytes, int box_rows, bool bytes);
 bool tc_linear_supported(int m, int n, int k, int dtype);
 // Split-K workspace of a group with m rows, output width ld, `tiles` 128-row weight tiles and depth k.
 size_t tc_workspace_bytes(int m, int ld, int tiles, int k);
+// The decode path's gate / up projection (SWIGLU): one equal share of the features per SM (gemm_gu.cu).  next (nullable): the weights
+// [next_n, next_k], of the same type, that the following launch streams.  cudaErrorNotSupported: left to tc_group_launch.
+cudaError_t gemm_gu_launch(const TcGroup& g, const TcOut& o, const void* next, int next_n, int next_k, cudaStream_t st);
 cudaError_t tc_group_launch(const TcGroup& g, const TcOut& o, cudaStream_t st);
 
 // SM count of the current device (cached per device: one process may drive several GPUs).

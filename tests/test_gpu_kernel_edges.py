@@ -195,3 +195,42 @@ def test_fp8_projection_of_rows_with_small_values():
     # f16 of a bf16 value and its planes are exact from 2^-13 up and off by at most 2^-24 below; fp32 sums of k products
     bound = (2.0 ** -24 + 2.0 ** -25) * np.abs(w).sum(1)[None] + 2.0 ** -20 * (np.abs(xv) @ np.abs(w).T)
     assert (np.abs(y - xv @ w.T) <= bound).all()
+
+
+# ---- gate / up of a decode step, one share of the features per SM: row counts at which the planes change, ragged last share and depth ----
+@pytest.mark.parametrize("base,inter,n", [(BF16, 2384, 17), (BF16, 2384, 33), (BF16, 2384, 64), (BF16, 1216, 31), (BF16, 19008, 24),
+                                          (FP8, 2416, 33), (FP8, 2416, 40), (FP8, 2416, 41), (FP8, 2416, 49), (FP8, 2416, 64)])
+def test_gate_up_shares(base, inter, n):
+    """(19008 features are more than 128 per SM and stay with the tiles; hidden: a last tile of 80 columns in the finalisation.)"""
+    shape = base.with_(n_layers=1, hidden=1104, intermediate=inter)
+    oracle, handle, _ = make_pair(shape, 5, max_seq=128, qkv_bias=True)
+    emb, toks = I.make_prefix(shape, 20, 20, 3)
+    oracle.prefill(I.as_numpy_storage(emb), toks.numpy())
+    handle.prefill(*upload_prefix(emb, toks))
+    assert replay_decode(oracle, handle, shape, n, orc.TOPK, 0.0, n)["steps"] == 1
+    handle.close()
+
+
+@pytest.mark.parametrize("shape,n", [(BF16, 33), (FP8, 64)], ids=["bf16", "fp8"])
+def test_give_up_path_of_the_gate_up_shares(shape, n):
+    """With the poison flag set every role leaves as after a wait that timed out; afterwards the step is what it was before, bit for bit."""
+    from paper_2604_06832_b200 import binding as B
+    h = B.Handle(shape, B.weights_to_device(I.make_weights(shape, 3)), max_seq=256, stream=torch.cuda.Stream())
+    toks = I.random_tokens(shape, 40, 4).cuda()
+
+    def step():
+        logits = torch.empty(n, shape.vocab, device="cuda")
+        h.reset()
+        h.prefill(None, toks)
+        h.block_begin(n)
+        h.block_step(B.RULE_TOPK, 0.0, n, logits=logits)
+        return logits
+
+    before = step()
+    h.debug_poison(True)
+    with pytest.raises(B.FdvlmError) as e:
+        step()
+    assert e.value.code == B.ERR_TIMEOUT
+    h.debug_poison(False)
+    assert torch.equal(before, step())
+    h.close()
