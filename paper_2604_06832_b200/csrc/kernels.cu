@@ -371,99 +371,124 @@ void launch_quantize_bf16_rows(const void* in, int m, int k, void* codes, float*
   quantize_bf16_rows_kernel<<<m, 256, 0, st>>>((const bf16*)in, k, (uint8_t*)codes, scale);
 }
 
-// Sum of S split-K partials p[i * stride].  These kernels are a handful of dependent L2 round trips long, so every
-// load that can be issued at once is: N loads in flight per call, added in index order (deterministic).
-template <int N> struct Partials { float r[N]; };
-template <int N>
-__device__ __forceinline__ void issue_partials(Partials<N>& v, const float* __restrict__ p, size_t stride, int i0, int S) {
-#pragma unroll
-  for (int j = 0; j < N; ++j) v.r[j] = (i0 + j < S) ? __ldcg(p + (size_t)(i0 + j) * stride) : 0.f;
-}
-template <int N>
-__device__ __forceinline__ float add_partials(const Partials<N>& v, float s) {
-#pragma unroll
-  for (int j = 0; j < N; ++j) s += v.r[j];
-  return s;
-}
-// the partials from index i0 on, added to s
-__device__ __forceinline__ float sum_partials_from(const float* __restrict__ p, size_t stride, int i0, int S, float s) {
-  for (; i0 < S; i0 += 16) {
-    Partials<16> v;
-    issue_partials(v, p, stride, i0, S);
-    s = add_partials(v, s);
+// Sums of S split-K partials, V consecutive columns a lane.  These kernels are a handful of dependent L2 round trips long, so every
+// load that can be issued at once is: NP partials in flight, added in index order (deterministic).
+template <int V> struct Cols { float v[V]; };
+template <int V>
+__device__ __forceinline__ Cols<V> load_cols(const float* __restrict__ p) {
+  Cols<V> c;
+  if (V == 4) {
+    const float4 x = __ldcg(reinterpret_cast<const float4*>(p));
+    c.v[0] = x.x; c.v[1] = x.y; c.v[V - 2] = x.z; c.v[V - 1] = x.w;
+  } else if (V == 2) {
+    const float2 x = __ldcg(reinterpret_cast<const float2*>(p));
+    c.v[0] = x.x; c.v[V - 1] = x.y;
+  } else {
+    c.v[0] = __ldcg(p);
   }
-  return s;
+  return c;
+}
+template <int V, int NP> struct Partials { Cols<V> c[NP]; };
+template <int V, int NP>
+__device__ __forceinline__ void issue_partials(Partials<V, NP>& x, const float* __restrict__ p, size_t stride, int i0, int S) {
+#pragma unroll
+  for (int j = 0; j < NP; ++j) {
+    if (i0 + j < S) x.c[j] = load_cols<V>(p + (size_t)(i0 + j) * stride);
+    else
+#pragma unroll
+      for (int k = 0; k < V; ++k) x.c[j].v[k] = 0.f;
+  }
+}
+template <int V, int NP>
+__device__ __forceinline__ void add_partials(const Partials<V, NP>& x, float* s) {
+#pragma unroll
+  for (int j = 0; j < NP; ++j)
+#pragma unroll
+    for (int k = 0; k < V; ++k) s[k] += x.c[j].v[k];
+}
+// the partials from index i0 on
+template <int V>
+__device__ __forceinline__ void sum_partials_from(const float* __restrict__ p, size_t stride, int i0, int S, float* s) {
+  for (; i0 < S; i0 += 8) {
+    Partials<V, 8> x;
+    issue_partials(x, p, stride, i0, S);
+    add_partials(x, s);
+  }
 }
 
 // QKV finalisation: sum the split-K partials, apply the folded norm factor and the bias, rotate q and k
-// (rotate-half pairs j, j + d/2), write q to its buffer and k, v into the layer's cache planes.
-// grid (hq + 2 hkv heads, m rows), d/2 threads: thread j owns the pair (j, j + d/2) of one head.
-template <typename T>
-__global__ void fin_qkv_kernel(const float* __restrict__ part, int S, int m, const float2* __restrict__ cs,
-                               const float* __restrict__ ssq, int nt, float inv_h, float eps,
-                               const float* __restrict__ bq, const float* __restrict__ bk, const float* __restrict__ bv,
-                               const float* __restrict__ sq, const float* __restrict__ sk, const float* __restrict__ sv,
-                               T* __restrict__ q, T* __restrict__ kc, T* __restrict__ vc, int pos0, int hq, int hkv,
-                               int d, int max_seq, const int* __restrict__ len_ptr, const float* __restrict__ x_scale,
-                               float* __restrict__ amax_zero, KStamp* stamp) {
+// (rotate-half pairs j, j + D/2), write q to its buffer and k, v into the layer's cache planes.  One warp per (row, head), D / 64
+// pairs a lane, four warps a CTA: a grid that is resident at once beside the GEMM CTAs which already hold their shared memory
+// (with one CTA of two warps per (row, head) it took two waves: 3.7 us a layer of the 3B shape and 32 rows).
+template <typename T, int D>
+__global__ void __launch_bounds__(128) fin_qkv_kernel(const float* __restrict__ part, int S, int m, const float2* __restrict__ cs,
+                                                      const float* __restrict__ ssq, int nt, float inv_h, float eps,
+                                                      const float* __restrict__ bq, const float* __restrict__ bk, const float* __restrict__ bv,
+                                                      const float* __restrict__ sq, const float* __restrict__ sk, const float* __restrict__ sv,
+                                                      T* __restrict__ q, T* __restrict__ kc, T* __restrict__ vc, int pos0, int hq, int hkv,
+                                                      int max_seq, const int* __restrict__ len_ptr, const float* __restrict__ x_scale,
+                                                      float* __restrict__ amax_zero, KStamp* stamp) {
+  constexpr int HALF = D / 2, V = D / 64;
   if (threadIdx.x == 0) stamp_start(stamp);
   pdl_trigger();
-  const int head = blockIdx.x, r = blockIdx.y, j = threadIdx.x, half = d >> 1;
+  const int heads = hq + 2 * hkv, unit = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  const int r = unit / heads, head = unit - r * heads, j = lane * V;
+  const bool live = r < m;
   // not written by any kernel of this forward: the cache length word, the scales and the biases
   if (len_ptr) pos0 = *len_ptr;
-  float sc_a = 1.f, sc_b = 1.f, bi_a = 0.f, bi_b = 0.f;
+  const int kind = head < hq ? 0 : (head < hq + hkv ? 1 : 2), hl = head - (kind == 0 ? 0 : (kind == 1 ? hq : hq + hkv));
+  float sc[2][V], bi[2][V];
   {
-    const int hl = head < hq ? head : (head < hq + hkv ? head - hq : head - hq - hkv);
-    const float* sc = head < hq ? sq : (head < hq + hkv ? sk : sv);
-    const float* bi = head < hq ? bq : (head < hq + hkv ? bk : bv);
-    if (sc) { sc_a = sc[hl * d + j]; sc_b = sc[hl * d + j + half]; }   // fp8 weights: per-output-channel factors
-    if (bi) { bi_a = bi[hl * d + j]; bi_b = bi[hl * d + j + half]; }
+    const float* scp = kind == 0 ? sq : (kind == 1 ? sk : sv);
+    const float* bip = kind == 0 ? bq : (kind == 1 ? bk : bv);
+#pragma unroll
+    for (int i = 0; i < 2 * V; ++i) {
+      const int c = hl * D + (i / V) * HALF + j + i % V;
+      sc[i / V][i % V] = live && scp ? scp[c] : 1.f;      // fp8 weights: per-output-channel factors
+      bi[i / V][i % V] = live && bip ? bip[c] : 0.f;
+    }
   }
   pdl_wait();
   if (threadIdx.x == 0) stamp_released(stamp);
-  __shared__ float s_rstd;
+  if (!live) return;
   // W8A8: the row's slot of the running maximum that this layer's gate/up epilogue raises; its last reader (the
   // quantisation in front of the previous layer's down projection) is long done, its next writers start after this kernel
-  if (amax_zero && head == 0 && threadIdx.x == 0) amax_zero[r] = 0.f;
+  if (amax_zero && head == 0 && lane == 0) amax_zero[r] = 0.f;
   // every load of this kernel is issued before the first result is needed
-  const int width = (hq + 2 * hkv) * d;
+  const int width = heads * D;
   const size_t sstride = (size_t)m * width;
-  const float* pa = part + (size_t)r * width + head * d + j;
-  float ssq_v = 0.f, xs = 1.f;
-  if (threadIdx.x < 32) {
-    for (int t = threadIdx.x; t < nt; t += 32) ssq_v += __ldcg(ssq + (size_t)r * nt + t);
-    if (x_scale) xs = __ldcg(x_scale + r);     // W8A8: the partial sums are sums of code products; the row's factor joins the norm's
-  }
-  const float2 c = (head < hq + hkv) ? __ldcg(&cs[r * half + j]) : make_float2(1.f, 0.f);
-  Partials<16> va, vb;
+  const float* pa = part + (size_t)r * width + head * D + j;
+  float ssq_v = 0.f;
+  for (int t = lane; t < nt; t += 32) ssq_v += __ldcg(ssq + (size_t)r * nt + t);
+  const float xs = x_scale ? __ldcg(x_scale + r) : 1.f;     // W8A8: the partial sums are sums of code products; the row's factor joins the norm's
+  float2 c[V];
+#pragma unroll
+  for (int k = 0; k < V; ++k) c[k] = kind < 2 ? __ldcg(&cs[r * HALF + j + k]) : make_float2(1.f, 0.f);
+  Partials<V, 16> va, vb;
   issue_partials(va, pa, sstride, 0, S);
-  issue_partials(vb, pa + half, sstride, 0, S);
-  if (threadIdx.x < 32) {
-    // fixed order: lanes hold disjoint strided subsets, combined by the butterfly below
-    const float t = warp_sum(ssq_v);
-    if (threadIdx.x == 0) s_rstd = rsqrtf(t * inv_h + eps) * xs;
+  issue_partials(vb, pa + HALF, sstride, 0, S);
+  const float rstd = rsqrtf(warp_sum(ssq_v) * inv_h + eps) * xs;
+  float a[V], b[V];
+#pragma unroll
+  for (int k = 0; k < V; ++k) a[k] = b[k] = 0.f;
+  add_partials(va, a);
+  add_partials(vb, b);
+  sum_partials_from<V>(pa, sstride, 16, S, a);
+  sum_partials_from<V>(pa + HALF, sstride, 16, S, b);
+  T oa[V], ob[V];
+#pragma unroll
+  for (int k = 0; k < V; ++k) {
+    const float x = a[k] * rstd * sc[0][k] + bi[0][k], y = b[k] * rstd * sc[1][k] + bi[1][k];
+    oa[k] = from_f32<T>(kind < 2 ? x * c[k].x - y * c[k].y : x);
+    ob[k] = from_f32<T>(kind < 2 ? y * c[k].x + x * c[k].y : y);
   }
-  float a = add_partials(va, 0.f), b = add_partials(vb, 0.f);
-  a = sum_partials_from(pa, sstride, 16, S, a);
-  b = sum_partials_from(pa + half, sstride, 16, S, b);
-  __syncthreads();
-  const float rstd = s_rstd;
-  a = a * rstd * sc_a + bi_a;
-  b = b * rstd * sc_b + bi_b;
-  if (head < hq) {
-    T* o = q + ((size_t)r * hq + head) * d;
-    o[j] = from_f32<T>(a * c.x - b * c.y);
-    o[j + half] = from_f32<T>(b * c.x + a * c.y);
-  } else if (head < hq + hkv) {
-    const int hk = head - hq;
-    T* o = kc + ((size_t)hk * max_seq + pos0 + r) * d;
-    o[j] = from_f32<T>(a * c.x - b * c.y);
-    o[j + half] = from_f32<T>(b * c.x + a * c.y);
+  T* o = kind == 0 ? q + ((size_t)r * hq + head) * D : (kind == 1 ? kc : vc) + ((size_t)hl * max_seq + pos0 + r) * D;
+  if (V == 2) {
+    *reinterpret_cast<uint32_t*>(o + j) = *reinterpret_cast<const uint32_t*>(oa);
+    *reinterpret_cast<uint32_t*>(o + j + HALF) = *reinterpret_cast<const uint32_t*>(ob);
   } else {
-    const int hk = head - hq - hkv;
-    T* o = vc + ((size_t)hk * max_seq + pos0 + r) * d;
-    o[j] = from_f32<T>(a);
-    o[j + half] = from_f32<T>(b);
+    o[j] = oa[0];
+    o[j + HALF] = ob[0];
   }
   if (threadIdx.x == 0) stamp_end(stamp, true);
 }
@@ -471,16 +496,21 @@ void launch_fin_qkv(const float* part, int S, int m, const float* cs, const floa
                     const float* bq, const float* bk, const float* bv, const float* sq, const float* sk, const float* sv, void* q, void* kc, void* vc, int pos0, int hq,
                     int hkv, int d, int max_seq, int kv_type, cudaStream_t st, const int* len_ptr, KStamp* stamp, const float* x_scale,
                     float* amax_zero) {
-  if (kv_type == KV_F16)
-    launch_pdl(fin_qkv_kernel<__half>, dim3(hq + 2 * hkv, m), dim3(d / 2), 0, st, part, S, m, (const float2*)cs, ssq, nt, 1.f / (float)hidden,
-               eps, bq, bk, bv, sq, sk, sv, (__half*)q, (__half*)kc, (__half*)vc, pos0, hq, hkv, d, max_seq, len_ptr, x_scale, amax_zero, stamp);
-  else
-    launch_pdl(fin_qkv_kernel<bf16>, dim3(hq + 2 * hkv, m), dim3(d / 2), 0, st, part, S, m, (const float2*)cs, ssq, nt, 1.f / (float)hidden,
-               eps, bq, bk, bv, sq, sk, sv, (bf16*)q, (bf16*)kc, (bf16*)vc, pos0, hq, hkv, d, max_seq, len_ptr, x_scale, amax_zero, stamp);
+  auto go = [&](auto kern, auto* qt, auto* kt, auto* vt) {
+    launch_pdl(kern, dim3(ceil_div(m * (hq + 2 * hkv), 4)), dim3(128), 0, st, part, S, m, (const float2*)cs, ssq, nt, 1.f / (float)hidden,
+               eps, bq, bk, bv, sq, sk, sv, qt, kt, vt, pos0, hq, hkv, max_seq, len_ptr, x_scale, amax_zero, stamp);
+  };
+  if (kv_type == KV_F16) {
+    if (d == 128) go(fin_qkv_kernel<__half, 128>, (__half*)q, (__half*)kc, (__half*)vc);
+    else go(fin_qkv_kernel<__half, 64>, (__half*)q, (__half*)kc, (__half*)vc);
+  } else {
+    if (d == 128) go(fin_qkv_kernel<bf16, 128>, (bf16*)q, (bf16*)kc, (bf16*)vc);
+    else go(fin_qkv_kernel<bf16, 64>, (bf16*)q, (bf16*)kc, (bf16*)vc);
+  }
 }
 
 // Residual finalisation: h += sum of split-K partials; xg = h * gain of the next norm (stored as `fmt`);
-// ssq[row][tile] = sum of h^2 over the tile's 128 columns.  grid (nt tiles, m rows), 128 threads.
+// ssq[row][tile] = sum of h^2 over the tile's 128 columns (hidden even).  Two warps per (row, tile), two columns a lane, two such pairs a CTA.
 __global__ void __launch_bounds__(128) fin_resid_kernel(const float* __restrict__ part, int S, int m, int hidden,
                                                         float* __restrict__ h, const float* __restrict__ g,
                                                         void* __restrict__ xg, size_t lo_off, int fmt, float* __restrict__ ssq, int nt,
@@ -488,40 +518,44 @@ __global__ void __launch_bounds__(128) fin_resid_kernel(const float* __restrict_
                                                         float* __restrict__ amax_out, KStamp* stamp) {
   if (threadIdx.x == 0) stamp_start(stamp);
   pdl_trigger();
-  const int t = blockIdx.x, r = blockIdx.y, c = t * 128 + threadIdx.x;
+  const int pair = threadIdx.x >> 6, unit = blockIdx.x * 2 + pair;
+  const int r = unit / nt, t = unit - r * nt, c = t * 128 + (threadIdx.x & 63) * 2;
+  const bool in = r < m && c < hidden;
   // weights (gain, scale) do not depend on the predecessor
-  const float gc = (c < hidden) ? g[c] : 0.f;
-  float sc = (c < hidden && scale) ? scale[c] : 1.f;
+  const float g0 = in ? g[c] : 0.f, g1 = in ? g[c + 1] : 0.f;
+  float s0 = in && scale ? scale[c] : 1.f, s1 = in && scale ? scale[c + 1] : 1.f;
   pdl_wait();
   if (threadIdx.x == 0) stamp_released(stamp);
-  const float xs = x_scale ? __ldcg(x_scale + r) : 1.f;     // W8A8: the partial sums are sums of code products
-  float v = 0.f;
-  Partials<32> pv;
-  float hv = 0.f;
-  const size_t idx = (size_t)r * hidden + c, sstride = (size_t)m * hidden;
-  if (c < hidden) {
+  float ss = 0.f, am = 0.f;
+  if (in) {
+    const size_t idx = (size_t)r * hidden + c, sstride = (size_t)m * hidden;
+    Partials<2, 18> pv;
     issue_partials(pv, part + idx, sstride, 0, S);
-    hv = __ldcg(h + idx);
+    const Cols<2> hv = load_cols<2>(h + idx);
+    if (x_scale) {     // W8A8: the partial sums are sums of code products
+      const float xs = __ldcg(x_scale + r);
+      s0 *= xs;
+      s1 *= xs;
+    }
+    float s[2] = {0.f, 0.f};
+    add_partials(pv, s);
+    sum_partials_from<2>(part + idx, sstride, 18, S, s);
+    const float x0 = hv.v[0] + s[0] * s0, x1 = hv.v[1] + s[1] * s1, a0 = x0 * g0, a1 = x1 * g1;
+    *reinterpret_cast<float2*>(h + idx) = make_float2(x0, x1);
+    store_act2(xg, lo_off, idx, a0, a1, fmt);
+    ss = fmaf(x0, x0, x1 * x1);
+    if (amax_out) am = fmaxf(abs_as_f16(a0), abs_as_f16(a1));
   }
-  sc *= xs;
-  if (c < hidden) {
-    v = hv + sum_partials_from(part + idx, sstride, 32, S, add_partials(pv, 0.f)) * sc;
-    h[idx] = v;
-    store_act(xg, lo_off, idx, v * gc, fmt);
-  }
-  // one pass for the tile's sum of squares and (W8A8: the next projection's quantiser) the maximum of the stored xg
+  // the tile's sum of squares and (W8A8: the next projection's quantiser) the maximum of the stored xg
   __shared__ float red_s[4], red_m[4];
-  {
-    const float ws = warp_sum(v * v);
-    const float wm = amax_out ? warp_max(c < hidden ? abs_as_f16(v * gc) : 0.f) : 0.f;
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) { red_s[threadIdx.x >> 5] = ws; red_m[threadIdx.x >> 5] = wm; }
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    ssq[(size_t)r * nt + t] = (red_s[0] + red_s[2]) + (red_s[1] + red_s[3]);
-    if (amax_out) amax_out[(size_t)r * nt + t] = fmaxf(fmaxf(red_m[0], red_m[1]), fmaxf(red_m[2], red_m[3]));
-    stamp_end(stamp, true);
+  ss = warp_sum(ss);
+  if (amax_out) am = warp_max(am);
+  if ((threadIdx.x & 31) == 0) { red_s[threadIdx.x >> 5] = ss; red_m[threadIdx.x >> 5] = am; }
+  __syncthreads();
+  if ((threadIdx.x & 63) == 0 && r < m) {
+    ssq[(size_t)r * nt + t] = red_s[2 * pair] + red_s[2 * pair + 1];
+    if (amax_out) amax_out[(size_t)r * nt + t] = fmaxf(red_m[2 * pair], red_m[2 * pair + 1]);
+    if (threadIdx.x == 0) stamp_end(stamp, true);
   }
 }
 // The same for the many rows of a prompt (hidden a multiple of 4, no W8A8): one warp per (row, tile of 128 columns), four
@@ -571,7 +605,7 @@ void launch_fin_resid_rows(const float* part, int S, int m, int hidden, float* h
 }
 void launch_fin_resid(const float* part, int S, int m, int hidden, float* h, const float* g, void* xg, size_t lo_off, int fmt,
                       float* ssq, int nt, const float* scale, cudaStream_t st, KStamp* stamp, const float* x_scale, float* amax_out) {
-  launch_pdl(fin_resid_kernel, dim3(nt, m), dim3(128), 0, st, part, S, m, hidden, h, g, xg, lo_off, fmt, ssq, nt, scale, x_scale,
+  launch_pdl(fin_resid_kernel, dim3(ceil_div(m * nt, 2)), dim3(128), 0, st, part, S, m, hidden, h, g, xg, lo_off, fmt, ssq, nt, scale, x_scale,
              amax_out, stamp);
 }
 
