@@ -142,6 +142,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
     constexpr bool F16 = !__is_same(E, bf16);
     const uint32_t id_s = F16 ? umma_idesc_f16(AT_STEP) : umma_idesc_bf16(AT_STEP);
     const uint32_t id_o = (F16 ? umma_idesc_f16(D) : umma_idesc_bf16(D)) | (1u << 16);      // (V: MN-major)
+    if (elect_one()) {      // one thread issues everything: every election costs what several MMAs do (see gemm_gu.cu)
     bool ok = mbar_wait(q_full, 0, abort_flag);
     auto score = [&](int w, int t) {
       if (t >= (w ? steps1 : steps0)) return;
@@ -149,7 +150,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
       ok = ok && mbar_wait(k_full(s), (uint32_t)(t / S::STAGES) & 1u, abort_flag);
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint32_t ka = base + S::KV_OFF + s * 2 * S::TILE_BYTES + w * (AT_STEP * 128);
-      if (elect_one() && ok) {
+      if (ok) {
 #pragma unroll
         for (int kk = 0; kk < D / 16; ++kk)
           umma_bf16(tmem + w * AT_STEP, umma_desc_sw128(base + (kk >> 2) * 16384) + 2u * (kk & 3), umma_desc_sw128(ka + (kk >> 2) * 16384) + 2u * (kk & 3),
@@ -164,7 +165,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
       ok = ok && mbar_wait(p_full(w), (uint32_t)t & 1u, abort_flag) && mbar_wait(v_full(s), (uint32_t)(t / S::STAGES) & 1u, abort_flag);
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint64_t vd = umma_desc_sw128_mn(base + S::KV_OFF + (s * 2 + 1) * S::TILE_BYTES + w * (AT_STEP * 128), 16384);
-      if (elect_one() && ok) {
+      if (ok) {
 #pragma unroll
         for (int kk = 0; kk < AT_STEP / 16; ++kk)
           umma_f16_ta(tmem + 256 + w * 128, tmem + w * AT_STEP + kk * 8, vd + (uint64_t)(kk * 128), id_o, (t > 0 || kk > 0) ? 1u : 0u);
@@ -177,11 +178,12 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
       value(0, t);
       score(0, t + 1);
       value(1, t);
-      if (elect_one() && ok) umma_commit(kv_empty(t % S::STAGES));
-      __syncwarp();
+      if (ok) umma_commit(kv_empty(t % S::STAGES));
       score(1, t + 1);
     }
     if (!ok && p.status) atomicCAS(p.status, 0, ST_ATTENTION);
+    }
+    __syncwarp();
   } else if (warp >= 4) {
     // Where this thread's pieces of Q come from and its rows of the result go is worked out before the wait: rows = heads x n,
     // row r -> head r / n, token r % n.
