@@ -130,14 +130,14 @@ __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const __gri
       }
     }
   } else if (warp == 1) {
-    {
+    if (elect_one()) {      // one thread issues everything: every election costs what several MMAs do (see gemm_gu.cu)
       constexpr bool F16 = sizeof(E) == 2 && !__is_same(E, bf16);
       const uint32_t id_s = F16 ? umma_idesc_f16(PA_STEP) : umma_idesc_bf16(PA_STEP);
       const uint32_t id_o = (F16 ? umma_idesc_f16(D) : umma_idesc_bf16(D)) | (1u << 16);      // (V: MN-major)
       bool ok = mbar_wait(q_full, 0, abort_flag);
       auto score = [&](int q, int t) {
         const uint32_t qa = base + q * S::TILE_BYTES, ka = base + S::K_OFF + ((t >> 1) & 1) * S::TILE_BYTES + (t & 1) * (PA_STEP * 128);
-        if (elect_one() && ok) {
+        if (ok) {
 #pragma unroll
         for (int kk = 0; kk < D / 16; ++kk)
           umma_bf16(tmem + q * 128 + (t & 1) * PA_STEP, umma_desc_sw128(qa + (kk >> 2) * 16384) + 2u * (kk & 3),
@@ -149,7 +149,7 @@ __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const __gri
         ok = ok && mbar_wait(p_full(q, t), (uint32_t)(t >> 1) & 1u, abort_flag);
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const uint64_t vd = umma_desc_sw128_mn(base + S::V_OFF + ((t >> 1) & 1) * S::TILE_BYTES + (t & 1) * (PA_STEP * 128), 16384);
-        if (elect_one() && ok) {
+        if (ok) {
 #pragma unroll
         for (int kk = 0; kk < PA_STEP / 16; ++kk)
           umma_f16_ta(tmem + 256 + q * 128, tmem + q * 128 + (t & 1) * PA_STEP + kk * 8, vd + (uint64_t)(kk * 128), id_o, (t > 0 || kk > 0) ? 1u : 0u);
@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const __gri
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         }
         if (t < (q ? n1 : n0)) score(q, t);
-        if (q == 1 && ((t & 1) || t + 1 == ns)) { if (elect_one() && ok) umma_commit(k_empty((t >> 1) & 1)); }
+        if (q == 1 && ((t & 1) || t + 1 == ns)) { if (ok) umma_commit(k_empty((t >> 1) & 1)); }
       };
       for (int t = 0; t < 2; ++t) { scores(0, t); scores(1, t); }
       for (int t = 0; t < ns; ++t) {
@@ -173,11 +173,12 @@ __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const __gri
         if (t < n0) value(0, t);
         scores(0, t + 2);
         if (t < n1) value(1, t);
-        if ((t & 1) || t + 1 == ns) { if (elect_one() && ok) umma_commit(v_empty((t >> 1) & 1)); }
+        if ((t & 1) || t + 1 == ns) { if (ok) umma_commit(v_empty((t >> 1) & 1)); }
         scores(1, t + 2);
       }
       if (!ok && p.status) atomicCAS(p.status, 0, ST_ATTENTION);
     }
+    __syncwarp();
   } else if (warp >= 4) {
     const int q = (warp - 4) >> 2, wq = warp & 3;
     const int nq = q ? n1 : n0;
