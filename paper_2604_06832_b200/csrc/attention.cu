@@ -42,6 +42,7 @@ struct AttnParams {
   const unsigned long long* row_mask;   // nullable: bit r' of word r = row r reads row r' of this forward (AttnArgs::row_mask)
   int* status;                // nullable: status words (see TcOut::status)
   KStamp* stamp;
+  NextWeights next;
 };
 
 template <int D, typename E>
@@ -71,7 +72,13 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
   }
   const int n = p.n, hq = p.hq, hkv = p.hkv, qh = p.qh;
   const int chunk = blockIdx.x, grp = blockIdx.y, hk = blockIdx.z;
-  if (chunk >= n_chunks) { pdl_trigger(); pdl_wait(); return; }
+  const int cta = chunk + gridDim.x * (grp + gridDim.y * hk), ctas = gridDim.x * gridDim.y * gridDim.z;
+  if (chunk >= n_chunks) {
+    pdl_trigger();
+    if (tid == 0) ask_for_next(p.next, cta, ctas);
+    pdl_wait();
+    return;
+  }
   if (tid == 0) {
     stamp_start(p.stamp);
     mbar_init(q_full, 8);
@@ -313,6 +320,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
       atomicCAS(p.status, 0, ST_ATTENTION);
     }
   } else {
+    if (warp == 2 && lane == 0) ask_for_next(p.next, cta, ctas);
     pdl_wait();
   }
   __syncwarp();
@@ -486,6 +494,7 @@ static cudaError_t attn_launch_t(const AttnArgs& a, const AttnPlan& pl, cudaStre
   p.part_ml = (float2*)((char*)a.workspace + ((slots * D * 4 + 255) / 256) * 256);
   p.n = a.n; p.L = a.cache_len; p.max_seq = a.max_seq; p.hq = a.hq; p.hkv = a.hkv; p.qh = pl.qh;
   p.chunk_keys = pl.chunk_keys; p.n_chunks = pl.n_chunks; p.causal = a.row_mask ? 0 : a.causal; p.row_mask = a.row_mask; p.len_ptr = a.len_ptr; p.status = a.status; p.stamp = a.stamp;
+  if (a.next_w[0] && !next_weights(&p.next, a.next_w[0], a.next_w[1], a.next_n, a.next_k, false, 3)) return cudaErrorInvalidValue;
   static bool attr_set[MAX_DEVICES] = {};
   cudaError_t e = ensure_dynamic_smem(attn_tc_kernel<D, E>, S::TOTAL, attr_set);
   if (e != cudaSuccess) return e;

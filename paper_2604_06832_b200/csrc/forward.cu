@@ -363,6 +363,11 @@ static int forward_rows_tc(fdvlm_t* h, int n, int mode, int logits_rows, int wan
     at.row_mask = (mode == MODE_MASKED) ? h->q_mask : (mode == MODE_FUSED ? h->f_mask : nullptr);
     at.dtype = h->dt; at.workspace = h->ws; at.kv_type = h->kv_type; at.out_fmt = h->xfmt; at.out_lo_off = h->ao_lo;
     at.status = h->info + 3;
+    // Memory idles from here to the gate / up projection.  Bringing a third of its bf16 weights into L2 meanwhile gains where they are
+    // streamed as fast as they come (gemm_gu.cu; 12 layers of the 3B shape, us a step without, with a quarter, a third, half of them: 32 rows
+    // 758, 738, 734, 758; 64 rows 858, 842, 834, 831; 32 rows behind 8000 positions 818, 800, 790, 790).  Up to 16 rows the
+    // tiles do not, and the cache's K and V come later (4 rows 685 : 710); with fp8 weights there is nothing to gain (32 rows 660 : 663).
+    if (h->dt == DT_BF16 && n > 16) { at.next_w[0] = lw.w_gate; at.next_w[1] = lw.w_up; at.next_n = I; at.next_k = H; }
     at.amax_out = a8 ? h->amax_ao : nullptr;
     at.stamp = stamp(FDVLM_K_ATTENTION);
     if (at.stamp && !stamp(FDVLM_K_ATTN_MERGE)) at.stamp = nullptr;     // the launcher uses two consecutive records

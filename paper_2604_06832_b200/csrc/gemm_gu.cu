@@ -20,9 +20,8 @@ constexpr int GU_STAGES = 10;
 enum { GU_BF16 = 0, GU_FP8 = 1, GU_A8 = 2 };      // operand kinds, as TC_KIND_* of gemm_tc.cu
 
 struct GuParams {
-  CUtensorMap tm_w[2], tm_x, tm_next;
-  // boxes of the next launch's weights to ask for in L2: of every 64 of its rows next_kb k-blocks, the first pair of every next_step pairs
-  int next_boxes, next_kb, next_step, next_kblocks;
+  CUtensorMap tm_w[2], tm_x;
+  NextWeights next;
   const float* scale[2];
   int m, mp, planes, inter, f, kblocks, kb_elems, stages, w_bytes, x_bytes, tmem_cols;
   void* act; size_t act_lo_off; int act_fmt;
@@ -104,10 +103,7 @@ __global__ void __launch_bounds__(GU_THREADS, 2) gemm_gu_kernel(const __grid_con
       if (weights) {
         // Memory would idle from here through the epilogue, the hand-over and the next launch's start: it brings part of the
         // next launch's weights into L2 instead.
-        for (int b = blockIdx.x; ok && b < p.next_boxes; b += gridDim.x) {
-          const int i = b % p.next_kb, kb_next = (i >> 1) * 2 * p.next_step + (i & 1);
-          if (kb_next < p.next_kblocks) tma_prefetch_2d(&p.tm_next, kb_next * p.kb_elems, (b / p.next_kb) * 64);
-        }
+        if (ok) ask_for_next(p.next, blockIdx.x, gridDim.x);
         pdl_wait();
       }
       if (!ok) {
@@ -284,15 +280,9 @@ cudaError_t gemm_gu_launch(const TcGroup& g, const TcOut& o, const void* next, i
     return cudaErrorInvalidValue;
   for (int i = 0; i < 2; ++i)
     if (!make_tmap(&p.tm_w[i], g.w[i], inter, g.k, p.f, xkind)) return cudaErrorInvalidValue;
-  // A quarter of the next launch's weights, up to 32 rows (3B shape, 32 rows, a layer's gate / up + down: 25.8 us without, 25.3 with a quarter,
-  // 25.4 with half; 7B fp8, 64 rows, 8 layers: 816 us a step without, 822 with).
-  if (next && g.m <= 32) {
-    if (!make_tmap(&p.tm_next, next, next_n, next_k, 64, xkind)) return cudaErrorInvalidValue;
-    p.next_step = 4;
-    p.next_kblocks = ceil_div(next_k, p.kb_elems);
-    p.next_kb = 2 * ceil_div(ceil_div(p.next_kblocks, 2), p.next_step);
-    p.next_boxes = ceil_div(next_n, 64) * p.next_kb;
-  }
+  // A third of the next launch's weights, up to 32 rows (12 layers of the 3B shape, 32 rows: a quarter 733.6, a third 734.5, half 731.6 us a step,
+  // none 10 us more; W8A8, 8 layers of the 7B shape: none 743.8, a quarter 743.8, a third 744.9, half 748; fp8, 64 rows: 816 without, 822 with).
+  if (next && g.m <= 32 && !next_weights(&p.next, next, nullptr, next_n, next_k, g.fp8, 3)) return cudaErrorInvalidValue;
   const int grid = ceil_div(inter, p.f);
   return kind == GU_A8 ? gu_launch_t<GU_A8>(p, grid, smem, st) : (kind == GU_FP8 ? gu_launch_t<GU_FP8>(p, grid, smem, st) : gu_launch_t<GU_BF16>(p, grid, smem, st));
 }

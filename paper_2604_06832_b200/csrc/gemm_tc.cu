@@ -516,6 +516,20 @@ bool make_tmap_planes(CUtensorMap* tm, const void* ptr, int rows, int cols, int 
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// (w1 nullable)
+bool next_weights(NextWeights* n, const void* w0, const void* w1, int rows, int k, bool fp8, int step) {
+  const void* w[2] = {w0, w1};
+  n->mats = w1 ? 2 : 1;
+  for (int i = 0; i < n->mats; ++i)
+    if (!make_tmap(&n->tm[i], w[i], rows, k, 64, fp8 ? TM_E4M3_128 : TM_BF16)) return false;
+  n->kb_elems = fp8 ? 2 * TC_BK : TC_BK;
+  n->kblocks = ceil_div(k, n->kb_elems);
+  n->step = step;
+  n->row_blocks = ceil_div(rows, 64);
+  n->units = n->row_blocks * ceil_div(ceil_div(n->kblocks, 2), step);
+  return true;
+}
+
 // SM count of the current device (cached per device: one process may drive several GPUs)
 int sm_count() {
   static int n[MAX_DEVICES] = {};

@@ -80,6 +80,23 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* tm,
 __device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap* tm, int c0, int c1) {
   asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];" ::"l"(tm), "r"(c0), "r"(c1) : "memory");
 }
+// Part of the weights that a later launch streams, asked for in L2 while memory would idle: of every 64 rows of one or two
+// matrices of `kblocks` k-blocks the first pair of every `step` pairs.  units (pairs of all rows) = 0: nothing.
+struct NextWeights {
+  CUtensorMap tm[2];
+  int mats, units, row_blocks, step, kblocks, kb_elems;
+};
+// one thread's share: units first, first + stride, ...
+__device__ __forceinline__ void ask_for_next(const NextWeights& n, int first, int stride) {
+  for (int u = first; u < n.units; u += stride) {
+    const int pair = u / n.row_blocks, row = (u - pair * n.row_blocks) * 64, kb = pair * 2 * n.step;
+    for (int i = 0; i < n.mats; ++i) {
+      tma_prefetch_2d(&n.tm[i], kb * n.kb_elems, row);
+      if (kb + 1 < n.kblocks) tma_prefetch_2d(&n.tm[i], (kb + 1) * n.kb_elems, row);
+    }
+  }
+}
+bool next_weights(NextWeights* n, const void* w0, const void* w1, int rows, int k, bool fp8, int step);
 __device__ __forceinline__ void tma_load_2d_plain(uint32_t dst, const CUtensorMap* tm, uint32_t bar, int c0, int c1) {
   asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
                ::"r"(dst), "l"(tm), "r"(bar), "r"(c0), "r"(c1)
