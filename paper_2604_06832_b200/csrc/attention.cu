@@ -483,6 +483,9 @@ static cudaError_t attn_launch_t(const AttnArgs& a, const AttnPlan& pl, cudaStre
   // with the length on the device the grid is sized for the most chunks any length can give
   int grid_x = pl.n_chunks;
   if (a.len_ptr) { grid_x = pl.bound; const int tmax = ceil_div(a.max_seq, AT_KEYS); if (grid_x > tmax) grid_x = tmax; }
+  // One CTA per SM where next weights are asked for: those without a chunk take their share (with 24 CTAs of 16 rows the boxes of 30 MB were
+  // still being issued when the attention was done: 766 us a step of 12 layers, 696 with 148)
+  if (a.next_w[0]) grid_x = pl.bound;
   const size_t slots = (size_t)a.hq * a.n * grid_x;
   AttnParams p;
   memset(&p, 0, sizeof(p));
@@ -494,7 +497,7 @@ static cudaError_t attn_launch_t(const AttnArgs& a, const AttnPlan& pl, cudaStre
   p.part_ml = (float2*)((char*)a.workspace + ((slots * D * 4 + 255) / 256) * 256);
   p.n = a.n; p.L = a.cache_len; p.max_seq = a.max_seq; p.hq = a.hq; p.hkv = a.hkv; p.qh = pl.qh;
   p.chunk_keys = pl.chunk_keys; p.n_chunks = pl.n_chunks; p.causal = a.row_mask ? 0 : a.causal; p.row_mask = a.row_mask; p.len_ptr = a.len_ptr; p.status = a.status; p.stamp = a.stamp;
-  if (a.next_w[0] && !next_weights(&p.next, a.next_w[0], a.next_w[1], a.next_n, a.next_k, false, 3)) return cudaErrorInvalidValue;
+  if (a.next_w[0] && !next_weights(&p.next, a.next_w[0], a.next_w[1], a.next_n, a.next_k, a.next_fp8 != 0, 3)) return cudaErrorInvalidValue;
   static bool attr_set[MAX_DEVICES] = {};
   cudaError_t e = ensure_dynamic_smem(attn_tc_kernel<D, E>, S::TOTAL, attr_set);
   if (e != cudaSuccess) return e;

@@ -363,11 +363,13 @@ static int forward_rows_tc(fdvlm_t* h, int n, int mode, int logits_rows, int wan
     at.row_mask = (mode == MODE_MASKED) ? h->q_mask : (mode == MODE_FUSED ? h->f_mask : nullptr);
     at.dtype = h->dt; at.workspace = h->ws; at.kv_type = h->kv_type; at.out_fmt = h->xfmt; at.out_lo_off = h->ao_lo;
     at.status = h->info + 3;
-    // Memory idles from here to the gate / up projection.  Bringing a third of its bf16 weights into L2 meanwhile gains where they are
-    // streamed as fast as they come (gemm_gu.cu; 12 layers of the 3B shape, us a step without, with a quarter, a third, half of them: 32 rows
-    // 758, 738, 734, 758; 64 rows 858, 842, 834, 831; 32 rows behind 8000 positions 818, 800, 790, 790).  Up to 16 rows the
-    // tiles do not, and the cache's K and V come later (4 rows 685 : 710); with fp8 weights there is nothing to gain (32 rows 660 : 663).
-    if (h->dt == DT_BF16 && n > 16) { at.next_w[0] = lw.w_gate; at.next_w[1] = lw.w_up; at.next_n = I; at.next_k = H; }
+    // Memory idles from here to the gate / up projection.  Bringing a third of its weights into L2 meanwhile gains where they are
+    // streamed as fast as they come (gemm_gu.cu; us a step without, with a quarter, a third, half of them, 12 layers of the 3B shape: 4 rows 694, 681,
+    // 679, 675; 16 rows 720, 697, 696, 694; 32 rows 758, 735, 731, 732; 64 rows 858, 841, 835, 842; 32 rows behind 8000 positions 818, 793, 781,
+    // 774; 7B fp8: 8 rows 610, 588, 587, 586; 32 rows 668, 642, 639, 635; 40 rows 700, 694, 687; but 64 rows 806, 817, 839).
+    if (h->dt == DT_BF16 || n <= 40) {
+      at.next_w[0] = lw.w_gate; at.next_w[1] = lw.w_up; at.next_n = I; at.next_k = H; at.next_fp8 = h->dt == DT_FP8;
+    }
     at.amax_out = a8 ? h->amax_ao : nullptr;
     at.stamp = stamp(FDVLM_K_ATTENTION);
     if (at.stamp && !stamp(FDVLM_K_ATTN_MERGE)) at.stamp = nullptr;     // the launcher uses two consecutive records

@@ -248,11 +248,11 @@ cudaError_t gemm_gu_launch(const TcGroup& g, const TcOut& o, const void* next, i
   const int kind = g.a8 ? GU_A8 : (g.fp8 ? GU_FP8 : GU_BF16), inter = g.n[0];
   if (g.m < 1 || g.m > 64 || g.n_mats != 2 || g.n[1] != inter || inter % 8 || !o.ssq_in || (kind == GU_BF16 && !g.x_lo)) return cudaErrorInvalidValue;
   if (kind == GU_A8 && (!o.x_scale || !o.amax_out)) return cudaErrorInvalidValue;
-  // Where the 64-feature tiles of gemm_tc_kernel, two CTAs per SM, are as good or better they keep the rows (us a step, tiles : shares; bf16, 12
-  // layers of the 3B shape: 8 rows 701 : 720, 16 rows 718 : 731, 20 rows 757 : 757, 32 rows 763 : 760, 40 rows 822 : 795, 64 rows 923 : 874;
-  // fp8, 8 layers of the 7B shape, whose 296 tiles fill the SMs evenly: 8 rows 610 : 620, 32 rows 670 : 670, 40 rows 711 : 694, 48 rows 728 : 739
-  // -- from 41 rows on their planes take two MMAs --, 64 rows 841 : 816; W8A8: 32 rows 734 : 727, 64 rows 822 : 807).
-  if (kind == GU_FP8 ? g.m <= 32 || (g.m > 40 && g.m <= 48) : g.m <= 16) return cudaErrorNotSupported;
+  // fp8 weights, 41 to 48 rows: three planes that take two MMAs and gain nothing from it yet (8 layers of the 7B shape, 48 rows: 739 us a step, 728
+  // with the 64-feature tiles of gemm_tc_kernel, two CTAs per SM; 40 rows 694 : 711, 64 rows 816 : 841).  Everywhere else the shares are the faster
+  // ones, up to 32 rows with the weights that the attention brings into L2 (forward.cu; 12 layers of the 3B shape, 4, 16, 32, 64 rows: 679, 696, 731,
+  // 835 us a step against 683, 707, 763, 923; 7B fp8, 8 and 32 rows: 587, 639 : 607, 661; W8A8, 8 and 32 rows: 628, 696 : 649, 732).
+  if (kind == GU_FP8 && g.m > 40 && g.m <= 48) return cudaErrorNotSupported;
   p.f = ((ceil_div(inter, sm_count()) + 7) / 8) * 8;
   if (p.f > 128) return cudaErrorNotSupported;        // N = 256 at most
   p.m = g.m; p.mp = ((g.m + 7) / 8) * 8; p.planes = kind == GU_FP8 ? 3 : (kind == GU_A8 ? 1 : 2); p.inter = inter;
