@@ -495,7 +495,7 @@ def run_ours(args, wl, block):
         # launches own in the production chain (in-chain timing, see above); frac x peak x that time = the bytes.
         "roofline": {"bound": "hbm", "achieved": gemm_gbs, "peak": peak, "unit": "GB/s", "frac": gemm_gbs / peak,
                      "traffic": traffic, "traffic_note": traffic_note, "peak_kind": peak_kind,
-                     "kernel": "gemm_tc_kernel: all projection launches of one denoise forward, in-chain",
+                     "kernel": "gemm_tc_kernel and gemm_gu_kernel: all projection launches of one denoise forward, in-chain",
                      "algorithmic_bytes_per_forward": wbytes, "in_chain_ms_per_forward": gemm_us_chain / 1000.0,
                      "forward_ms_in_chain_timing": statistics.median(chain_total) / 1000.0 if chain_total else None,
                      "isolated": {"ms_per_forward": gemm_ms_isolated, "achieved": wbytes / (gemm_ms_isolated / 1000.0) / 1e9,
