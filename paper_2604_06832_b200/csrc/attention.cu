@@ -9,7 +9,7 @@
 // lie wholly in the committed cache are requested before the wait for the predecessor kernel.  Each CTA leaves an
 // unnormalised partial (O, maximum, sum) and a small second kernel merges the chunks.  The in-block mask is applied by key
 // index: denoise rows see all L + n keys, commit / prefill rows see keys <= L + i, or the caller gives bit masks.
-// What bounds it is the chain through one CTA: rows to shared memory 1.5 us, S, softmax, P V, store (with mma.sync on 64-row CTAs: 13.4 us a layer at 8224 keys and 32 rows, 8.6 now; 5.5 both at 2052 keys and 4 rows).
+// What bounds it is the chain through one CTA: rows to shared memory 1.5 us, S, softmax, P V, store (with mma.sync on 64-row CTAs: 13.4 us a layer at 8224 keys and 32 rows, 8.1 now; 5.5 and 5.3 at 2052 keys and 4 rows).
 // Every mbarrier wait is bounded; a wait that gives up records ST_ATTENTION in the status word and the CTA drains its
 // copies in flight and returns.
 #include "attn_plan.cuh"
