@@ -312,7 +312,8 @@ int fdvlm_profile_read_chain(fdvlm_t *h, fdvlm_kernel_record *records, int cap, 
 /* Test hook for the give-up path of the kernels' bounded waits.  While `on` is non-zero, every tensor-core GEMM of
  * this handle reads the flag when it starts and each of its roles (TMA producer, MMA issuer, converters, epilogue)
  * waits for nothing, as after a timed-out wait -- nothing issued, nothing in flight, tensor memory freed -- and
- * records its role in the status word, so the next synchronous call returns FDVLM_ERR_TIMEOUT.  Outputs of such
+ * records its role in the status word, so the next synchronous call returns FDVLM_ERR_TIMEOUT.  With `on` = 2 the other roles
+ * give up while the producers, which have not heard of it, go on to issue what fits into their rings.  Outputs of such
  * calls are undefined; committed cache positions are not written.  Takes effect in stream order. */
 int fdvlm_debug_poison(fdvlm_t *h, int on);
 

@@ -204,7 +204,7 @@ class Handle:
     def synchronize(self):
         self._check(lib().fdvlm_synchronize(self._h))
 
-    def debug_poison(self, on: bool):
+    def debug_poison(self, on: int):
         self._check(lib().fdvlm_debug_poison(self._h, int(on)))
 
     def decode_block(self, block_size: int, rule: int, threshold: float = 0.9, k: int = 8,

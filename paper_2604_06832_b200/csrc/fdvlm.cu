@@ -347,7 +347,7 @@ extern "C" int fdvlm_debug_poison(fdvlm_t* h, int on) {
   if (!h) return FDVLM_ERR_INVALID_ARG;
   int32_t* stage = (int32_t*)(h->host_stage + 960);      // pinned, beyond what the *_host variants use
   CU(h, cudaStreamSynchronize(h->st));                   // an earlier value may still be in flight from the same slot
-  *stage = on ? 1 : 0;
+  *stage = on == 2 ? 2 : (on ? 1 : 0);
   CU(h, cudaMemcpyAsync(h->info + 4, stage, 4, cudaMemcpyHostToDevice, h->st));
   return FDVLM_OK;
 }

@@ -34,7 +34,7 @@ struct GuParams {
 template <int KIND>
 __global__ void __launch_bounds__(GU_THREADS, 2) gemm_gu_kernel(const __grid_constant__ GuParams p) {
   extern __shared__ uint8_t smem_raw[];
-  __shared__ __align__(8) uint64_t bars[3 * GU_STAGES + 1];
+  __shared__ __align__(8) uint64_t bars[3 * GU_STAGES + 2];
   __shared__ uint32_t tmem_slot_s;
   __shared__ int abort_s, amax_s[64];
   __shared__ float rs[64], sc[2][128];
@@ -43,14 +43,14 @@ __global__ void __launch_bounds__(GU_THREADS, 2) gemm_gu_kernel(const __grid_con
   auto wfull = [&](int s) { return bar0 + 8u * s; };
   auto xfull = [&](int s) { return bar0 + 8u * (GU_STAGES + s); };
   auto empty = [&](int s) { return bar0 + 8u * (2 * GU_STAGES + s); };
-  const uint32_t tfull = bar0 + 8u * (3 * GU_STAGES);
+  const uint32_t tfull = bar0 + 8u * (3 * GU_STAGES), mma_done = tfull + 8u;
   volatile int* abort_flag = &abort_s;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int stage_bytes = p.x_bytes + p.w_bytes;      // the rows first: the MMA reads 128 of them, whatever follows the real ones
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < p.stages; ++s) { mbar_init(wfull(s), 1); mbar_init(xfull(s), 1); mbar_init(empty(s), 1); }
-    mbar_init(tfull, 1);
+    mbar_init(tfull, 1); mbar_init(mma_done, 1);
     stamp_start(p.stamp);
     abort_s = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -73,9 +73,7 @@ __global__ void __launch_bounds__(GU_THREADS, 2) gemm_gu_kernel(const __grid_con
     if (elect_one()) {
       const bool weights = warp == 0;
       const uint64_t pol = weights ? policy_evict_first() : policy_evict_last();
-      const bool poisoned = p.status && *reinterpret_cast<const volatile int*>(p.status + 1) != 0;      // (test hook: see gemm_tc.cu)
-      if (poisoned) *abort_flag = 1;
-      bool ok = !poisoned;
+      bool ok = may_issue(p.status, abort_flag);
       if (!weights) {
         pdl_wait();
         stamp_released(p.stamp);
@@ -106,14 +104,11 @@ __global__ void __launch_bounds__(GU_THREADS, 2) gemm_gu_kernel(const __grid_con
         if (ok) ask_for_next(p.next, blockIdx.x, gridDim.x);
         pdl_wait();
       }
-      if (!ok) {
-        atomicCAS(p.status, 0, ST_PRODUCER);
-        // drain: wait (bounded) for the bulk copies in flight, the last ones into each stage
-        for (int i = max(0, issued - p.stages); i < issued; ++i) {
-          const long long t0 = clock64();
-          while (!mbar_try_wait(weights ? wfull(i % p.stages) : xfull(i % p.stages), (uint32_t)(i / p.stages) & 1u) && clock64() - t0 < TC_TIMEOUT) {}
-        }
-      }
+      if (!ok) atomicCAS(p.status, 0, ST_PRODUCER);
+      // The CTA leaves no copy in flight, whether its reader has waited for it or has given up (which this thread does not hear of
+      // where all its k-blocks fit into the ring): the last ones into each stage.
+      for (int i = max(0, issued - p.stages); i < issued; ++i)
+        mbar_drain(weights ? wfull(i % p.stages) : xfull(i % p.stages), (uint32_t)(i / p.stages) & 1u);
     }
     __syncwarp();
   } else if (warp == 1) {
@@ -144,6 +139,8 @@ __global__ void __launch_bounds__(GU_THREADS, 2) gemm_gu_kernel(const __grid_con
       }
       if (ok) umma_commit(tfull);
       else atomicCAS(p.status, 0, ST_MMA);
+      umma_commit(mma_done);      // no MMA outlives the stages and the tensor memory that it uses, whoever gives up
+      mbar_drain(mma_done, 0);
     }
     __syncwarp();
   } else {

@@ -57,6 +57,23 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     if (clock64() - t0 > TC_TIMEOUT) { *abort_flag = 1; return false; }
   }
 }
+// What a CTA must not leave behind (bulk copies, MMAs): a bounded wait that no abort ends.
+__device__ __forceinline__ void mbar_drain(uint32_t bar, uint32_t parity) {
+  const long long t0 = clock64();
+  while (!mbar_try_wait(bar, parity) && clock64() - t0 < TC_TIMEOUT) {}
+}
+// The host-set test hook (status[1]; written by the host only, never by a kernel of the chain, so it may be read before the wait for
+// the predecessor).  1: the abort flag is raised, which every other role's first wait sees, and the producer is to issue nothing
+// (returns false): all leave by the path a timed-out wait takes.  2: the flag is raised, the others are given the time to see it, and
+// the producer goes on as one that has waited for nothing yet.  Only the producers pay for the read.
+__device__ __forceinline__ bool may_issue(const int* status, volatile int* abort_flag) {
+  const int hook = status ? *reinterpret_cast<const volatile int*>(status + 1) : 0;
+  if (hook == 0) return true;
+  *abort_flag = 1;
+  const long long t0 = clock64();
+  while (hook == 2 && clock64() - t0 < (1ll << 17)) {}
+  return hook == 2;
+}
 // Barrier 1 of N threads that also tells every thread whether all of them came with `ok`.
 template <int N>
 __device__ __forceinline__ bool named_barrier_and(bool ok) {

@@ -234,3 +234,31 @@ def test_give_up_path_of_the_gate_up_shares(shape, n):
     h.debug_poison(False)
     assert torch.equal(before, step())
     h.close()
+
+
+@pytest.mark.parametrize("shape,n", [(BF16, 33), (BF16.with_(hidden=1104), 64), (FP8, 40), (FP8.with_(hidden=1104), 64), (FP8.with_(dtype=I.W8A8), 17)],
+                         ids=["bf16", "bf16-deep", "fp8", "fp8-deep", "w8a8"])
+def test_producers_that_do_not_hear_of_an_abort(shape, n):
+    """The other roles give up before the producers issue anything.  Where all k-blocks fit into the ring no wait of a producer fails, and
+    the CTA must wait for its copies all the same; afterwards the step is what it was before, bit for bit."""
+    from paper_2604_06832_b200 import binding as B
+    h = B.Handle(shape, B.weights_to_device(I.make_weights(shape, 3)), max_seq=256, stream=torch.cuda.Stream())
+    toks = I.random_tokens(shape, 40, 4).cuda()
+
+    def step():
+        logits = torch.empty(n, shape.vocab, device="cuda")
+        h.reset()
+        h.prefill(None, toks)
+        h.block_begin(n)
+        h.block_step(B.RULE_TOPK, 0.0, n, logits=logits)
+        return logits
+
+    before = step()
+    for _ in range(2):
+        h.debug_poison(2)
+        with pytest.raises(B.FdvlmError) as e:
+            step()
+        assert e.value.code == B.ERR_TIMEOUT
+        h.debug_poison(False)
+        assert torch.equal(before, step())
+    h.close()
