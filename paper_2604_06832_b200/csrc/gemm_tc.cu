@@ -116,6 +116,7 @@ __global__ void __launch_bounds__(TC_THREADS) gemm_tc_kernel(const __grid_consta
   // SwiGLU epilogue, per warp pair pr: exchange buffer written (exw) / read (exr), two arrivals each
   auto exw_bar = [&](int pr) { return bar0 + 8u * (2 * TC_STAGES + 6 + pr); };
   auto exr_bar = [&](int pr) { return bar0 + 8u * (2 * TC_STAGES + 8 + pr); };
+  const uint32_t done_bar = bar0 + 8u * (2 * TC_STAGES + 10);      // every MMA of the CTA is complete
   volatile uint32_t* tmem_slot = (volatile uint32_t*)(sm + L::BAR_OFF + 8 * (2 * TC_STAGES + 4));
   volatile int* abort_flag = (volatile int*)(sm + L::BAR_OFF + 8 * (2 * TC_STAGES + 4) + 8);
 
@@ -130,6 +131,7 @@ __global__ void __launch_bounds__(TC_THREADS) gemm_tc_kernel(const __grid_consta
     for (int s = 0; s < TC_STAGES; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
     for (int a = 0; a < 2; ++a) { mbar_init(tfull_bar(a), 1); mbar_init(tempty_bar(a), 4); }
     for (int pr = 0; pr < 2; ++pr) { mbar_init(exw_bar(pr), 2); mbar_init(exr_bar(pr), 2); }
+    mbar_init(done_bar, 1);
     stamp_start(p.stamp);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -154,16 +156,11 @@ __global__ void __launch_bounds__(TC_THREADS) gemm_tc_kernel(const __grid_consta
     // ------------------------------------------------ TMA producer ------------------------------------------------
     if (lane == 0) {
       const uint64_t pol_w = policy_evict_first(), pol_x = policy_evict_last();
-      // The host-set test hook (status[1]; written by the host only, never by a kernel of the chain, so it may be read
-      // before the wait): the producer issues nothing and raises the abort flag, which every other role's first wait
-      // sees -- all leave by the path a timed-out wait takes.  Only this thread pays for the read.
-      const bool poisoned = p.status && *reinterpret_cast<const volatile int*>(p.status + 1) != 0;
-      if (poisoned) *abort_flag = 1;
       int stage = 0;
       uint32_t phase = 0;
-      uint32_t armed = 0;           // bit s: full[s] armed and not yet known complete
-      uint32_t armed_parity = 0;    // bit s: parity of that arming
-      bool ok = !poisoned;
+      uint32_t armed = 0;           // bit s: full[s] armed
+      uint32_t armed_parity = 0;    // bit s: parity of the last arming
+      bool ok = may_issue(p.status, abort_flag);
       bool waited = false;
       int n_pend = 0, pend_stage[TC_STAGES], pend_kb[TC_STAGES];
       const uint32_t stage_tx = L::W_BYTES + (X3 ? 3 : (p.has_lo ? 2 : 1)) * L::B_BYTES;
@@ -222,16 +219,11 @@ __global__ void __launch_bounds__(TC_THREADS) gemm_tc_kernel(const __grid_consta
         stamp_released(p.stamp);
         for (int j = 0; j < n_pend; ++j) load_x(pend_stage[j], pend_kb[j]);
       }
-      if (!ok) {
-        atomicCAS(p.status, 0, TC_ERR_PRODUCER);
-        // drain: wait (bounded) for every bulk copy this thread has in flight
-        for (int s = 0; s < TC_STAGES; ++s) {
-          if (!(armed & (1u << s))) continue;
-          const uint32_t par = (armed_parity >> s) & 1u;
-          const long long t0 = clock64();
-          while (!mbar_try_wait(full_bar(s), par) && clock64() - t0 < TC_TIMEOUT) {}
-        }
-      }
+      if (!ok) atomicCAS(p.status, 0, TC_ERR_PRODUCER);
+      // no copy stays in flight, whether its reader has waited for it or has given up (which this thread does not hear of where
+      // all its k-blocks fit into the ring)
+      for (int s = 0; s < TC_STAGES; ++s)
+        if (armed & (1u << s)) mbar_drain(full_bar(s), (armed_parity >> s) & 1u);
     }
   } else if (warp == 1) {
     // ------------------------------------------------ MMA issuer --------------------------------------------------
@@ -273,6 +265,10 @@ __global__ void __launch_bounds__(TC_THREADS) gemm_tc_kernel(const __grid_consta
         if (elect_one() && ok) umma_commit(tfull_bar(acc));
       }
       if (!ok) atomicCAS(p.status, 0, TC_ERR_MMA);
+      if (elect_one()) {      // no MMA outlives the stages and the tensor memory that it uses, whoever gives up
+        umma_commit(done_bar);
+        mbar_drain(done_bar, 0);
+      }
     }
   } else {
     // ------------------------------------------------ epilogue warps ----------------------------------------------

@@ -236,8 +236,9 @@ def test_give_up_path_of_the_gate_up_shares(shape, n):
     h.close()
 
 
-@pytest.mark.parametrize("shape,n", [(BF16, 33), (BF16.with_(hidden=1104), 64), (FP8, 40), (FP8.with_(hidden=1104), 64), (FP8.with_(dtype=I.W8A8), 17)],
-                         ids=["bf16", "bf16-deep", "fp8", "fp8-deep", "w8a8"])
+@pytest.mark.parametrize("shape,n", [(BF16, 33), (BF16.with_(hidden=1104), 64), (FP8, 40), (FP8.with_(hidden=1104), 64), (FP8.with_(dtype=I.W8A8), 17),
+                                     (BF16.with_(hidden=2048, intermediate=4096), 32), (FP8.with_(hidden=2048, intermediate=8192), 16)],
+                         ids=["bf16", "bf16-deep", "fp8", "fp8-deep", "w8a8", "bf16-items", "fp8-items"])
 def test_producers_that_do_not_hear_of_an_abort(shape, n):
     """The other roles give up before the producers issue anything.  Where all k-blocks fit into the ring no wait of a producer fails, and
     the CTA must wait for its copies all the same; afterwards the step is what it was before, bit for bit."""
