@@ -61,6 +61,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
   auto s_full = [&](int w) { return bar0 + 80u + 8u * w; };
   auto p_full = [&](int w) { return bar0 + 96u + 8u * w; };
   auto o_full = [&](int w) { return bar0 + 112u + 8u * w; };     // the last P V of a warpgroup's steps is complete
+  const uint32_t mma_done = bar0 + 136u;
   volatile uint32_t* tmem_slot = (volatile uint32_t*)(sm + S::BAR_OFF + 128);
   volatile int* abort_flag = (volatile int*)(sm + S::BAR_OFF + 132);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -81,7 +82,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
   }
   if (tid == 0) {
     stamp_start(p.stamp);
-    mbar_init(q_full, 8);
+    mbar_init(q_full, 8); mbar_init(mma_done, 1);
     for (int i = 0; i < S::STAGES; ++i) { mbar_init(k_full(i), 1); mbar_init(v_full(i), 1); mbar_init(kv_empty(i), 1); }
     for (int w = 0; w < 2; ++w) { mbar_init(s_full(w), 1); mbar_init(p_full(w), 4); mbar_init(o_full(w), 1); }
     *abort_flag = 0;
@@ -110,11 +111,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
   if (warp == 0) {
     if (lane == 0) {
       const uint64_t pol = policy_evict_last();     // the cache is read again by the other head groups and by the next step
-      // The host-set test hook (status[1], never written by a kernel): the producer issues nothing and raises the abort
-      // flag, so every other wait gives up.
-      const bool poisoned = p.status && *reinterpret_cast<const volatile int*>(p.status + 1) != 0;
-      if (poisoned) *abort_flag = 1;
-      bool ok = !poisoned, waited = false;
+      bool ok = may_issue(p.status, abort_flag), waited = false;
       uint32_t armed = 0, parity = 0;
       for (int t = 0; t < n_tiles && ok; ++t) {
         const int s = t % S::STAGES;
@@ -134,61 +131,61 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
         for (int b = 0; b < D / 64; ++b) tma_load_2d(dst + S::TILE_BYTES + b * 16384, &p.tm_v, v_full(s), b * 64, row, pol);
       }
       if (!waited) pdl_wait();
-      if (!ok) {
-        if (p.status) atomicCAS(p.status, 0, ST_ATTENTION);
-        for (int s = 0; s < S::STAGES; ++s) {      // drain: wait (bounded) for every bulk copy in flight
-          if (!(armed & (1u << s))) continue;
-          for (int v = 0; v < 2; ++v) {
-            const long long t0 = clock64();
-            while (!mbar_try_wait(v ? v_full(s) : k_full(s), (parity >> s) & 1u) && clock64() - t0 < TC_TIMEOUT) {}
-          }
+      if (!ok && p.status) atomicCAS(p.status, 0, ST_ATTENTION);
+      // no copy stays in flight, whether its reader has waited for it or has given up (which this thread does not hear of where all
+      // its tiles fit into the ring)
+      for (int s = 0; s < S::STAGES; ++s)
+        if (armed & (1u << s)) {
+          mbar_drain(k_full(s), (parity >> s) & 1u);
+          mbar_drain(v_full(s), (parity >> s) & 1u);
         }
-      }
     }
   } else if (warp == 1) {
     constexpr bool F16 = !__is_same(E, bf16);
     const uint32_t id_s = F16 ? umma_idesc_f16(AT_STEP) : umma_idesc_bf16(AT_STEP);
     const uint32_t id_o = (F16 ? umma_idesc_f16(D) : umma_idesc_bf16(D)) | (1u << 16);      // (V: MN-major)
     if (elect_one()) {      // one thread issues everything: every election costs what several MMAs do (see gemm_gu.cu)
-    bool ok = mbar_wait(q_full, 0, abort_flag);
-    auto score = [&](int w, int t) {
-      if (t >= (w ? steps1 : steps0)) return;
-      const int s = t % S::STAGES;
-      ok = ok && mbar_wait(k_full(s), (uint32_t)(t / S::STAGES) & 1u, abort_flag);
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint32_t ka = base + S::KV_OFF + s * 2 * S::TILE_BYTES + w * (AT_STEP * 128);
-      if (ok) {
+      bool ok = mbar_wait(q_full, 0, abort_flag);
+      auto score = [&](int w, int t) {
+        if (t >= (w ? steps1 : steps0)) return;
+        const int s = t % S::STAGES;
+        ok = ok && mbar_wait(k_full(s), (uint32_t)(t / S::STAGES) & 1u, abort_flag);
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t ka = base + S::KV_OFF + s * 2 * S::TILE_BYTES + w * (AT_STEP * 128);
+        if (ok) {
 #pragma unroll
-        for (int kk = 0; kk < D / 16; ++kk)
-          umma_bf16(tmem + w * AT_STEP, umma_desc_sw128(base + (kk >> 2) * 16384) + 2u * (kk & 3), umma_desc_sw128(ka + (kk >> 2) * 16384) + 2u * (kk & 3),
-                    id_s, kk > 0 ? 1u : 0u);
-        umma_commit(s_full(w));
-      }
-    };
-    auto value = [&](int w, int t) {
-      const int steps = w ? steps1 : steps0;
-      if (t >= steps) return;
-      const int s = t % S::STAGES;
-      ok = ok && mbar_wait(p_full(w), (uint32_t)t & 1u, abort_flag) && mbar_wait(v_full(s), (uint32_t)(t / S::STAGES) & 1u, abort_flag);
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint64_t vd = umma_desc_sw128_mn(base + S::KV_OFF + (s * 2 + 1) * S::TILE_BYTES + w * (AT_STEP * 128), 16384);
-      if (ok) {
+          for (int kk = 0; kk < D / 16; ++kk)
+            umma_bf16(tmem + w * AT_STEP, umma_desc_sw128(base + (kk >> 2) * 16384) + 2u * (kk & 3), umma_desc_sw128(ka + (kk >> 2) * 16384) + 2u * (kk & 3),
+                      id_s, kk > 0 ? 1u : 0u);
+          umma_commit(s_full(w));
+        }
+      };
+      auto value = [&](int w, int t) {
+        const int steps = w ? steps1 : steps0;
+        if (t >= steps) return;
+        const int s = t % S::STAGES;
+        ok = ok && mbar_wait(p_full(w), (uint32_t)t & 1u, abort_flag) && mbar_wait(v_full(s), (uint32_t)(t / S::STAGES) & 1u, abort_flag);
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint64_t vd = umma_desc_sw128_mn(base + S::KV_OFF + (s * 2 + 1) * S::TILE_BYTES + w * (AT_STEP * 128), 16384);
+        if (ok) {
 #pragma unroll
-        for (int kk = 0; kk < AT_STEP / 16; ++kk)
-          umma_f16_ta(tmem + 256 + w * 128, tmem + w * AT_STEP + kk * 8, vd + (uint64_t)(kk * 128), id_o, (t > 0 || kk > 0) ? 1u : 0u);
-        if (t + 1 == steps) umma_commit(o_full(w));
+          for (int kk = 0; kk < AT_STEP / 16; ++kk)
+            umma_f16_ta(tmem + 256 + w * 128, tmem + w * AT_STEP + kk * 8, vd + (uint64_t)(kk * 128), id_o, (t > 0 || kk > 0) ? 1u : 0u);
+          if (t + 1 == steps) umma_commit(o_full(w));
+        }
+      };
+      score(0, 0);
+      score(1, 0);
+      for (int t = 0; t < n_tiles; ++t) {
+        value(0, t);
+        score(0, t + 1);
+        value(1, t);
+        if (ok) umma_commit(kv_empty(t % S::STAGES));
+        score(1, t + 1);
       }
-    };
-    score(0, 0);
-    score(1, 0);
-    for (int t = 0; t < n_tiles; ++t) {
-      value(0, t);
-      score(0, t + 1);
-      value(1, t);
-      if (ok) umma_commit(kv_empty(t % S::STAGES));
-      score(1, t + 1);
-    }
-    if (!ok && p.status) atomicCAS(p.status, 0, ST_ATTENTION);
+      if (!ok && p.status) atomicCAS(p.status, 0, ST_ATTENTION);
+      umma_commit(mma_done);      // no MMA outlives the tiles and the tensor memory that it uses, whoever gives up
+      mbar_drain(mma_done, 0);
     }
     __syncwarp();
   } else if (warp >= 4) {
@@ -325,7 +322,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
   }
   __syncwarp();
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();     // the producer's copies have all been consumed (or drained) before any thread leaves
+  __syncthreads();     // the producer's copies have all landed before any thread leaves
   if (warp == 1) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
