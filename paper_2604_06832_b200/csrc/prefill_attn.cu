@@ -56,12 +56,13 @@ __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const __gri
   auto p_full = [&](int q, int t) { return bar0 + 104u + 16u * q + 8u * (t & 1); };
   auto o_done = [&](int q) { return bar0 + 136u + 8u * q; };                            // a step's P V is complete
   auto o_full = [&](int q) { return bar0 + 152u + 8u * q; };                            // the last one is
+  const uint32_t mma_done = bar0 + 176u;
   volatile uint32_t* tmem_slot = (volatile uint32_t*)(sm + S::BAR_OFF + 168);
   volatile int* abort_flag = (volatile int*)(sm + S::BAR_OFF + 172);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid == 0) {
     stamp_start(p.stamp);
-    mbar_init(q_full, 1);
+    mbar_init(q_full, 1); mbar_init(mma_done, 1);
     for (int i = 0; i < 2; ++i) {
       mbar_init(k_full(i), 1); mbar_init(k_empty(i), 1); mbar_init(v_full(i), 1); mbar_init(v_empty(i), 1);
       for (int t = 0; t < 2; ++t) { mbar_init(s_full(i, t), 1); mbar_init(p_full(i, t), 4); }
@@ -93,9 +94,8 @@ __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const __gri
 
   if (warp == 0) {
     if (lane == 0) {
-      const bool poisoned = p.status && *reinterpret_cast<const volatile int*>(p.status + 1) != 0;   // host-set test hook
-      if (poisoned) *abort_flag = 1;
-      bool ok = !poisoned;
+      const bool issue = may_issue(p.status, abort_flag);
+      bool ok = issue;
       uint32_t k_armed = 0, v_armed = 0, k_par = 0, v_par = 0;
       if (ok) {
         mbar_expect_tx(q_full, 2 * S::TILE_BYTES);
@@ -116,17 +116,12 @@ __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const __gri
         v_armed |= 1u << s; v_par = (v_par & ~(1u << s)) | (ph << s);
         for (int b = 0; b < D / 64; ++b) tma_load_2d_plain(base + S::V_OFF + s * S::TILE_BYTES + b * 16384, &p.tm_v, v_full(s), b * 64, row);
       }
-      if (!ok) {
-        if (p.status) atomicCAS(p.status, 0, ST_ATTENTION);
-        auto drain = [&](uint32_t bar, uint32_t par) {       // wait (bounded) for the copies in flight
-          const long long t0 = clock64();
-          while (!mbar_try_wait(bar, par) && clock64() - t0 < TC_TIMEOUT) {}
-        };
-        if (!poisoned) drain(q_full, 0);
-        for (int s = 0; s < 2; ++s) {
-          if (k_armed & (1u << s)) drain(k_full(s), (k_par >> s) & 1u);
-          if (v_armed & (1u << s)) drain(v_full(s), (v_par >> s) & 1u);
-        }
+      if (!ok && p.status) atomicCAS(p.status, 0, ST_ATTENTION);
+      // no copy stays in flight, whether its reader has waited for it or has given up
+      if (issue) mbar_drain(q_full, 0);
+      for (int s = 0; s < 2; ++s) {
+        if (k_armed & (1u << s)) mbar_drain(k_full(s), (k_par >> s) & 1u);
+        if (v_armed & (1u << s)) mbar_drain(v_full(s), (v_par >> s) & 1u);
       }
     }
   } else if (warp == 1) {
@@ -177,6 +172,8 @@ __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const __gri
         scores(1, t + 2);
       }
       if (!ok && p.status) atomicCAS(p.status, 0, ST_ATTENTION);
+      umma_commit(mma_done);      // no MMA outlives the tiles and the tensor memory that it uses, whoever gives up
+      mbar_drain(mma_done, 0);
     }
     __syncwarp();
   } else if (warp >= 4) {
@@ -255,7 +252,7 @@ __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attn_kernel(const __gri
   }
   __syncwarp();
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();     // the producer's copies have all been consumed (or drained) before any thread leaves
+  __syncthreads();     // the producer's copies have all landed before any thread leaves
   if (warp == 1) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");

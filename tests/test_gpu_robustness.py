@@ -97,6 +97,38 @@ def test_give_up_path_of_the_prompt_kernels(shape, n):
     handle.close()
 
 
+@pytest.mark.parametrize("shape,n", [(SMALL_BF16, 140), (SMALL_FP8, 150),
+                                     (SMALL_BF16.with_(n_layers=2, hidden=1536, intermediate=2560, vocab=512, mask_id=511), 770),
+                                     (SMALL_FP8.with_(n_layers=2, hidden=2048, n_q_heads=32, n_kv_heads=4, intermediate=1792, vocab=512, mask_id=511), 1290)],
+                         ids=["bf16", "fp8", "bf16-pieces", "fp8-pieces"])
+def test_prompt_producers_that_do_not_hear_of_an_abort(shape, n):
+    """The other roles give up before the producers of the prompt kernels (in both CTAs of a pair) issue anything; the CTAs wait for the copies
+    all the same, and afterwards the handle gives what it gave before, bit for bit."""
+    b = B()
+    handle = b.Handle(shape, b.weights_to_device(I.make_weights(shape, 31)), max_seq=n + 64, stream=torch.cuda.Stream())
+    toks = I.random_tokens(shape, n, 8).cuda()
+
+    def prompt():
+        last = torch.zeros(shape.vocab, dtype=torch.float32, device="cuda")
+        torch.cuda.synchronize()
+        handle.reset()
+        handle.prefill(None, toks, last)
+        handle.synchronize()
+        kv = [handle.cache_read(l, w, 0, n) for l in range(shape.n_layers) for w in (0, 1)]
+        torch.cuda.synchronize()
+        return [last] + kv
+
+    before = prompt()
+    for _ in range(2):
+        handle.debug_poison(2)
+        with pytest.raises(b.FdvlmError) as e:
+            prompt()
+        assert e.value.code == b.ERR_TIMEOUT
+        handle.debug_poison(False)
+        assert all(torch.equal(x, y) for x, y in zip(before, prompt()))
+    handle.close()
+
+
 def test_poisoned_operator_call_reports_through_its_status_query():
     b = B()
     m, n, k = 32, 1024, 512
