@@ -273,7 +273,7 @@ cudaError_t gemm_gu_launch(const TcGroup& g, const TcOut& o, const void* next, i
   if (smem > 224 * 1024) return cudaErrorNotSupported;
   const int xkind = g.fp8 ? TM_E4M3_128 : TM_BF16;
   if (kind == GU_A8 ? !make_tmap(&p.tm_x, g.x, g.m, g.k, p.mp, xkind)
-                    : !make_tmap_planes(&p.tm_x, g.x, g.m, g.k, p.planes, (const char*)g.x_lo - (const char*)g.x, p.mp, g.fp8))
+                    : !make_tmap_planes(&p.tm_x, g.x, g.m, g.k, p.planes, (const char*)g.x_lo - (const char*)g.x, p.mp, xkind))
     return cudaErrorInvalidValue;
   for (int i = 0; i < 2; ++i)
     if (!make_tmap(&p.tm_w[i], g.w[i], inter, g.k, p.f, xkind)) return cudaErrorInvalidValue;

@@ -471,27 +471,28 @@ static EncodeTiledFn encode_fn() {
   return fn;
 }
 
-// 2-D row-major [rows, cols] tensor, box {64 columns, box_rows}, zero OOB fill.  16-bit elements (TM_BF16, TM_F16):
-// 128-byte swizzle (rows of the box are 128 bytes); e4m3 bytes: TM_E4M3 no swizzle (rows of 64 bytes, widened by the
-// converter warps of the prompt path), TM_E4M3_128 a box of 128 columns with the 128-byte swizzle (the tile is an MMA operand as it lands).
-bool make_tmap(CUtensorMap* tm, const void* ptr, int rows, int cols, int box_rows, int kind) {
-  typedef std::tuple<const void*, int, int, int, int> Key;
+// Row-major [rows, cols] matrix, or `planes` > 0 of them plane_bytes apart as one 3-D tensor; box {64 columns, box_rows(, planes)}, zero
+// OOB fill.  16-bit elements (TM_BF16, TM_F16): 128-byte swizzle (rows of the box are 128 bytes); e4m3 bytes: TM_E4M3 no swizzle (rows of
+// 64 bytes, widened by the converter warps of the prompt path), TM_E4M3_128 a box of 128 columns with the 128-byte swizzle (the tile is an
+// MMA operand as it lands).  A map is a function of these arguments alone: those made before are kept, at most 4096 of them.
+static bool encode_tmap(CUtensorMap* tm, const void* ptr, int rows, int cols, int box_rows, int kind, int planes, size_t plane_bytes) {
+  typedef std::tuple<const void*, int, int, int, int, int, size_t> Key;
   static std::map<Key, CUtensorMap> cache;
   static std::mutex mu;
   std::lock_guard<std::mutex> lock(mu);
   const bool fp8 = kind == TM_E4M3 || kind == TM_E4M3_128;
   const bool wide = kind == TM_E4M3_128;
-  Key key(ptr, rows, cols, box_rows, kind);
+  Key key(ptr, rows, cols, box_rows, kind, planes, plane_bytes);
   auto it = cache.find(key);
   if (it != cache.end()) { *tm = it->second; return true; }
   EncodeTiledFn fn = encode_fn();
   if (!fn) return false;
-  cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-  cuuint64_t strides[1] = {(cuuint64_t)cols * (fp8 ? 1 : 2)};
-  cuuint32_t box[2] = {(cuuint32_t)(wide ? 2 * TC_BK : TC_BK), (cuuint32_t)box_rows};
-  cuuint32_t estr[2] = {1, 1};
+  cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)rows, (cuuint64_t)planes};
+  cuuint64_t strides[2] = {(cuuint64_t)cols * (fp8 ? 1 : 2), (cuuint64_t)plane_bytes};
+  cuuint32_t box[3] = {(cuuint32_t)(wide ? 2 * TC_BK : TC_BK), (cuuint32_t)box_rows, (cuuint32_t)planes};
+  cuuint32_t estr[3] = {1, 1, 1};
   const CUtensorMapDataType dt = fp8 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : (kind == TM_F16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16);
-  CUresult r = fn(tm, dt, 2, const_cast<void*>(ptr), dims, strides,
+  CUresult r = fn(tm, dt, planes ? 3 : 2, const_cast<void*>(ptr), dims, strides,
                   box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, (fp8 && !wide) ? CU_TENSOR_MAP_SWIZZLE_NONE : CU_TENSOR_MAP_SWIZZLE_128B,
                   CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) return false;
@@ -499,17 +500,11 @@ bool make_tmap(CUtensorMap* tm, const void* ptr, int rows, int cols, int box_row
   cache[key] = *tm;
   return true;
 }
-
-// The planes of a GEMM input, equally far apart, as one 3-D tensor [planes, rows, cols]: one box fetches a k-block of all of them.
-bool make_tmap_planes(CUtensorMap* tm, const void* ptr, int rows, int cols, int planes, size_t plane_bytes, int box_rows, bool bytes) {
-  EncodeTiledFn fn = encode_fn();
-  if (!fn) return false;
-  cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)rows, (cuuint64_t)planes};
-  cuuint64_t strides[2] = {(cuuint64_t)cols * (bytes ? 1 : 2), (cuuint64_t)plane_bytes};
-  cuuint32_t box[3] = {(cuuint32_t)(bytes ? 2 * TC_BK : TC_BK), (cuuint32_t)box_rows, (cuuint32_t)planes};
-  cuuint32_t estr[3] = {1, 1, 1};
-  return fn(tm, bytes ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), dims, strides, box, estr,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+bool make_tmap(CUtensorMap* tm, const void* ptr, int rows, int cols, int box_rows, int kind) {
+  return encode_tmap(tm, ptr, rows, cols, box_rows, kind, 0, 0);
+}
+bool make_tmap_planes(CUtensorMap* tm, const void* ptr, int rows, int cols, int planes, size_t plane_bytes, int box_rows, int kind) {
+  return encode_tmap(tm, ptr, rows, cols, box_rows, kind, planes, plane_bytes);
 }
 
 // (w1 nullable)

@@ -120,7 +120,8 @@ struct TcOut {
 // TM_E4M3_128: bytes, box of 128 columns, 128-byte swizzle.  False when the driver entry point is missing or the encode fails.
 enum { TM_BF16 = 0, TM_E4M3 = 1, TM_F16 = 2, TM_E4M3_128 = 3 };
 bool make_tmap(CUtensorMap* tm, const void* ptr, int rows, int cols, int box_rows, int kind = TM_BF16);
-bool make_tmap_planes(CUtensorMap* tm, const void* ptr, int rows, int cols, int planes, size_t plane_bytes, int box_rows, bool bytes);
+// The planes of a GEMM input, equally far apart, as one 3-D tensor [planes, rows, cols]: one box fetches a k-block of all of them.
+bool make_tmap_planes(CUtensorMap* tm, const void* ptr, int rows, int cols, int planes, size_t plane_bytes, int box_rows, int kind);
 bool tc_linear_supported(int m, int n, int k, int dtype);
 // Split-K workspace of a group with m rows, output width ld, `tiles` 128-row weight tiles and depth k.
 size_t tc_workspace_bytes(int m, int ld, int tiles, int k);
