@@ -392,8 +392,7 @@ static int forward_rows_tc(fdvlm_t* h, int n, int mode, int logits_rows, int wan
     gu.scale[0] = lw.s_gate; gu.scale[1] = lw.s_up;
     gu = quantised(gu, h->amax_a, nt);
     prof_begin(h, 0);
-    e = gemm_gu_launch(gu, o, lw.w_down, H, I, h->st);
-    if (e == cudaErrorNotSupported) e = tc_group_launch(gu, o, h->st);
+    e = gemm_gu_supported(gu) ? gemm_gu_launch(gu, o, lw.w_down, H, I, h->st) : tc_group_launch(gu, o, h->st);
     prof_end(h);
     h->launches++;
     if (e != cudaSuccess)

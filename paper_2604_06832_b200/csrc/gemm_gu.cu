@@ -239,41 +239,56 @@ static cudaError_t gu_launch_t(const GuParams& p, int grid, size_t smem, cudaStr
   return launch_pdl(gemm_gu_kernel<KIND>, dim3(grid), dim3(GU_THREADS), smem, st, p);
 }
 
-cudaError_t gemm_gu_launch(const TcGroup& g, const TcOut& o, const void* next, int next_n, int next_k, cudaStream_t st) {
-  GuParams p;
-  memset(&p, 0, sizeof(p));
-  const int kind = g.a8 ? GU_A8 : (g.fp8 ? GU_FP8 : GU_BF16), inter = g.n[0];
-  if (g.m < 1 || g.m > 64 || g.n_mats != 2 || g.n[1] != inter || inter % 8 || !o.ssq_in || (kind == GU_BF16 && !g.x_lo)) return cudaErrorInvalidValue;
-  if (kind == GU_A8 && (!o.x_scale || !o.amax_out)) return cudaErrorInvalidValue;
+// The launch for g: shares and shared memory.  False: g is left to gemm_tc_kernel.
+struct GuPlan { int kind, f, mp, planes, kblocks, stages; size_t smem; };
+static bool gu_plan(const TcGroup& g, GuPlan* pl) {
+  pl->kind = g.a8 ? GU_A8 : (g.fp8 ? GU_FP8 : GU_BF16);
   // fp8 weights, 41 to 48 rows: three planes that take two MMAs and gain nothing from it yet (8 layers of the 7B shape, 48 rows: 739 us a step, 728
   // with the 64-feature tiles of gemm_tc_kernel, two CTAs per SM; 40 rows 694 : 711, 64 rows 816 : 841).  Everywhere else the shares are the faster
   // ones, up to 32 rows with the weights that the attention brings into L2 (forward.cu; 12 layers of the 3B shape, 4, 16, 32, 64 rows: 679, 696, 731,
   // 835 us a step against 683, 707, 763, 923; 7B fp8, 8 and 32 rows: 587, 639 : 607, 661; W8A8, 8 and 32 rows: 628, 696 : 649, 732).
-  if (kind == GU_FP8 && g.m > 40 && g.m <= 48) return cudaErrorNotSupported;
-  p.f = ((ceil_div(inter, sm_count()) + 7) / 8) * 8;
-  if (p.f > 128) return cudaErrorNotSupported;        // N = 256 at most
-  p.m = g.m; p.mp = ((g.m + 7) / 8) * 8; p.planes = kind == GU_FP8 ? 3 : (kind == GU_A8 ? 1 : 2); p.inter = inter;
-  p.kb_elems = g.fp8 ? 2 * TC_BK : TC_BK; p.kblocks = ceil_div(g.k, p.kb_elems);
+  if (pl->kind == GU_FP8 && g.m > 40 && g.m <= 48) return false;
+  pl->f = ((ceil_div(g.n[0], sm_count()) + 7) / 8) * 8;
+  if (pl->f > 128) return false;        // N = 256 at most
+  pl->mp = ((g.m + 7) / 8) * 8; pl->planes = pl->kind == GU_FP8 ? 3 : (pl->kind == GU_A8 ? 1 : 2);
+  pl->kblocks = ceil_div(g.k, g.fp8 ? 2 * TC_BK : TC_BK);
+  const int lanes = pl->planes * pl->mp, n = 2 * pl->f, stage = (n + lanes) * 128;
+  pl->stages = 221 * 1024 / stage;
+  if (pl->stages > GU_STAGES) pl->stages = GU_STAGES;
+  if (pl->stages > pl->kblocks) pl->stages = pl->kblocks;
+  // the ring; the rows that the MMA reads behind the last stage's real ones; the turned accumulators
+  size_t smem = (size_t)pl->stages * stage;
+  const size_t reach = (size_t)(pl->stages - 1) * stage + (lanes > 128 ? 32768 : 16384), turned = (size_t)n * (lanes | 1) * 4;
+  if (smem < reach) smem = reach;
+  if (smem < turned) smem = turned;
+  pl->smem = smem + 1024;
+  return pl->smem <= 224 * 1024;
+}
+
+bool gemm_gu_supported(const TcGroup& g) {
+  GuPlan pl;
+  return g.m >= 1 && g.m <= 64 && gu_plan(g, &pl);
+}
+
+cudaError_t gemm_gu_launch(const TcGroup& g, const TcOut& o, const void* next, int next_n, int next_k, cudaStream_t st) {
+  GuParams p;
+  GuPlan pl;
+  memset(&p, 0, sizeof(p));
+  const int inter = g.n[0];
+  if (g.m < 1 || g.m > 64 || g.n_mats != 2 || g.n[1] != inter || inter % 8 || !o.ssq_in || !gu_plan(g, &pl)) return cudaErrorInvalidValue;
+  if (pl.kind == GU_A8 ? (!o.x_scale || !o.amax_out) : !g.x_lo) return cudaErrorInvalidValue;
+  p.f = pl.f; p.m = g.m; p.mp = pl.mp; p.planes = pl.planes; p.inter = inter; p.stages = pl.stages; p.kblocks = pl.kblocks;
+  p.kb_elems = g.fp8 ? 2 * TC_BK : TC_BK;
   p.w_bytes = 2 * p.f * 128; p.x_bytes = p.planes * p.mp * 128;
   p.scale[0] = g.scale[0]; p.scale[1] = g.scale[1];
   p.act = o.act; p.act_lo_off = o.act_lo_off; p.act_fmt = o.act_fmt;
   p.ssq_in = o.ssq_in; p.nt = o.nt_in; p.inv_h = o.hidden > 0 ? 1.f / (float)o.hidden : 0.f; p.eps = o.eps;
   p.x_scale = o.x_scale; p.amax_out = o.amax_out; p.status = o.status; p.stamp = o.stamp;
-  const int lanes = p.planes * p.mp, n = 2 * p.f, stage = p.w_bytes + p.x_bytes;
+  const int lanes = p.planes * p.mp, n = 2 * p.f;
   p.tmem_cols = lanes > 128 ? 512 : (n <= 32 ? 32 : (n <= 64 ? 64 : (n <= 128 ? 128 : 256)));
-  p.stages = 221 * 1024 / stage;
-  if (p.stages > GU_STAGES) p.stages = GU_STAGES;
-  if (p.stages > p.kblocks) p.stages = p.kblocks;
-  // the ring; the rows that the MMA reads behind the last stage's real ones; the turned accumulators
-  size_t smem = (size_t)p.stages * stage;
-  const size_t reach = (size_t)(p.stages - 1) * stage + (lanes > 128 ? 32768 : 16384), turned = (size_t)n * (lanes | 1) * 4;
-  if (smem < reach) smem = reach;
-  if (smem < turned) smem = turned;
-  smem += 1024;
-  if (smem > 224 * 1024) return cudaErrorNotSupported;
   const int xkind = g.fp8 ? TM_E4M3_128 : TM_BF16;
-  if (kind == GU_A8 ? !make_tmap(&p.tm_x, g.x, g.m, g.k, p.mp, xkind)
-                    : !make_tmap_planes(&p.tm_x, g.x, g.m, g.k, p.planes, (const char*)g.x_lo - (const char*)g.x, p.mp, xkind))
+  if (pl.kind == GU_A8 ? !make_tmap(&p.tm_x, g.x, g.m, g.k, p.mp, xkind)
+                       : !make_tmap_planes(&p.tm_x, g.x, g.m, g.k, p.planes, (const char*)g.x_lo - (const char*)g.x, p.mp, xkind))
     return cudaErrorInvalidValue;
   for (int i = 0; i < 2; ++i)
     if (!make_tmap(&p.tm_w[i], g.w[i], inter, g.k, p.f, xkind)) return cudaErrorInvalidValue;
@@ -281,7 +296,8 @@ cudaError_t gemm_gu_launch(const TcGroup& g, const TcOut& o, const void* next, i
   // none 10 us more; W8A8, 8 layers of the 7B shape: none 743.8, a quarter 743.8, a third 744.9, half 748; fp8, 64 rows: 816 without, 822 with).
   if (next && g.m <= 32 && !next_weights(&p.next, next, nullptr, next_n, next_k, g.fp8, 3)) return cudaErrorInvalidValue;
   const int grid = ceil_div(inter, p.f);
-  return kind == GU_A8 ? gu_launch_t<GU_A8>(p, grid, smem, st) : (kind == GU_FP8 ? gu_launch_t<GU_FP8>(p, grid, smem, st) : gu_launch_t<GU_BF16>(p, grid, smem, st));
+  return pl.kind == GU_A8 ? gu_launch_t<GU_A8>(p, grid, pl.smem, st)
+                          : (pl.kind == GU_FP8 ? gu_launch_t<GU_FP8>(p, grid, pl.smem, st) : gu_launch_t<GU_BF16>(p, grid, pl.smem, st));
 }
 
 }  // namespace fdk

@@ -126,7 +126,8 @@ bool tc_linear_supported(int m, int n, int k, int dtype);
 // Split-K workspace of a group with m rows, output width ld, `tiles` 128-row weight tiles and depth k.
 size_t tc_workspace_bytes(int m, int ld, int tiles, int k);
 // The decode path's gate / up projection (SWIGLU): one equal share of the features per SM (gemm_gu.cu).  next (nullable): the weights
-// [next_n, next_k], of the same type, that the following launch streams.  cudaErrorNotSupported: left to tc_group_launch.
+// [next_n, next_k], of the same type, that the following launch streams.  Groups that are not supported go to tc_group_launch.
+bool gemm_gu_supported(const TcGroup& g);
 cudaError_t gemm_gu_launch(const TcGroup& g, const TcOut& o, const void* next, int next_n, int next_k, cudaStream_t st);
 cudaError_t tc_group_launch(const TcGroup& g, const TcOut& o, cudaStream_t st);
 
