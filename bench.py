@@ -442,18 +442,17 @@ def run_ours(args, wl, block):
     gemm_us_chain = sum(chain_us.get(k_, 0.0) for k_ in gemm_kinds)
     if gemm_us_chain <= 0:          # exact fp32 path: no in-chain stamps, the one-by-one figure stands in
         gemm_us_chain = gemm_ms_isolated * 1000.0
-    gemm_gbs = wbytes / (gemm_us_chain * 1e-6) / 1e9
     kv_bytes = shape.kv_bytes_per_token() * L_step
     attn_us_chain = chain_us.get("attention", 0.0) + chain_us.get("attn_merge", 0.0)
-    # DRAM bytes of the same launches: dram read + write over algorithmic bytes of the layer projections, from the ncu
-    # capture summarised in profiles/ncu_traffic.json (taken on the 4-layer cut of the shape; traffic grows in
-    # proportion to the weight bytes).  Null when there is no capture of the kernel as it stands.
+    # DRAM bytes of one forward: those of the projections (dram read + write over algorithmic bytes of the layer projections, from
+    # the ncu captures summarised in profiles/ncu_traffic.json, taken on the 4-layer cut of the shape; traffic grows in proportion
+    # to the weight bytes) and the cached K / V once.  Null when there is no capture of the kernels as they stand.
     traffic, traffic_note = None, None
     try:
         with open(os.path.join(ROOT, "profiles", "ncu_traffic.json")) as f:
-            cap = json.load(f).get("gemm_tc", {}).get(shape.dtype)
+            cap = json.load(f).get("projections", {}).get(shape.dtype)
         if cap and block == cap.get("block"):
-            traffic = wbytes * cap["dram_bytes"] / cap["algorithmic_bytes"]
+            traffic = wbytes * cap["dram_bytes"] / cap["algorithmic_bytes"] + kv_bytes
             traffic_note = cap.get("note")
     except (OSError, ValueError, KeyError):
         pass
@@ -491,15 +490,19 @@ def run_ours(args, wl, block):
                 "d2h_bytes_per_step": n_steps * (block * 13 + 32)},
         "gpu_launches": n_launch,
         "clocks": clocks,
-        # dominant kernel: the projection GEMMs.  achieved = every linear weight byte of one forward / the time those
-        # launches own in the production chain (in-chain timing, see above); frac x peak x that time = the bytes.
-        "roofline": {"bound": "hbm", "achieved": gemm_gbs, "peak": peak, "unit": "GB/s", "frac": gemm_gbs / peak,
-                     "traffic": traffic, "traffic_note": traffic_note, "peak_kind": peak_kind,
-                     "kernel": "gemm_tc_kernel and gemm_gu_kernel: all projection launches of one denoise forward, in-chain",
-                     "algorithmic_bytes_per_forward": wbytes, "in_chain_ms_per_forward": gemm_us_chain / 1000.0,
+        # The whole denoise step: weights and cached K / V once, over the step's time.  (No launch has a bandwidth of its own: each asks
+        # for its first weights while its predecessors run, and attention and gate / up bring part of the next weights into L2.)
+        "roofline": {"bound": "hbm", "achieved": step_bytes / (step_med / 1000.0) / 1e9, "peak": peak, "unit": "GB/s",
+                     "frac": step_bytes / (step_med / 1000.0) / 1e9 / peak, "traffic": traffic, "traffic_note": traffic_note, "peak_kind": peak_kind,
+                     "kernel": "every kernel of one denoise step (projections: gemm_tc_kernel, gemm_gu_kernel)",
+                     "algorithmic_bytes_per_forward": step_bytes,
                      "forward_ms_in_chain_timing": statistics.median(chain_total) / 1000.0 if chain_total else None,
-                     "isolated": {"ms_per_forward": gemm_ms_isolated, "achieved": wbytes / (gemm_ms_isolated / 1000.0) / 1e9,
-                                  "note": "the same launches timed one by one with CUDA events, without the chain's overlap"}},
+                     "projections": {"weight_bytes_per_forward": wbytes, "in_chain_ms_per_forward": gemm_us_chain / 1000.0,
+                                     "isolated_ms_per_forward": gemm_ms_isolated,
+                                     "isolated_gbs": wbytes / (gemm_ms_isolated / 1000.0) / 1e9,
+                                     "note": "in_chain: the time that the projection launches own in the replayed forward; part of their weights "
+                                             "reaches L2 and shared memory before it, so bytes over this time is no HBM rate. "
+                                             "isolated: the same launches timed one by one with CUDA events"}},
         "attention": {"kernel": "attn_tc_kernel + attn_combine_kernel, in-chain", "kv_bytes_per_forward": kv_bytes,
                       "in_chain_ms_per_forward": attn_us_chain / 1000.0,
                       "achieved_gbs": kv_bytes / (attn_us_chain * 1e-6) / 1e9 if attn_us_chain > 0 else None},
