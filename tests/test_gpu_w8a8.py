@@ -158,3 +158,44 @@ def test_w8a8_give_up_path_and_recovery():
         h.synchronize()
     assert torch.equal(lg[0], lg[1])
     h.close()
+
+
+@pytest.mark.parametrize("n,inter", [(1, 2416), (17, 2416), (33, 2416), (64, 2416), (16, 18928), (64, 18928), (40, 19008)])
+def test_w8a8_mlp_of_one_layer(n, inter):
+    """Gate / up and down of one layer whose attention adds nothing (wo = 0): rows of every padding, a ragged depth (1104 = 8 x 128 + 80),
+    a last share of 16 and of 112 features, shares of 128 features, and more than an SM's 128.
+    The rows of the first quantiser are bf16 embeddings (gains of 1), which f16 holds exactly, and none of their quotients lies on a tie: 448 x / max
+    is a midpoint of two codes (an odd multiple, 17 to 31, of a power of two) only where 7 divides the mantissa of max, or for 21 where three
+    times that mantissa has 8 bits.  So both sides give the same codes.  The input of the second is stored as f16,
+    which moves a quotient by up to 2^-12 of itself, 2^-13 on the mean, against a spacing of some 2^-3.5: one code in 2^9.5 lands elsewhere, by
+    a whole spacing s, where quantising moves every element by s / sqrt(12) rms.  The ratio is sqrt(12 / 2^9.5) = 0.13."""
+    b = B()
+    shape = SMALL.with_(n_layers=1, hidden=1104, intermediate=inter, vocab=1000, mask_id=999, tie_embeddings=True)
+    w = I.make_weights(shape, 11)
+    w["layers"][0]["wo"].zero_()
+    mantissa = (w["embed"].abs().max(1).values.view(torch.int16).int() & 127) + 128
+    odd = mantissa // (mantissa & -mantissa)
+    untied = ((odd % 7 != 0) & (odd > 85)).nonzero().flatten().to(torch.int32)
+    w["embed"][shape.mask_id] = w["embed"][untied[-1]]
+    assert len(untied) > 80
+    init = untied[:n].clone()
+    init[-1] = shape.mask_id
+    wn = I.weights_to_numpy(w)
+    toks = I.random_tokens(shape, 9, 13)
+    ref = []
+    for o in (orc.Oracle(shape, wn, act_fp8=True), orc.Oracle(shape, wn)):
+        o.prefill(None, toks.numpy(), want_logits=False)
+        o.block_begin(n, init.numpy())
+        ref.append(o.block_step(orc.TOPK, 0.0, 1)["logits"])
+    h = b.Handle(shape, b.weights_to_device(w), max_seq=128, max_block=64, stream=torch.cuda.Stream())
+    lg = torch.empty(n, shape.vocab, dtype=torch.float32, device="cuda")
+    torch.cuda.synchronize()
+    h.prefill(None, toks.cuda())
+    h.block_begin(n, init.cuda())
+    h.block_step(b.RULE_TOPK, 0.0, 1, logits=lg)
+    h.close()
+    d8, noise = lg.double().cpu().numpy() - ref[0], ref[0] - ref[1]
+    assert _rms(noise) > 1e-2
+    assert _rms(d8) <= 0.25 * _rms(noise), (_rms(d8), _rms(noise))
+    # no row is off as a whole
+    assert np.sqrt((d8 ** 2).mean(1)).max() <= 0.5 * _rms(noise), np.sqrt((d8 ** 2).mean(1)).max()
