@@ -30,8 +30,10 @@
  *     (info / *_host variants) synchronise that stream before returning; others are asynchronous.
  *   - Every function returns FDVLM_OK (0) or a negative fdvlm_status; argument and state errors are
  *     detected on the host before anything is launched.  fdvlm_last_error gives a message.
- *   - A handle is not thread-safe; distinct handles are independent.  There is no CPU fallback: with
- *     no usable GPU fdvlm_create fails with FDVLM_ERR_CUDA.
+ *   - A handle is not thread-safe; distinct handles are independent.  A forward takes the whole GPU (one CTA per SM that holds
+ *     nearly all of its shared memory, in attention too, whose spare CTAs fetch the next weights): forwards of handles on
+ *     several streams queue for SMs rather than run side by side.  There is no CPU fallback: with no usable GPU fdvlm_create
+ *     fails with FDVLM_ERR_CUDA.
  */
 #ifndef FDVLM_H_
 #define FDVLM_H_

@@ -480,7 +480,7 @@ static cudaError_t attn_launch_t(const AttnArgs& a, const AttnPlan& pl, cudaStre
   // with the length on the device the grid is sized for the most chunks any length can give
   int grid_x = pl.n_chunks;
   if (a.len_ptr) { grid_x = pl.bound; const int tmax = ceil_div(a.max_seq, AT_KEYS); if (grid_x > tmax) grid_x = tmax; }
-  // One CTA per SM where next weights are asked for: those without a chunk take their share (with 24 CTAs of 16 rows the boxes of 30 MB were
+  // One CTA per SM where next weights are asked for: those without a chunk take their share (with 24 CTAs of 16 rows the boxes of 34 MB were
   // still being issued when the attention was done: 766 us a step of 12 layers, 696 with 148)
   if (a.next_w[0]) grid_x = pl.bound;
   const size_t slots = (size_t)a.hq * a.n * grid_x;

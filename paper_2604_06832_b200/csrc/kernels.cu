@@ -376,11 +376,9 @@ void launch_quantize_bf16_rows(const void* in, int m, int k, void* codes, float*
 template <int V> struct Cols { float v[V]; };
 template <int V>
 __device__ __forceinline__ Cols<V> load_cols(const float* __restrict__ p) {
+  static_assert(V == 1 || V == 2, "columns a lane");
   Cols<V> c;
-  if (V == 4) {
-    const float4 x = __ldcg(reinterpret_cast<const float4*>(p));
-    c.v[0] = x.x; c.v[1] = x.y; c.v[V - 2] = x.z; c.v[V - 1] = x.w;
-  } else if (V == 2) {
+  if (V == 2) {
     const float2 x = __ldcg(reinterpret_cast<const float2*>(p));
     c.v[0] = x.x; c.v[V - 1] = x.y;
   } else {

@@ -191,7 +191,7 @@ struct AttnArgs {
   const int* len_ptr;   // nullable: device word holding the cache length (overrides cache_len)
   int* status;          // nullable: device status words (see TcOut::status)
   float* amax_out;      // nullable (tensor-core kernel): [n][hq] maxima of |out| as stored, per row and head
-  // tensor-core kernel, nullable: matrices [next_n, next_k] (bf16 or e4m3) of a launch that follows soon, a third of which is asked for in L2
+  // tensor-core kernel, nullable: matrices [next_n, next_k] (bf16 or e4m3) of a launch that follows soon, every third pair of k-blocks of which is asked for in L2, by CTAs on every SM
   const void* next_w[2]; int next_n, next_k, next_fp8;
   KStamp* stamp;        // nullable: decode: two consecutive entries (attention, chunk merge); prompt path: one
 };

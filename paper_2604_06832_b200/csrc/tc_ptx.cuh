@@ -98,7 +98,8 @@ __device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap* tm, int c0, i
   asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];" ::"l"(tm), "r"(c0), "r"(c1) : "memory");
 }
 // Part of the weights that a later launch streams, asked for in L2 while memory would idle: of every 64 rows of one or two
-// matrices of `kblocks` k-blocks the first pair of every `step` pairs.  units (pairs of all rows) = 0: nothing.
+// matrices of `kblocks` k-blocks every step-th pair of k-blocks from the first on (step 3, 32 k-blocks: 6 of 16 pairs, 37.5 %; one or
+// two k-blocks: all).  units (pairs of all rows) = 0: nothing.
 struct NextWeights {
   CUtensorMap tm[2];
   int mats, units, row_blocks, step, kblocks, kb_elems;
@@ -129,9 +130,10 @@ __device__ __forceinline__ uint64_t policy_evict_last() {
   asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(p));
   return p;
 }
-// True in one lane of a converged warp.  MMAs and commits are issued inside `if (elect_one())` by warps that wait together:
-// the operands are then known to be the same for all that execute the instruction.  Issued inside `if (lane == 0)` each
-// cost some 100 clocks of the issuing thread.
+// True in one lane of a converged warp, the same one every time.  MMAs and commits are issued inside `if (elect_one())`: one thread is
+// then known to execute them.  Inside `if (lane == 0)` each costs some 100 clocks of the issuing thread; an election in front of a group
+// of MMAs costs some 250.  So where that is not hidden, the whole loop, waits included, runs in one elected thread (gemm_gu.cu,
+// attention.cu, prefill_attn.cu); gemm_tc.cu (two CTAs per SM) and prefill_gemm.cu (N = 256) elect per k-block, which costs them nothing.
 __device__ __forceinline__ bool elect_one() {
   uint32_t r;
   asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r));
