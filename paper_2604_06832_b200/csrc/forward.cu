@@ -363,11 +363,12 @@ static int forward_rows_tc(fdvlm_t* h, int n, int mode, int logits_rows, int wan
     at.row_mask = (mode == MODE_MASKED) ? h->q_mask : (mode == MODE_FUSED ? h->f_mask : nullptr);
     at.dtype = h->dt; at.workspace = h->ws; at.kv_type = h->kv_type; at.out_fmt = h->xfmt; at.out_lo_off = h->ao_lo;
     at.status = h->info + 3;
-    // Memory idles from here to the gate / up projection.  Bringing a third of its weights into L2 meanwhile gains where they are
-    // streamed as fast as they come (gemm_gu.cu; us a step without, with a quarter, a third, half of them, 12 layers of the 3B shape: 4 rows 694, 681,
-    // 679, 675; 16 rows 720, 697, 696, 694; 32 rows 758, 735, 731, 732; 64 rows 858, 841, 835, 842; 32 rows behind 8000 positions 818, 793, 781,
-    // 774; 7B fp8: 8 rows 610, 588, 587, 586; 32 rows 668, 642, 639, 635; 40 rows 700, 694, 687; but 64 rows 806, 817, 839).
-    if (h->dt == DT_BF16 || n <= 40) {
+    // Memory idles from here to the gate / up projection: part of its weights is brought into L2 meanwhile (NextWeights, every third pair).
+    // Not with fp8 weights from 41 rows on, where gate / up is bound by its MMAs (three planes) and not by its weights.
+    // us a step without : with, 3B shape, 12 layers: 4 rows 687 : 672, 32 rows 758 : 737, 64 rows 866 : 841.  7B shape, 8 layers, fp8: 8 rows
+    // 610 : 596, 33 rows 708 : 699, 36 rows 719 : 710, 40 rows 729 : 731, 41 rows 760 : 776, 48 rows 784 : 790, 64 rows 877 : 891;
+    // W8A8 (one plane): 8 rows 656 : 634, 32 rows 721 : 697, 41 rows 732 : 723, 48 rows 741 : 730, 56 rows 782 : 771, 64 rows 805 : 799.
+    if (h->dt == DT_BF16 || a8 || n <= 40) {
       at.next_w[0] = lw.w_gate; at.next_w[1] = lw.w_up; at.next_n = I; at.next_k = H; at.next_fp8 = h->dt == DT_FP8;
     }
     at.amax_out = a8 ? h->amax_ao : nullptr;

@@ -243,10 +243,10 @@ static cudaError_t gu_launch_t(const GuParams& p, int grid, size_t smem, cudaStr
 struct GuPlan { int kind, f, mp, planes, kblocks, stages; size_t smem; };
 static bool gu_plan(const TcGroup& g, GuPlan* pl) {
   pl->kind = g.a8 ? GU_A8 : (g.fp8 ? GU_FP8 : GU_BF16);
-  // fp8 weights, 41 to 48 rows: three planes that take two MMAs and gain nothing from it yet (8 layers of the 7B shape, 48 rows: 739 us a step, 728
-  // with the 64-feature tiles of gemm_tc_kernel, two CTAs per SM; 40 rows 694 : 711, 64 rows 816 : 841).  Everywhere else the shares are the faster
-  // ones, up to 32 rows with the weights that the attention brings into L2 (forward.cu; 12 layers of the 3B shape, 4, 16, 32, 64 rows: 679, 696, 731,
-  // 835 us a step against 683, 707, 763, 923; 7B fp8, 8 and 32 rows: 587, 639 : 607, 661; W8A8, 8 and 32 rows: 628, 696 : 649, 732).
+  // fp8 weights, 41 to 48 rows: more than 128 lanes take a second MMA, which eats up what the shares gain, while the 64-feature tiles still
+  // have three stages (two from 49 rows on).  us a step, shares : tiles, 8 layers of the 7B shape: 40 rows 729 : 749, 41 rows 760 : 760,
+  // 44 rows 771 : 766, 48 rows 784 : 789 (no difference; two runs differ by 8), 49 rows 831 : 878, 56 rows 841 : 903, 64 rows 877 : 911.
+  // Everywhere else the shares are as fast or faster: 12 layers of the 3B shape, 4, 16, 32, 64 rows: 679, 696, 731, 835 : 683, 707, 763, 923.
   if (pl->kind == GU_FP8 && g.m > 40 && g.m <= 48) return false;
   pl->f = ((ceil_div(g.n[0], sm_count()) + 7) / 8) * 8;
   if (pl->f > 128) return false;        // N = 256 at most
@@ -292,9 +292,12 @@ cudaError_t gemm_gu_launch(const TcGroup& g, const TcOut& o, const void* next, i
     return cudaErrorInvalidValue;
   for (int i = 0; i < 2; ++i)
     if (!make_tmap(&p.tm_w[i], g.w[i], inter, g.k, p.f, xkind)) return cudaErrorInvalidValue;
-  // A third of the next launch's weights, up to 32 rows (12 layers of the 3B shape, 32 rows: a quarter 733.6, a third 734.5, half 731.6 us a step,
-  // none 10 us more; W8A8, 8 layers of the 7B shape: none 743.8, a quarter 743.8, a third 744.9, half 748; fp8, 64 rows: 816 without, 822 with).
-  if (next && g.m <= 32 && !next_weights(&p.next, next, nullptr, next_n, next_k, g.fp8, 3)) return cudaErrorInvalidValue;
+  // Part of the next launch's weights (NextWeights, every third pair).  us a step without : with, 3B shape, 12 layers: 4 and 8 rows the
+  // same, 16 rows 699 : 706, 24 rows 721 : 719, 32 rows 737 : 732, 33 rows 757 : 751, 48 rows 782 : 778, 64 rows 840 : 836.  7B shape, 8 layers, fp8:
+  // 4 rows 596 : 589, 8 rows 596 : 591, 16 rows 610 : 603, 24 rows 650 : 653, 33 rows 704 : 711, 64 rows 877 : 904; W8A8: up to 32 rows the same,
+  // 40 rows 720 : 731, 48 rows 730 : 741.  So bf16 weights from 17 rows on, fp8 weights up to 16, W8A8 never.
+  const bool ask = pl.kind == GU_BF16 ? g.m > 16 : pl.kind == GU_FP8 && g.m <= 16;
+  if (next && ask && !next_weights(&p.next, next, nullptr, next_n, next_k, g.fp8, 3)) return cudaErrorInvalidValue;
   const int grid = ceil_div(inter, p.f);
   return pl.kind == GU_A8 ? gu_launch_t<GU_A8>(p, grid, pl.smem, st)
                           : (pl.kind == GU_FP8 ? gu_launch_t<GU_FP8>(p, grid, pl.smem, st) : gu_launch_t<GU_BF16>(p, grid, pl.smem, st));
