@@ -248,6 +248,11 @@ static bool gu_plan(const TcGroup& g, GuPlan* pl) {
   // 44 rows 771 : 766, 48 rows 784 : 789 (no difference; two runs differ by 8), 49 rows 831 : 878, 56 rows 841 : 903, 64 rows 877 : 911.
   // Everywhere else the shares are as fast or faster: 12 layers of the 3B shape, 4, 16, 32, 64 rows: 679, 696, 731, 835 : 683, 707, 763, 923.
   if (pl->kind == GU_FP8 && g.m > 40 && g.m <= 48) return false;
+  // A few MB of weights and few rows: everything is latency, and the smaller CTAs of the tiles start sooner.  us a step, shares : tiles: 12 layers of
+  // hidden 512, intermediate 1376 in bf16 (2.8 MB): 2 rows 360 : 349, 4 rows 367 : 352, 8 rows 378 : 365, 16 rows 366 : 366, 32 rows 422 : 454;
+  // of 1024 and 2816 in fp8 (5.8 MB): 391 : 374, 391 : 379, 396 : 374, 405 : 387, 427 : 462; of 1536 and 8960 in bf16 (55 MB): 2 rows 480 : 485,
+  // 8 rows 503 : 510.
+  if (g.m <= 8 && (size_t)g.n[0] * g.k * (g.fp8 ? 2 : 4) <= (8u << 20)) return false;
   pl->f = ((ceil_div(g.n[0], sm_count()) + 7) / 8) * 8;
   if (pl->f > 128) return false;        // N = 256 at most
   pl->mp = ((g.m + 7) / 8) * 8; pl->planes = pl->kind == GU_FP8 ? 3 : (pl->kind == GU_A8 ? 1 : 2);
@@ -294,9 +299,9 @@ cudaError_t gemm_gu_launch(const TcGroup& g, const TcOut& o, const void* next, i
     if (!make_tmap(&p.tm_w[i], g.w[i], inter, g.k, p.f, xkind)) return cudaErrorInvalidValue;
   // Part of the next launch's weights (NextWeights, every third pair).  us a step without : with, 3B shape, 12 layers: 4 and 8 rows the
   // same, 16 rows 699 : 706, 24 rows 721 : 719, 32 rows 737 : 732, 33 rows 757 : 751, 48 rows 782 : 778, 64 rows 840 : 836.  7B shape, 8 layers, fp8:
-  // 4 rows 596 : 589, 8 rows 596 : 591, 16 rows 610 : 603, 24 rows 650 : 653, 33 rows 704 : 711, 64 rows 877 : 904; W8A8: up to 32 rows the same,
-  // 40 rows 720 : 731, 48 rows 730 : 741.  So bf16 weights from 17 rows on, fp8 weights up to 16, W8A8 never.
-  const bool ask = pl.kind == GU_BF16 ? g.m > 16 : pl.kind == GU_FP8 && g.m <= 16;
+  // 8 rows 596 : 591, 16 rows 613 : 604, 24 rows 653 : 653, 32 rows 670 : 669, 33 rows 704 : 711, 64 rows 877 : 904; W8A8: up to 32 rows the same,
+  // 40 rows 720 : 731, 48 rows 730 : 741.  So bf16 weights from 17 rows on, fp8 weights up to 32, W8A8 never.
+  const bool ask = pl.kind == GU_BF16 ? g.m > 16 : pl.kind == GU_FP8 && g.m <= 32;
   if (next && ask && !next_weights(&p.next, next, nullptr, next_n, next_k, g.fp8, 3)) return cudaErrorInvalidValue;
   const int grid = ceil_div(inter, p.f);
   return pl.kind == GU_A8 ? gu_launch_t<GU_A8>(p, grid, pl.smem, st)

@@ -199,9 +199,9 @@ def test_fp8_projection_of_rows_with_small_values():
 
 # ---- gate / up of a decode step, one share of the features per SM: row counts at which the planes change, ragged last share and depth ----
 @pytest.mark.parametrize("base,inter,n", [(BF16, 2384, 1), (BF16, 2384, 16), (BF16, 2384, 17), (BF16, 2384, 33), (BF16, 2384, 64), (BF16, 1216, 31), (BF16, 19008, 24),
-                                          (FP8, 2416, 3), (FP8, 2416, 33), (FP8, 2416, 40), (FP8, 2416, 41), (FP8, 2416, 49), (FP8, 2416, 64)])
+                                          (FP8, 2416, 3), (FP8, 4816, 3), (FP8, 2416, 33), (FP8, 2416, 40), (FP8, 2416, 41), (FP8, 2416, 49), (FP8, 2416, 64)])
 def test_gate_up_shares(base, inter, n):
-    """(19008 features are more than 128 per SM and stay with the tiles; hidden: a last tile of 80 columns in the finalisation.)"""
+    """(19008 features are more than 128 per SM and stay with the tiles, as do 2416 of fp8 weights up to 8 rows; hidden: a last tile of 80 columns in the finalisation.)"""
     shape = base.with_(n_layers=1, hidden=1104, intermediate=inter)
     oracle, handle, _ = make_pair(shape, 5, max_seq=128, qkv_bias=True)
     emb, toks = I.make_prefix(shape, 20, 20, 3)

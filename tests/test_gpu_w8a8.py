@@ -160,7 +160,7 @@ def test_w8a8_give_up_path_and_recovery():
     h.close()
 
 
-@pytest.mark.parametrize("n,inter", [(1, 2416), (17, 2416), (33, 2416), (64, 2416), (16, 18928), (64, 18928), (40, 19008)])
+@pytest.mark.parametrize("n,inter", [(1, 2416), (1, 4816), (8, 4816), (17, 2416), (33, 2416), (64, 2416), (16, 18928), (64, 18928), (40, 19008)])
 def test_w8a8_mlp_of_one_layer(n, inter):
     """Gate / up and down of one layer whose attention adds nothing (wo = 0): rows of every padding, a ragged depth (1104 = 8 x 128 + 80),
     a last share of 16 and of 112 features, shares of 128 features, and more than an SM's 128.
