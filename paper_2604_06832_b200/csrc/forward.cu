@@ -364,11 +364,11 @@ static int forward_rows_tc(fdvlm_t* h, int n, int mode, int logits_rows, int wan
     at.dtype = h->dt; at.workspace = h->ws; at.kv_type = h->kv_type; at.out_fmt = h->xfmt; at.out_lo_off = h->ao_lo;
     at.status = h->info + 3;
     // Memory idles from here to the gate / up projection: part of its weights is brought into L2 meanwhile (NextWeights, every third pair).
-    // Not with fp8 weights from 41 rows on, where gate / up is bound by its MMAs (three planes) and not by its weights.
-    // us a step without : with, 3B shape, 12 layers: 4 rows 687 : 672, 32 rows 758 : 737, 64 rows 866 : 841.  7B shape, 8 layers, fp8: 8 rows
-    // 610 : 596, 33 rows 708 : 699, 36 rows 719 : 710, 40 rows 729 : 731, 41 rows 760 : 776, 48 rows 784 : 790, 64 rows 877 : 891;
-    // W8A8 (one plane): 8 rows 656 : 634, 32 rows 721 : 697, 41 rows 732 : 723, 48 rows 741 : 730, 56 rows 782 : 771, 64 rows 805 : 799.
-    if (h->dt == DT_BF16 || a8 || n <= 40) {
+    // Not with fp8 weights from 33 rows on, where gate / up is bound by its MMAs (three planes) and not by its weights.
+    // us a step without : with, a process each: 3B shape, 12 layers: 4 rows 687 : 672, 32 rows 762 : 739, 64 rows 862 : 842.  7B shape, 8 layers,
+    // fp8: 8 rows 608 : 597, 32 rows 658 : 647, 33 rows 682 : 685, 36 rows 686 : 691, 40 rows 697 : 705, 64 rows 855 : 867;
+    // W8A8 (one plane): 8 rows 652 : 633, 32 rows 721 : 697, 33 rows 719 : 706, 41 rows 724 : 718, 48 rows 725 : 722, 64 rows 804 : 798.
+    if (h->dt == DT_BF16 || a8 || n <= 32) {
       at.next_w[0] = lw.w_gate; at.next_w[1] = lw.w_up; at.next_n = I; at.next_k = H; at.next_fp8 = h->dt == DT_FP8;
     }
     at.amax_out = a8 ? h->amax_ao : nullptr;

@@ -249,8 +249,8 @@ struct GuPlan { int kind, f, mp, planes, kblocks, stages; size_t smem; };
 static bool gu_plan(const TcGroup& g, GuPlan* pl) {
   pl->kind = g.a8 ? GU_A8 : (g.fp8 ? GU_FP8 : GU_BF16);
   // fp8 weights, 41 to 48 rows: more than 128 lanes take a second MMA, which eats up what the shares gain, while the 64-feature tiles still
-  // have three stages (two from 49 rows on).  us a step, shares : tiles, 8 layers of the 7B shape: 40 rows 729 : 749, 41 rows 760 : 760,
-  // 44 rows 771 : 766, 48 rows 784 : 789 (no difference; two runs differ by 8), 49 rows 831 : 878, 56 rows 841 : 903, 64 rows 877 : 911.
+  // have three stages (two from 49 rows on).  us a step, shares : tiles, 8 layers of the 7B shape: 32 rows 658 : 658, 33 rows 682 : 694, 40 rows
+  // 697 : 719, 41 rows 740 : 722, 44 rows 750 : 727, 48 rows 767 : 742, 49 rows 815 : 830, 56 rows 805 : 830, 64 rows 855 : 866.
   // Everywhere else the shares are as fast or faster: 12 layers of the 3B shape, 4, 16, 32, 64 rows: 679, 696, 731, 835 : 683, 707, 763, 923.
   if (pl->kind == GU_FP8 && g.m > 40 && g.m <= 48) return false;
   // A few MB of weights and few rows: everything is latency, and the smaller CTAs of the tiles start sooner.  us a step, shares : tiles: 12 layers of
@@ -302,12 +302,11 @@ cudaError_t gemm_gu_launch(const TcGroup& g, const TcOut& o, const void* next, i
     return cudaErrorInvalidValue;
   for (int i = 0; i < 2; ++i)
     if (!make_tmap(&p.tm_w[i], g.w[i], inter, g.k, p.f, xkind)) return cudaErrorInvalidValue;
-  // Part of the next launch's weights (NextWeights, every third pair).  us a step without : with, 3B shape, 12 layers: 4 and 8 rows the
-  // same, 16 rows 699 : 706, 24 rows 721 : 719, 32 rows 737 : 732, 33 rows 757 : 751, 48 rows 782 : 778, 64 rows 840 : 836.  7B shape, 8 layers, fp8:
-  // 8 rows 596 : 591, 16 rows 613 : 604, 24 rows 653 : 653, 32 rows 670 : 669, 33 rows 704 : 711, 64 rows 877 : 904; W8A8: up to 32 rows the same,
-  // 40 rows 720 : 731, 48 rows 730 : 741.  So bf16 weights from 17 rows on, fp8 weights up to 32, W8A8 never.
-  const bool ask = pl.kind == GU_BF16 ? g.m > 16 : pl.kind == GU_FP8 && g.m <= 32;
-  if (next && ask && !next_weights(&p.next, next, nullptr, next_n, next_k, g.fp8, 3)) return cudaErrorInvalidValue;
+  // Part of the next launch's weights (NextWeights, every third pair), up to 32 rows.  us a step without : with, a process each: 3B shape, 12
+  // layers: 4 rows 672 : 672, 16 rows 706 : 701, 24 rows 723 : 717, 32 rows 739 : 734, 33 rows 754 : 754, 48 rows 782 : 780, 64 rows 842 : 839
+  // (7B shape in bf16, 6 layers, 48 rows 865 : 873).  7B shape, 8 layers, fp8: 4 rows 597 : 588, 16 rows 610 : 600, 32 rows 648 : 644, 33 rows
+  // 684 : 686, 40 rows 705 : 707; W8A8: 8 rows 633 : 625, 16 rows 646 : 645, 32 rows 697 : 696, 33 rows 706 : 709, 48 rows 722 : 730.
+  if (next && g.m <= 32 && !next_weights(&p.next, next, nullptr, next_n, next_k, g.fp8, 3)) return cudaErrorInvalidValue;
   const int grid = ceil_div(inter, p.f);
   return pl.kind == GU_A8 ? gu_launch_t<GU_A8>(p, grid, pl.smem, st)
                           : (pl.kind == GU_FP8 ? gu_launch_t<GU_FP8>(p, grid, pl.smem, st) : gu_launch_t<GU_BF16>(p, grid, pl.smem, st));
