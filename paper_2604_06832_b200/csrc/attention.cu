@@ -62,7 +62,6 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
   auto p_full = [&](int w) { return bar0 + 96u + 8u * w; };
   auto o_full = [&](int w) { return bar0 + 112u + 8u * w; };     // the last P V of a warpgroup's steps is complete
   const uint32_t mma_done = bar0 + 136u;                         // every MMA is complete (after an abort)
-  volatile uint32_t* armed_slot = (volatile uint32_t*)(sm + S::BAR_OFF + 144);      // stages armed, parity of the last time << 16
   volatile uint32_t* tmem_slot = (volatile uint32_t*)(sm + S::BAR_OFF + 128);
   volatile int* abort_flag = (volatile int*)(sm + S::BAR_OFF + 132);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -133,7 +132,12 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
       }
       if (!waited) pdl_wait();
       if (!ok && p.status) atomicCAS(p.status, 0, ST_ATTENTION);
-      *armed_slot = armed | (parity << 16);
+      if (*abort_flag)      // (see linger)
+        for (int s = 0; s < S::STAGES; ++s)
+          if (armed & (1u << s)) {
+            mbar_drain(k_full(s), (parity >> s) & 1u);
+            mbar_drain(v_full(s), (parity >> s) & 1u);
+          }
     }
   } else if (warp == 1) {
     constexpr bool F16 = !__is_same(E, bf16);
@@ -179,6 +183,11 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
         score(1, t + 1);
       }
       if (!ok && p.status) atomicCAS(p.status, 0, ST_ATTENTION);
+      if (*abort_flag) {
+        umma_commit(mma_done);
+        mbar_drain(mma_done, 0);
+        linger();
+      }
     }
     __syncwarp();
   } else if (warp >= 4) {
@@ -306,8 +315,9 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
         for (int i = 0; i < 4; ++i)
           if (out_row[i] >= 0) *reinterpret_cast<float4*>(p.part_o + (size_t)out_row[i] * D + c + lc) = o[i];
       }
-    } else if (lane == 0 && p.status) {
-      atomicCAS(p.status, 0, ST_ATTENTION);
+    } else {
+      if (lane == 0 && p.status) atomicCAS(p.status, 0, ST_ATTENTION);
+      linger();
     }
   } else {
     if (warp == 2 && lane == 0) ask_for_next(p.next, cta, ctas);
@@ -315,20 +325,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
   }
   __syncwarp();
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();     // the producer's copies have all been consumed
-  if (*abort_flag) {
-    // ... unless somebody gave up: then others may not have waited for what is in flight (a producer whose tiles all fit into the ring does not
-    // even hear of it), and the last copies into each stage and the last MMAs end before any thread leaves.
-    if (tid == 0)
-      for (int s = 0; s < S::STAGES; ++s)
-        if (*armed_slot & (1u << s)) {
-          mbar_drain(k_full(s), (*armed_slot >> (16 + s)) & 1u);
-          mbar_drain(v_full(s), (*armed_slot >> (16 + s)) & 1u);
-        }
-    __syncwarp();
-    if (warp == 1 && elect_one()) { umma_commit(mma_done); mbar_drain(mma_done, 0); }
-    __syncthreads();
-  }
+  __syncthreads();     // nothing is in flight any more (see linger)
   if (warp == 1) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");

@@ -36,7 +36,7 @@ __global__ void __launch_bounds__(GU_THREADS, 2) gemm_gu_kernel(const __grid_con
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t bars[3 * GU_STAGES + 2];
   __shared__ uint32_t tmem_slot_s;
-  __shared__ int abort_s, issued_s[2], amax_s[64];
+  __shared__ int abort_s, amax_s[64];
   __shared__ float rs[64], sc[2][128];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   const uint32_t bar0 = smem_u32(bars);
@@ -52,7 +52,7 @@ __global__ void __launch_bounds__(GU_THREADS, 2) gemm_gu_kernel(const __grid_con
     for (int s = 0; s < p.stages; ++s) { mbar_init(wfull(s), 1); mbar_init(xfull(s), 1); mbar_init(empty(s), 1); }
     mbar_init(tfull, 1); mbar_init(mma_done, 1);
     stamp_start(p.stamp);
-    abort_s = issued_s[0] = issued_s[1] = 0;
+    abort_s = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
@@ -105,7 +105,9 @@ __global__ void __launch_bounds__(GU_THREADS, 2) gemm_gu_kernel(const __grid_con
         pdl_wait();
       }
       if (!ok) atomicCAS(p.status, 0, ST_PRODUCER);
-      issued_s[weights ? 0 : 1] = issued;
+      if (*abort_flag)      // (see linger) the last copies into each stage
+        for (int i = max(0, issued - p.stages); i < issued; ++i)
+          mbar_drain(weights ? wfull(i % p.stages) : xfull(i % p.stages), (uint32_t)(i / p.stages) & 1u);
     }
     __syncwarp();
   } else if (warp == 1) {
@@ -136,6 +138,11 @@ __global__ void __launch_bounds__(GU_THREADS, 2) gemm_gu_kernel(const __grid_con
       }
       if (ok) umma_commit(tfull);
       else atomicCAS(p.status, 0, ST_MMA);
+      if (*abort_flag) {
+        umma_commit(mma_done);
+        mbar_drain(mma_done, 0);
+        linger();
+      }
     }
     __syncwarp();
   } else {
@@ -213,22 +220,15 @@ __global__ void __launch_bounds__(GU_THREADS, 2) gemm_gu_kernel(const __grid_con
       asm volatile("bar.sync 1, %0;" ::"n"(GU_EPI) : "memory");
       if (ok && t < p.m && amax_s[t] > 0) atomicMax(reinterpret_cast<int*>(p.amax_out) + t, amax_s[t]);
     }
-    if (!ok && lane == 0) atomicCAS(p.status, 0, ST_EPILOGUE);
+    if (!ok) {
+      if (lane == 0) atomicCAS(p.status, 0, ST_EPILOGUE);
+      linger();
+    }
   }
 
   // ---- teardown: every thread arrives here, whatever happened ----
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
-  if (*abort_flag) {
-    // Somebody gave up, so others may not have waited for what is in flight (a producer whose k-blocks all fit into the ring does not even
-    // hear of it): the last copies into each stage and the last MMAs end before the shared and tensor memory they use is left.
-    if (threadIdx.x < 2)
-      for (int n = issued_s[threadIdx.x], i = max(0, n - p.stages); i < n; ++i)
-        mbar_drain(threadIdx.x == 0 ? wfull(i % p.stages) : xfull(i % p.stages), (uint32_t)(i / p.stages) & 1u);
-    __syncwarp();
-    if (warp == 1 && elect_one()) { umma_commit(mma_done); mbar_drain(mma_done, 0); }
-    __syncthreads();
-  }
   if (warp == 1) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(p.tmem_cols) : "memory");

@@ -117,7 +117,6 @@ __global__ void __launch_bounds__(TC_THREADS) gemm_tc_kernel(const __grid_consta
   auto exw_bar = [&](int pr) { return bar0 + 8u * (2 * TC_STAGES + 6 + pr); };
   auto exr_bar = [&](int pr) { return bar0 + 8u * (2 * TC_STAGES + 8 + pr); };
   const uint32_t done_bar = bar0 + 8u * (2 * TC_STAGES + 10);      // every MMA of the CTA is complete (after an abort)
-  volatile uint32_t* armed_slot = (volatile uint32_t*)(sm + L::BAR_OFF + 8 * (2 * TC_STAGES + 11));      // stages armed, parity of the last time << 16
   volatile uint32_t* tmem_slot = (volatile uint32_t*)(sm + L::BAR_OFF + 8 * (2 * TC_STAGES + 4));
   volatile int* abort_flag = (volatile int*)(sm + L::BAR_OFF + 8 * (2 * TC_STAGES + 4) + 8);
 
@@ -221,7 +220,9 @@ __global__ void __launch_bounds__(TC_THREADS) gemm_tc_kernel(const __grid_consta
         for (int j = 0; j < n_pend; ++j) load_x(pend_stage[j], pend_kb[j]);
       }
       if (!ok) atomicCAS(p.status, 0, TC_ERR_PRODUCER);
-      *armed_slot = armed | (armed_parity << 16);
+      if (*abort_flag)      // (see linger)
+        for (int s = 0; s < TC_STAGES; ++s)
+          if (armed & (1u << s)) mbar_drain(full_bar(s), (armed_parity >> s) & 1u);
     }
   } else if (warp == 1) {
     // ------------------------------------------------ MMA issuer --------------------------------------------------
@@ -263,6 +264,13 @@ __global__ void __launch_bounds__(TC_THREADS) gemm_tc_kernel(const __grid_consta
         if (elect_one() && ok) umma_commit(tfull_bar(acc));
       }
       if (!ok) atomicCAS(p.status, 0, TC_ERR_MMA);
+      if (__any_sync(0xffffffffu, *abort_flag != 0)) {
+        if (elect_one()) {
+          umma_commit(done_bar);
+          mbar_drain(done_bar, 0);
+        }
+        linger();
+      }
     }
   } else {
     // ------------------------------------------------ epilogue warps ----------------------------------------------
@@ -432,22 +440,15 @@ __global__ void __launch_bounds__(TC_THREADS) gemm_tc_kernel(const __grid_consta
         }
       }
     }
-    if (!ok) atomicCAS(p.status, 0, TC_ERR_EPILOGUE);
+    if (!ok) {
+      atomicCAS(p.status, 0, TC_ERR_EPILOGUE);
+      linger();
+    }
   }
 
   // ---- teardown: every thread arrives here, whatever happened ----
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
-  if (*abort_flag) {
-    // Somebody gave up, so others may not have waited for what is in flight (a producer whose k-blocks all fit into the ring does not even
-    // hear of it): the last copies into each stage and the last MMAs end before the shared and tensor memory they use is left.
-    if (threadIdx.x == 0)
-      for (int s = 0; s < TC_STAGES; ++s)
-        if (*armed_slot & (1u << s)) mbar_drain(full_bar(s), (*armed_slot >> (16 + s)) & 1u);
-    __syncwarp();
-    if (warp == 1 && elect_one()) { umma_commit(done_bar); mbar_drain(done_bar, 0); }
-    __syncthreads();
-  }
   if (warp == 1) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS) : "memory");

@@ -62,6 +62,15 @@ __device__ __forceinline__ void mbar_drain(uint32_t bar, uint32_t parity) {
   const long long t0 = clock64();
   while (!mbar_try_wait(bar, parity) && clock64() - t0 < TC_TIMEOUT) {}
 }
+// No CTA leaves with a copy or an MMA in flight, whoever gives up.  A producer or MMA thread that finds the abort flag raised when its loop has
+// ended (no wait of its own may have failed: where all k-blocks fit into the ring a producer waits for nothing) drains what it issued.  Where
+// the flag is raised later, all of that has been issued before: whoever gives up lingers for a time (0.5 ms) that copies and MMAs need many
+// times over, before it comes to the CTA's last barrier.  (Waiting in every CTA, or reading the flag behind the last barrier, where the code is
+// fetched in vain, cost 0.2 to 1 % of a decode step.)
+__device__ __forceinline__ void linger() {
+  const long long t0 = clock64();
+  while (clock64() - t0 < (1ll << 20)) {}
+}
 // The host-set test hook (status[1]; written by the host only, never by a kernel of the chain, so it may be read before the wait for
 // the predecessor).  1: the abort flag is raised, which every other role's first wait sees, and the producer is to issue nothing
 // (returns false): all leave by the path a timed-out wait takes.  2: the flag is raised, the others are given the time to see it, and
