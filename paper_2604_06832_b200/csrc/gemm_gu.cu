@@ -5,9 +5,9 @@
 // steps of 8 features where the MMA's M goes in steps of 128: 11008 features are 138 equal CTAs instead of 172 tiles
 // on 148 SMs.  The rows (all planes of them: bf16 hi + lo, or three e5m2 planes) are the MMA's M; they come from L2 once
 // per SM, all planes in one box.  All shared memory is one ring: 7 stages of 28 KB at 32 rows of bf16 (with 4 the launch takes 3 us longer).
-// What bounds it is memory: 90 MB of the 3B shape's gate and up at 32 rows take 12.3 us behind the predecessor, 20 MB having come before
-// its end; the rest is 2 us of epilogue and 0.9 us of hand-over.  A layer's gate / up and down launches together: 26.9 -> 25.3 us at 32
-// rows, 34.4 -> 28.4 at 64 (7B fp8, 64 rows: 48.6 -> 45.1).
+// What bounds it is memory: of the 90 MB of the 3B shape's gate and up at 32 rows 34 MB lie in L2 (brought by the attention) and 20 MB in the
+// rings when its predecessor ends; 14 us from there, 0.9 of them the hand-over, 2 the epilogue.  A layer's gate / up and down launches together,
+// with 64-feature tiles : now: 26.9 : 23.0 us at 32 rows, 34.3 : 26.2 at 64 (7B fp8, 64 rows 48.8 : 45.9).
 // Every mbarrier wait is bounded (see gemm_tc.cu).
 #include "kernels.h"
 #include "tc_ptx.cuh"
